@@ -14,15 +14,13 @@
 // each chunk (Re chunks then Im chunks), padded to 16. A frame whose widths
 // are all zero has length 0 (the all-zero run elision).
 //
-// Encoding is single-pass: each CTA encodes one frame, takes a ticket so that
-// frames are processed in order, and finds its byte offset inside the block's
-// stream with a decoupled look-back over the preceding frames' sizes. Every
-// spin-wait is bounded and reports QSIM_E_TIMEOUT instead of hanging.
+// A frame is coded by a team of threads, one per chunk pair (codec_team.cuh).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "codec.cuh"
 #include "codec_dev.cuh"
+#include "codec_team.cuh"
 #include "device_common.cuh"
 #include "gates.cuh"
 
@@ -32,299 +30,319 @@ namespace {
 
 using namespace cdev;
 
-// NP: the most leading phase ops the kernel applies (pre.count <= NP).
+// One frame per team of max(32, C) threads, which is the CTA. Blocks are read from table[ids[j]] (ids null: block
+// b0 + j). NP: the most leading phase ops the kernel applies (pre.count <= NP). Five CTAs of 128 threads per SM: 102
+// registers hold a chunk pair's 64 bit-plane words (the wide path) without spills, and 35 KB of tile each fit six.
 template <int NP, bool REL>
-__global__ void __launch_bounds__(NT, 3) k_decode(const BlockRef *__restrict__ in, const BlockSlot *__restrict__ table,
-                                               const uint32_t *__restrict__ ids, uint32_t nblocks, int m,
-                                               float2 *__restrict__ wv, uint32_t *__restrict__ hist,
-                                               int *status, PreOps pre) {
+__global__ void __launch_bounds__(kTeamMax, 5) k_decode(const BlockSlot *__restrict__ table,
+                                                        const uint32_t *__restrict__ ids, uint64_t b0,
+                                                        uint32_t nblocks, int m, float2 *__restrict__ wv,
+                                                        uint32_t *__restrict__ hist, int *status, PreOps pre) {
+    extern __shared__ __align__(16) uint8_t tile[];
     const FrameGeom g = geom(m);
     __shared__ OpDev s_pre[NP > 0 ? NP : 1];
     __shared__ uint2 s_pre_ab[NP > 0 ? NP : 1];
-    __shared__ uint32_t s_hist[NW][32];
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
     if (NP > 0 && threadIdx.x < pre.count) {
         s_pre[threadIdx.x] = pre.ops[threadIdx.x];
         s_pre_ab[threadIdx.x] = pre_setup(pre.ops[threadIdx.x]);
     }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5;
+    if (NP > 0) __syncthreads();
     const uint64_t items = uint64_t(nblocks) * g.nframes;
-    for (uint64_t item = uint64_t(blockIdx.x) * NW + warp; item < items; item += uint64_t(gridDim.x) * NW) {
+    for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
-        const uint8_t *sp;
-        uint64_t bytes;
-        if (table) {
-            const BlockSlot sl = table[ids[j]];
-            sp = sl.ptr;
-            bytes = sl.bytes;
-        } else {
-            sp = in[j].ptr;
-            bytes = in[j].bytes;
-        }
-        decode_frame_warp<NP, false, REL>(sp, bytes, g, m, f, wv + (uint64_t(j) << m) + uint64_t(f) * g.F,
-                                         hist ? hist + uint64_t(j) * 32 : nullptr, s_hist[warp], status, s_pre,
-                                         s_pre_ab, pre.count, pre.mats, pre.count ? (uint64_t(j % pre.G) << m) : 0,
-                                         pre.count ? pre.gbase[j / pre.G] : 0);
+        const BlockSlot sl = table[ids ? ids[j] : b0 + j];
+        decode_frame_team<NP, REL>(tm, S, tile, sl.ptr, sl.bytes, g, m, f, wv + (uint64_t(j) << m) + uint64_t(f) * g.F,
+                                   hist ? hist + uint64_t(j) * 32 : nullptr, status, s_pre, s_pre_ab, pre.count,
+                                   pre.mats, pre.count ? (uint64_t(j % pre.G) << m) : 0,
+                                   pre.count ? pre.gbase[j / pre.G] : 0);
+        tm.sync();
     }
 }
 
-// Random access: frame frames[i].y of block frames[i].x (slot table entry) decoded into out + i * F, one warp per
-// frame; no leading phase ops, no histogram.
-template <bool REL>
-__global__ void __launch_bounds__(NT, 3) k_decode_frames(const BlockSlot *__restrict__ table,
-                                                      const uint2 *__restrict__ frames, uint32_t nitems, int m,
-                                                      float2 *__restrict__ out, int *status) {
+// One block given by pointer, its format (QSZ1 or QSZR) read from the stream's magic number.
+__global__ void __launch_bounds__(kTeamMax, 5) k_decode_block(BlockRef in, int m, float2 *__restrict__ out,
+                                                              CallResult res) {
+    extern __shared__ __align__(16) uint8_t tile[];
     const FrameGeom g = geom(m);
-    __shared__ uint32_t s_hist[NW][32];
-    const int warp = threadIdx.x >> 5;
-    for (uint64_t item = uint64_t(blockIdx.x) * NW + warp; item < nitems; item += uint64_t(gridDim.x) * NW) {
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
+    const uint32_t f = blockIdx.x;
+    float2 *dst = out + uint64_t(f) * g.F;
+    const bool rel = in.bytes >= g.data_start && !(reinterpret_cast<uintptr_t>(in.ptr) & 15) &&
+                     __ldg(reinterpret_cast<const uint32_t *>(in.ptr)) == kQszrMagic;
+    if (rel)
+        decode_frame_team<0, true>(tm, S, tile, in.ptr, in.bytes, g, m, f, dst, nullptr, res.status, nullptr, nullptr,
+                                   0, nullptr, 0, 0);
+    else
+        decode_frame_team<0, false>(tm, S, tile, in.ptr, in.bytes, g, m, f, dst, nullptr, res.status, nullptr, nullptr,
+                                    0, nullptr, 0, 0);
+    call_done(res, tm, gridDim.x);
+}
+
+// Random access: frame frames[i].y of block frames[i].x (slot table entry) decoded into out + i * F; no leading phase
+// ops, no histogram.
+template <bool REL>
+__global__ void __launch_bounds__(kTeamMax, 5) k_decode_frames(const BlockSlot *__restrict__ table,
+                                                               const uint2 *__restrict__ frames, uint32_t nitems,
+                                                               int m, float2 *__restrict__ out, int *status) {
+    extern __shared__ __align__(16) uint8_t tile[];
+    const FrameGeom g = geom(m);
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
+    for (uint64_t item = blockIdx.x; item < nitems; item += gridDim.x) {
         const uint2 bf = frames[item];
         const BlockSlot sl = table[bf.x];
-        decode_frame_warp<0, false, REL>(sl.ptr, sl.bytes, g, m, bf.y, out + item * g.F, nullptr, s_hist[warp],
-                                         status, nullptr, nullptr, 0, nullptr, 0, 0);
+        decode_frame_team<0, REL>(tm, S, tile, sl.ptr, sl.bytes, g, m, bf.y, out + item * g.F, nullptr, status, nullptr,
+                                  nullptr, 0, nullptr, 0, 0);
+        tm.sync();
     }
 }
 
-__global__ void __launch_bounds__(NT) k_encode(const float2 *__restrict__ wv, uint32_t nblocks, int m, int e,
-                                               const EncTarget *__restrict__ tgt, EncResult *__restrict__ res,
-                                               int only_overflowed, const uint32_t *__restrict__ ids,
-                                               BlockSlot *__restrict__ table, StageAccum *acc,
-                                               LookbackScratch scr, int *status) {
+// Encoder of a batch of blocks, one frame per team of max(32, C) threads (the CTA). A frame is read once, coded in
+// shared memory and
+//  - blocks of one frame (m <= 12): written to its slot, reserved here, header included; nothing is left to copy;
+//  - larger blocks: its bit-plane words go over the frame's own amplitudes (they never need more room) and the part
+//    of its image before them to the frame's side record; the CTA that finishes a block's last frame turns the frame
+//    lengths into offsets and reserves the block's slot, while other blocks are still being coded. k_frame_copy then
+//    moves the images. (The exact slot needs the size of the whole block, so its frames cannot go there directly.)
+// arrive: one counter per block, zero before and after. keep_fitting (learned sizing): a block keeps the slot reserved
+// for it beforehand when its exact size fits, and only a block whose prediction was too small gets an exact slot
+// (counted as an overflowed block).
+template <bool REL>
+__global__ void __launch_bounds__(kTeamMax, 5) k_encode(float2 *wv, uint32_t nblocks, int m, int e, ArenaDev dev,
+                                                        ArenaDev host, EncTarget *__restrict__ tgt,
+                                                        EncResult *__restrict__ res,
+                                                        const uint32_t *__restrict__ ids,
+                                                        BlockSlot *__restrict__ table, StageAccum *acc,
+                                                        FrameRecords fr, unsigned long long *arrive, int keep_fitting,
+                                                        int *status) {
+    extern __shared__ __align__(16) uint8_t tile[];
     const FrameGeom g = geom(m);
-    __shared__ __align__(16) uint32_t s_stage[kStageWords];
-    __shared__ EncSmem SE;
-    __shared__ uint32_t s_item, s_epoch;
-    __shared__ int s_skip;
-    __shared__ bool s_last;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
+    const uint64_t items = uint64_t(nblocks) * g.nframes;
+    for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+        const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
+        float2 *frame = wv + (uint64_t(j) << m) + uint64_t(f) * g.F;
+        load_rows_team(tm, tile, frame, g.C);
+        const EncFrame r = encode_frame_team<REL>(tm, S, tile, g, e, status);
+        uint32_t total = uint32_t(g.data_start) + r.len;
+        double err = r.err_sq, nrm = r.norm_sq;
+        bool last = true;
+        if (g.nframes > 1) {
+            if (r.len) {
+                uint4 *pay = reinterpret_cast<uint4 *>(frame), *side = reinterpret_cast<uint4 *>(fr.side + item * fr.side_bytes);
+                const uint4 *img = reinterpret_cast<const uint4 *>(tile);
+                const uint32_t h = r.head / 16u, n = r.len / 16u;
+                for (uint32_t i = tm.t; i < n; i += tm.n) {
+                    if (i < h) side[i] = img[i];
+                    else pay[i - h] = img[i];
+                }
+            }
+            if (tm.t == 0) {
+                fr.len[item] = r.len;
+                if (REL) fr.head[item] = r.head;
+                fr.part[item] = make_float2(r.err_sq, r.norm_sq);
+                __threadfence();  // the frame's records before its arrival: the block's last CTA reads them all
+                S.flag = atomicAdd(arrive + j, 1ull) == g.nframes - 1;
+            }
+            tm.sync();
+            last = S.flag != 0;
+            if (last) {
+                __threadfence();
+                const uint64_t b = uint64_t(j) * g.nframes;
+                total = block_offsets_team(tm, S, fr.len + b, fr.part + b, fr.off + b, g.nframes,
+                                           uint32_t(g.data_start), err, nrm);
+            }
+        }
+        if (last && tm.t == 0) {
+            EncTarget t{};
+            if (keep_fitting) t = tgt[j];
+            if (!keep_fitting || t.ptr == nullptr || total > t.cap) {
+                if (keep_fitting && acc) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+                reserve_slot(total, dev, host, &t, status);
+                tgt[j] = t;
+            }
+            EncResult out{};
+            out.err_sq = err;
+            out.norm_sq = nrm;
+            const bool fits = t.ptr != nullptr && total <= t.cap;  // false after a failed reservation only
+            if (g.nframes == 1) {
+                out.total = total;
+                out.overflow = fits ? 0u : 1u;
+                if (fits) {
+                    BlockSlot *sl = table + (ids ? ids[j] : j);
+                    sl->ptr = t.ptr;
+                    sl->bytes = total;
+                    sl->tier = t.tier;
+                }
+                S.bc = fits ? reinterpret_cast<uint64_t>(t.ptr) : 0ull;
+            } else {
+                arrive[j] = 0;
+            }
+            res[j] = out;
+            if (acc) {
+                atomicAdd(&acc->err_sq, err);
+                atomicAdd(&acc->norm_sq, nrm);
+                if (g.nframes == 1) {
+                    if (fits) count_block(acc, total, t);
+                    else atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+                }
+            }
+        }
+        tm.sync();
+        if (g.nframes == 1) {
+            uint8_t *out = reinterpret_cast<uint8_t *>(S.bc);
+            if (out) {
+                for (uint32_t i = tm.t; i < uint32_t(g.data_start) / 4u; i += tm.n)
+                    reinterpret_cast<uint32_t *>(out)[i] = header_word(i, REL, g, m, e, 0, r.len);
+                uint4 *d = reinterpret_cast<uint4 *>(out + g.data_start);
+                for (uint32_t i = tm.t; i < r.len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
+            }
+            tm.sync();
+        }
+    }
+}
 
-    if (tid == 0) {
-        s_item = atomicAdd(scr.ticket, 1u);
-        s_epoch = ld_relaxed_u32(scr.epoch) & kEpochMask;
-    }
-    __syncthreads();
-    const uint32_t item = s_item, epoch = s_epoch;
-    const uint32_t j = item / g.nframes, f = item % g.nframes;
-    if (tid == 0) s_skip = (j >= nblocks) || (only_overflowed && res[j].overflow == 0);
-    __syncthreads();
-    if (!s_skip)
-        encode_frame_cta(wv + (uint64_t(j) << m) + uint64_t(f) * g.F, g, m, e, f, scr.state + uint64_t(j) * g.nframes,
-                         epoch, tgt[j], res + j, table ? table + ids[j] : nullptr, acc,
-                         scr.part ? scr.part + item : nullptr, only_overflowed, s_stage, SE, status);
-    // ---- last CTA: reduce the frame partials, reset the ticket counter, advance the epoch ----
-    __syncthreads();  // the frame's writes by every thread of the CTA come before its arrival
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(scr.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (scr.part && !only_overflowed) {
-        // warp per block: sum its frames' partials in FP64
-        double ta = 0, tb = 0;
-        for (uint32_t jb = warp; jb < nblocks; jb += NW) {
-            double a = 0, b = 0;
-            for (uint32_t f2 = lane; f2 < g.nframes; f2 += 32) {
-                const float2 p = scr.part[uint64_t(jb) * g.nframes + f2];
-                a += double(p.x);
-                b += double(p.y);
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                a += __shfl_xor_sync(kFull, a, o);
-                b += __shfl_xor_sync(kFull, b, o);
-            }
-            if (lane == 0) {
-                res[jb].err_sq = a;
-                res[jb].norm_sq = b;
-            }
-            ta += a;
-            tb += b;
+// Second step of blocks of several frames (C = 128): frame f's image (side record, then the words over its amplitudes)
+// copied to its offset in the block's slot. The block's last frame writes the header, the table slot and the totals.
+template <bool REL>
+__global__ void __launch_bounds__(kTeamMax) k_frame_copy(const float2 *__restrict__ wv, uint32_t nblocks, int m, int e,
+                                                         const EncTarget *__restrict__ tgt,
+                                                         EncResult *__restrict__ res,
+                                                         const uint32_t *__restrict__ ids,
+                                                         BlockSlot *__restrict__ table, StageAccum *acc,
+                                                         FrameRecords fr) {
+    const FrameGeom g = geom(m);
+    const uint64_t items = uint64_t(nblocks) * g.nframes;
+    for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
+        const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
+        const uint32_t len = fr.len[item], off = fr.off[item], head = REL ? fr.head[item] : 256u;
+        const EncTarget t = tgt[j];
+        const bool fits = t.ptr != nullptr && uint64_t(off) + len <= t.cap;
+        if (fits && len) {
+            const uint4 *side = reinterpret_cast<const uint4 *>(fr.side + item * fr.side_bytes);
+            const uint4 *pay = reinterpret_cast<const uint4 *>(wv + (uint64_t(j) << m) + uint64_t(f) * g.F);
+            uint4 *d = reinterpret_cast<uint4 *>(t.ptr + off);
+            const uint32_t h = head / 16u, n = len / 16u;
+#pragma unroll 4
+            for (uint32_t i = threadIdx.x; i < n; i += kTeamMax) d[i] = i < h ? side[i] : pay[i - h];
         }
-        if (lane == 0) {
-            SE.red[0][warp] = ta;
-            SE.red[1][warp] = tb;
-        }
-        __syncthreads();
-        if (tid == 0 && acc) {
-            double a = 0, b = 0;
-            for (int w = 0; w < NW; ++w) { a += SE.red[0][w]; b += SE.red[1][w]; }
-            atomicAdd(&acc->err_sq, a);
-            atomicAdd(&acc->norm_sq, b);
+        if (threadIdx.x == 0) {
+            if (!fits) atomicOr(&res[j].overflow, 1u);
+            if (t.ptr && g.data_start <= t.cap) reinterpret_cast<uint32_t *>(t.ptr + 32)[f] = off;
+            if (f == g.nframes - 1) {
+                const uint64_t total = uint64_t(off) + len;
+                res[j].total = total;
+                if (t.ptr && total <= t.cap) {
+                    uint32_t *h32 = reinterpret_cast<uint32_t *>(t.ptr);
+                    for (uint32_t i = 0; i < 8; ++i) h32[i] = header_word(i, REL, g, m, e, f, uint32_t(total - g.data_start));
+                    for (uint32_t i = 8 + g.nframes; i < uint32_t(g.data_start) / 4u; ++i)
+                        h32[i] = i == 8 + g.nframes ? uint32_t(total) : 0u;
+                    BlockSlot *sl = table + (ids ? ids[j] : j);
+                    sl->ptr = t.ptr;
+                    sl->bytes = total;
+                    sl->tier = t.tier;
+                    if (acc) count_block(acc, total, t);
+                } else if (acc) {
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+                }
+            }
         }
     }
-    if (tid == 0) {
+}
+
+// One block into the caller's buffer in one pass: each CTA codes one frame, takes a ticket so that frames are
+// processed in order, and finds its byte offset with a decoupled look-back over the preceding frames' sizes. Every
+// spin-wait is bounded and reports QSIM_E_TIMEOUT instead of hanging. The record receives the stream's size (also when
+// it exceeds cap; the header is then not written) and the status.
+template <bool REL>
+__global__ void __launch_bounds__(kTeamMax, 5) k_encode_block(const float2 *__restrict__ amps, int m, int e,
+                                                              uint8_t *__restrict__ out, uint64_t cap,
+                                                              LookbackScratch scr, CallResult res) {
+    extern __shared__ __align__(16) uint8_t tile[];
+    const FrameGeom g = geom(m);
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
+    if (tm.t == 0) {
+        S.bc = atomicAdd(scr.ticket, 1u);
+        S.bc2 = ld_relaxed_u32(scr.epoch) & kEpochMask;
+    }
+    tm.sync();
+    const uint32_t f = uint32_t(S.bc), epoch = uint32_t(S.bc2);
+    load_rows_team(tm, tile, amps + uint64_t(f) * g.F, g.C);
+    const EncFrame r = encode_frame_team<REL>(tm, S, tile, g, e, res.status);
+    if (tm.t < 32) {
+        const uint32_t excl = lookback_warp(scr.state, f, epoch, r.len, res.status);
+        if (tm.t == 0) S.flag = excl;
+    }
+    tm.sync();
+    const uint64_t off = g.data_start + S.flag, total = off + r.len;
+    if (total <= cap) {
+        uint4 *d = reinterpret_cast<uint4 *>(out + off);
+        for (uint32_t i = tm.t; i < r.len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
+    }
+    if (tm.t == 0 && g.data_start <= cap) reinterpret_cast<uint32_t *>(out + 32)[f] = uint32_t(off);
+    if (f == g.nframes - 1) {
+        if (total <= cap) {
+            uint32_t *h32 = reinterpret_cast<uint32_t *>(out);
+            if (tm.t < 8) h32[tm.t] = header_word(tm.t, REL, g, m, e, f, uint32_t(total - g.data_start));
+            const uint32_t i = 8 + g.nframes + tm.t;
+            if (i < uint32_t(g.data_start) / 4u) h32[i] = tm.t ? 0u : uint32_t(total);
+        }
+        if (tm.t == 0) res.record->bytes = total;
+    }
+    if (call_done(res, tm, gridDim.x)) {
         *scr.ticket = 0;
-        *scr.done = 0;
-        __threadfence();
         atomicExch(scr.epoch, (epoch + 1) & kEpochMask);
     }
 }
 
-// Sizing pass (one CTA per frame) whose last CTA reserves every block's slot
-// from the summed frame lengths; sizes are left zeroed for the next use.
-__global__ void __launch_bounds__(NT, 3) k_encode_size(const float2 *__restrict__ wv, uint32_t nblocks, int m, int e,
-                                                    uint64_t *__restrict__ sizes, uint32_t *done_ctr,
-                                                    ArenaDev dev, ArenaDev host, EncTarget *__restrict__ tgt,
-                                                    EncResult *__restrict__ res, int *status) {
-    const FrameGeom g = geom(m);
-    __shared__ uint32_t s_words[NW];
-    __shared__ bool s_last;
-    const int tid = threadIdx.x;
-    const uint64_t items = uint64_t(nblocks) * g.nframes;
-    for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
-        const uint32_t len = size_frame_cta(wv + (uint64_t(j) << m) + uint64_t(f) * g.F, g, e, s_words, status);
-        if (tid == 0 && len) atomicAdd(reinterpret_cast<unsigned long long *>(&sizes[j]), uint64_t(len));
-    }
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(done_ctr, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (uint32_t j = tid; j < nblocks; j += NT) {
-        const uint64_t want = ld_relaxed_u64(&sizes[j]) + g.data_start;
-        sizes[j] = 0;
-        res[j].total = 0;
-        res[j].overflow = 0;
-        res[j].err_sq = 0;
-        res[j].norm_sq = 0;
-        reserve_slot(want, dev, host, &tgt[j], status);
-    }
-    if (tid == 0) *done_ctr = 0;
-}
-
-// In-place exact encoder, pass 1: one warp per frame encodes the frame over
-// its own amplitudes (Im-plane words to im, F words per frame) and records
-// its length and word counts; the last CTA turns the frame lengths into frame
-// offsets, reserves each block's exact slot and folds the frames' error
-// partials into the blocks' and the stage's totals.
-// REL: the relative-bound format (e is the shift k, side records of kQszrSideBytes, mixed sign words counted
-// in fmixed). Without a device arena (dev.bump null) the targets are the caller's and nothing is reserved; with
-// keep_fitting (learned sizing) a block keeps the slot reserved for it beforehand when its exact size fits, and
-// only a block whose prediction was too small gets an exact slot (counted as an overflowed block).
+// Initial store (Sec. 4.2): every block's stream written directly. All but block b0 are zero: a header and an offset
+// table. b0 holds the basis state's single amplitude 1 at local index loc: its one non-empty frame is coded here.
 template <bool REL>
-__global__ void __launch_bounds__(NT, 4) k_encode_ip(float2 *wv, uint32_t *__restrict__ im, uint32_t nblocks, int m,
-                                                  int e, uint32_t *done_ctr, ArenaDev dev, ArenaDev host,
-                                                  EncTarget *__restrict__ tgt, EncResult *__restrict__ res,
-                                                  StageAccum *acc, uint8_t *__restrict__ wrec,
-                                                  uint32_t *__restrict__ flen, uint32_t *__restrict__ fwords,
-                                                  uint32_t *__restrict__ fmixed, uint32_t *__restrict__ foff,
-                                                  float2 *__restrict__ part, int keep_fitting, int *status) {
+__global__ void __launch_bounds__(kTeamMax) k_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e,
+                                                         BlockSlot *__restrict__ table, ArenaDev dev, ArenaDev host,
+                                                         StageAccum *acc, int *status) {
+    extern __shared__ __align__(16) uint8_t tile[];
     const FrameGeom g = geom(m);
-    constexpr uint32_t kSide = REL ? kQszrSideBytes : 256u;
-    __shared__ bool s_last;
-    __shared__ double s_red[2][NW];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint64_t items = uint64_t(nblocks) * g.nframes;
-    for (uint64_t item = uint64_t(blockIdx.x) * NW + warp; item < items; item += uint64_t(gridDim.x) * NW) {
-        const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
-        uint32_t words, mixed;
-        const uint32_t len = encode_frame_warp_ip<REL>(wv + (uint64_t(j) << m) + uint64_t(f) * g.F, im + item * g.F,
-                                                       g, e, wrec + item * kSide, words, mixed, part + item, status);
-        if (lane == 0) {
-            flen[item] = len;
-            fwords[item] = words;
-            if (REL) fmixed[item] = mixed;
-            __threadfence();  // the frame's records (and its error partial) before the CTA's arrival below
+    __shared__ TeamSmem S;
+    const Team tm{threadIdx.x, blockDim.x, 1};
+    unsigned long long bytes = 0;  // thread 0
+    for (uint64_t b = blockIdx.x; b < nblocks; b += gridDim.x) {
+        uint32_t len = 0;
+        const uint32_t f0 = uint32_t(loc >> g.fl), at = uint32_t(loc) & (g.F - 1u);
+        if (b == b0) {
+            for (uint32_t i = tm.t; i < team_tile_bytes(g.C) / 16u; i += tm.n)
+                reinterpret_cast<uint4 *>(tile)[i] = make_uint4(0, 0, 0, 0);
+            tm.sync();
+            if (tm.t == 0) *reinterpret_cast<float *>(tile + kRowBytes * (at >> 5) + 8u * (at & 31u)) = 1.f;
+            tm.sync();
+            len = encode_frame_team<REL>(tm, S, tile, g, e, status).len;
         }
-    }
-    // every warp of the CTA has written its frames' records before the CTA counts as arrived: the last CTA
-    // reads all of them
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(done_ctr, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // warp per block: frame offsets = data_start + exclusive prefix of the frame lengths; exact slot;
-    // the block's error sums in FP64
-    double ta = 0, tb = 0;
-    for (uint32_t jb = warp; jb < nblocks; jb += NW) {
-        uint32_t run = uint32_t(g.data_start);
-        double a = 0, b = 0;
-        for (uint32_t f0 = 0; f0 < g.nframes; f0 += 32) {
-            const uint64_t it = uint64_t(jb) * g.nframes + f0 + lane;
-            const bool live = f0 + lane < g.nframes;
-            const uint32_t v = live ? __ldcg(flen + it) : 0u;
-            if (live) {
-                const float2 pp = __ldcg(part + it);
-                a += double(pp.x);
-                b += double(pp.y);
-            }
-            uint32_t incl = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (live) foff[it] = run + incl - v;
-            run += __shfl_sync(kFull, incl, 31);
+        if (tm.t == 0) {
+            const uint64_t total = g.data_start + len;
+            EncTarget t;
+            reserve_slot(total, dev, host, &t, status);
+            table[b].ptr = t.ptr;
+            table[b].bytes = total;
+            table[b].tier = t.tier;
+            S.bc = reinterpret_cast<uint64_t>(t.ptr);
+            bytes += total;
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            a += __shfl_xor_sync(kFull, a, o);
-            b += __shfl_xor_sync(kFull, b, o);
+        tm.sync();
+        uint8_t *out = reinterpret_cast<uint8_t *>(S.bc);
+        if (out) {
+            for (uint32_t i = tm.t; i < uint32_t(g.data_start) / 4u; i += tm.n)
+                reinterpret_cast<uint32_t *>(out)[i] = header_word(i, REL, g, m, e, f0, len);
+            uint4 *d = reinterpret_cast<uint4 *>(out + g.data_start);
+            for (uint32_t i = tm.t; i < len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
         }
-        if (lane == 0) {
-            res[jb].total = 0;
-            res[jb].overflow = 0;
-            res[jb].err_sq = a;
-            res[jb].norm_sq = b;
-            if (dev.bump) {
-                if (!keep_fitting) {
-                    reserve_slot(run, dev, host, &tgt[jb], status);
-                } else if (tgt[jb].ptr == nullptr || run > tgt[jb].cap) {
-                    if (acc) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
-                    reserve_slot(run, dev, host, &tgt[jb], status);
-                }
-            }
-        }
-        ta += a;
-        tb += b;
+        tm.sync();
     }
-    if (lane == 0) {
-        s_red[0][warp] = ta;
-        s_red[1][warp] = tb;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        if (acc) {
-            double a = 0, b = 0;
-            for (int w = 0; w < NW; ++w) { a += s_red[0][w]; b += s_red[1][w]; }
-            atomicAdd(&acc->err_sq, a);
-            atomicAdd(&acc->norm_sq, b);
-        }
-        *done_ctr = 0;
-    }
-}
-
-// In-place exact encoder, pass 2: one warp per frame copies the frame's
-// pieces to its offset in the block's slot.
-template <bool REL>
-__global__ void __launch_bounds__(NT) k_frame_copy(const float2 *__restrict__ wv, const uint32_t *__restrict__ im,
-                                                   uint32_t nblocks, int m, int e, const EncTarget *__restrict__ tgt,
-                                                   EncResult *__restrict__ res, const uint32_t *__restrict__ ids,
-                                                   BlockSlot *__restrict__ table, StageAccum *acc,
-                                                   const uint8_t *__restrict__ wrec, const uint32_t *__restrict__ flen,
-                                                   const uint32_t *__restrict__ fwords,
-                                                   const uint32_t *__restrict__ fmixed,
-                                                   const uint32_t *__restrict__ foff) {
-    const FrameGeom g = geom(m);
-    constexpr uint32_t kSide = REL ? kQszrSideBytes : 256u;
-    const int warp = threadIdx.x >> 5;
-    const uint64_t items = uint64_t(nblocks) * g.nframes;
-    for (uint64_t item = uint64_t(blockIdx.x) * NW + warp; item < items; item += uint64_t(gridDim.x) * NW) {
-        const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
-        copy_frame_warp<REL>(reinterpret_cast<const uint32_t *>(wv + (uint64_t(j) << m) + uint64_t(f) * g.F),
-                             im + item * g.F, wrec + item * kSide, fwords[item], REL ? fmixed[item] : 0u, flen[item],
-                             foff[item], g, m, e, f, tgt[j], res + j, table ? table + ids[j] : nullptr, acc);
-    }
+    if (tm.t == 0 && bytes) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->store_bytes), bytes);
 }
 
 // ---------------------------------------------------------------------------
@@ -399,13 +417,14 @@ __global__ void k_copy_blocks_in(const BlockRef *__restrict__ in, uint32_t nbloc
     }
 }
 
-// Gather the input block references of one group from the block table.
+// Gather block references from the block table (ids null: its first `count` entries).
 __global__ void k_gather_refs(const BlockSlot *__restrict__ table, const uint32_t *__restrict__ ids, uint32_t count,
                               BlockRef *__restrict__ out) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < count) {
-        out[j].ptr = table[ids[j]].ptr;
-        out[j].bytes = table[ids[j]].bytes;
+        const uint32_t b = ids ? ids[j] : j;
+        out[j].ptr = table[b].ptr;
+        out[j].bytes = table[b].bytes;
     }
 }
 
@@ -418,95 +437,114 @@ static unsigned grid_for(uint64_t items, unsigned cap) {
     return unsigned(items < cap ? (items ? items : 1) : cap);
 }
 
-void launch_decode(const BlockRef *in, uint32_t nblocks, int m, float2 *wv, uint32_t *hist, int *status,
-                   cudaStream_t s, bool rel) {
+// Team kernels: one CTA of team_threads(C) threads per frame, team_tile_bytes(C) of dynamic shared memory.
+struct TeamShape {
+    uint32_t threads;
+    size_t smem;
+};
+static TeamShape team_shape(int m) {
+    const uint32_t C = (1u << frame_log_for(m)) / 32u;
+    return {cdev::team_threads(C), cdev::team_tile_bytes(C)};
+}
+constexpr unsigned kMaxGrid = 1u << 30;
+
+template <bool REL>
+static void decode_table(const BlockSlot *table, const uint32_t *ids, uint64_t b0, uint32_t nblocks, int m, float2 *wv,
+                         uint32_t *hist, int *status, const PreOps &pre, cudaStream_t s) {
     const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    const unsigned grid = grid_for((items + NW - 1) / NW, 152 * 8);
-    if (rel)
-        k_decode<0, true><<<grid, NT, 0, s>>>(in, nullptr, nullptr, nblocks, m, wv, hist, status, PreOps{});
+    const TeamShape ts = team_shape(m);
+    // with leading phase ops each CTA copies their descriptors once and takes several frames
+    const unsigned grid = grid_for(items, pre.count ? 152 * 5 * 3 : kMaxGrid);
+    if (pre.count == 0)
+        k_decode<0, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
+    else if (pre.count <= 2)
+        k_decode<2, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
     else
-        k_decode<0, false><<<grid, NT, 0, s>>>(in, nullptr, nullptr, nblocks, m, wv, hist, status, PreOps{});
+        k_decode<kMaxPreOps, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
+}
+
+void launch_decode(const BlockSlot *table, uint64_t b0, uint32_t nblocks, int m, float2 *wv, int *status,
+                   cudaStream_t s, bool rel) {
+    if (rel)
+        decode_table<true>(table, nullptr, b0, nblocks, m, wv, nullptr, status, PreOps{}, s);
+    else
+        decode_table<false>(table, nullptr, b0, nblocks, m, wv, nullptr, status, PreOps{}, s);
     count_launch();
 }
 
-template <bool REL>
-static void decode_table(const BlockSlot *table, const uint32_t *ids, uint32_t nblocks, int m, float2 *wv,
-                         uint32_t *hist, int *status, const PreOps &pre, cudaStream_t s) {
-    const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    const unsigned grid = grid_for((items + NW - 1) / NW, 152 * 8);
-    if (pre.count == 0)
-        k_decode<0, REL><<<grid, NT, 0, s>>>(nullptr, table, ids, nblocks, m, wv, hist, status, pre);
-    else if (pre.count <= 2)
-        k_decode<2, REL><<<grid, NT, 0, s>>>(nullptr, table, ids, nblocks, m, wv, hist, status, pre);
-    else
-        k_decode<kMaxPreOps, REL><<<grid, NT, 0, s>>>(nullptr, table, ids, nblocks, m, wv, hist, status, pre);
+void launch_decode_block(const BlockRef &in, int m, float2 *out, const CallResult &res, cudaStream_t s) {
+    const TeamShape ts = team_shape(m);
+    k_decode_block<<<unsigned(qsz_nframes(m)), ts.threads, ts.smem, s>>>(in, m, out, res);
+    count_launch();
 }
 
 void launch_decode_frames(const BlockSlot *table, const uint2 *frames, uint32_t nitems, int m, float2 *out,
                           int *status, cudaStream_t s, bool rel) {
-    const unsigned grid = grid_for((uint64_t(nitems) + NW - 1) / NW, 152 * 8);
+    const TeamShape ts = team_shape(m);
+    const unsigned grid = grid_for(nitems, kMaxGrid);
     if (rel)
-        k_decode_frames<true><<<grid, NT, 0, s>>>(table, frames, nitems, m, out, status);
+        k_decode_frames<true><<<grid, ts.threads, ts.smem, s>>>(table, frames, nitems, m, out, status);
     else
-        k_decode_frames<false><<<grid, NT, 0, s>>>(table, frames, nitems, m, out, status);
+        k_decode_frames<false><<<grid, ts.threads, ts.smem, s>>>(table, frames, nitems, m, out, status);
     count_launch();
 }
 
 void launch_decode_table(const BlockSlot *table, const uint32_t *ids, uint32_t nblocks, int m, float2 *wv,
                          uint32_t *hist, int *status, const PreOps &pre, cudaStream_t s, bool rel) {
     if (rel)
-        decode_table<true>(table, ids, nblocks, m, wv, hist, status, pre, s);
+        decode_table<true>(table, ids, 0, nblocks, m, wv, hist, status, pre, s);
     else
-        decode_table<false>(table, ids, nblocks, m, wv, hist, status, pre, s);
+        decode_table<false>(table, ids, 0, nblocks, m, wv, hist, status, pre, s);
     count_launch();
 }
 
-void launch_encode(const float2 *wv, uint32_t nblocks, int m, int e, const EncTarget *tgt, EncResult *res,
-                   int only_overflowed, const uint32_t *ids, BlockSlot *table, StageAccum *acc,
-                   const LookbackScratch &scr, int *status, cudaStream_t s) {
-    const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    k_encode<<<unsigned(items), NT, 0, s>>>(wv, nblocks, m, e, tgt, res, only_overflowed, ids, table, acc, scr,
-                                             status);
-    count_launch();
-}
-
-
-void launch_size_reserve(const float2 *wv, uint32_t nblocks, int m, int e, uint64_t *sizes, uint32_t *done_ctr,
-                         const ArenaDev &dev, const ArenaDev &host, EncTarget *tgt, EncResult *res, int *status,
-                         cudaStream_t s) {
-    const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    k_encode_size<<<grid_for(items, 152 * 8), NT, 0, s>>>(wv, nblocks, m, e, sizes, done_ctr, dev, host, tgt, res,
-                                                           status);
-    count_launch();
-}
-
-
-void launch_encode_ip(float2 *wv, uint32_t *im, uint32_t nblocks, int m, int e, uint32_t *done_ctr,
-                      const ArenaDev &dev, const ArenaDev &host, EncTarget *tgt, EncResult *res, StageAccum *acc,
-                      uint8_t *wrec, uint32_t *flen, uint32_t *fwords, uint32_t *foff, float2 *part, int *status,
-                      cudaStream_t s, bool rel, uint32_t *fmixed, bool keep_fitting) {
-    const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    const unsigned grid = grid_for((items + NW - 1) / NW, 152 * 8);
+void launch_encode(float2 *wv, uint32_t nblocks, int m, int e, const ArenaDev &dev, const ArenaDev &host,
+                   EncTarget *tgt, EncResult *res, const uint32_t *ids, BlockSlot *table, StageAccum *acc,
+                   const FrameRecords &fr, uint64_t *arrive, int *status, cudaStream_t s, bool rel,
+                   bool keep_fitting) {
+    const unsigned grid = grid_for(uint64_t(nblocks) * qsz_nframes(m), kMaxGrid);
+    const TeamShape ts = team_shape(m);
+    unsigned long long *arr = reinterpret_cast<unsigned long long *>(arrive);
     if (rel)
-        k_encode_ip<true><<<grid, NT, 0, s>>>(wv, im, nblocks, m, e, done_ctr, dev, host, tgt, res, acc, wrec, flen,
-                                              fwords, fmixed, foff, part, keep_fitting ? 1 : 0, status);
+        k_encode<true><<<grid, ts.threads, ts.smem, s>>>(wv, nblocks, m, e, dev, host, tgt, res, ids, table, acc, fr,
+                                                         arr, keep_fitting ? 1 : 0, status);
     else
-        k_encode_ip<false><<<grid, NT, 0, s>>>(wv, im, nblocks, m, e, done_ctr, dev, host, tgt, res, acc, wrec, flen,
-                                               fwords, fmixed, foff, part, keep_fitting ? 1 : 0, status);
+        k_encode<false><<<grid, ts.threads, ts.smem, s>>>(wv, nblocks, m, e, dev, host, tgt, res, ids, table, acc, fr,
+                                                          arr, keep_fitting ? 1 : 0, status);
     count_launch();
 }
-void launch_frame_copy(const float2 *wv, const uint32_t *im, uint32_t nblocks, int m, int e, const EncTarget *tgt,
-                       EncResult *res, const uint32_t *ids, BlockSlot *table, StageAccum *acc, const uint8_t *wrec,
-                       const uint32_t *flen, const uint32_t *fwords, const uint32_t *foff, cudaStream_t s, bool rel,
-                       const uint32_t *fmixed) {
-    const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
-    const unsigned grid = grid_for((items + NW - 1) / NW, 152 * 16);
+
+void launch_frame_copy(const float2 *wv, uint32_t nblocks, int m, int e, const EncTarget *tgt, EncResult *res,
+                       const uint32_t *ids, BlockSlot *table, StageAccum *acc, const FrameRecords &fr, cudaStream_t s,
+                       bool rel) {
+    const unsigned grid = grid_for(uint64_t(nblocks) * qsz_nframes(m), kMaxGrid);
     if (rel)
-        k_frame_copy<true><<<grid, NT, 0, s>>>(wv, im, nblocks, m, e, tgt, res, ids, table, acc, wrec, flen, fwords,
-                                               fmixed, foff);
+        k_frame_copy<true><<<grid, cdev::kTeamMax, 0, s>>>(wv, nblocks, m, e, tgt, res, ids, table, acc, fr);
     else
-        k_frame_copy<false><<<grid, NT, 0, s>>>(wv, im, nblocks, m, e, tgt, res, ids, table, acc, wrec, flen, fwords,
-                                                fmixed, foff);
+        k_frame_copy<false><<<grid, cdev::kTeamMax, 0, s>>>(wv, nblocks, m, e, tgt, res, ids, table, acc, fr);
+    count_launch();
+}
+
+void launch_encode_block(const float2 *amps, int m, int e, uint8_t *out, uint64_t cap, const LookbackScratch &scr,
+                         const CallResult &res, cudaStream_t s, bool rel) {
+    const TeamShape ts = team_shape(m);
+    const unsigned grid = unsigned(qsz_nframes(m));
+    if (rel)
+        k_encode_block<true><<<grid, ts.threads, ts.smem, s>>>(amps, m, e, out, cap, scr, res);
+    else
+        k_encode_block<false><<<grid, ts.threads, ts.smem, s>>>(amps, m, e, out, cap, scr, res);
+    count_launch();
+}
+
+void launch_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e, BlockSlot *table,
+                       const ArenaDev &dev, const ArenaDev &host, StageAccum *acc, int *status, cudaStream_t s,
+                       bool rel) {
+    const TeamShape ts = team_shape(m);
+    const unsigned grid = grid_for(nblocks, 152 * 8);
+    if (rel)
+        k_init_store<true><<<grid, ts.threads, ts.smem, s>>>(nblocks, b0, loc, m, e, table, dev, host, acc, status);
+    else
+        k_init_store<false><<<grid, ts.threads, ts.smem, s>>>(nblocks, b0, loc, m, e, table, dev, host, acc, status);
     count_launch();
 }
 

@@ -57,41 +57,57 @@ struct ArenaDev {
     uint64_t *bump;  // device counter
 };
 
-// look-back scratch of the encoder
+// look-back scratch of the single-block encoder
 struct LookbackScratch {
     uint64_t *state;    // one status word per frame
-    uint32_t *ticket;
-    uint32_t *done;
-    uint32_t *epoch;
-    float2 *part;       // per-frame (err_sq, norm_sq) partials, or null (then per-CTA atomics)
+    uint32_t *ticket;   // left zero
+    uint32_t *epoch;    // tags the status words; advanced by every launch
 };
 
 void count_launch();
 
-// rel: the stream is QSZR (relative bound) rather than QSZ1
-void launch_decode(const BlockRef *in, uint32_t nblocks, int m, float2 *wv, uint32_t *hist, int *status,
+// What a single-block call tells the host: written by the launch itself, to mapped pinned memory where the call may
+// hold some, so that the call needs one launch and one synchronisation and no copy.
+struct CallHost {
+    uint64_t bytes;   // compressed size
+    int32_t status;   // QSIM_OK or the first error
+    uint32_t pad;
+};
+struct CallResult {
+    int *status;       // device status word of the launch, left zero
+    uint32_t *done;    // device counter, left zero
+    CallHost *record;  // device address of the record
+};
+
+// Blocks b0 .. b0 + nblocks - 1 of a table decoded back to back. rel: the streams are QSZR (relative bound)
+void launch_decode(const BlockSlot *table, uint64_t b0, uint32_t nblocks, int m, float2 *wv, int *status,
                    cudaStream_t s, bool rel = false);
-void launch_encode(const float2 *wv, uint32_t nblocks, int m, int e, const EncTarget *tgt, EncResult *res,
-                   int only_overflowed, const uint32_t *ids, BlockSlot *table, StageAccum *acc,
-                   const LookbackScratch &scr, int *status, cudaStream_t s);
-// sizing pass whose last CTA reserves every block's slot (sizes are left zeroed)
-void launch_size_reserve(const float2 *wv, uint32_t nblocks, int m, int e, uint64_t *sizes, uint32_t *done_ctr,
-                         const ArenaDev &dev, const ArenaDev &host, EncTarget *tgt, EncResult *res, int *status,
-                         cudaStream_t s);
-// In-place exact encoder: pass 1 encodes every frame over its own amplitudes (Im-plane words to im, 4 bytes
-// per amplitude), records the frames' lengths, word counts (fwords) and offsets and reserves each block's
-// exact slot; pass 2 (launch_frame_copy) copies the frames into the slots. wv is overwritten.
-// rel: QSZR (e is the shift k, wrec holds kQszrSideBytes per frame, fmixed one word per frame); without a
-// device arena (dev.bump null) tgt is the caller's and nothing is reserved. keep_fitting: learned sizing, a
-// block keeps its predicted slot (tgt, reserved beforehand) when it fits, else gets an exact one.
-void launch_encode_ip(float2 *wv, uint32_t *im, uint32_t nblocks, int m, int e, uint32_t *done_ctr,
-                      const ArenaDev &dev, const ArenaDev &host, EncTarget *tgt, EncResult *res, StageAccum *acc,
-                      uint8_t *wrec, uint32_t *flen, uint32_t *fwords, uint32_t *foff, float2 *part, int *status,
-                      cudaStream_t s, bool rel = false, uint32_t *fmixed = nullptr, bool keep_fitting = false);
-void launch_frame_copy(const float2 *wv, const uint32_t *im, uint32_t nblocks, int m, int e, const EncTarget *tgt,
-                       EncResult *res, const uint32_t *ids, BlockSlot *table, StageAccum *acc, const uint8_t *wrec,
-                       const uint32_t *flen, const uint32_t *fwords, const uint32_t *foff, cudaStream_t s,
-                       bool rel = false, const uint32_t *fmixed = nullptr);
+// One block given by pointer, QSZ1 or QSZR by its magic number
+void launch_decode_block(const BlockRef &in, int m, float2 *out, const CallResult &res, cudaStream_t s);
+// Per-frame records of the encoder, in work-item order (blocks of more than one frame)
+struct FrameRecords {
+    uint8_t *side;        // image bytes before the bit-plane words (at most side_bytes)
+    uint32_t side_bytes;  // 256, or kQszrSideBytes for the relative-bound codec
+    uint32_t *len, *off;  // stream bytes, offset in the block's stream
+    uint32_t *head;       // relative-bound codec: bytes in `side`
+    float2 *part;         // (sum (x - x')^2, sum x'^2)
+};
+// Encode a batch of blocks with exact slots (see k_encode); wv is overwritten. Blocks of more than one frame need
+// launch_frame_copy after it. arrive: one zero word per block, left zero. rel: QSZR (e is the shift k).
+void launch_encode(float2 *wv, uint32_t nblocks, int m, int e, const ArenaDev &dev, const ArenaDev &host,
+                   EncTarget *tgt, EncResult *res, const uint32_t *ids, BlockSlot *table, StageAccum *acc,
+                   const FrameRecords &fr, uint64_t *arrive, int *status, cudaStream_t s, bool rel,
+                   bool keep_fitting);
+void launch_frame_copy(const float2 *wv, uint32_t nblocks, int m, int e, const EncTarget *tgt, EncResult *res,
+                       const uint32_t *ids, BlockSlot *table, StageAccum *acc, const FrameRecords &fr, cudaStream_t s,
+                       bool rel);
+// One block into a caller's buffer (rel: QSZR, e is the shift k)
+void launch_encode_block(const float2 *amps, int m, int e, uint8_t *out, uint64_t cap, const LookbackScratch &scr,
+                         const CallResult &res, cudaStream_t s, bool rel = false);
+// The compressed store of a basis state: block b0 holds amplitude 1 at index loc, the others are zero
+void launch_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e, BlockSlot *table,
+                       const ArenaDev &dev, const ArenaDev &host, StageAccum *acc, int *status, cudaStream_t s,
+                       bool rel);
 // leading phase ops of a stage for the decoder (count <= kMaxPreOps)
 struct OpDev;
 struct PreOps {

@@ -13,10 +13,6 @@ namespace qsim {
 namespace cdev {
 
 
-constexpr int NT = 256;          // threads per CTA (8 warps)
-constexpr int NW = NT / 32;
-constexpr int MAX_C = 128;       // chunks per plane per frame (F = 4096)
-constexpr int MAX_CPW = MAX_C / NW;  // chunk pairs per warp
 constexpr uint32_t kFlagA = 1u, kFlagP = 2u;
 constexpr uint32_t kEpochMask = (1u << 30) - 1;
 constexpr long long kSpinLimit = 1ll << 22;
@@ -385,245 +381,6 @@ __device__ __forceinline__ void decode_frame_warp(const uint8_t *sp, uint64_t by
 }
 
 // ---------------------------------------------------------------------------
-// Encode: one CTA per frame, ticket-ordered, decoupled look-back. The frame
-// image (widths, then bit-plane words) is assembled in shared memory while
-// warp 0 finds the frame's byte offset, then copied out with 16-byte stores.
-// The bit planes of a chunk, W_b = ballot(bit b of z_j), are produced for all
-// b at once by a 32x32 bit transpose across the warp (five shuffle stages).
-// ---------------------------------------------------------------------------
-constexpr uint32_t kStageWords = (256 + 8 * 4096) / 4 + 4;  // widths + worst-case payload + pad
-
-// Shared memory of the frame encoder.
-struct EncSmem {
-    uint32_t w[2 * MAX_C];
-    uint32_t off[2 * MAX_C];
-    uint32_t warp_sums[NW];
-    uint32_t total;
-    uint64_t excl;
-    double red[2][NW];
-};
-
-// Encode frame f of one block with the whole CTA (NT threads): src is the
-// frame's amplitudes, lb_block the block's look-back words, tgt its slot,
-// s_stage kStageWords words of shared memory for the frame image.
-template <bool CG = false>
-__device__ __forceinline__ void encode_frame_cta(const float2 *__restrict__ src, const FrameGeom &g, int m, int e,
-                                                 uint32_t f, uint64_t *lb_block, uint32_t epoch, EncTarget tgt,
-                                                 EncResult *res_j, BlockSlot *table_slot, StageAccum *acc,
-                                                 float2 *part_item, int only_overflowed, uint32_t *s_stage,
-                                                 EncSmem &SE, int *status) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t *s_w = SE.w, *s_off = SE.off, *s_warp = SE.warp_sums;
-    uint32_t &s_total = SE.total;
-    uint64_t &s_excl = SE.excl;
-    double (&s_red)[2][NW] = SE.red;
-    const float inv_step = exp2i(-e);
-    const float step = exp2i(e);
-    // x - x' is exact in FP32 (|x - x'| <= s/2 <= |x'|/2 when q != 0, x' = 0 otherwise), so the
-    // per-thread sums are FP32 and only the per-CTA totals are accumulated in FP64
-    float err_sq = 0.f, norm_sq = 0.f;
-    int bad = 0;
-    float2 vin[MAX_CPW];
-#pragma unroll
-    for (int i = 0; i < MAX_CPW; ++i) {
-        const uint32_t c = warp + i * NW;
-        vin[i] = c < g.C ? (CG ? __ldcg(src + c * 32 + lane) : __ldcs(src + c * 32 + lane)) : make_float2(0.f, 0.f);
-    }
-    uint32_t zr[MAX_CPW], zi[MAX_CPW];
-#pragma unroll
-    for (int i = 0; i < MAX_CPW; ++i) {
-        zr[i] = zi[i] = 0;
-        const uint32_t c = warp + i * NW;
-        if (c < g.C) {
-            int32_t q[2];
-            const float x[2] = {vin[i].x, vin[i].y};
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (!isfinite(x[p])) {
-                    bad = QSIM_E_INVALID;
-                    q[p] = 0;
-                } else {
-                    const float t = x[p] * inv_step;  // exact: power-of-two scaling
-                    if (fabsf(t) >= 1073741824.0f) {
-                        bad = bad ? bad : QSIM_E_RANGE;
-                        q[p] = 0;
-                    } else {
-                        q[p] = __float2int_rn(t);
-                    }
-                }
-                const float xr = float(q[p]) * step;
-                const float dx = x[p] - xr;
-                err_sq = fmaf(dx, dx, err_sq);
-                norm_sq = fmaf(xr, xr, norm_sq);
-            }
-            const int32_t pr = __shfl_up_sync(kFull, q[0], 1);
-            const int32_t pi = __shfl_up_sync(kFull, q[1], 1);
-            zr[i] = zigzag(lane ? int32_t(uint32_t(q[0]) - uint32_t(pr)) : q[0]);
-            zi[i] = zigzag(lane ? int32_t(uint32_t(q[1]) - uint32_t(pi)) : q[1]);
-            const uint32_t wr = 32 - __clz(__reduce_or_sync(kFull, zr[i]));
-            const uint32_t wi = 32 - __clz(__reduce_or_sync(kFull, zi[i]));
-            if (lane == 0) {
-                s_w[c] = wr;
-                s_w[g.C + c] = wi;
-            }
-        }
-    }
-    if (bad) raise_status(status, bad);
-    __syncthreads();
-    const uint32_t my_w = tid < int(2 * g.C) ? s_w[tid] : 0;
-    const uint32_t my_off = block_exclusive_scan<NT>(my_w, s_warp, &s_total);
-    const uint32_t padw = (2u * g.C + 15u) & ~15u;
-    if (tid < int(2 * g.C)) s_off[tid] = my_off;
-    // width bytes (and their zero padding) at the head of the frame image
-    if (tid < int(padw) / 4) {
-        uint32_t wbytes = 0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const uint32_t x = 4 * tid + t;
-            wbytes |= (x < 2 * g.C ? s_w[x] : 0u) << (8 * t);
-        }
-        s_stage[tid] = wbytes;
-    }
-    const uint32_t words = s_total;
-    const uint32_t len = words ? uint32_t(padw + ((4ull * words + 15) & ~15ull)) : 0u;
-    __syncthreads();
-
-    // ---- warp 0: decoupled look-back over the preceding frames of this block ----
-    if (warp == 0) {
-        uint64_t *st = lb_block;
-        if (f == 0) {
-            if (lane == 0) {
-                st_relaxed_u64(st, lb_word(epoch, kFlagP, len));
-                s_excl = 0;
-            }
-        } else {
-            if (lane == 0) st_relaxed_u64(st + f, lb_word(epoch, kFlagA, len));
-            uint64_t excl = 0;
-            int64_t end = int64_t(f) - 1;
-            bool timed_out = false;
-            while (true) {
-                const int64_t p = end - lane;
-                uint32_t flag = kFlagP, val = 0;
-                if (p >= 0) {
-                    long long spins = 0;
-                    const uint64_t t0 = global_ns();
-                    while (true) {
-                        const uint64_t w = ld_relaxed_u64(st + p);
-                        const uint32_t fl = uint32_t(w >> 32) & 3u;
-                        if (fl != 0 && uint32_t(w >> 34) == epoch) {
-                            flag = fl;
-                            val = uint32_t(w);
-                            break;
-                        }
-                        if (++spins > kSpinLimit || global_ns() - t0 > kLookbackWaitNs) {
-                            timed_out = true;
-                            flag = kFlagP;
-                            val = 0;
-                            break;
-                        }
-                        __nanosleep(32);
-                    }
-                }
-                const uint32_t pmask = __ballot_sync(kFull, flag == kFlagP);
-                const int first = pmask ? __ffs(pmask) - 1 : 32;
-                uint64_t contrib = lane <= first ? val : 0;
-#pragma unroll
-                for (int o = 16; o; o >>= 1) contrib += __shfl_xor_sync(kFull, contrib, o);
-                excl += contrib;
-                if (pmask) break;
-                end -= 32;
-            }
-            if (__any_sync(kFull, timed_out) && lane == 0) raise_status(status, QSIM_E_TIMEOUT);
-            if (lane == 0) {
-                st_relaxed_u64(st + f, lb_word(epoch, kFlagP, uint32_t(excl + len)));
-                s_excl = excl;
-            }
-        }
-    }
-    // ---- bit-plane words into the frame image: W_b = ballot(bit b of z) ----
-    uint32_t *stage_words = s_stage + padw / 4;
-#pragma unroll
-    for (int i = 0; i < MAX_CPW; ++i) {
-        const uint32_t c = warp + i * NW;
-        if (c < g.C) {
-            const uint32_t wr = s_w[c], wi = s_w[g.C + c];
-            // lane b receives W_b = ballot(bit b of z): the bit-matrix transpose of the chunk's codes
-            const uint32_t word_r = warp_bit_transpose(zr[i], lane);
-            const uint32_t word_i = warp_bit_transpose(zi[i], lane);
-            if (lane < int(wr)) stage_words[s_off[c] + lane] = word_r;
-            if (lane < int(wi)) stage_words[s_off[g.C + c] + lane] = word_i;
-        }
-    }
-    if (words + uint32_t(tid) < (len > padw ? (len - padw) / 4 : 0u)) stage_words[words + tid] = 0;  // pad
-    __syncthreads();
-    const uint64_t frame_off = g.data_start + s_excl;
-    uint8_t *out = tgt.ptr;
-    const uint64_t cap = tgt.cap;
-    const bool fits = frame_off + len <= cap;
-    if (fits && len) {
-        uint4 *o4 = reinterpret_cast<uint4 *>(out + frame_off);
-        const uint4 *s4 = reinterpret_cast<const uint4 *>(s_stage);
-        for (uint32_t i = tid; i < len / 16; i += NT) o4[i] = s4[i];
-    }
-    if (!fits && tid == 0) atomicOr(&res_j->overflow, 1u);
-    if (tid == 0 && g.data_start <= cap)
-        reinterpret_cast<uint32_t *>(out + 32)[f] = uint32_t(frame_off);
-    if (f == g.nframes - 1 && tid == 0) {
-        const uint64_t total = frame_off + len;
-        res_j->total = total;
-        if (total <= cap) {
-            uint32_t *h32 = reinterpret_cast<uint32_t *>(out);
-            h32[0] = kQszMagic;
-            h32[1] = 1u;  // version 1, flags 0
-            h32[2] = uint32_t(m) | (uint32_t(g.fl) << 8) | (uint32_t(uint8_t(int8_t(e))) << 16);
-            h32[3] = g.nframes;
-            reinterpret_cast<uint64_t *>(out)[2] = total;
-            reinterpret_cast<uint64_t *>(out)[3] = 0;
-            h32[8 + g.nframes] = uint32_t(total);
-            for (uint64_t b = 32 + 4ull * (g.nframes + 1); b < g.data_start; ++b) out[b] = 0;
-            if (table_slot) {
-                table_slot->ptr = out;
-                table_slot->bytes = total;
-                table_slot->tier = tgt.tier;
-            }
-            if (acc) {
-                atomicAdd(reinterpret_cast<unsigned long long *>(&acc->store_bytes), total);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&acc->reserved_bytes), cap);
-                if (tgt.tier) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->host_bytes), cap);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&acc->blocks), 1ull);
-            }
-        } else if (acc) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
-        }
-    }
-    // error norms of this frame (only counted once: not on the overflow retry)
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        err_sq += __shfl_xor_sync(kFull, err_sq, o);
-        norm_sq += __shfl_xor_sync(kFull, norm_sq, o);
-    }
-    if (lane == 0) {
-        s_red[0][warp] = double(err_sq);
-        s_red[1][warp] = double(norm_sq);
-    }
-    __syncthreads();
-    if (tid == 0 && !only_overflowed) {
-        double a = 0, b = 0;
-        for (int w = 0; w < NW; ++w) { a += s_red[0][w]; b += s_red[1][w]; }
-        if (part_item) {
-            *part_item = make_float2(float(a), float(b));  // reduced once the block's frames are done
-        } else {
-            atomicAdd(&res_j->err_sq, a);
-            atomicAdd(&res_j->norm_sq, b);
-            if (acc) {
-                atomicAdd(&acc->err_sq, a);
-                atomicAdd(&acc->norm_sq, b);
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Reservation of one block's slot from the two-tier pool: device arena
 // first, then the pinned host arena; slots are padded to 256 bytes.
 // ---------------------------------------------------------------------------
@@ -651,61 +408,6 @@ __device__ __forceinline__ void reserve_slot(uint64_t want, const ArenaDev &dev,
     t->tier = 0;
     raise_status(status, QSIM_E_NOMEM);
 }
-
-// ---------------------------------------------------------------------------
-// Sizing pass: exact stream size of every block (reads the data once more),
-// then the last CTA to finish reserves each block's slot and clears the size
-// counters for the next launch.
-// ---------------------------------------------------------------------------
-// Stream bytes of frame f (zero for an all-zero frame), computed by the whole
-// CTA; the result is returned to every thread. s_words holds NW words.
-template <bool CG = false>
-__device__ __forceinline__ uint32_t size_frame_cta(const float2 *__restrict__ src, const FrameGeom &g, int e,
-                                                   uint32_t *s_words, int *status) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float inv_step = exp2i(-e);
-    float2 vin[MAX_CPW];
-#pragma unroll
-    for (int i = 0; i < MAX_CPW; ++i) {
-        const uint32_t c = warp + i * NW;
-        vin[i] = c < g.C ? (CG ? __ldcg(src + c * 32 + lane) : src[c * 32 + lane]) : make_float2(0.f, 0.f);
-    }
-    uint32_t words = 0;
-    int bad = 0;
-#pragma unroll
-    for (int i = 0; i < MAX_CPW; ++i) {
-        const uint32_t c = warp + i * NW;
-        if (c >= g.C) break;
-        int32_t q[2];
-        const float x[2] = {vin[i].x, vin[i].y};
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const float t = x[p] * inv_step;  // exact: power-of-two scaling
-            if (fabsf(t) < 1073741824.0f) {
-                q[p] = __float2int_rn(t);
-            } else {  // NaN, Inf or out of range
-                q[p] = 0;
-                bad = isfinite(x[p]) ? (bad ? bad : QSIM_E_RANGE) : QSIM_E_INVALID;
-            }
-        }
-        int32_t pr = __shfl_up_sync(kFull, q[0], 1);
-        int32_t pi = __shfl_up_sync(kFull, q[1], 1);
-        const uint32_t zr = zigzag(lane ? int32_t(uint32_t(q[0]) - uint32_t(pr)) : q[0]);
-        const uint32_t zi = zigzag(lane ? int32_t(uint32_t(q[1]) - uint32_t(pi)) : q[1]);
-        const uint32_t wr = 32 - __clz(__reduce_or_sync(kFull, zr)), wi = 32 - __clz(__reduce_or_sync(kFull, zi));
-        words += wr + wi;
-    }
-    if (bad) raise_status(status, bad);
-    if (lane == 0) s_words[warp] = words;
-    __syncthreads();
-    uint32_t tot = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) tot += s_words[w];
-    __syncthreads();
-    const uint64_t padw = (2ull * g.C + 15) & ~15ull;
-    return tot ? uint32_t(padw + ((4ull * tot + 15) & ~15ull)) : 0u;
-}
-
 
 // Chunk widths of one frame with one warp (no block-wide barrier): lane l
 // receives the Re widths of chunks 4l .. 4l+3 packed in wre and the Im widths

@@ -66,34 +66,4 @@ __device__ __forceinline__ uint32_t warp_bit_transpose(uint32_t x, int lane) {
     return x;
 }
 
-// Exclusive scan of `count` (<= blockDim.x) values held by threads 0..count-1
-// in a block of `NT` threads; returns the thread's exclusive prefix and writes
-// the total to *total (shared). `warp_sums` must hold NT/32 entries.
-template <int NT>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *warp_sums,
-                                                         uint32_t *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < NT / 32 ? warp_sums[lane] : 0;
-        uint32_t wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t t = __shfl_up_sync(kFull, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < NT / 32) warp_sums[lane] = wi - w;
-        if (lane == NT / 32 - 1) *total = wi;
-    }
-    __syncthreads();
-    return warp_sums[warp] + incl - v;
-}
-
 }  // namespace qsim

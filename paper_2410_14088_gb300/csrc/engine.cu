@@ -255,15 +255,11 @@ struct DevBuf {
 // ---------------------------------------------------------------------------
 struct DeviceCtx {
     std::mutex mu;  // serialises the single-block entry points
-    // relative-bound block compression: a copy of the block, the Im-plane scratch and the per-frame records
-    uint8_t *rel_buf = nullptr;
-    size_t rel_cap = 0;
     int *status = nullptr;
     uint64_t *lb_state = nullptr;
-    uint32_t *lb_ctr = nullptr;  // ticket, done, epoch
-    EncTarget *tgt = nullptr;
-    EncResult *res = nullptr;
-    BlockRef *ref = nullptr;
+    uint32_t *lb_ctr = nullptr;  // single-block encoder: ticket, -, epoch; [16] arrivals of a call's CTAs
+    CallResult call;             // single-block calls: device words and the mapped record of the last CTA
+    CallHost *call_host = nullptr;
     bool ready = false;
     // learned size predictor of this device
     float *pred_params = nullptr;
@@ -287,25 +283,17 @@ static int ensure_device_ctx(DeviceCtx &c) {
     CUDA_TRY(alloc(&c.status, 256));
     CUDA_TRY(alloc(&c.lb_state, max_frames * sizeof(uint64_t)));
     CUDA_TRY(alloc(&c.lb_ctr, 256));
-    CUDA_TRY(alloc(&c.tgt, sizeof(EncTarget)));
-    CUDA_TRY(alloc(&c.res, sizeof(EncResult)));
-    CUDA_TRY(alloc(&c.ref, sizeof(BlockRef)));
     CUDA_TRY(alloc(&c.pred_params, kMlpParams * sizeof(float)));
     CUDA_TRY(cudaMemset(c.status, 0, 256));
     CUDA_TRY(cudaMemset(c.lb_state, 0, max_frames * sizeof(uint64_t)));
     CUDA_TRY(cudaMemset(c.lb_ctr, 0, 256));
+    CUDA_TRY(cudaHostAlloc(reinterpret_cast<void **>(&c.call_host), sizeof(CallHost), cudaHostAllocMapped));
+    g_allocs.fetch_add(1, std::memory_order_relaxed);
+    CUDA_TRY(cudaHostGetDevicePointer(reinterpret_cast<void **>(&c.call.record), c.call_host, 0));
+    c.call.status = c.status + 1;  // the run engine's status is word 0
+    c.call.done = c.lb_ctr + 16;
     c.ready = true;
     return QSIM_OK;
-}
-
-static LookbackScratch make_scratch(uint64_t *state, uint32_t *ctr, float2 *part = nullptr) {
-    LookbackScratch s{};
-    s.part = part;
-    s.state = state;
-    s.ticket = ctr;
-    s.done = ctr + 1;
-    s.epoch = ctr + 2;
-    return s;
 }
 
 static int read_status(int *d_status, cudaStream_t s) {
@@ -317,6 +305,14 @@ static int read_status(int *d_status, cudaStream_t s) {
         CUDA_TRY(cudaStreamSynchronize(s));
     }
     return h;
+}
+
+// Wait for a single-block call's launch, before which call_host->status was set to QSIM_E_CUDA (it stays so when the
+// launch did not run); *code receives its device status.
+static int call_status(DeviceCtx &c, cudaStream_t s, int *code) {
+    CUDA_TRY(cudaStreamSynchronize(s));
+    *code = static_cast<volatile CallHost *>(c.call_host)->status;
+    return QSIM_OK;
 }
 
 static const char *status_text(int code) {
@@ -1025,17 +1021,29 @@ struct StreamWork {
     DevBuf<BlockRef> refs;
     DevBuf<EncTarget> tgt;
     DevBuf<EncResult> res;
-    DevBuf<uint64_t> sizes;
-    DevBuf<uint64_t> lb_state;
-    DevBuf<uint32_t> lb_ctr;
+    DevBuf<uint64_t> sizes;  // per block: frames coded (the encoder's arrival counters, left zero)
+    DevBuf<uint32_t> ctr;    // gate-pass tile counter (two words, left zero)
     DevBuf<float2> part;
     DevBuf<uint32_t> hist;   // per block: 32-bin histogram of code bit lengths (decoder)
     DevBuf<float> pred;      // per block: predicted log2 stream bytes
-    DevBuf<uint8_t> wrec;    // per frame: chunk widths recorded by the sizing pass
-    DevBuf<uint32_t> flen, foff;  // per frame: stream bytes and offset
-    DevBuf<uint32_t> fwords;      // per frame: Re words | Im words << 16 (in-place encoder)
-    DevBuf<uint32_t> fmixed;      // per frame: Re | Im mixed sign chunks << 16 (relative-bound codec)
-    DevBuf<uint32_t> imsc;        // Im-plane words of the in-place encoder, one word per amplitude
+    DevBuf<uint8_t> side;               // per frame: its image before the bit-plane words
+    DevBuf<uint32_t> flen, foff, fhead;  // per frame: stream bytes, offset, bytes in `side`
+    FrameRecords records(bool rel) const {
+        return {side.p, rel ? kQszrSideBytes : 256u, flen.p, foff.p, fhead.p, part.p};
+    }
+    // encode and decode buffers of `blocks` blocks of 2^m amplitudes in nframes frames each; the counters zeroed on s
+    int alloc_codec(uint64_t blocks, uint32_t m, uint64_t nframes, bool rel, cudaStream_t st) {
+        int rc;
+        const uint64_t nf = nframes > 1 ? blocks * nframes : 0;  // one-frame blocks keep no frame records
+        if ((rc = wv.alloc(blocks << m)) || (rc = refs.alloc(blocks)) || (rc = tgt.alloc(blocks)) ||
+            (rc = res.alloc(blocks)) || (rc = sizes.alloc(blocks)) || (rc = hist.alloc(blocks * 32)) ||
+            (rc = pred.alloc(blocks)) || (rc = part.alloc(nf)) || (rc = side.alloc(nf * (rel ? kQszrSideBytes : 256))) ||
+            (rc = flen.alloc(nf)) || (rc = foff.alloc(nf)) || (rel && (rc = fhead.alloc(nf))) || (rc = ctr.alloc(2)))
+            return rc;
+        CUDA_TRY(cudaMemsetAsync(ctr.p, 0, 2 * sizeof(uint32_t), st));
+        CUDA_TRY(cudaMemsetAsync(sizes.p, 0, blocks * sizeof(uint64_t), st));
+        return QSIM_OK;
+    }
 };
 
 static StageFeatures stage_features(const qsim_plan *p, size_t si, int e) {
@@ -1178,43 +1186,35 @@ static int alloc_run(RunCtx &R, uint64_t dev_budget, uint64_t host_limit, cudaSt
     return QSIM_OK;
 }
 
-// Initial store (Sec. 4.2): encode the basis block and one zero block once, every
-// other block gets a copy of the zero stream. Runs on w.s; w.wv holds two blocks.
-static int init_store(RunCtx &R, StreamWork &w, int *status) {
+// Initial store (Sec. 4.2) on stream s: the compressed streams of the basis block and the zero blocks are written in one
+// launch. An uncompressed store is built from two blocks in w (w.wv holds two): the basis block and one zero block,
+// which every other block gets a copy of.
+static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
     const qsim_config &cfg = R.p->cfg;
     const uint32_t m = R.m;
-    const uint32_t b0 = uint32_t(cfg.init_basis >> m);
+    const uint64_t b0 = cfg.init_basis >> m;
     const uint64_t loc = cfg.init_basis & ((1ull << m) - 1);
-    k_init_blocks<<<256, 256, 0, w.s>>>(w.wv.p, m, loc);
+    BlockSlot *tab0 = R.tables.p;
+    if (!R.raw) {
+        launch_init_store(R.nblocks, b0, loc, int(m), R.e, tab0, R.arena_dev(0), R.arena_host(0), R.accs.p + R.nst,
+                          status, s, R.rel);
+        return QSIM_OK;
+    }
+    k_init_blocks<<<256, 256, 0, s>>>(w->wv.p, m, loc);
     count_launch();
     static const uint32_t h_ids[2] = {0, 1};
-    CUDA_TRY(cudaMemcpyAsync(R.init_ids.p, h_ids, sizeof(h_ids), cudaMemcpyHostToDevice, w.s));
-    // encode both blocks into slots of arena 0; tmpl[0] is the basis block, tmpl[1] the zero template
-    if (R.raw) {
-        launch_reserve(2, nullptr, R.worst, nullptr, 0, R.worst, R.arena_dev(0), R.arena_host(0), w.tgt.p, w.res.p, 0,
-                       status, w.s);
-        launch_copy_out(w.wv.p, 2, m, w.tgt.p, R.init_ids.p, R.tmpl.p, nullptr, status, w.s);
-    } else if (R.rel) {
-        // the in-place encoder and its frame copy (relative-bound streams)
-        launch_encode_ip(w.wv.p, w.imsc.p, 2, int(m), R.e, w.lb_ctr.p + 3, R.arena_dev(0), R.arena_host(0), w.tgt.p,
-                         w.res.p, nullptr, w.wrec.p, w.flen.p, w.fwords.p, w.foff.p, w.part.p, status, w.s, true,
-                         w.fmixed.p);
-        launch_frame_copy(w.wv.p, w.imsc.p, 2, int(m), R.e, w.tgt.p, w.res.p, R.init_ids.p, R.tmpl.p, nullptr, w.wrec.p,
-                          w.flen.p, w.fwords.p, w.foff.p, w.s, true, w.fmixed.p);
-    } else {
-        launch_size_reserve(w.wv.p, 2, m, R.e, w.sizes.p, w.lb_ctr.p + 3, R.arena_dev(0), R.arena_host(0), w.tgt.p,
-                            w.res.p, status, w.s);
-        LookbackScratch scr = make_scratch(w.lb_state.p, w.lb_ctr.p);
-        launch_encode(w.wv.p, 2, m, R.e, w.tgt.p, w.res.p, 0, R.init_ids.p, R.tmpl.p, nullptr, scr, status, w.s);
-    }
-    BlockSlot *tab0 = R.tables.p;
-    k_copy_slot<<<1, 1, 0, w.s>>>(tab0 + b0, R.tmpl.p + 0);
+    CUDA_TRY(cudaMemcpyAsync(R.init_ids.p, h_ids, sizeof(h_ids), cudaMemcpyHostToDevice, s));
+    // tmpl[0] is the basis block, tmpl[1] the zero template
+    launch_reserve(2, nullptr, R.worst, nullptr, 0, R.worst, R.arena_dev(0), R.arena_host(0), w->tgt.p, w->res.p, 0,
+                   status, s);
+    launch_copy_out(w->wv.p, 2, m, w->tgt.p, R.init_ids.p, R.tmpl.p, nullptr, status, s);
+    k_copy_slot<<<1, 1, 0, s>>>(tab0 + b0, R.tmpl.p + 0);
     count_launch();
     // the zero template slot stays allocated in arena 0 until stage 0 has read its copies
-    k_replicate_zero<<<unsigned(std::min<uint64_t>(R.nblocks, 152 * 8)), 128, 0, w.s>>>(
-        tab0, uint32_t(R.nblocks), b0, R.tmpl.p + 1, R.arena_dev(0), R.arena_host(0), status);
+    k_replicate_zero<<<unsigned(std::min<uint64_t>(R.nblocks, 152 * 8)), 128, 0, s>>>(
+        tab0, uint32_t(R.nblocks), uint32_t(b0), R.tmpl.p + 1, R.arena_dev(0), R.arena_host(0), status);
     count_launch();
-    k_sum_table<<<64, 256, 0, w.s>>>(tab0, R.nblocks, R.accs.p + R.nst);
+    k_sum_table<<<64, 256, 0, s>>>(tab0, R.nblocks, R.accs.p + R.nst);
     count_launch();
     return QSIM_OK;
 }
@@ -1688,7 +1688,7 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
     int rc = prepare_run(RC, p, dctx);
     if (rc) return rc;
     PlanDev *pd = RC.pd;
-    const bool persistent = RC.persistent, raw = RC.raw;
+    const bool persistent = RC.persistent;
     const uint32_t m = RC.m;
     const uint64_t nframes = RC.nframes;
 
@@ -1716,26 +1716,11 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
         max_batch_blocks = std::max<uint64_t>(max_batch_blocks, gpb * sd.G);
     }
     max_batch_blocks = std::max<uint64_t>(max_batch_blocks, 2);
-    if (persistent) max_batch_blocks = 2;  // the stream buffers only serve the initial store
     for (uint32_t i = 0; i < nstreams; ++i) {
         StreamWork &w = sw[i];
         CUDA_TRY(cudaStreamCreateWithFlags(&w.s, cudaStreamNonBlocking));
         CUDA_TRY(cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming));
-        if ((rc = w.wv.alloc(max_batch_blocks << m)) || (rc = w.refs.alloc(max_batch_blocks)) ||
-            (rc = w.tgt.alloc(max_batch_blocks)) || (rc = w.res.alloc(max_batch_blocks)) ||
-            (rc = w.sizes.alloc(max_batch_blocks)) || (rc = w.lb_state.alloc(max_batch_blocks * nframes)) ||
-            (rc = w.part.alloc(max_batch_blocks * nframes)) || (rc = w.hist.alloc(max_batch_blocks * 32)) ||
-            (rc = w.pred.alloc(max_batch_blocks)) ||
-            ((!persistent || RC.rel) && (rc = w.wrec.alloc(max_batch_blocks * nframes * (RC.rel ? kQszrSideBytes : 256)))) ||
-            ((!persistent || RC.rel) && !raw && (rc = w.imsc.alloc(max_batch_blocks << m))) ||
-            ((!persistent || RC.rel) && (rc = w.fwords.alloc(max_batch_blocks * nframes))) ||
-            (RC.rel && (rc = w.fmixed.alloc(max_batch_blocks * nframes))) ||
-            (rc = w.flen.alloc(max_batch_blocks * nframes)) || (rc = w.foff.alloc(max_batch_blocks * nframes)) ||
-            (rc = w.lb_ctr.alloc(16)))
-            return rc;
-        CUDA_TRY(cudaMemsetAsync(w.lb_state.p, 0, max_batch_blocks * nframes * sizeof(uint64_t), main));
-        CUDA_TRY(cudaMemsetAsync(w.lb_ctr.p, 0, 16 * sizeof(uint32_t), main));  // [8], [9]: gate-pass tile counter
-        CUDA_TRY(cudaMemsetAsync(w.sizes.p, 0, max_batch_blocks * sizeof(uint64_t), main));
+        if (!persistent && (rc = w.alloc_codec(max_batch_blocks, m, nframes, RC.rel, main))) return rc;
     }
     CUDA_TRY(cudaEventCreate(&S.ev_start));
     CUDA_TRY(cudaEventCreate(&S.ev_stop));
@@ -1749,7 +1734,7 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
         StreamWork &w = sw[0];
         CUDA_TRY(cudaEventRecord(S.ev_fork, main));
         CUDA_TRY(cudaStreamWaitEvent(w.s, S.ev_fork, 0));
-        if ((rc = init_store(RC, w, S.status))) return rc;
+        if ((rc = init_store(RC, &w, S.status, w.s))) return rc;
         CUDA_TRY(cudaEventRecord(w.done, w.s));
         CUDA_TRY(cudaStreamWaitEvent(main, w.done, 0));
     }
@@ -1849,7 +1834,7 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
             for (uint32_t pi = 0; pi < sd.npasses; ++pi) {
                 prof.begin(P_PASS, w.s);
                 launch_pass(w.wv.p, sd.W, ng, &sd.passes_host[pi], pd->blob.p, pd->mats.p, pd->bfr.p, gb_stage + g0,
-                            cfg.prec, w.s, w.lb_ctr.p + 8, status);
+                            cfg.prec, w.s, w.ctr.p, status);
                 prof.end(w.s);
             }
             if (raw) {
@@ -1862,31 +1847,21 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
                 prof.end(w.s);
             } else {
                 if (predict) {
-                    // reserve 2^pred (1 + margin) bytes per block ahead of the encoder; the in-place encoder keeps
-                    // every slot its block fits and reserves exact slots for under-estimated blocks; copy
+                    // learned sizing: 2^pred (1 + margin) bytes per block ahead of the encoder, which keeps every
+                    // slot its block fits and reserves exact slots for under-estimated blocks
                     prof.begin(P_RESERVE, w.s);
                     launch_reserve(nb, nullptr, 0, w.pred.p, cfg.predictor_margin, worst, arena_dev(out_par),
                                    arena_host(out_par), w.tgt.p, w.res.p, 0, status, w.s);
                     prof.end(w.s);
-                    prof.begin(P_ENCODE, w.s);
-                    launch_encode_ip(w.wv.p, w.imsc.p, nb, m, e, w.lb_ctr.p + 3, arena_dev(out_par),
-                                     arena_host(out_par), w.tgt.p, w.res.p, acc, w.wrec.p, w.flen.p, w.fwords.p,
-                                     w.foff.p, w.part.p, status, w.s, RC.rel, w.fmixed.p, true);
-                    prof.end(w.s);
+                }
+                const FrameRecords fr = w.records(RC.rel);
+                prof.begin(P_ENCODE, w.s);
+                launch_encode(w.wv.p, nb, int(m), e, arena_dev(out_par), arena_host(out_par), w.tgt.p, w.res.p, ids,
+                              tab_out, acc, fr, w.sizes.p, status, w.s, RC.rel, predict);
+                prof.end(w.s);
+                if (RC.nframes > 1) {
                     prof.begin(P_FRAME_COPY, w.s);
-                    launch_frame_copy(w.wv.p, w.imsc.p, nb, m, e, w.tgt.p, w.res.p, ids, tab_out, acc, w.wrec.p,
-                                      w.flen.p, w.fwords.p, w.foff.p, w.s, RC.rel, w.fmixed.p);
-                    prof.end(w.s);
-                } else {
-                    // exact sizing: encode every frame in place, reserve exact slots, copy the frames over
-                    prof.begin(P_ENCODE, w.s);
-                    launch_encode_ip(w.wv.p, w.imsc.p, nb, m, e, w.lb_ctr.p + 3, arena_dev(out_par),
-                                     arena_host(out_par), w.tgt.p, w.res.p, acc, w.wrec.p, w.flen.p, w.fwords.p,
-                                     w.foff.p, w.part.p, status, w.s, RC.rel, w.fmixed.p);
-                    prof.end(w.s);
-                    prof.begin(P_FRAME_COPY, w.s);
-                    launch_frame_copy(w.wv.p, w.imsc.p, nb, m, e, w.tgt.p, w.res.p, ids, tab_out, acc, w.wrec.p,
-                                      w.flen.p, w.fwords.p, w.foff.p, w.s, RC.rel, w.fmixed.p);
+                    launch_frame_copy(w.wv.p, nb, int(m), e, w.tgt.p, w.res.p, ids, tab_out, acc, fr, w.s, RC.rel);
                     prof.end(w.s);
                 }
                 if (collect) {
@@ -1951,7 +1926,6 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     int rc;
     uint64_t sum_need = 0;
     std::map<uint32_t, uint64_t> w_groups;  // working-vector sizes of the batch and their group counts
-    uint32_t mmax = 0;
     for (size_t c = 0; c < count; ++c) {
         const qsim_plan *p = plans[c];
         if (!p) return set_error(QSIM_E_INVALID, "batch entry %zu is null", c);
@@ -1968,19 +1942,18 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
         if ((rc = prepare_run(*rs[c], p, dctx))) return rc;
         for (const StageDev &sd : rs[c]->pd->stages) w_groups[sd.W] += sd.ngroups;
         sum_need += rs[c]->need_per_parity;
-        mmax = std::max(mmax, rs[c]->m);
     }
     const uint64_t slot_budget = 1ull << 27;  // working-vector slots of the launch: about 1 GiB
     size_t free_b = 0, total_b = 0;
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     free_b += cached_dev_bytes();
-    // working-vector slot rings (one per size) with their frame scratch, and the initial-store buffers
+    // working-vector slot rings (one per size) with their frame scratch
     uint64_t ring_amps = 0;
     for (const auto &kv : w_groups)
         ring_amps += std::min<uint64_t>(kv.second, std::max<uint64_t>(2, slot_budget >> kv.first)) << kv.first;
     const bool rel = plans[0]->cfg.codec == QSIM_CODEC_QSZR;
     // 8 B per amplitude and a quarter for the frame scratch; the relative codec adds its 4 B imaginary words
-    const uint64_t work_bytes = ring_amps * (rel ? 12 : 10) + (16ull << (mmax + 1)) * (rel ? 2 : 1);
+    const uint64_t work_bytes = ring_amps * (rel ? 14 : 10);
     const double dev_budget = free_b > work_bytes ? 0.85 * double(free_b - work_bytes) : 0.0;
     const double host_budget = 0.3 * double(host_phys_bytes());
     // each circuit's share of both levels follows its worst-case need
@@ -1988,19 +1961,6 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
         const double f = double(rs[c]->need_per_parity) / double(sum_need);
         if ((rc = alloc_run(*rs[c], uint64_t(dev_budget * f), uint64_t(host_budget * f), main))) return rc;
     }
-    StreamWork w;
-    const uint64_t nframes_max = qsz_nframes(int(mmax));
-    if ((rc = w.wv.alloc(2ull << mmax)) || (rc = w.tgt.alloc(2)) || (rc = w.res.alloc(2)) || (rc = w.sizes.alloc(2)) ||
-        (rc = w.lb_state.alloc(2 * nframes_max)) || (rc = w.lb_ctr.alloc(4)) ||
-        (rel && ((rc = w.imsc.alloc(2ull << mmax)) || (rc = w.wrec.alloc(2 * nframes_max * kQszrSideBytes)) ||
-                 (rc = w.fwords.alloc(2 * nframes_max)) || (rc = w.fmixed.alloc(2 * nframes_max)) ||
-                 (rc = w.flen.alloc(2 * nframes_max)) || (rc = w.foff.alloc(2 * nframes_max)) ||
-                 (rc = w.part.alloc(2 * nframes_max)))))
-        return rc;
-    CUDA_TRY(cudaMemsetAsync(w.lb_state.p, 0, 2 * nframes_max * sizeof(uint64_t), main));
-    CUDA_TRY(cudaMemsetAsync(w.lb_ctr.p, 0, 4 * sizeof(uint32_t), main));
-    CUDA_TRY(cudaMemsetAsync(w.sizes.p, 0, 2 * sizeof(uint64_t), main));
-    w.s = main;  // the initial stores run on the caller's stream, one after another
     cudaEvent_t ev_start, ev_stop;
     CUDA_TRY(cudaEventCreate(&ev_start));
     CUDA_TRY(cudaEventCreate(&ev_stop));
@@ -2008,8 +1968,7 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     Profiler prof;
     prof.on = (g_profile.load() != 0 || launch_stat) && !plans[0]->cfg.graph;
     CUDA_TRY(cudaEventRecord(ev_start, main));
-    for (size_t c = 0; c < count && !rc; ++c) rc = init_store(*rs[c], w, status);
-    w.s = nullptr;  // not ours to destroy
+    for (size_t c = 0; c < count && !rc; ++c) rc = init_store(*rs[c], nullptr, status, main);
     if (rc) return rc;
     if ((rc = run_persistent(rp, true, main, status, prof, dctx, slot_budget))) return rc;
     CUDA_TRY(cudaEventRecord(ev_stop, main));
@@ -2056,16 +2015,16 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     return QSIM_OK;
 }
 
-// decode blocks [b0, b0 + count) of a state (block order) into dst
+// Decode blocks [b0, b0 + count) of a state (block order) into dst: one launch, not synchronised. refs serves an
+// uncompressed state only.
 static int decode_state_blocks(const qsim_state *st, uint64_t b0, uint32_t count, float2 *dst, BlockRef *refs,
-                               uint32_t *ids_dev, int *status, cudaStream_t s) {
-    std::vector<uint32_t> ids(count);
-    for (uint32_t i = 0; i < count; ++i) ids[i] = uint32_t(b0 + i);
-    CUDA_TRY(cudaMemcpyAsync(ids_dev, ids.data(), count * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-    launch_gather_refs(st->table, ids_dev, count, refs, s);
-    if (st->codec == QSIM_CODEC_NONE) launch_copy_in(refs, count, st->m, dst, status, s);
-    else launch_decode(refs, count, st->m, dst, nullptr, status, s, st->codec == QSIM_CODEC_QSZR);
-    CUDA_TRY(cudaStreamSynchronize(s));
+                               int *status, cudaStream_t s) {
+    if (st->codec == QSIM_CODEC_NONE) {
+        launch_gather_refs(st->table + b0, nullptr, count, refs, s);
+        launch_copy_in(refs, count, st->m, dst, status, s);
+    } else {
+        launch_decode(st->table, b0, count, int(st->m), dst, status, s, st->codec == QSIM_CODEC_QSZR);
+    }
     return QSIM_OK;
 }
 
@@ -2677,14 +2636,14 @@ int qsim_state_decompress(const qsim_state *st, float *d_out, void *cuda_stream)
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const uint64_t nblocks = 1ull << (st->n - st->m);
     DevBuf<BlockRef> refs;
-    DevBuf<uint32_t> ids;
     int rc;
-    const uint32_t chunk = uint32_t(std::min<uint64_t>(nblocks, 4096));
-    if ((rc = refs.alloc(chunk)) || (rc = ids.alloc(chunk))) return rc;
+    if (st->codec == QSIM_CODEC_NONE && (rc = refs.alloc(nblocks))) return rc;
     int *status = device_ctx(st->device).status;
-    for (uint64_t b = 0; b < nblocks; b += chunk) {
-        uint32_t cnt = uint32_t(std::min<uint64_t>(chunk, nblocks - b));
-        rc = decode_state_blocks(st, b, cnt, reinterpret_cast<float2 *>(d_out) + (b << st->m), refs.p, ids.p, status, s);
+    // launches of at most 2^28 blocks (32-bit block and grid counts)
+    for (uint64_t b = 0, cnt; b < nblocks; b += cnt) {
+        cnt = std::min<uint64_t>(nblocks - b, 1ull << 28);
+        rc = decode_state_blocks(st, b, uint32_t(cnt), reinterpret_cast<float2 *>(d_out) + (b << st->m), refs.p + b,
+                                 status, s);
         if (rc) return rc;
     }
     int code = read_status(status, s);
@@ -2793,8 +2752,7 @@ int qsim_amplitudes(const qsim_state *st, const uint64_t *idx, size_t count, flo
         const uint32_t cnt = uint32_t(std::min<size_t>(chunk, bids.size() - b0));
         CUDA_TRY(cudaMemcpyAsync(ids.p, bids.data() + b0, cnt * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
         launch_gather_refs(st->table, ids.p, cnt, refs.p, s);
-        if (st->codec == QSIM_CODEC_NONE) launch_copy_in(refs.p, cnt, m, blocks.p, status, s);
-        else launch_decode(refs.p, cnt, m, blocks.p, nullptr, status, s, st->codec == QSIM_CODEC_QSZR);
+        launch_copy_in(refs.p, cnt, m, blocks.p, status, s);
         std::vector<uint32_t> sel_slot, sel_local;
         std::vector<size_t> sel_pos;
         for (size_t i = 0; i < count; ++i)
@@ -2834,12 +2792,11 @@ static int reduce_state(const qsim_state *st, const double *ref, double acc_out[
     CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     const uint32_t chunk = uint32_t(std::min<uint64_t>(nblocks, std::max<uint64_t>(1, (1ull << 24) >> m)));
     DevBuf<BlockRef> refs;
-    DevBuf<uint32_t> ids;
     DevBuf<float2> blocks;
     DevBuf<double2> rbuf;
     DevBuf<double> acc;
     int rc;
-    if ((rc = refs.alloc(chunk)) || (rc = ids.alloc(chunk)) || (rc = blocks.alloc(uint64_t(chunk) << m)) ||
+    if ((rc = refs.alloc(chunk)) || (rc = blocks.alloc(uint64_t(chunk) << m)) ||
         (rc = acc.alloc(4)) || (ref && !ref_dev && (rc = rbuf.alloc(uint64_t(chunk) << m)))) {
         cudaStreamDestroy(s);
         return rc;
@@ -2848,7 +2805,7 @@ static int reduce_state(const qsim_state *st, const double *ref, double acc_out[
     int *status = device_ctx(st->device).status;
     for (uint64_t b = 0; b < nblocks; b += chunk) {
         const uint32_t cnt = uint32_t(std::min<uint64_t>(chunk, nblocks - b));
-        rc = decode_state_blocks(st, b, cnt, blocks.p, refs.p, ids.p, status, s);
+        rc = decode_state_blocks(st, b, cnt, blocks.p, refs.p, status, s);
         if (rc) { cudaStreamDestroy(s); return rc; }
         const uint64_t amps = uint64_t(cnt) << m;
         const double2 *r = nullptr;
@@ -2905,6 +2862,23 @@ int qsim_state_block_stream(const qsim_state *st, uint64_t block, void *host_out
     return QSIM_OK;
 }
 
+// One block compressed into the caller's buffer (the context's lock held): one launch, one synchronisation.
+static int compress_call(DeviceCtx &c, const float *d_amps, uint32_t m, int e, void *d_out, size_t cap,
+                         size_t *out_bytes, cudaStream_t s, bool rel, const char *what) {
+    c.call_host->status = QSIM_E_CUDA;
+    launch_encode_block(reinterpret_cast<const float2 *>(d_amps), int(m), e, static_cast<uint8_t *>(d_out), cap,
+                        {c.lb_state, c.lb_ctr, c.lb_ctr + 2}, c.call, s, rel);
+    int code = 0;
+    int rc = call_status(c, s, &code);
+    if (rc) return rc;
+    if (code) return set_error(code, "%s: %s", what, status_text(code));
+    const uint64_t bytes = static_cast<volatile CallHost *>(c.call_host)->bytes;
+    *out_bytes = size_t(bytes);
+    if (bytes > cap)
+        return set_error(QSIM_E_CAPACITY, "stream needs %llu bytes, cap is %zu", (unsigned long long)bytes, cap);
+    return QSIM_OK;
+}
+
 int qsim_compress_block(const float *d_amps, uint32_t m, double eb, void *d_out, size_t cap, size_t *out_bytes,
                         void *cuda_stream) {
     if (!d_amps || !d_out || !out_bytes) return set_error(QSIM_E_INVALID, "null argument");
@@ -2920,21 +2894,7 @@ int qsim_compress_block(const float *d_amps, uint32_t m, double eb, void *d_out,
     int rc = ensure_device_ctx(c);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    EncTarget t{};
-    t.ptr = static_cast<uint8_t *>(d_out);
-    t.cap = cap;
-    EncResult r{};
-    CUDA_TRY(cudaMemcpyAsync(c.tgt, &t, sizeof(t), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(c.res, &r, sizeof(r), cudaMemcpyHostToDevice, s));
-    launch_encode(reinterpret_cast<const float2 *>(d_amps), 1, int(m), e, c.tgt, c.res, 0, nullptr, nullptr, nullptr,
-                  make_scratch(c.lb_state, c.lb_ctr), c.status, s);
-    CUDA_TRY(cudaMemcpyAsync(&r, c.res, sizeof(r), cudaMemcpyDeviceToHost, s));
-    int code = read_status(c.status, s);
-    if (code) return set_error(code, "compress: %s", status_text(code));
-    *out_bytes = r.total;
-    if (r.overflow) return set_error(QSIM_E_CAPACITY, "stream needs %llu bytes, cap is %zu",
-                                     (unsigned long long)r.total, cap);
-    return QSIM_OK;
+    return compress_call(c, d_amps, m, e, d_out, cap, out_bytes, s, false, "compress");
 }
 
 int qsim_compress_block_rel(const float *d_amps, uint32_t m, double rel, void *d_out, size_t cap,
@@ -2952,45 +2912,7 @@ int qsim_compress_block_rel(const float *d_amps, uint32_t m, double rel, void *d
     int rc = ensure_device_ctx(c);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    // scratch layout: block copy (8 B / amplitude), Im words (4 B), side records, then five per-frame arrays
-    const uint64_t N = 1ull << m, nf = qsz_nframes(int(m));
-    const size_t need = size_t(12 * N + nf * (kQszrSideBytes + 4 * 4 + 8));
-    if (need > c.rel_cap) {
-        if (c.rel_buf) CUDA_TRY(cudaFree(c.rel_buf));
-        c.rel_buf = nullptr;
-        c.rel_cap = 0;
-        if (cudaMalloc(&c.rel_buf, need) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(QSIM_E_NOMEM, "relative-codec scratch of %zu bytes", need);
-        }
-        g_allocs.fetch_add(1, std::memory_order_relaxed);
-        c.rel_cap = need;
-    }
-    float2 *wv = reinterpret_cast<float2 *>(c.rel_buf);
-    uint32_t *im = reinterpret_cast<uint32_t *>(c.rel_buf + 8 * N);
-    uint8_t *side = c.rel_buf + 12 * N;
-    uint32_t *flen = reinterpret_cast<uint32_t *>(side + nf * kQszrSideBytes);
-    uint32_t *fwords = flen + nf, *fmixed = fwords + nf, *foff = fmixed + nf;
-    float2 *part = reinterpret_cast<float2 *>(foff + nf);
-    CUDA_TRY(cudaMemcpyAsync(wv, d_amps, 8 * N, cudaMemcpyDeviceToDevice, s));
-    EncTarget t{};
-    t.ptr = static_cast<uint8_t *>(d_out);
-    t.cap = cap;
-    EncResult r{};
-    CUDA_TRY(cudaMemcpyAsync(c.tgt, &t, sizeof(t), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(c.res, &r, sizeof(r), cudaMemcpyHostToDevice, s));
-    const ArenaDev none{};
-    launch_encode_ip(wv, im, 1, int(m), k, c.lb_ctr + 3, none, none, c.tgt, c.res, nullptr, side, flen, fwords, foff,
-                     part, c.status, s, true, fmixed);
-    launch_frame_copy(wv, im, 1, int(m), k, c.tgt, c.res, nullptr, nullptr, nullptr, side, flen, fwords, foff, s, true,
-                      fmixed);
-    CUDA_TRY(cudaMemcpyAsync(&r, c.res, sizeof(r), cudaMemcpyDeviceToHost, s));
-    int code = read_status(c.status, s);
-    if (code) return set_error(code, "compress_rel: %s", status_text(code));
-    *out_bytes = r.total;
-    if (r.overflow) return set_error(QSIM_E_CAPACITY, "stream needs %llu bytes, cap is %zu",
-                                     (unsigned long long)r.total, cap);
-    return QSIM_OK;
+    return compress_call(c, d_amps, m, k, d_out, cap, out_bytes, s, true, "compress_rel");
 }
 
 int qsim_decompress_block(const void *d_in, size_t in_bytes, float *d_amps, uint32_t m, void *cuda_stream) {
@@ -3005,15 +2927,11 @@ int qsim_decompress_block(const void *d_in, size_t in_bytes, float *d_amps, uint
     int rc = ensure_device_ctx(c);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    BlockRef r{static_cast<const uint8_t *>(d_in), in_bytes};
-    uint32_t magic = 0;  // the format: QSZ1 or QSZR (any other value fails the kernel's header check)
-    if (in_bytes >= 4) {
-        CUDA_TRY(cudaMemcpyAsync(&magic, d_in, 4, cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-    }
-    CUDA_TRY(cudaMemcpyAsync(c.ref, &r, sizeof(r), cudaMemcpyHostToDevice, s));
-    launch_decode(c.ref, 1, int(m), reinterpret_cast<float2 *>(d_amps), nullptr, c.status, s, magic == kQszrMagic);
-    int code = read_status(c.status, s);
+    const BlockRef r{static_cast<const uint8_t *>(d_in), in_bytes};
+    c.call_host->status = QSIM_E_CUDA;
+    launch_decode_block(r, int(m), reinterpret_cast<float2 *>(d_amps), c.call, s);
+    int code = 0;
+    if ((rc = call_status(c, s, &code))) return rc;
     if (code) return set_error(code, "decompress: %s", status_text(code));
     return QSIM_OK;
 }

@@ -29,7 +29,7 @@ namespace {
 
 constexpr uint32_t kNoAllocMaxFrames = 1u << (QSIM_NOALLOC_MAX_M - kQszMaxFrameLog);
 constexpr size_t kLookbackBytes = size_t(kNoAllocMaxFrames) * sizeof(uint64_t);
-// layout of the tail: counters [0,16), status [16,20), target [32,56), result [64,96)
+// layout of the tail: counters [0,16), status [16,20), the call's record [32,48)
 constexpr size_t kTailBytes = 256;
 constexpr size_t kScratchBytes = kLookbackBytes + kTailBytes;
 
@@ -91,42 +91,30 @@ extern "C" int qsim_compress_block_noalloc(const float *d_amps, uint32_t m, doub
     unsigned char *tail = base + kLookbackBytes;
     uint32_t *counters = reinterpret_cast<uint32_t *>(tail);
     int *status = reinterpret_cast<int *>(tail + 16);
-    EncTarget *tgt = reinterpret_cast<EncTarget *>(tail + 32);
-    EncResult *res = reinterpret_cast<EncResult *>(tail + 64);
+    CallHost *record = reinterpret_cast<CallHost *>(tail + 32);
 
     // The array keeps the previous call's contents: clear the look-back words
     // of the frames this block uses and the whole tail (counters, status,
-    // result) so the encoder starts from zero.
+    // record) so the encoder starts from zero.
     const size_t nframes = size_t(qsz_nframes(int(m)));
     cudaError_t ce = cudaMemsetAsync(lookback, 0, nframes * sizeof(uint64_t), s);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(tail, 0, kTailBytes, s);
-    EncTarget t;
-    memset(&t, 0, sizeof(t));
-    t.ptr = static_cast<uint8_t *>(d_out);
-    t.cap = cap;
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(tgt, &t, sizeof(t), cudaMemcpyHostToDevice, s);
     if (ce != cudaSuccess) return set_error(QSIM_E_CUDA, "scratch set-up: %s", cudaGetErrorString(ce));
 
-    LookbackScratch scr{};
-    scr.state = lookback;
-    scr.ticket = counters;
-    scr.done = counters + 1;
-    scr.epoch = counters + 2;
-    launch_encode(reinterpret_cast<const float2 *>(d_amps), 1, int(m), e, tgt, res, 0, nullptr, nullptr, nullptr, scr,
-                  status, s);
+    launch_encode_block(reinterpret_cast<const float2 *>(d_amps), int(m), e, static_cast<uint8_t *>(d_out), cap,
+                        {lookback, counters, counters + 2}, {status, counters + 1, record}, s);
 
-    EncResult r;
-    int h_status = 0;
-    ce = cudaMemcpyAsync(&r, res, sizeof(r), cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, s);
+    CallHost r;
+    r.status = QSIM_E_CUDA;
+    ce = cudaMemcpyAsync(&r, record, sizeof(r), cudaMemcpyDeviceToHost, s);
     // Once the encoder is queued, wait for the stream on every path, failed copies included: the next call
     // (possibly on another stream) clears the shared array and must not do so under a running encoder.
     const cudaError_t se = cudaStreamSynchronize(s);
     if (ce == cudaSuccess) ce = se;
     if (ce != cudaSuccess) return set_error(QSIM_E_CUDA, "compress (no-alloc): %s", cudaGetErrorString(ce));
-    if (h_status) return set_error(h_status, "compress (no-alloc): device status %d", h_status);
-    *out_bytes = size_t(r.total);
-    if (r.overflow)
-        return set_error(QSIM_E_CAPACITY, "stream needs %llu bytes, cap is %zu", (unsigned long long)r.total, cap);
+    if (r.status) return set_error(r.status, "compress (no-alloc): device status %d", r.status);
+    *out_bytes = size_t(r.bytes);
+    if (r.bytes > cap)
+        return set_error(QSIM_E_CAPACITY, "stream needs %llu bytes, cap is %zu", (unsigned long long)r.bytes, cap);
     return QSIM_OK;
 }
