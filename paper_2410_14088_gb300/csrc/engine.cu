@@ -2487,7 +2487,7 @@ int qsim_mlp_loss_grad(const float *d_params, const float *d_x, const float *d_t
     DevBuf<float> dl;
     int rc = dl.alloc(1);
     if (rc) return rc;
-    rc = launch_mlp_loss_grad(d_params, d_x, kMlpIn, d_t, 1, nullptr, 0, uint32_t(batch), d_grad, dl.p, s);
+    rc = launch_mlp_loss_grad(d_params, d_x, kMlpIn, d_t, 1, uint32_t(batch), d_grad, dl.p, s);
     if (rc) return set_error(rc, "loss/grad launch failed");
     float h = 0;
     CUDA_TRY(cudaMemcpyAsync(&h, dl.p, sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -2550,10 +2550,11 @@ int qsim_predictor_train(const float *rows, size_t count, const qsim_train_confi
     int rc = predictor_ctx(&c);
     if (rc) return rc;
     const size_t rowf = kMlpIn + 1;
-    DevBuf<float> d_rows, p, g, m1, m2, loss;
+    DevBuf<float> d_rows, p, m1, m2;
+    DevBuf<double> loss;
     DevBuf<uint32_t> perm;
-    if ((rc = d_rows.alloc(count * rowf)) || (rc = p.alloc(kMlpParams)) || (rc = g.alloc(kMlpParams)) ||
-        (rc = m1.alloc(kMlpParams)) || (rc = m2.alloc(kMlpParams)) || (rc = loss.alloc(1)) || (rc = perm.alloc(count)))
+    if ((rc = d_rows.alloc(count * rowf)) || (rc = p.alloc(kMlpParams)) || (rc = m1.alloc(kMlpParams)) ||
+        (rc = m2.alloc(kMlpParams)) || (rc = loss.alloc(1)))
         return rc;
     cudaStream_t s = nullptr;
     CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
@@ -2574,30 +2575,40 @@ int qsim_predictor_train(const float *rows, size_t count, const qsim_train_confi
     CUDA_TRY(cudaMemcpyAsync(p.p, hp.data(), kMlpParams * sizeof(float), cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemsetAsync(m1.p, 0, kMlpParams * sizeof(float), s));
     CUDA_TRY(cudaMemsetAsync(m2.p, 0, kMlpParams * sizeof(float), s));
-    std::vector<uint32_t> hperm(count);
-    int t = 0;
-    for (uint32_t ep = 0; ep < tc->epochs; ++ep) {
-        for (size_t i = 0; i < count; ++i) hperm[i] = uint32_t(i);
-        for (size_t i = count - 1; i > 0; --i) std::swap(hperm[i], hperm[splitmix_next(st) % (i + 1)]);
-        CUDA_TRY(cudaStreamSynchronize(s));  // hperm is reused: the previous upload must have landed
-        CUDA_TRY(cudaMemcpyAsync(perm.p, hperm.data(), count * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-        for (size_t b0 = 0; b0 < count; b0 += tc->batch) {
-            const uint32_t nb = uint32_t(std::min<size_t>(tc->batch, count - b0));
-            rc = launch_mlp_loss_grad(p.p, d_rows.p, rowf, d_rows.p + kMlpIn, rowf, perm.p, uint32_t(b0), nb, g.p,
-                                      nullptr, s);
-            if (rc) { cudaStreamDestroy(s); return set_error(rc, "loss/grad launch failed"); }
-            launch_adam(p.p, g.p, m1.p, m2.p, kMlpParams, ++t, tc->lr, 0.9f, 0.999f, 1e-8f, s);
-        }
+    CUDA_TRY(cudaMemsetAsync(loss.p, 0, sizeof(double), s));
+    // launches of whole epochs whose sample orders (shuffled on the host) take at most 16 MB, and of about 2^17 steps
+    // (under a second), one after another
+    const size_t steps = (count + tc->batch - 1) / tc->batch;  // of an epoch
+    const uint64_t most = std::min<uint64_t>((4ull << 20) / count, (1ull << 17) / steps);
+    const uint32_t per_launch = uint32_t(std::min<uint64_t>(tc->epochs, std::max<uint64_t>(1, most)));
+    std::vector<uint32_t> hperm(count * per_launch);
+    if ((rc = perm.alloc(hperm.size()))) {
+        cudaStreamDestroy(s);
+        return rc;
     }
-    rc = launch_mlp_loss_grad(p.p, d_rows.p, rowf, d_rows.p + kMlpIn, rowf, nullptr, 0, uint32_t(count), g.p, loss.p, s);
-    float hl = 0;
-    CUDA_TRY(cudaMemcpyAsync(&hl, loss.p, sizeof(float), cudaMemcpyDeviceToHost, s));
+    for (uint32_t ep = 0; ep < tc->epochs; ep += per_launch) {
+        const uint32_t ne = std::min(per_launch, tc->epochs - ep);
+        if (ep) CUDA_TRY(cudaStreamSynchronize(s));  // hperm is reused: the previous upload must have landed
+        for (uint32_t k = 0; k < ne; ++k) {
+            uint32_t *o = hperm.data() + size_t(k) * count;
+            for (size_t i = 0; i < count; ++i) o[i] = uint32_t(i);
+            for (size_t i = count - 1; i > 0; --i) std::swap(o[i], o[splitmix_next(st) % (i + 1)]);
+        }
+        CUDA_TRY(cudaMemcpyAsync(perm.p, hperm.data(), ne * count * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+        rc = launch_mlp_train(p.p, d_rows.p, uint32_t(rowf), perm.p, uint64_t(ne) * count, uint32_t(count), tc->batch,
+                              m1.p, m2.p, int(ep * steps), tc->lr, 0.9f, 0.999f, 1e-8f, s);
+        if (rc) { cudaStreamDestroy(s); return set_error(rc, "training launch failed"); }
+    }
+    rc = launch_mlp_loss(p.p, d_rows.p, uint32_t(rowf), count, loss.p, s);
+    if (rc) { cudaStreamDestroy(s); return set_error(rc, "loss launch failed"); }
+    double hl = 0;
+    CUDA_TRY(cudaMemcpyAsync(&hl, loss.p, sizeof(double), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaMemcpyAsync(c->pred_params, p.p, kMlpParams * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     cudaStreamDestroy(s);
     c->pred_bf16 = int(tc->bf16_inference);
     c->pred_ready = true;
-    if (final_loss) *final_loss = hl;
+    if (final_loss) *final_loss = double(float(hl));  // an FP32 value, as qsim_mlp_loss_grad's
     return QSIM_OK;
 }
 

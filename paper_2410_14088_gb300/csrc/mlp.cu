@@ -14,9 +14,12 @@
 // i.e. minus the log2 of the block's compression ratio.
 // Parameter layout (6913 floats): W1[64][41], b1[64], W2[64][64], b2[64],
 // W3[64], b3.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <atomic>
 
 #include "codec.cuh"
 #include "device_common.cuh"
@@ -108,115 +111,311 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
     if (j < nblocks) rows[uint64_t(j) * (IN + 1) + IN] = log2f(float(res[j].total)) - float(m + 3);
 }
 
-// Mean-squared-error loss 0.5/B sum (y - t)^2 and its gradient over a batch
-// of samples (perm selects them; null = 0..count-1), one CTA, deterministic:
-// every gradient entry is one thread's dot product over the batch.
-constexpr int CH = 64;  // samples per chunk
-__global__ void __launch_bounds__(256) k_mlp_loss_grad(const float *__restrict__ params, const float *__restrict__ x,
-                                                      uint32_t xstride, const float *__restrict__ t,
-                                                      uint32_t tstride, const uint32_t *__restrict__ perm,
-                                                      uint32_t start, uint32_t count, float *__restrict__ grad,
-                                                      float *__restrict__ loss_out) {
-    extern __shared__ float sm[];
-    float *w = sm;                  // NP
-    float *g = w + NP;              // NP
-    float *X = g + NP;              // CH x IN
-    float *A1 = X + CH * IN;        // CH x HID (pre-activation), then dH1
-    float *A2 = A1 + CH * HID;      // CH x HID (pre-activation), then dH2
-    float *H1 = A2 + CH * HID;      // CH x HID
-    float *dY = H1 + CH * HID;      // CH
-    __shared__ float s_loss;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int i = tid; i < NP; i += nt) {
-        w[i] = params[i];
-        g[i] = 0.f;
+// ---------------------------------------------------------------------------
+// Training. One cluster of eight CTAs runs a whole sequence of steps: each CTA takes an eighth of a batch's samples
+// through the forward and backward pass with its own copy of the weights in shared memory, the gradient is reduced
+// through distributed shared memory (each CTA sums an eighth of the parameters over the eight partials, in rank
+// order, so the result is deterministic), and the same CTA applies Adam to that eighth, whose moments it keeps in
+// registers, and writes the new weights into all eight copies. Two cluster barriers per step, no launch and no global
+// round trip. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases: latency bounds it, so the split is
+// the smallest that leaves every phase two outputs per thread (8 samples x 64 units on 256 threads). W2's rows are
+// padded to 65 words: both directions through it read conflict-free.
+// ---------------------------------------------------------------------------
+constexpr int CR = 8;                            // CTAs of the cluster
+constexpr int SB = 8;                            // samples a CTA takes at a time (one warp each in the output layer)
+constexpr int TT = 256;                          // threads
+constexpr int SHARD = 868;                       // parameters per CTA (8 x 868 >= NP), four per thread at most
+constexpr int W2S = HID + 1;
+
+struct __align__(16) TrainSmem {
+    float w1[HID * IN], b1[HID], w2[HID * W2S], b2[HID], w3[HID], b3[4];
+    float g[CR * SHARD];                         // partial gradient, flat parameter order
+    float h1[SB][HID], h2[SB][HID], d1[SB][HID], d2[SB][HID];
+    float x[SB * IN], t[SB], dy[SB], sq[SB];
+    float loss;
+};
+
+// parameter i's place in the weights' shared copy
+__device__ __forceinline__ float *train_weight(TrainSmem &S, int i) {
+    if (i < OB1) return S.w1 + i;
+    if (i < OW2) return S.b1 + (i - OB1);
+    if (i < OB2) return S.w2 + ((i - OW2) / HID) * W2S + (i - OW2) % HID;
+    if (i < OW3) return S.b2 + (i - OB2);
+    if (i < OB3) return S.w3 + (i - OW3);
+    return S.b3;
+}
+
+// The rows of the samples a CTA takes at once, two values per thread (IN features and the target per sample), held in
+// registers so that a step's rows are on their way while the step before it is computed.
+struct TrainRows {
+    float v[2];
+};
+__device__ __forceinline__ TrainRows train_fetch(const float *x, uint32_t xstride, const float *t, uint32_t tstride,
+                                                 const uint32_t *perm, uint64_t first, uint32_t n) {
+    TrainRows r{{0.f, 0.f}};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t i = threadIdx.x + TT * k, b = i / (IN + 1), j = i % (IN + 1);
+        if (b < n && b < uint32_t(SB)) {
+            const uint64_t s = perm ? __ldg(perm + first + b) : first + b;
+            r.v[k] = j < uint32_t(IN) ? __ldg(x + s * xstride + j) : __ldg(t + s * tstride);
+        }
     }
-    if (tid == 0) s_loss = 0.f;
+    return r;
+}
+__device__ __forceinline__ void train_put(TrainSmem &S, const TrainRows &r) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t i = threadIdx.x + TT * k, b = i / (IN + 1), j = i % (IN + 1);
+        if (b >= uint32_t(SB)) continue;
+        if (j < uint32_t(IN)) S.x[b * IN + j] = r.v[k];
+        else S.t[b] = r.v[k];
+    }
+}
+
+// Forward pass of the n (<= SB) samples in S.x; each sample's residual y - t to S.dy (0 past n). Ends unsynchronised:
+// warp b wrote sample b's.
+__device__ __forceinline__ void train_forward(TrainSmem &S, uint32_t n) {
+    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID, lane = tid & 31, warp = tid >> 5;
+    float a0 = S.b1[h], a1 = a0;
+#pragma unroll
+    for (int j = 0; j < IN; ++j) {
+        const float w = S.w1[h * IN + j];
+        a0 = fmaf(w, S.x[q * IN + j], a0);
+        a1 = fmaf(w, S.x[(q + 4) * IN + j], a1);
+    }
+    S.h1[q][h] = fmaxf(a0, 0.f);
+    S.h1[q + 4][h] = fmaxf(a1, 0.f);
     __syncthreads();
-    const float invB = 1.0f / float(count);
-    for (uint32_t c0 = 0; c0 < count; c0 += CH) {
-        const uint32_t nb = min(uint32_t(CH), count - c0);
-        for (uint32_t i = tid; i < nb * IN; i += nt) {
-            const uint32_t b = i / IN, jx = i % IN;
-            const uint32_t s = perm ? perm[start + c0 + b] : start + c0 + b;
-            X[b * IN + jx] = x[uint64_t(s) * xstride + jx];
+    a0 = a1 = S.b2[h];
+#pragma unroll 16
+    for (int j = 0; j < HID; ++j) {
+        const float w = S.w2[h * W2S + j];
+        a0 = fmaf(w, S.h1[q][j], a0);
+        a1 = fmaf(w, S.h1[q + 4][j], a1);
+    }
+    S.h2[q][h] = fmaxf(a0, 0.f);
+    S.h2[q + 4][h] = fmaxf(a1, 0.f);
+    __syncthreads();
+    float y = S.w3[lane] * S.h2[warp][lane] + S.w3[lane + 32] * S.h2[warp][lane + 32];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+    if (lane == 0) S.dy[warp] = uint32_t(warp) < n ? y + S.b3[0] - S.t[warp] : 0.f;
+    __syncwarp();
+}
+
+// Gradient of the chunk in S.x (n samples), written to S.g (first) or added; the loss terms go to S.loss.
+__device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_b, bool first) {
+    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID, lane = tid & 31, warp = tid >> 5;
+    train_forward(S, n);
+    {
+        const float r = S.dy[warp], dy = r * inv_b;
+        __syncwarp();
+        if (lane == 0) {
+            S.dy[warp] = dy;
+            S.sq[warp] = 0.5f * r * dy;
         }
+        S.d2[warp][lane] = S.h2[warp][lane] > 0.f ? dy * S.w3[lane] : 0.f;
+        S.d2[warp][lane + 32] = S.h2[warp][lane + 32] > 0.f ? dy * S.w3[lane + 32] : 0.f;
+    }
+    __syncthreads();
+    // back through W2
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll 16
+    for (int i = 0; i < HID; ++i) {
+        const float w = S.w2[i * W2S + h];
+        a0 = fmaf(S.d2[q][i], w, a0);
+        a1 = fmaf(S.d2[q + 4][i], w, a1);
+    }
+    S.d1[q][h] = S.h1[q][h] > 0.f ? a0 : 0.f;
+    S.d1[q + 4][h] = S.h1[q + 4][h] > 0.f ? a1 : 0.f;
+    auto put = [&](int i, float v) { S.g[i] = first ? v : S.g[i] + v; };
+    {  // W2: a 4 x 4 tile per thread
+        const int r0 = (tid >> 4) * 4, c0 = (tid & 15) * 4;
+        float acc[4][4] = {};
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            const float4 d = *reinterpret_cast<const float4 *>(&S.d2[b][r0]);
+            const float4 x = *reinterpret_cast<const float4 *>(&S.h1[b][c0]);
+            const float dd[4] = {d.x, d.y, d.z, d.w}, xx[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], xx[j], acc[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) put(OW2 + (r0 + i) * HID + c0 + j, acc[i][j]);
+    }
+    if (q == 0) {  // W3, b2 and b3
+        float gw = 0.f, gb = 0.f;
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            gw = fmaf(S.dy[b], S.h2[b][h], gw);
+            gb += S.d2[b][h];
+        }
+        put(OW3 + h, gw);
+        put(OB2 + h, gb);
+        if (h == 0) {
+            float g3 = 0.f, ls = 0.f;
+#pragma unroll
+            for (int b = 0; b < SB; ++b) {
+                g3 += S.dy[b];
+                ls += S.sq[b];
+            }
+            put(OB3, g3);
+            S.loss = first ? ls : S.loss + ls;
+        }
+    }
+    __syncthreads();
+    {  // W1 and b1: four threads per unit
+        const int u = tid >> 2, j0 = tid & 3;
+        float d[SB];
+#pragma unroll
+        for (int b = 0; b < SB; ++b) d[b] = S.d1[b][u];
+        for (int j = j0; j < IN; j += 4) {
+            float v = 0.f;
+#pragma unroll
+            for (int b = 0; b < SB; ++b) v = fmaf(d[b], S.x[b * IN + j], v);
+            put(OW1 + u * IN + j, v);
+        }
+        if (j0 == 0) {
+            float v = 0.f;
+#pragma unroll
+            for (int b = 0; b < SB; ++b) v += d[b];
+            put(OB1 + u, v);
+        }
+    }
+}
+
+// Samples [r0, r0 + per) of a batch of nb belong to rank r.
+__device__ __forceinline__ void train_share(uint32_t nb, uint32_t rank, uint32_t &r0, uint32_t &per) {
+    const uint32_t each = (nb + CR - 1) / CR;
+    r0 = min(each * rank, nb);
+    per = min(each, nb - r0);
+}
+
+// `total` samples in the order of perm (null: as they are), `batch` per step; TRAIN: Adam's step number t0 + 1 and on,
+// params, m1 and m2 updated at the end. Else one batch of all samples: gradient and loss.
+template <bool TRAIN>
+__global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
+    k_mlp_train(float *__restrict__ params, const float *__restrict__ x, uint32_t xstride, const float *__restrict__ t,
+                uint32_t tstride, const uint32_t *__restrict__ perm, uint64_t total, uint32_t epoch, uint32_t batch,
+                float *__restrict__ m1, float *__restrict__ m2, int t0, float lr, float beta1, float beta2, float eps,
+                float *__restrict__ grad, float *__restrict__ loss_out) {
+    extern __shared__ __align__(16) uint8_t train_smem[];
+    TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const uint32_t rank = cl.block_rank();
+    const int tid = threadIdx.x;
+    for (int i = tid; i < NP; i += TT) *train_weight(S, i) = params[i];
+    // the thread's parameters: SHARD * rank + tid + 256 k
+    float p[4] = {}, ma[4] = {}, mb[4] = {};
+    int own[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int o = tid + TT * k, i = SHARD * int(rank) + o;
+        own[k] = o < SHARD && i < NP ? i : -1;
+        if (own[k] >= 0) {
+            p[k] = params[own[k]];
+            if (TRAIN) {
+                ma[k] = m1[own[k]];
+                mb[k] = m2[own[k]];
+            }
+        }
+    }
+    // batches do not cross epochs: the last one of an epoch may be smaller
+    uint64_t pos = 0;
+    uint32_t in_epoch = 0;
+    int step = t0;
+    auto batch_at = [&](uint32_t e) { return min(batch, epoch - e); };
+    uint32_t r0, per;
+    train_share(batch_at(0), rank, r0, per);
+    TrainRows next = train_fetch(x, xstride, t, tstride, perm, r0, min(per, uint32_t(SB)));
+    cl.sync();
+    while (pos < total) {
+        const uint32_t nb = batch_at(in_epoch);
+        train_share(nb, rank, r0, per);
+        const float inv_b = 1.0f / float(nb);
+        const uint64_t npos = pos + nb;
+        const uint32_t nin = in_epoch + nb == epoch ? 0u : in_epoch + nb;
+        uint32_t nr0 = 0, nper = 0;
+        if (npos < total) train_share(batch_at(nin), rank, nr0, nper);
+        // at least one chunk: a rank without samples contributes zeros
+        for (uint32_t c = 0; c == 0 || c < per; c += SB) {
+            const uint32_t n = per > c ? min(per - c, uint32_t(SB)) : 0u;
+            train_put(S, next);
+            __syncthreads();
+            if (c + SB < per)
+                next = train_fetch(x, xstride, t, tstride, perm, pos + r0 + c + SB, min(per - c - SB, uint32_t(SB)));
+            else if (npos < total)
+                next = train_fetch(x, xstride, t, tstride, perm, npos + nr0, min(nper, uint32_t(SB)));
+            train_chunk(S, n, inv_b, c == 0);
+            __syncthreads();
+        }
+        cl.sync();  // every rank's partial gradient is complete
+        ++step;
+        const float c1 = TRAIN ? 1.f - powf(beta1, float(step)) : 1.f, c2 = TRAIN ? 1.f - powf(beta2, float(step)) : 1.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (own[k] < 0) continue;
+            float g = 0.f;
+#pragma unroll
+            for (int r = 0; r < CR; ++r) g += cl.map_shared_rank(S.g, r)[own[k]];
+            if (TRAIN) {
+                const float a = beta1 * ma[k] + (1.f - beta1) * g;
+                const float b = beta2 * mb[k] + (1.f - beta2) * g * g;
+                ma[k] = a;
+                mb[k] = b;
+                p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+                float *w = train_weight(S, own[k]);
+#pragma unroll
+                for (int r = 0; r < CR; ++r) *cl.map_shared_rank(w, r) = p[k];
+            } else {
+                grad[own[k]] = g;
+            }
+        }
+        if (!TRAIN && rank == 0 && tid == 0 && loss_out) {
+            float ls = 0.f;
+            for (int r = 0; r < CR; ++r) ls += *cl.map_shared_rank(&S.loss, r);
+            *loss_out = ls;
+        }
+        cl.sync();  // the new weights are in every copy, the partials have been read
+        pos = npos;
+        in_epoch = nin;
+    }
+    if (TRAIN) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (own[k] >= 0) {
+                params[own[k]] = p[k];
+                m1[own[k]] = ma[k];
+                m2[own[k]] = mb[k];
+            }
+    }
+}
+
+// Loss 0.5/B sum (y - t)^2 over count samples, summed in FP64 (loss: one zero double).
+__global__ void __launch_bounds__(TT) k_mlp_loss(const float *__restrict__ params, const float *__restrict__ x,
+                                                 uint32_t xstride, const float *__restrict__ t, uint32_t tstride,
+                                                 uint64_t count, double *loss) {
+    extern __shared__ __align__(16) uint8_t train_smem[];
+    TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
+    for (int i = threadIdx.x; i < NP; i += TT) *train_weight(S, i) = params[i];
+    double sum = 0;
+    for (uint64_t c = uint64_t(blockIdx.x) * SB; c < count; c += uint64_t(gridDim.x) * SB) {
+        const uint32_t n = uint32_t(min(count - c, uint64_t(SB)));
+        train_put(S, train_fetch(x, xstride, t, tstride, nullptr, c, n));
         __syncthreads();
-        for (uint32_t i = tid; i < nb * HID; i += nt) {  // layer 1
-            const uint32_t b = i / HID, h = i % HID;
-            float a = w[OB1 + h];
-            for (int jx = 0; jx < IN; ++jx) a = fmaf(w[OW1 + h * IN + jx], X[b * IN + jx], a);
-            A1[b * HID + h] = a;
-            H1[b * HID + h] = fmaxf(a, 0.f);
-        }
+        train_forward(S, n);
         __syncthreads();
-        for (uint32_t i = tid; i < nb * HID; i += nt) {  // layer 2
-            const uint32_t b = i / HID, h = i % HID;
-            float a = w[OB2 + h];
-            for (int jx = 0; jx < HID; ++jx) a = fmaf(w[OW2 + h * HID + jx], H1[b * HID + jx], a);
-            A2[b * HID + h] = a;
-        }
-        __syncthreads();
-        for (uint32_t b = tid; b < nb; b += nt) {  // output and dL/dy
-            float y = w[OB3];
-            for (int h = 0; h < HID; ++h) y = fmaf(w[OW3 + h], fmaxf(A2[b * HID + h], 0.f), y);
-            const uint32_t s = perm ? perm[start + c0 + b] : start + c0 + b;
-            const float r = y - t[uint64_t(s) * tstride];
-            dY[b] = r * invB;
-            atomicAdd(&s_loss, 0.5f * r * r * invB);
-        }
-        __syncthreads();
-        // output layer gradients, and dH2 (overwrites A2 after use: keep the ReLU mask)
-        for (int h = tid; h < HID; h += nt) {
-            float gw = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) gw = fmaf(dY[b], fmaxf(A2[b * HID + h], 0.f), gw);
-            g[OW3 + h] += gw;
-        }
-        if (tid == 0) {
-            float gb = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) gb += dY[b];
-            g[OB3] += gb;
-        }
-        __syncthreads();
-        for (uint32_t i = tid; i < nb * HID; i += nt) {
-            const uint32_t b = i / HID, h = i % HID;
-            A2[b * HID + h] = A2[b * HID + h] > 0.f ? dY[b] * w[OW3 + h] : 0.f;  // dA2
-        }
-        __syncthreads();
-        for (int i = tid; i < HID * HID; i += nt) {  // gW2 = dA2^T H1
-            const int h = i / HID, jx = i % HID;
-            float a = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) a = fmaf(A2[b * HID + h], H1[b * HID + jx], a);
-            g[OW2 + i] += a;
-        }
-        for (int h = tid; h < HID; h += nt) {
-            float a = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) a += A2[b * HID + h];
-            g[OB2 + h] += a;
-        }
-        __syncthreads();
-        for (uint32_t i = tid; i < nb * HID; i += nt) {  // dA1 = (dA2 W2) * relu'(A1)
-            const uint32_t b = i / HID, jx = i % HID;
-            float a = 0.f;
-            for (int h = 0; h < HID; ++h) a = fmaf(A2[b * HID + h], w[OW2 + h * HID + jx], a);
-            A1[b * HID + jx] = A1[b * HID + jx] > 0.f ? a : 0.f;
-        }
-        __syncthreads();
-        for (int i = tid; i < HID * IN; i += nt) {  // gW1 = dA1^T X
-            const int h = i / IN, jx = i % IN;
-            float a = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) a = fmaf(A1[b * HID + h], X[b * IN + jx], a);
-            g[OW1 + i] += a;
-        }
-        for (int h = tid; h < HID; h += nt) {
-            float a = 0.f;
-            for (uint32_t b = 0; b < nb; ++b) a += A1[b * HID + h];
-            g[OB1 + h] += a;
-        }
+        if (threadIdx.x == 0)
+            for (int b = 0; b < SB; ++b) sum += 0.5 * double(S.dy[b]) * double(S.dy[b]) / double(count);
         __syncthreads();
     }
-    for (int i = tid; i < NP; i += nt) grad[i] = g[i];
-    if (tid == 0 && loss_out) *loss_out = s_loss;
+    if (threadIdx.x == 0) atomicAdd(loss, sum);
 }
 
 // Adam (Kingma & Ba 2015) with bias correction; t is 1-based.
@@ -232,8 +431,6 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
     m2[i] = b;
     p[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
 }
-
-size_t grad_smem_bytes() { return sizeof(float) * (2 * NP + CH * IN + 3 * CH * HID + CH); }
 
 }  // namespace
 
@@ -255,18 +452,48 @@ void launch_log_targets(const EncResult *res, uint32_t nblocks, int m, float *ro
     count_launch();
 }
 
+// dynamic shared memory of a training kernel, allowed once per kernel and device
+template <auto *kernel>
+static int train_smem_ok() {
+    static std::atomic<uint64_t> done{0};  // per kernel: a bit per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return QSIM_E_CUDA;
+    if (done.load() >> (dev & 63) & 1) return QSIM_OK;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(TrainSmem))) != cudaSuccess)
+        return QSIM_E_CUDA;
+    done.fetch_or(1ull << (dev & 63));
+    return QSIM_OK;
+}
+
 int launch_mlp_loss_grad(const float *params, const float *x, uint32_t xstride, const float *t, uint32_t tstride,
-                         const uint32_t *perm, uint32_t start, uint32_t count, float *grad, float *loss,
-                         cudaStream_t s) {
-    static bool attr = false;
-    const size_t smem = grad_smem_bytes();
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_mlp_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess)
-            return QSIM_E_CUDA;
-        attr = true;
-    }
-    k_mlp_loss_grad<<<1, 256, smem, s>>>(params, x, xstride, t, tstride, perm, start, count, grad, loss);
+                         uint32_t count, float *grad, float *loss, cudaStream_t s) {
+    int rc = train_smem_ok<k_mlp_train<false>>();
+    if (rc) return rc;
+    k_mlp_train<false><<<CR, TT, sizeof(TrainSmem), s>>>(const_cast<float *>(params), x, xstride, t, tstride, nullptr,
+                                                         count, count, count, nullptr, nullptr, 0, 0.f, 0.f, 0.f, 0.f,
+                                                         grad, loss);
+    count_launch();
+    return QSIM_OK;
+}
+
+int launch_mlp_train(float *params, const float *rows, uint32_t stride, const uint32_t *perm, uint64_t total,
+                     uint32_t epoch, uint32_t batch, float *m1, float *m2, int t0, float lr, float beta1, float beta2,
+                     float eps, cudaStream_t s) {
+    int rc = train_smem_ok<k_mlp_train<true>>();
+    if (rc) return rc;
+    k_mlp_train<true><<<CR, TT, sizeof(TrainSmem), s>>>(params, rows, stride, rows + IN, stride, perm, total, epoch,
+                                                        batch, m1, m2, t0, lr, beta1, beta2, eps, nullptr, nullptr);
+    count_launch();
+    return QSIM_OK;
+}
+
+int launch_mlp_loss(const float *params, const float *rows, uint32_t stride, uint64_t count, double *loss,
+                    cudaStream_t s) {
+    int rc = train_smem_ok<k_mlp_loss>();
+    if (rc) return rc;
+    const uint64_t chunks = (count + SB - 1) / SB;
+    k_mlp_loss<<<unsigned(chunks < 304 ? chunks : 304), TT, sizeof(TrainSmem), s>>>(params, rows, stride, rows + IN,
+                                                                                   stride, count, loss);
     count_launch();
     return QSIM_OK;
 }

@@ -63,8 +63,15 @@ void launch_predict_sizes(const uint32_t *hist, uint32_t nblocks, uint32_t G, in
                           const float *params, int bf16, float *pred, float *feat_out, cudaStream_t s);
 void launch_log_targets(const EncResult *res, uint32_t nblocks, int m, float *rows, cudaStream_t s);
 int launch_mlp_loss_grad(const float *params, const float *x, uint32_t xstride, const float *t, uint32_t tstride,
-                         const uint32_t *perm, uint32_t start, uint32_t count, float *grad, float *loss,
-                         cudaStream_t s);
+                         uint32_t count, float *grad, float *loss, cudaStream_t s);
+// Adam steps t0 + 1 .. over `total` samples (rows of `stride` floats: features, then the target) in the order of perm,
+// `batch` per step, a shorter one at the end of every `epoch` samples; params, m1 and m2 are updated
+int launch_mlp_train(float *params, const float *rows, uint32_t stride, const uint32_t *perm, uint64_t total,
+                     uint32_t epoch, uint32_t batch, float *m1, float *m2, int t0, float lr, float beta1, float beta2,
+                     float eps, cudaStream_t s);
+// 0.5/count sum (y - t)^2 added to *loss
+int launch_mlp_loss(const float *params, const float *rows, uint32_t stride, uint64_t count, double *loss,
+                    cudaStream_t s);
 void launch_adam(float *p, const float *g, float *m1, float *m2, uint32_t n, int t, float lr, float beta1, float beta2,
                  float eps, cudaStream_t s);
 
