@@ -81,22 +81,33 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_decode_block(BlockRef in, int m
     call_done(res, tm, gridDim.x);
 }
 
-// Random access: frame frames[i].y of block frames[i].x (slot table entry) decoded into out + i * F; no leading phase
-// ops, no histogram.
+// Random access: amplitude idx[i] of a state to out[i], one warp each. It reads the frame's widths and the words of two
+// chunks (about 0.5 KB) instead of decoding the frame's 4096 amplitudes to memory first, so its cost, about 0.3 ns an
+// index, stays below that of moving the index and the amplitude to and from the host however many a frame is asked for.
 template <bool REL>
-__global__ void __launch_bounds__(kTeamMax, 5) k_decode_frames(const BlockSlot *__restrict__ table,
-                                                               const uint2 *__restrict__ frames, uint32_t nitems,
-                                                               int m, float2 *__restrict__ out, int *status) {
-    extern __shared__ __align__(16) uint8_t tile[];
+__global__ void __launch_bounds__(256) k_amplitudes(const BlockSlot *__restrict__ table,
+                                                    const uint64_t *__restrict__ idx, uint64_t count, int m,
+                                                    float2 *__restrict__ out, int *status) {
     const FrameGeom g = geom(m);
-    __shared__ TeamSmem S;
-    const Team tm{threadIdx.x, blockDim.x, 1};
-    for (uint64_t item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const uint2 bf = frames[item];
-        const BlockSlot sl = table[bf.x];
-        decode_frame_team<0, REL>(tm, S, tile, sl.ptr, sl.bytes, g, m, bf.y, out + item * g.F, nullptr, status, nullptr,
-                                  nullptr, 0, nullptr, 0, 0);
-        tm.sync();
+    for (uint64_t i = blockIdx.x * 8ull + (threadIdx.x >> 5); i < count; i += gridDim.x * 8ull) {
+        const uint64_t x = idx[i];
+        const uint32_t local = uint32_t(x & ((1ull << m) - 1));
+        const BlockSlot sl = table[x >> m];
+        const float2 v = amplitude_warp<REL>(sl.ptr, sl.bytes, g, m, local >> g.fl, local & (g.F - 1u), status);
+        if ((threadIdx.x & 31) == 0) out[i] = v;
+    }
+}
+
+// the same from an uncompressed store
+__global__ void k_amplitudes_raw(const BlockSlot *__restrict__ table, const uint64_t *__restrict__ idx, uint64_t count,
+                                 int m, float2 *__restrict__ out, int *status) {
+    for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < count; i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint64_t x = idx[i];
+        const BlockSlot sl = table[x >> m];
+        float2 v = make_float2(0.f, 0.f);
+        if (sl.ptr == nullptr || sl.bytes < (8ull << m)) raise_status(status, QSIM_E_CORRUPT);
+        else v = reinterpret_cast<const float2 *>(sl.ptr)[x & ((1ull << m) - 1)];
+        out[i] = v;
     }
 }
 
@@ -478,14 +489,14 @@ void launch_decode_block(const BlockRef &in, int m, float2 *out, const CallResul
     count_launch();
 }
 
-void launch_decode_frames(const BlockSlot *table, const uint2 *frames, uint32_t nitems, int m, float2 *out,
-                          int *status, cudaStream_t s, bool rel) {
-    const TeamShape ts = team_shape(m);
-    const unsigned grid = grid_for(nitems, kMaxGrid);
-    if (rel)
-        k_decode_frames<true><<<grid, ts.threads, ts.smem, s>>>(table, frames, nitems, m, out, status);
+void launch_amplitudes(const BlockSlot *table, const uint64_t *idx, uint64_t count, int m, float2 *out, int *status,
+                       cudaStream_t s, uint32_t codec) {
+    if (codec == QSIM_CODEC_NONE)
+        k_amplitudes_raw<<<grid_for((count + 255) / 256, 152 * 16), 256, 0, s>>>(table, idx, count, m, out, status);
+    else if (codec == QSIM_CODEC_QSZR)
+        k_amplitudes<true><<<grid_for((count + 7) / 8, 152 * 64), 256, 0, s>>>(table, idx, count, m, out, status);
     else
-        k_decode_frames<false><<<grid, ts.threads, ts.smem, s>>>(table, frames, nitems, m, out, status);
+        k_amplitudes<false><<<grid_for((count + 7) / 8, 152 * 64), 256, 0, s>>>(table, idx, count, m, out, status);
     count_launch();
 }
 

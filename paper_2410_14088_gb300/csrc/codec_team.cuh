@@ -114,19 +114,18 @@ __device__ __forceinline__ bool call_done(const CallResult &res, const Team &tm,
 // ---------------------------------------------------------------------------
 // decode
 // ---------------------------------------------------------------------------
-// Frame f of one block (stream sp, `bytes` long) into dst (F amplitudes). tile: team_tile_bytes(C), 16-byte aligned.
-// hist_j (nullable): the block's code-width histogram. pre_*: leading phase ops, as decode of a stage. The team may
-// reuse tile and S after its next sync().
-template <int NP, bool REL>
-__device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, uint8_t *tile, const uint8_t *sp,
-                                                  uint64_t bytes, const FrameGeom &g, int m, uint32_t f,
-                                                  float2 *__restrict__ dst, uint32_t *hist_j, int *status,
-                                                  const OpDev *pre_ops, const uint2 *pre_ab, uint32_t npre,
-                                                  const float2 *__restrict__ mats, uint64_t wbase, uint64_t gb) {
-    const uint32_t t = tm.t, lane = t & 31u, warp = t >> 5, nw = tm.n >> 5, C = g.C;
+struct FrameHead {
+    bool ok;          // the stream's header and frame f's offsets are consistent
+    uint32_t fa, fb;  // frame f's image in the stream
+    int e;            // step exponent (QSZ1) or code shift (QSZR)
+};
+
+// Header and offsets of frame f of a stream, read and checked by a whole warp, one load per lane.
+template <bool REL>
+__device__ __forceinline__ FrameHead frame_head(const uint8_t *sp, uint64_t bytes, const FrameGeom &g, int m, uint32_t f) {
+    const uint32_t lane = threadIdx.x & 31u, C = g.C;
     const uint32_t padw = (2u * C + 15u) & ~15u;
     const uint32_t tbp = REL ? ((((2u * C + 3u) / 4u) + 15u) & ~15u) : 0u;  // sign chunk types, padded
-    // ---- header and offsets, one load per lane (every warp of the team reads them) ----
     const bool can = sp != nullptr && !(reinterpret_cast<uintptr_t>(sp) & 15) && bytes >= g.data_start;
     uint32_t hv = 0;
     if (can) {
@@ -141,16 +140,120 @@ __device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, u
     const uint32_t w2 = __shfl_sync(kFull, hv, 2), nfr = __shfl_sync(kFull, hv, 3);
     const uint64_t total = uint64_t(__shfl_sync(kFull, hv, 4)) | (uint64_t(__shfl_sync(kFull, hv, 5)) << 32);
     const uint64_t rsv = uint64_t(__shfl_sync(kFull, hv, 6)) | (uint64_t(__shfl_sync(kFull, hv, 7)) << 32);
-    const uint32_t o0 = __shfl_sync(kFull, hv, 8), fa = __shfl_sync(kFull, hv, 9);
-    const uint32_t fb = __shfl_sync(kFull, hv, 10), on = __shfl_sync(kFull, hv, 11);
-    const int e = REL ? int(uint8_t(w2 >> 16)) : int(int8_t(uint8_t(w2 >> 16)));
-    bool ok = can && magic == (REL ? kQszrMagic : kQszMagic) && w1 == 1u && (w2 & 0xff) == uint32_t(m) &&
-              ((w2 >> 8) & 0xff) == uint32_t(g.fl) && (w2 >> 24) == 0 && nfr == g.nframes && rsv == 0 &&
-              (REL ? (e >= kQszrKMin && e <= kQszrKMax) : (e >= kQszEMin && e <= kQszEMax)) && total <= bytes &&
-              total >= g.data_start && o0 == g.data_start && on == total && fb >= fa && fb <= total &&
-              fa >= g.data_start && !((fa | fb) & 15u) &&
-              (fb == fa || (fb - fa >= padw + tbp && fb - fa <= team_tile_bytes(C)));
-    const uint32_t flen = ok ? fb - fa : 0u;
+    const uint32_t o0 = __shfl_sync(kFull, hv, 8), on = __shfl_sync(kFull, hv, 11);
+    FrameHead r;
+    r.fa = __shfl_sync(kFull, hv, 9);
+    r.fb = __shfl_sync(kFull, hv, 10);
+    r.e = REL ? int(uint8_t(w2 >> 16)) : int(int8_t(uint8_t(w2 >> 16)));
+    r.ok = can && magic == (REL ? kQszrMagic : kQszMagic) && w1 == 1u && (w2 & 0xff) == uint32_t(m) &&
+           ((w2 >> 8) & 0xff) == uint32_t(g.fl) && (w2 >> 24) == 0 && nfr == g.nframes && rsv == 0 &&
+           (REL ? (r.e >= kQszrKMin && r.e <= kQszrKMax) : (r.e >= kQszEMin && r.e <= kQszEMax)) && total <= bytes &&
+           total >= g.data_start && o0 == g.data_start && on == total && r.fb >= r.fa && r.fb <= total &&
+           r.fa >= g.data_start && !((r.fa | r.fb) & 15u) &&
+           (r.fb == r.fa || (r.fb - r.fa >= padw + tbp && r.fb - r.fa <= team_tile_bytes(C)));
+    return r;
+}
+
+// The amplitude at index `at` of frame f of one block, decoded by a whole warp from the two chunks that hold it: the
+// widths are read 8 per lane and scanned for the chunks' words, each plane's words go through one transpose, and the
+// codes up to the index are summed. Every lane returns the amplitude.
+template <bool REL>
+__device__ __forceinline__ float2 amplitude_warp(const uint8_t *sp, uint64_t bytes, const FrameGeom &g, int m,
+                                                 uint32_t f, uint32_t at, int *status) {
+    const uint32_t lane = threadIdx.x & 31u, C = g.C, c = at >> 5, l = at & 31u;
+    const uint32_t padw = (2u * C + 15u) & ~15u;
+    const uint32_t tbp = REL ? ((((2u * C + 3u) / 4u) + 15u) & ~15u) : 0u;
+    const FrameHead fh = frame_head<REL>(sp, bytes, g, m, f);
+    bool ok = fh.ok;
+    const uint32_t flen = ok ? fh.fb - fh.fa : 0u;
+    if (ok && !flen) return make_float2(0.f, 0.f);
+    const uint8_t *img = sp + fh.fa;
+    uint64_t wb = 0;  // widths 8 lane .. 8 lane + 7 (bytes past 2C are zero padding)
+    if (ok && 8u * lane < 2u * C) wb = *reinterpret_cast<const uint64_t *>(img + 8u * lane);
+    uint32_t sum = 0, mx = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        const uint32_t w = uint32_t(wb >> (8u * k)) & 0xffu;
+        sum += w;
+        mx = max(mx, w);
+    }
+    uint32_t tw = 0, cnt = 0;  // REL: sign chunk types 16 lane .. 16 lane + 15; stored words | run records << 16
+    if constexpr (REL) {
+        if (ok && 16u * lane < 2u * C) tw = *reinterpret_cast<const uint32_t *>(img + padw + 4u * lane);
+        const uint32_t hi = tw & 0xAAAAAAAAu, t3 = hi & (tw << 1);
+        cnt = __popc(hi ^ t3) | (__popc(t3) << 16);
+    }
+    uint32_t incl = sum, icnt = cnt;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint32_t a = __shfl_up_sync(kFull, incl, o);
+        const uint32_t b = REL ? __shfl_up_sync(kFull, icnt, o) : 0u;
+        if (lane >= o) {
+            incl += a;
+            icnt += b;
+        }
+    }
+    const uint32_t words = __shfl_sync(kFull, incl, 31), ctot = __shfl_sync(kFull, icnt, 31);
+    const uint32_t n2 = ctot & 0xffffu, n3 = ctot >> 16, signs = REL ? (4u * n2 + 2u * n3 + 15u) & ~15u : 0u;
+    ok = ok && __reduce_max_sync(kFull, mx) <= 32 && words > 0 &&
+         uint64_t(flen) == padw + tbp + signs + ((4ull * words + 15) & ~15ull);
+    if (!ok) {
+        if (lane == 0) raise_status(status, QSIM_E_CORRUPT);
+        return make_float2(0.f, 0.f);
+    }
+    const uint32_t *pay = reinterpret_cast<const uint32_t *>(img + padw + tbp + signs);
+    float v[2];
+    bool bad = false;
+#pragma unroll
+    for (uint32_t p = 0; p < 2; ++p) {
+        const uint32_t i = p * C + c;  // the chunk among the frame's 2C
+        const uint64_t own = __shfl_sync(kFull, wb, i >> 3);
+        uint32_t off = __shfl_sync(kFull, incl - sum, i >> 3);
+        for (uint32_t k = 0; k < (i & 7u); ++k) off += uint32_t(own >> (8u * k)) & 0xffu;
+        const uint32_t w = uint32_t(own >> (8u * (i & 7u))) & 0xffu;
+        const uint32_t z = warp_bit_transpose(lane < w ? __ldg(pay + off + lane) : 0u, int(lane));
+        const int32_t q = __reduce_add_sync(kFull, lane <= l ? unzigzag(z) : 0);
+        if constexpr (REL) {
+            const uint32_t types = __shfl_sync(kFull, tw, i >> 4), s = 2u * (i & 15u);
+            const uint32_t before = __shfl_sync(kFull, icnt - cnt, i >> 4), below = (1u << s) - 1u;
+            const uint32_t t3 = types & 0xAAAAAAAAu & (types << 1), t2 = (types & 0xAAAAAAAAu) ^ t3;
+            const uint32_t ty = (types >> s) & 3u;
+            const uint32_t *mixw = reinterpret_cast<const uint32_t *>(img + padw + tbp);
+            uint32_t sw = ty == 1u ? 0xFFFFFFFFu : 0u;
+            if (ty == 2u) sw = __ldg(mixw + (before & 0xffffu) + __popc(t2 & below));
+            if (ty == 3u) {
+                bool rok;
+                const uint16_t *runw = reinterpret_cast<const uint16_t *>(mixw + n2);
+                sw = sign_run_word(__ldg(runw + (before >> 16) + __popc(t3 & below)), rok);
+                bad |= !rok;
+            }
+            bad |= uint32_t(q) > (kQszrMaxU >> fh.e);
+            v[p] = __uint_as_float((uint32_t(q) << fh.e) ^ (((sw >> l) & 1u) << 31));
+        } else {
+            v[p] = float(q) * exp2i(fh.e);
+        }
+    }
+    if (bad && lane == 0) raise_status(status, QSIM_E_CORRUPT);
+    return make_float2(v[0], v[1]);
+}
+
+// Frame f of one block (stream sp, `bytes` long) into dst (F amplitudes). tile: team_tile_bytes(C), 16-byte aligned.
+// hist_j (nullable): the block's code-width histogram. pre_*: leading phase ops, as decode of a stage. The team may
+// reuse tile and S after its next sync().
+template <int NP, bool REL>
+__device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, uint8_t *tile, const uint8_t *sp,
+                                                  uint64_t bytes, const FrameGeom &g, int m, uint32_t f,
+                                                  float2 *__restrict__ dst, uint32_t *hist_j, int *status,
+                                                  const OpDev *pre_ops, const uint2 *pre_ab, uint32_t npre,
+                                                  const float2 *__restrict__ mats, uint64_t wbase, uint64_t gb) {
+    const uint32_t t = tm.t, lane = t & 31u, warp = t >> 5, nw = tm.n >> 5, C = g.C;
+    const uint32_t padw = (2u * C + 15u) & ~15u;
+    const uint32_t tbp = REL ? ((((2u * C + 3u) / 4u) + 15u) & ~15u) : 0u;  // sign chunk types, padded
+    const FrameHead fh = frame_head<REL>(sp, bytes, g, m, f);  // every warp of the team reads it
+    const uint32_t fa = fh.fa;
+    const int e = fh.e;
+    bool ok = fh.ok;
+    const uint32_t flen = ok ? fh.fb - fa : 0u;
     // ---- the frame's image to shared memory ----
     for (uint32_t i = t; i < flen / 16u; i += tm.n) team_cp16(tile + 16u * i, sp + fa + 16u * i);
     team_cp_wait();

@@ -91,3 +91,14 @@ def test_state_decompress_into_an_8_byte_aligned_tensor(codec):
     room = torch.zeros((1 << 15) + 1, dtype=torch.complex64, device="cuda")
     st.decompress(out=room[1:])
     assert torch.equal(room[1:], want)
+
+
+@pytest.mark.parametrize("codec", [qsim.CODEC_QSZ1, qsim.CODEC_QSZR, qsim.CODEC_NONE])
+@pytest.mark.parametrize("m", [5, 6, 7, 8, 10, 12, 14])
+def test_single_amplitudes_equal_the_decompressed_state(m, codec):
+    """Every index of a small state, unsorted and repeated, decoded one by one from its chunks."""
+    c = inputs.random_brick(15, 4, 21)
+    c.gates += [inputs.X(3), inputs.CP(2, 9, 0.3)]
+    st = qsim.run(qsim.plan_stages(c, m=m, inner=2, k=4, codec=codec))
+    idx = np.concatenate([np.random.default_rng(m).permutation(1 << 15), [0, 0, (1 << 15) - 1]]).astype(np.uint64)
+    np.testing.assert_array_equal(st.amplitudes(idx), st.decompress().cpu().numpy()[idx.astype(np.int64)])
