@@ -637,6 +637,88 @@ static int upload_plan(const qsim_plan *p, PlanDev **out) {
             if (ps.T == 12)
                 for (uint32_t a = 0; a < P.op_count; ++a)
                     if (ops[P.op_begin + a].type == OP_DIAG) quad[a] = diag_quadratic(st.ops[ps.ops[a]], &qpoly[a]);
+            // The summed phase polynomial of the run headed by op a (angles in turns, 32-bit fixed point: 2^32 = one
+            // turn, so that sums wrap exactly) over 12 index bits, tile bit t at index bit pos[t]: G[t][t'] (t < t'),
+            // the run's quadratic part over tile bits 7..11 (Q7, 32 values) and 8..11 (Q8, 16), the linear
+            // coefficients A0[t], the constant C0, then *ncst records {t or -1, source, source or kNoSrc, coefficient}
+            // of the terms with bits constant over the tile (a working bit outside the tile, or 64 + an outer qubit):
+            // index bit t's linear coefficient, or (t = -1) the constant, gains the coefficient when those bits are 1.
+            // With reg (register passes) G leaves out the pairs of tile bits 7..11, word 205 is the mask of the index
+            // bits 0..6 that are tile bits 7..11, and word 206 the offset of a table T[r][u] after the records: the
+            // quadratic part over index bits 7..11 = u plus Q7 where the masked bits spell r (lowest first), so that
+            // the angles are those of the identity arrangement to the last bit.
+            auto poly_tables = [&](const PassDev &P, uint32_t a, const uint32_t *pos, bool reg, uint32_t *ncst) {
+                const uint32_t r = ops[P.op_begin + a].run;
+                double G[12][12] = {}, A0[12] = {}, C0 = 0;  // by tile bit
+                std::map<std::array<uint32_t, 3>, double> terms;
+                for (uint32_t d = 0; d < r; ++d) {
+                    const OpDev &rd = ops[P.op_begin + a + d];
+                    const DiagPoly &q = qpoly[a + d];
+                    C0 += q.c;
+                    for (uint32_t j = 0; j < rd.k; ++j) {
+                        if (rd.dtile[j] != 255) A0[rd.dtile[j]] += q.a[j];
+                        else terms[{kPolyConst, rd.dsrc[j], kNoSrc}] += q.a[j];
+                        for (uint32_t l = j + 1; l < rd.k; ++l) {
+                            const uint32_t tj = rd.dtile[j], tl = rd.dtile[l];
+                            if (tj != 255 && tl != 255) G[std::min(tj, tl)][std::max(tj, tl)] += q.g[j][l];
+                            else if (tj != 255) terms[{tj, rd.dsrc[l], kNoSrc}] += q.g[j][l];
+                            else if (tl != 255) terms[{tl, rd.dsrc[j], kNoSrc}] += q.g[j][l];
+                            else
+                                terms[{kPolyConst, std::min(rd.dsrc[j], rd.dsrc[l]), std::max(rd.dsrc[j], rd.dsrc[l])}] +=
+                                    q.g[j][l];
+                        }
+                    }
+                }
+                auto red = [](double t) {
+                    const double f = t - std::floor(t);
+                    return uint32_t(uint64_t(std::llround(f * 4294967296.0)) & 0xffffffffull);
+                };
+                std::vector<uint32_t> w(kPolyHeadWords, 0u);
+                for (uint32_t t = 0; t < 12; ++t)
+                    for (uint32_t t2 = t + 1; t2 < 12; ++t2)
+                        if (!reg || t < 7) w[12 * std::min(pos[t], pos[t2]) + std::max(pos[t], pos[t2])] = red(G[t][t2]);
+                for (uint32_t u = 0; u < 32; ++u) {
+                    double qv = 0, qv8 = 0;
+                    for (uint32_t b = 7; b < 12; ++b)
+                        for (uint32_t b2 = b + 1; b2 < 12; ++b2) {
+                            const bool on = ((u >> (b - 7)) & 1u) && ((u >> (b2 - 7)) & 1u);
+                            if (on) qv += G[b][b2];
+                            if (b >= 8 && u < 16 && ((u >> (b - 8)) & 1u) && ((u >> (b2 - 8)) & 1u)) qv8 += G[b][b2];
+                        }
+                    w[144 + u] = red(qv);
+                    if (u < 16) w[176 + u] = red(qv8);
+                }
+                for (uint32_t t = 0; t < 12; ++t) w[192 + pos[t]] = red(A0[t]);
+                w[204] = red(C0);
+                for (const auto &kv : terms)
+                    w.insert(w.end(), {kv.first[0] == kPolyConst ? kPolyConst : pos[kv.first[0]], kv.first[1],
+                                       kv.first[2], red(kv.second)});
+                *ncst = uint32_t(terms.size());
+                if (reg) {
+                    uint32_t tile_bit[12], rows[7], nr = 0;
+                    for (uint32_t t = 0; t < 12; ++t) tile_bit[pos[t]] = t;
+                    for (uint32_t t = 0; t < 7; ++t)
+                        if (tile_bit[t] >= 7) {
+                            w[205] |= 1u << t;
+                            rows[nr++] = tile_bit[t] - 7;
+                        }
+                    w[206] = uint32_t(w.size());
+                    for (uint32_t x = 0; x < (1u << nr); ++x)
+                        for (uint32_t u = 0; u < 32; ++u) {
+                            uint32_t high = 0, v = 0;
+                            for (uint32_t k = 0; k < nr; ++k) high |= ((x >> k) & 1u) << rows[k];
+                            for (uint32_t b = 0; b < 5; ++b) {
+                                if (!((u >> b) & 1u)) continue;
+                                if (tile_bit[7 + b] >= 7) high |= 1u << (tile_bit[7 + b] - 7);
+                                for (uint32_t b2 = b + 1; b2 < 5; ++b2)
+                                    if ((u >> b2) & 1u) v += w[12 * (7 + b) + 7 + b2];
+                            }
+                            w.push_back(v + w[144 + high]);
+                            if (u == 31) w.resize(w.size() + kRegRow - 32, 0u);
+                        }
+                }
+                return w;
+            };
             // runs of consecutive diagonal ops applied in one sweep: up to kDiagRun table ops, or any number of
             // polynomial ops (one phase per amplitude for the whole run; the head becomes an OP_POLY descriptor)
             for (uint32_t a = P.op_begin; a < P.op_begin + P.op_count;) {
@@ -665,64 +747,12 @@ static int upload_plan(const qsim_plan *p, PlanDev **out) {
                     const Op &op = st.ops[ps.ops[a]];
                     od.tab = kNoTab;
                     if (od.type == OP_POLY) {
-                        // the run's summed phase polynomial (angles in turns, 32-bit fixed point) over the tile bits t (the bits of a
-                        // 4096-amplitude tile): G[t][t'] (t < t'), the run's quadratic part over tile bits 7..11
-                        // (Q7, 32 values) and 8..11 (Q8, 16), the linear coefficients A0[t], the constant C0, then
-                        // records {t or -1, source, source or kNoSrc, coefficient} of the terms with bits constant
-                        // over the tile (a working bit outside the tile, or 64 + an outer qubit): tile bit t's linear
-                        // coefficient, or (t = -1) the constant, gains the coefficient when those bits are 1
-                        const uint32_t r = od.run;
-                        double G[12][12] = {}, A0[12] = {}, C0 = 0;
-                        std::map<std::array<uint32_t, 3>, double> terms;
-                        for (uint32_t d = 0; d < r; ++d) {
-                            const OpDev &rd = ops[P.op_begin + a + d];
-                            const DiagPoly &q = qpoly[a + d];
-                            C0 += q.c;
-                            for (uint32_t j = 0; j < rd.k; ++j) {
-                                if (rd.dtile[j] != 255) A0[rd.dtile[j]] += q.a[j];
-                                else terms[{kPolyConst, rd.dsrc[j], kNoSrc}] += q.a[j];
-                                for (uint32_t l = j + 1; l < rd.k; ++l) {
-                                    const uint32_t tj = rd.dtile[j], tl = rd.dtile[l];
-                                    if (tj != 255 && tl != 255) G[std::min(tj, tl)][std::max(tj, tl)] += q.g[j][l];
-                                    else if (tj != 255) terms[{tj, rd.dsrc[l], kNoSrc}] += q.g[j][l];
-                                    else if (tl != 255) terms[{tl, rd.dsrc[j], kNoSrc}] += q.g[j][l];
-                                    else
-                                        terms[{kPolyConst, std::min(rd.dsrc[j], rd.dsrc[l]),
-                                               std::max(rd.dsrc[j], rd.dsrc[l])}] += q.g[j][l];
-                                }
-                            }
-                        }
-                        // angles as 32-bit fixed point in turns (2^32 = one turn): sums wrap exactly modulo a turn
-                        auto red = [](double t) {
-                            const double f = t - std::floor(t);
-                            return uint32_t(uint64_t(std::llround(f * 4294967296.0)) & 0xffffffffull);
-                        };
-                        std::vector<uint32_t> w(kPolyHeadWords, 0u);
-                        for (uint32_t t = 0; t < 12; ++t)
-                            for (uint32_t t2 = t + 1; t2 < 12; ++t2) w[12 * t + t2] = red(G[t][t2]);
-                        for (uint32_t u = 0; u < 32; ++u) {
-                            double qv = 0, qv8 = 0;
-                            for (uint32_t b = 7; b < 12; ++b)
-                                for (uint32_t b2 = b + 1; b2 < 12; ++b2) {
-                                    const bool on = ((u >> (b - 7)) & 1u) && ((u >> (b2 - 7)) & 1u);
-                                    if (on) qv += G[b][b2];
-                                    if (b >= 8 && u < 16 && ((u >> (b - 8)) & 1u) && ((u >> (b2 - 8)) & 1u)) qv8 += G[b][b2];
-                                }
-                            w[144 + u] = red(qv);
-                            if (u < 16) w[176 + u] = red(qv8);
-                        }
-                        for (uint32_t t = 0; t < 12; ++t) w[192 + t] = red(A0[t]);
-                        w[204] = red(C0);
                         align16();
                         od.tab = uint32_t(pb.size() / 4);
-                        od.ncst = uint32_t(terms.size());
+                        const uint32_t same[12] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11};
+                        const std::vector<uint32_t> w = poly_tables(P, a, same, false, &od.ncst);
                         const uint8_t *wb = reinterpret_cast<const uint8_t *>(w.data());
                         pb.insert(pb.end(), wb, wb + 4 * w.size());
-                        for (const auto &kv : terms) {
-                            const uint32_t rec[4] = {kv.first[0], kv.first[1], kv.first[2], red(kv.second)};
-                            const uint8_t *rb = reinterpret_cast<const uint8_t *>(rec);
-                            pb.insert(pb.end(), rb, rb + 16);
-                        }
                     } else if (od.type == OP_DIAG && quad[a]) {
                         // inside a polynomial run: nothing of its own in the blob
                     } else if (od.type == OP_DIAG) {
@@ -849,6 +879,92 @@ static int upload_plan(const qsim_plan *p, PlanDev **out) {
                 memcpy(blob.data() + w0, pb.data(), pb.size());
             }
             P.mat_elems = (P.mat_elems + 1) & ~1u;
+            // The pass's form that keeps its tiles in registers, when every op is a width-5 dense op on tcgen05 or a
+            // polynomial run: the tables of gates_reg.cuh.
+            {
+                std::vector<uint32_t> dense, polys, steps;
+                bool fits = (P.umma & 1u) && !(P.umma & 8u);
+                for (uint32_t a = 0; a < P.op_count && fits; ++a) {
+                    const OpDev &od = ops[P.op_begin + a];
+                    if (od.type == OP_DENSE) {
+                        fits = od.k == 5;
+                        steps.push_back(uint32_t(dense.size()));
+                        dense.push_back(a);
+                    } else if (od.type == OP_POLY) {
+                        steps.push_back(kRegPoly | uint32_t(polys.size()));
+                        polys.push_back(a);
+                    } else {
+                        fits = od.type == OP_DIAG && quad[a];  // inside a run
+                    }
+                }
+                if (fits && !dense.empty() && polys.size() <= kRegMaxPoly && steps.size() <= kRegMaxSteps) {
+                    // index bits of dense op d: 0..6 its complement (the group number's bits), 7..11 its matrix bits
+                    auto index_bits = [&](uint32_t d, uint32_t *bits) {
+                        const OpDev &od = ops[P.op_begin + dense[d]];
+                        for (uint32_t t = 0; t < 7; ++t) bits[t] = od.comp[t];
+                        for (uint32_t t = 0; t < 5; ++t) bits[7 + t] = od.tq[t];
+                    };
+                    auto swz = [](uint32_t i) { return i ^ (((i >> 4) ^ (i >> 8) ^ (i >> 12)) & 15u); };
+                    const uint32_t nd = uint32_t(dense.size()), np = uint32_t(polys.size());
+                    std::vector<uint32_t> w(kRegHead + kRegDense * nd, 0u);
+                    w[0] = uint32_t(steps.size());
+                    w[1] = nd;
+                    w[2] = np;
+                    for (size_t i = 0; i < steps.size(); ++i) w[4 + i] = steps[i];
+                    uint32_t bits[12];
+                    for (uint32_t d = 0; d < nd; ++d) {
+                        index_bits(d, bits);
+                        uint32_t *o = w.data() + kRegHead + kRegDense * d;
+                        for (uint32_t x = 0; x < 64; ++x)
+                            for (uint32_t t = 0; t < 6; ++t) {
+                                if (!((x >> t) & 1u)) continue;
+                                o[x] ^= swz(1u << bits[t]);
+                                if (t < 1) o[64 + x] ^= swz(1u << bits[6 + t]);
+                            }
+                        for (uint32_t t = 0; t < 5; ++t) o[128 + t] = swz(1u << bits[7 + t]);
+                        o[133] = ops[P.op_begin + dense[d]].bfrag;
+                        // a thread's neighbours hold the tile's lowest three bits, unless the op takes them: then its
+                        // groups pass through the staged tile at that end
+                        bool low = false;
+                        for (uint32_t t = 0; t < 5; ++t) low |= bits[7 + t] < 3;
+                        for (uint32_t t = 0; t < 12; ++t) {
+                            if (d == 0) w[28 + t] = ps.tile_pos[bits[t]];
+                            if (d == nd - 1) w[40 + t] = ps.tile_pos[bits[t]];
+                        }
+                        if (d == 0 && !low) w[3] |= kRegIn;
+                        if (d == nd - 1 && !low) w[3] |= kRegOut;
+                    }
+                    uint32_t before = 0;  // dense ops before the step
+                    for (uint32_t st2 : steps) {
+                        if (!(st2 & kRegPoly)) {
+                            ++before;
+                            continue;
+                        }
+                        uint32_t pos[12];
+                        index_bits(before ? before - 1 : 0, bits);
+                        for (uint32_t t = 0; t < 12; ++t) pos[bits[t]] = t;
+                        const uint32_t p2 = st2 & 0xffffu;
+                        uint32_t ncst = 0;
+                        const std::vector<uint32_t> t = poly_tables(P, polys[p2], pos, true, &ncst);
+                        w[52 + p2] = uint32_t(w.size());
+                        w[56 + p2] = ncst;
+                        w.insert(w.end(), t.begin(), t.end());
+                    }
+                    w.resize((w.size() + 3) & ~size_t(3), 0u);
+                    P.reg_off = uint32_t(blob.size());
+                    P.reg_words = uint32_t(w.size());
+                    P.reg_dense = nd;
+                    P.reg_poly = np;
+                    P.reg_flags = w[3];
+                    const size_t w0 = blob.size();
+                    blob.resize(w0 + w.size() / 4);
+                    memcpy(blob.data() + w0, w.data(), w.size() * 4);
+                    if (!reg_pass_fits(P, int(p->cfg.prec))) {
+                        blob.resize(w0);
+                        P.reg_words = 0;
+                    }
+                }
+            }
             sd.passes_host.push_back(P);
             passes.push_back(P);
         }

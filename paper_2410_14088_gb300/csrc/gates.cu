@@ -24,6 +24,7 @@
 #include "device_common.cuh"
 #include "gates.cuh"
 #include "gates_dev.cuh"
+#include "gates_reg.cuh"
 
 namespace qsim {
 
@@ -132,6 +133,53 @@ void launch_pass_k(dim3 grid, size_t smem, cudaStream_t s, float2 *wv, uint32_t 
     launch_pass_ku<KMAX, PREC, false>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status);
 }
 
+template <int PREC, int H>
+__global__ void __launch_bounds__(128 * H, 4 / H)
+    k_pass_reg(float2 *__restrict__ wv, uint32_t W, uint64_t ntiles, const __grid_constant__ PassDev P,
+               const uint4 *__restrict__ blob, const uint32_t *__restrict__ bfr, const uint64_t *__restrict__ gbase,
+               uint32_t *ctr, int *status) {
+    extern __shared__ float4 dyn_smem[];
+    __shared__ RegSmem<H> S;
+    pass_reg_tiles<PREC, H>(wv, W, ntiles, P, blob, bfr, gbase, S, reinterpret_cast<uint8_t *>(dyn_smem), ctr, status);
+}
+
+// Shared memory a CTA of k_pass_reg may take for two (H = 2) to be resident: 228 KB per SM, 1 KB reserved per CTA, and
+// RegSmem.
+constexpr uint32_t kRegSmemTwo = 228u * 512u - 1024u - uint32_t(sizeof(RegSmem<2>)) - 64u;
+
+// Two tiles per CTA when every dense op's B operand fits beside them at two CTAs per SM (four tiles in flight, B read
+// once per CTA); else one tile per CTA and B reloaded per op.
+template <int PREC>
+bool reg_two(const PassDev &P) {
+    return reg_shape<PREC, 2>(P.reg_dense, P.reg_poly, P.reg_flags, P.reg_words).bytes <= kRegSmemTwo;
+}
+
+template <int PREC, int H>
+void launch_reg(uint64_t ntiles, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
+                const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaFuncSetAttribute(k_pass_reg<PREC, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_pass_reg<PREC, H>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             int(cudaSharedmemCarveoutMaxShared));
+        attr_set = true;
+    }
+    const uint32_t smem = reg_shape<PREC, H>(P.reg_dense, P.reg_poly, P.reg_flags, P.reg_words).bytes;
+    const uint64_t by_smem = (228u * 1024u) / (smem + sizeof(RegSmem<H>) + 1024u);
+    const uint64_t per_sm = std::max<uint64_t>(1, std::min<uint64_t>(by_smem, 4 / H));
+    // twice the resident CTAs, as launch_pass_ku
+    const uint64_t want = (ntiles + H - 1) / H, resident = 2 * per_sm * num_sms();
+    k_pass_reg<PREC, H><<<unsigned(std::min(want, resident)), 128 * H, smem, s>>>(wv, W, ntiles, P, blob, bfr, gbase,
+                                                                                 ctr, status);
+}
+
+template <int PREC>
+void launch_reg_prec(uint64_t ntiles, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
+                     const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {
+    if (reg_two<PREC>(P)) launch_reg<PREC, 2>(ntiles, s, wv, W, P, blob, bfr, gbase, ctr, status);
+    else launch_reg<PREC, 1>(ntiles, s, wv, W, P, blob, bfr, gbase, ctr, status);
+}
+
 template <int PREC>
 void launch_pass_prec(uint32_t kmax, dim3 grid, size_t smem, cudaStream_t s, float2 *wv, uint32_t W,
                       const PassDev &P, const uint4 *blob, const float2 *mats, const uint32_t *bfr,
@@ -230,6 +278,17 @@ size_t pass_smem_bytes(const PassDev &P) {
            size_t(P.mat_elems) * sizeof(float2);
 }
 
+// (the reload form keeps three CTAs per SM up to 75 KB each)
+bool reg_pass_fits(const PassDev &P, int prec) {
+    constexpr uint32_t most = 228u * 1024u / 3u - 1024u - uint32_t(sizeof(RegSmem<1>)) - 64u;
+    if (prec == QSIM_PREC_TF32)
+        return reg_two<QSIM_PREC_TF32>(P) ||
+               reg_shape<QSIM_PREC_TF32, 1>(P.reg_dense, P.reg_poly, P.reg_flags, P.reg_words).bytes <= most;
+    return prec == QSIM_PREC_BF16X3 &&
+           (reg_two<QSIM_PREC_BF16X3>(P) ||
+            reg_shape<QSIM_PREC_BF16X3, 1>(P.reg_dense, P.reg_poly, P.reg_flags, P.reg_words).bytes <= most);
+}
+
 void build_umma_b(const double *u, uint32_t *out) {
     constexpr uint32_t D = 32;
     for (uint32_t n = 0; n < 2 * D; ++n)
@@ -280,6 +339,15 @@ void launch_pass(float2 *wv, uint32_t W, uint32_t ngroups, const PassDev *pass_h
                  const float2 *mats_dev, const uint32_t *bfr_dev, const uint64_t *gbase_dev, int prec,
                  cudaStream_t s, uint32_t *ctr, int *status) {
     const PassDev &P = *pass_host;
+    if (P.reg_words) {
+        const uint64_t ntiles = uint64_t(ngroups) << P.nout;
+        if (prec == QSIM_PREC_TF32)
+            launch_reg_prec<QSIM_PREC_TF32>(ntiles, s, wv, W, P, blob_dev, bfr_dev, gbase_dev, ctr, status);
+        else
+            launch_reg_prec<QSIM_PREC_BF16X3>(ntiles, s, wv, W, P, blob_dev, bfr_dev, gbase_dev, ctr, status);
+        count_launch();
+        return;
+    }
     const size_t smem = pass_smem_bytes(P);
     dim3 grid(1u << P.nout, ngroups);
     const uint32_t kmax = P.kmax;

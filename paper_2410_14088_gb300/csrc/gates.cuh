@@ -25,6 +25,9 @@ struct PassDev {
                              // swizzled form); bit 1: test hook, no MMA is issued or committed to the mbarrier;
                              // bit 2: split-BF16 B operands (three parts, 24 KB); bit 3: a TF32 width-6 op
                              // (B operand 64 KB, 128 TMEM columns)
+    // the pass's form that keeps its tiles in registers (gates_reg.cuh), 0 words when it has none: tables at reg_off (in
+    // 16-byte words) of the plan's blob array, their 32-bit words, dense ops, diagonal runs and kRegIn / kRegOut
+    uint32_t reg_off, reg_words, reg_dense, reg_poly, reg_flags;
     uint64_t out_mask;       // working-index mask of the non-tile bits
     uint32_t tile_pos[16];   // working bit of tile bit t (ascending)
     uint32_t out_pos[32];    // working bit of CTA-index bit t
@@ -71,6 +74,19 @@ constexpr uint32_t kNoSrc = 0xffffffffu;      // term record: no second source b
 constexpr uint32_t kNoTab = 0xffffffffu;
 constexpr uint32_t kPassBlobMax = 40960;    // bytes of one pass blob (shared memory next to the tile)
 
+// Tables of a register pass (32-bit words, in the plan's blob array at PassDev::reg_off):
+//   0 steps, 1 dense ops, 2 diagonal runs, 3 flags (1: first op's groups straight from memory, 2: last op's to memory)
+//   4.. the steps in order: dense op d, or kRegPoly | run p
+//   28.. / 40.. working bits of the first / last dense op's index-group bits (7) and matrix bits (5)
+//   52.. / 56.. word offset and record count of run p
+//   64 + 136 d: dense op d: swizzled group bases (128, as OpDev::dlut), swizzled offsets of its matrix bits (5), the
+//       word offset of its B operand in the plan's B array
+//   runs: kPolyHeadWords words as OP_POLY's, in the index bits of the dense op before it (else after it): bits 0..6 the
+//       group number's, 7..11 the matrix bits; its term records; its table T (words 205 and 206 of the head)
+constexpr uint32_t kRegHead = 64, kRegDense = 136, kRegMaxSteps = 24, kRegMaxPoly = 4, kRegPoly = 0x10000u;
+constexpr uint32_t kRegRow = 33;  // words per row of a run's table T: rows read by one warp fall on different banks
+constexpr uint32_t kRegIn = 1u, kRegOut = 2u;
+
 // wv: ngroups consecutive working vectors of 2^W amplitudes; gbase[g] is the
 // full-index value of group g's outer bits.
 // B-fragment tables (tensor-core precisions): the real matrix U_r^T of every
@@ -105,6 +121,9 @@ void build_umma_b3(const double *u_interleaved, uint32_t *out);
 void launch_pass(float2 *wv, uint32_t W, uint32_t ngroups, const PassDev *pass_host, const uint4 *blob_dev,
                  const float2 *mats_dev, const uint32_t *bfr_dev, const uint64_t *gbase_dev, int prec,
                  cudaStream_t s, uint32_t *ctr, int *status);
+
+// whether a pass with register tables (reg_words) gets at least two CTAs' worth of threads per SM in that form
+bool reg_pass_fits(const PassDev &P, int prec);
 
 // dynamic shared memory of one tile pass (tile, B operand and alignment when on tcgen05, blob, matrices)
 size_t pass_smem_bytes(const PassDev &P);
