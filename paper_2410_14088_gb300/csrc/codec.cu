@@ -143,15 +143,7 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_encode(float2 *wv, uint32_t nbl
         double err = r.err_sq, nrm = r.norm_sq;
         bool last = true;
         if (g.nframes > 1) {
-            if (r.len) {
-                uint4 *pay = reinterpret_cast<uint4 *>(frame), *side = reinterpret_cast<uint4 *>(fr.side + item * fr.side_bytes);
-                const uint4 *img = reinterpret_cast<const uint4 *>(tile);
-                const uint32_t h = r.head / 16u, n = r.len / 16u;
-                for (uint32_t i = tm.t; i < n; i += tm.n) {
-                    if (i < h) side[i] = img[i];
-                    else pay[i - h] = img[i];
-                }
-            }
+            stage_frame(tm, tile, r, frame, fr.side + item * fr.side_bytes);
             if (tm.t == 0) {
                 fr.len[item] = r.len;
                 if (REL) fr.head[item] = r.head;
@@ -169,56 +161,29 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_encode(float2 *wv, uint32_t nbl
             }
         }
         if (last && tm.t == 0) {
-            EncTarget t{};
-            if (keep_fitting) t = tgt[j];
-            if (!keep_fitting || t.ptr == nullptr || total > t.cap) {
-                if (keep_fitting && acc) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
-                reserve_slot(total, dev, host, &t, status);
-                tgt[j] = t;
-            }
+            const EncTarget t = reserve_block(total, keep_fitting != 0, tgt + j, dev, host, acc, status);
             EncResult out{};
             out.err_sq = err;
             out.norm_sq = nrm;
-            const bool fits = t.ptr != nullptr && total <= t.cap;  // false after a failed reservation only
-            if (g.nframes == 1) {
-                out.total = total;
-                out.overflow = fits ? 0u : 1u;
-                if (fits) {
-                    BlockSlot *sl = table + (ids ? ids[j] : j);
-                    sl->ptr = t.ptr;
-                    sl->bytes = total;
-                    sl->tier = t.tier;
-                }
-                S.bc = fits ? reinterpret_cast<uint64_t>(t.ptr) : 0ull;
-            } else {
+            if (g.nframes == 1)
+                S.bc = reinterpret_cast<uint64_t>(finish_single_frame(total, t, out, table + (ids ? ids[j] : j), acc));
+            else
                 arrive[j] = 0;
-            }
             res[j] = out;
             if (acc) {
                 atomicAdd(&acc->err_sq, err);
                 atomicAdd(&acc->norm_sq, nrm);
-                if (g.nframes == 1) {
-                    if (fits) count_block(acc, total, t);
-                    else atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
-                }
             }
         }
         tm.sync();
         if (g.nframes == 1) {
-            uint8_t *out = reinterpret_cast<uint8_t *>(S.bc);
-            if (out) {
-                for (uint32_t i = tm.t; i < uint32_t(g.data_start) / 4u; i += tm.n)
-                    reinterpret_cast<uint32_t *>(out)[i] = header_word(i, REL, g, m, e, 0, r.len);
-                uint4 *d = reinterpret_cast<uint4 *>(out + g.data_start);
-                for (uint32_t i = tm.t; i < r.len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
-            }
+            store_single_frame<REL>(tm, tile, g, m, e, r.len, reinterpret_cast<uint8_t *>(S.bc));
             tm.sync();
         }
     }
 }
 
-// Second step of blocks of several frames (C = 128): frame f's image (side record, then the words over its amplitudes)
-// copied to its offset in the block's slot. The block's last frame writes the header, the table slot and the totals.
+// Second step of blocks of several frames (C = 128), one CTA per frame (copy_frame_team).
 template <bool REL>
 __global__ void __launch_bounds__(kTeamMax) k_frame_copy(const float2 *__restrict__ wv, uint32_t nblocks, int m, int e,
                                                          const EncTarget *__restrict__ tgt,
@@ -227,41 +192,13 @@ __global__ void __launch_bounds__(kTeamMax) k_frame_copy(const float2 *__restric
                                                          BlockSlot *__restrict__ table, StageAccum *acc,
                                                          FrameRecords fr) {
     const FrameGeom g = geom(m);
+    const Team tm{threadIdx.x, kTeamMax, 1};
     const uint64_t items = uint64_t(nblocks) * g.nframes;
     for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
-        const uint32_t len = fr.len[item], off = fr.off[item], head = REL ? fr.head[item] : 256u;
-        const EncTarget t = tgt[j];
-        const bool fits = t.ptr != nullptr && uint64_t(off) + len <= t.cap;
-        if (fits && len) {
-            const uint4 *side = reinterpret_cast<const uint4 *>(fr.side + item * fr.side_bytes);
-            const uint4 *pay = reinterpret_cast<const uint4 *>(wv + (uint64_t(j) << m) + uint64_t(f) * g.F);
-            uint4 *d = reinterpret_cast<uint4 *>(t.ptr + off);
-            const uint32_t h = head / 16u, n = len / 16u;
-#pragma unroll 4
-            for (uint32_t i = threadIdx.x; i < n; i += kTeamMax) d[i] = i < h ? side[i] : pay[i - h];
-        }
-        if (threadIdx.x == 0) {
-            if (!fits) atomicOr(&res[j].overflow, 1u);
-            if (t.ptr && g.data_start <= t.cap) reinterpret_cast<uint32_t *>(t.ptr + 32)[f] = off;
-            if (f == g.nframes - 1) {
-                const uint64_t total = uint64_t(off) + len;
-                res[j].total = total;
-                if (t.ptr && total <= t.cap) {
-                    uint32_t *h32 = reinterpret_cast<uint32_t *>(t.ptr);
-                    for (uint32_t i = 0; i < 8; ++i) h32[i] = header_word(i, REL, g, m, e, f, uint32_t(total - g.data_start));
-                    for (uint32_t i = 8 + g.nframes; i < uint32_t(g.data_start) / 4u; ++i)
-                        h32[i] = i == 8 + g.nframes ? uint32_t(total) : 0u;
-                    BlockSlot *sl = table + (ids ? ids[j] : j);
-                    sl->ptr = t.ptr;
-                    sl->bytes = total;
-                    sl->tier = t.tier;
-                    if (acc) count_block(acc, total, t);
-                } else if (acc) {
-                    atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
-                }
-            }
-        }
+        copy_frame_team<REL>(tm, wv + (uint64_t(j) << m) + uint64_t(f) * g.F, fr.side + item * fr.side_bytes, fr.len[item],
+                             REL ? fr.head[item] : 256u, fr.off[item], g, m, e, f, tgt[j], res + j,
+                             table + (ids ? ids[j] : j), acc);
     }
 }
 

@@ -44,12 +44,16 @@ struct TeamSmem {
     uint32_t hist[32];
 };
 
-// n threads (a multiple of 32, numbered t) meeting on hardware barrier `bar`
+// n threads (a multiple of 32, numbered t) meeting on hardware barrier `bar` (1 to 4; unused by a team of one warp)
 struct Team {
     uint32_t t, n, bar;
     __device__ __forceinline__ void sync() const {
+        // barrier ids 1 to 4 as constants: an id in a register would reserve all sixteen for the CTA
         if (n == 32u) __syncwarp();
-        else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n) : "memory");
+        else if (bar == 1u) asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory");
+        else if (bar == 2u) asm volatile("bar.sync 2, %0;" ::"r"(n) : "memory");
+        else if (bar == 3u) asm volatile("bar.sync 3, %0;" ::"r"(n) : "memory");
+        else asm volatile("bar.sync 4, %0;" ::"r"(n) : "memory");
     }
 };
 
@@ -730,6 +734,24 @@ __device__ __forceinline__ uint32_t block_offsets_team(const Team &tm, TeamSmem 
     return run;
 }
 
+// Reserve block j's slot for `total` bytes (thread 0). keep: it keeps the slot reserved for it beforehand when it fits,
+// and is counted as overflowed when it does not.
+__device__ __forceinline__ EncTarget reserve_block(uint32_t total, bool keep, EncTarget *tgt_j, const ArenaDev &dev,
+                                                   const ArenaDev &host, StageAccum *acc, int *status) {
+    EncTarget t{};
+    if (keep) {
+        t.ptr = reinterpret_cast<uint8_t *>(__ldcg(reinterpret_cast<const unsigned long long *>(&tgt_j->ptr)));
+        t.cap = __ldcg(reinterpret_cast<const unsigned long long *>(&tgt_j->cap));
+        t.tier = __ldcg(&tgt_j->tier);
+    }
+    if (!keep || t.ptr == nullptr || total > t.cap) {
+        if (keep && acc) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+        reserve_slot(total, dev, host, &t, status);
+        *tgt_j = t;
+    }
+    return t;
+}
+
 // 32-bit word i of a stream's header and offset table (data_start bytes) for a block whose frames up to f0 are empty,
 // frame f0 has len bytes and the later ones are empty
 __device__ __forceinline__ uint32_t header_word(uint32_t i, bool rel, const FrameGeom &g, int m, int e, uint32_t f0,
@@ -752,6 +774,82 @@ __device__ __forceinline__ void count_block(StageAccum *acc, uint64_t total, con
     atomicAdd(reinterpret_cast<unsigned long long *>(&acc->reserved_bytes), t.cap);
     if (t.tier) atomicAdd(reinterpret_cast<unsigned long long *>(&acc->host_bytes), t.cap);
     atomicAdd(reinterpret_cast<unsigned long long *>(&acc->blocks), 1ull);
+}
+
+// A one-frame block (header, offsets and the frame's image in the tile) to its slot `out` (null: nothing).
+template <bool REL>
+__device__ __forceinline__ void store_single_frame(const Team &tm, const uint8_t *tile, const FrameGeom &g, int m, int e,
+                                                   uint32_t len, uint8_t *out) {
+    if (!out) return;
+    for (uint32_t i = tm.t; i < uint32_t(g.data_start) / 4u; i += tm.n)
+        reinterpret_cast<uint32_t *>(out)[i] = header_word(i, REL, g, m, e, 0, len);
+    uint4 *d = reinterpret_cast<uint4 *>(out + g.data_start);
+    for (uint32_t i = tm.t; i < len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
+}
+
+// Thread 0 after a one-frame block's slot is known: result, table slot and totals. Returns the slot, null when the
+// reservation failed.
+__device__ __forceinline__ uint8_t *finish_single_frame(uint32_t total, const EncTarget &t, EncResult &out,
+                                                        BlockSlot *slot, StageAccum *acc) {
+    const bool fits = t.ptr != nullptr && total <= t.cap;
+    out.total = total;
+    out.overflow = fits ? 0u : 1u;
+    if (fits) {
+        slot->ptr = t.ptr;
+        slot->bytes = total;
+        slot->tier = t.tier;
+        if (acc) count_block(acc, total, t);
+    } else if (acc) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+    }
+    return fits ? t.ptr : nullptr;
+}
+
+// The frame's image from the tile to where the copy step finds it: the bit-plane words over the frame's own amplitudes
+// (they never need more room), the part before them to the side record.
+__device__ __forceinline__ void stage_frame(const Team &tm, const uint8_t *tile, const EncFrame &r, float2 *frame,
+                                            uint8_t *side) {
+    uint4 *pay = reinterpret_cast<uint4 *>(frame), *s = reinterpret_cast<uint4 *>(side);
+    const uint4 *img = reinterpret_cast<const uint4 *>(tile);
+    const uint32_t h = r.head / 16u, n = r.len / 16u;  // n = 0 for an all-zero frame
+    for (uint32_t i = tm.t; i < n; i += tm.n) {
+        if (i < h) s[i] = img[i];
+        else pay[i - h] = img[i];
+    }
+}
+
+// Second step of blocks of several frames: frame f's staged image (read through L2) to its offset in the block's slot t;
+// the block's last frame writes the header, the table slot and the totals. 128 threads.
+template <bool REL>
+__device__ __forceinline__ void copy_frame_team(const Team &tm, const float2 *frame, const uint8_t *side, uint32_t len,
+                                                uint32_t head, uint32_t off, const FrameGeom &g, int m, int e, uint32_t f,
+                                                const EncTarget &t, EncResult *res_j, BlockSlot *slot, StageAccum *acc) {
+    const bool fits = t.ptr != nullptr && uint64_t(off) + len <= t.cap;
+    if (fits && len) {
+        const uint4 *s = reinterpret_cast<const uint4 *>(side), *pay = reinterpret_cast<const uint4 *>(frame);
+        uint4 *d = reinterpret_cast<uint4 *>(t.ptr + off);
+        const uint32_t h = head / 16u, n = len / 16u;
+#pragma unroll 4
+        for (uint32_t i = tm.t; i < n; i += tm.n) d[i] = __ldcg(i < h ? s + i : pay + (i - h));
+    }
+    if (tm.t != 0) return;
+    if (!fits) atomicOr(&res_j->overflow, 1u);
+    if (t.ptr && g.data_start <= t.cap) reinterpret_cast<uint32_t *>(t.ptr + 32)[f] = off;
+    if (f != g.nframes - 1) return;
+    const uint64_t total = uint64_t(off) + len;
+    res_j->total = total;
+    if (t.ptr && total <= t.cap) {
+        uint32_t *h32 = reinterpret_cast<uint32_t *>(t.ptr);
+        for (uint32_t i = 0; i < 8; ++i) h32[i] = header_word(i, REL, g, m, e, f, uint32_t(total - g.data_start));
+        for (uint32_t i = 8 + g.nframes; i < uint32_t(g.data_start) / 4u; ++i)
+            h32[i] = i == 8 + g.nframes ? uint32_t(total) : 0u;
+        slot->ptr = t.ptr;
+        slot->bytes = total;
+        slot->tier = t.tier;
+        if (acc) count_block(acc, total, t);
+    } else if (acc) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&acc->overflow_blocks), 1ull);
+    }
 }
 
 }  // namespace cdev

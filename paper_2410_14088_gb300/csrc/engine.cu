@@ -1337,9 +1337,14 @@ static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
 struct PBlockBufs {
     DevBuf<EncTarget> tgt;
     DevBuf<EncResult> res;
-    DevBuf<uint64_t> sizes;
     DevBuf<uint32_t> hist;
 };
+
+// SV groups of a stage that the persistent kernel takes as one unit: about 2^22 amplitudes (a power of two that divides
+// the stage's groups, a power of two itself)
+static uint32_t unit_groups(const StageDev &sd) {
+    return uint32_t(std::min<uint64_t>(sd.ngroups, sd.W < 22 ? 1ull << (22 - sd.W) : 1ull));
+}
 
 static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cudaStream_t main, int *status,
                           Profiler &prof, const DeviceCtx &dctx, uint64_t slot_budget_amps) {
@@ -1367,7 +1372,7 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
     for (const SegRef &sr : order) {
         const RunCtx &R = *rs[sr.c];
         const StageDev &sd = R.pd->stages[sr.si];
-        total_groups += sd.ngroups;
+        total_groups += sd.ngroups / unit_groups(sd);
         for (const PassDev &ps : sd.passes_host) {
             max_pass_bytes = std::max(max_pass_bytes, (size_t(1) << ps.T) * sizeof(float2) + size_t(ps.blob_words) * 16 +
                                                           size_t(ps.mat_elems) * sizeof(float2) +
@@ -1385,15 +1390,14 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         const RunCtx &R = *rs[c];
         bb[c].reset(new PBlockBufs());
         PBlockBufs &b = *bb[c];
-        if ((rc = b.tgt.alloc(R.nblocks)) || (rc = b.res.alloc(R.nblocks)) || (rc = b.sizes.alloc(R.nblocks)) ||
+        if ((rc = b.tgt.alloc(R.nblocks)) || (rc = b.res.alloc(R.nblocks)) ||
             (R.predict && (rc = b.hist.alloc(R.nblocks * 32))))
             return rc;
-        CUDA_TRY(cudaMemsetAsync(b.sizes.p, 0, R.nblocks * sizeof(uint64_t), main));
         if (R.predict) CUDA_TRY(cudaMemsetAsync(b.hist.p, 0, R.nblocks * 32 * sizeof(uint32_t), main));
     }
-    // Working-vector slots, planned per launch: one ring of slots per working-vector size (2^W amplitudes),
-    // each ring about slot_budget_amps large (at least 2 slots, at most the launch's groups of that size);
-    // a group takes the next slot of its ring and waits for the slot's previous group.
+    // Working-vector slots, planned per launch: one ring of slots per unit size (amplitudes), each ring about
+    // slot_budget_amps large (at least 2 slots, at most the launch's units of that size); a unit takes the next slot
+    // of its ring and waits for the slot's previous unit.
     std::vector<uint64_t> g_wv(total_groups);
     std::vector<uint32_t> g_frame(total_groups), g_prev(total_groups, kNoGroup);
     uint64_t wv_total = 0, frames_total = 0;
@@ -1406,14 +1410,15 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
                 uint64_t amps = 0, frames = 0, groups = 0, slots = 0, used = 0, wv_base = 0, fr_base = 0;
                 std::vector<uint32_t> last;  // per slot: launch group that used it last
             };
-            std::map<uint32_t, Ring> rings;  // by W
+            std::map<uint64_t, Ring> rings;  // by amplitudes of a unit
             for (size_t k = k0; k < k1; ++k) {
                 const RunCtx &R = *rs[order[k].c];
                 const StageDev &sd = R.pd->stages[order[k].si];
-                Ring &rg = rings[sd.W];
-                rg.amps = 1ull << sd.W;
-                rg.frames = std::max<uint64_t>(rg.frames, uint64_t(sd.G) * R.nframes);
-                rg.groups += sd.ngroups;
+                const uint64_t ug = unit_groups(sd);
+                Ring &rg = rings[ug << sd.W];
+                rg.amps = ug << sd.W;
+                rg.frames = std::max<uint64_t>(rg.frames, ug * sd.G * R.nframes);
+                rg.groups += sd.ngroups / ug;
             }
             uint64_t wv_l = 0, fr_l = 0;
             for (auto &kv : rings) {
@@ -1431,8 +1436,9 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
             uint32_t q_local = 0;
             for (size_t k = k0; k < k1; ++k) {
                 const StageDev &sd = rs[order[k].c]->pd->stages[order[k].si];
-                Ring &rg = rings[sd.W];
-                for (uint32_t gi = 0; gi < sd.ngroups; ++gi, ++q_local, ++q_global) {
+                const uint32_t ug = unit_groups(sd);
+                Ring &rg = rings[uint64_t(ug) << sd.W];
+                for (uint32_t gi = 0; gi < sd.ngroups / ug; ++gi, ++q_local, ++q_global) {
                     const uint64_t slot = rg.used++ % rg.slots;
                     g_wv[q_global] = rg.wv_base + slot * rg.amps;
                     g_frame[q_global] = uint32_t(rg.fr_base + slot * rg.frames);
@@ -1445,23 +1451,22 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
     }
     const bool rel = rs[0]->rel;  // one codec per launch (the batch entry points check it)
     DevBuf<float2> wv, part;
-    DevBuf<uint8_t> wrec;
-    DevBuf<uint32_t> flen, foff, fwords, fmixed, im;
-    DevBuf<uint64_t> lb, dg_wv;
+    DevBuf<uint8_t> side;
+    DevBuf<uint32_t> flen, foff, fhead;
+    DevBuf<uint64_t> dg_wv;
     DevBuf<uint32_t> sync, fin, ctr, dg_frame, dg_prev;
     DevBuf<PSeg> dsegs;
-    if ((rc = wv.alloc(wv_total)) || (rc = lb.alloc(frames_total)) || (rc = part.alloc(frames_total)) ||
+    const uint32_t side_bytes = rel ? kQszrSideBytes : 256u;
+    if ((rc = wv.alloc(wv_total)) || (rc = part.alloc(frames_total)) ||
         (rc = sync.alloc(2 * total_groups * kMaxPhases)) || (rc = fin.alloc(2 * nseg)) || (rc = ctr.alloc(4)) ||
         (rc = dsegs.alloc(nseg)) || (rc = dg_wv.alloc(total_groups)) || (rc = dg_frame.alloc(total_groups)) ||
-        (rc = dg_prev.alloc(total_groups)) || (rc = wrec.alloc(frames_total * (rel ? kQszrSideBytes : 256))) ||
-        (rc = flen.alloc(frames_total)) || (rc = foff.alloc(frames_total)) ||
-        (rel && ((rc = fwords.alloc(frames_total)) || (rc = fmixed.alloc(frames_total)) || (rc = im.alloc(wv_total)))))
+        (rc = dg_prev.alloc(total_groups)) || (rc = side.alloc(frames_total * side_bytes)) ||
+        (rc = flen.alloc(frames_total)) || (rc = foff.alloc(frames_total)) || (rel && (rc = fhead.alloc(frames_total))))
         return rc;
     CUDA_TRY(cudaMemcpyAsync(dg_wv.p, g_wv.data(), total_groups * sizeof(uint64_t), cudaMemcpyHostToDevice, main));
     CUDA_TRY(cudaMemcpyAsync(dg_frame.p, g_frame.data(), total_groups * sizeof(uint32_t), cudaMemcpyHostToDevice,
                              main));
     CUDA_TRY(cudaMemcpyAsync(dg_prev.p, g_prev.data(), total_groups * sizeof(uint32_t), cudaMemcpyHostToDevice, main));
-    CUDA_TRY(cudaMemsetAsync(lb.p, 0, lb.n * sizeof(uint64_t), main));
     CUDA_TRY(cudaMemsetAsync(sync.p, 0, sync.n * sizeof(uint32_t), main));
     CUDA_TRY(cudaMemsetAsync(fin.p, 0, fin.n * sizeof(uint32_t), main));
     CUDA_TRY(cudaMemsetAsync(ctr.p, 0, 4 * sizeof(uint32_t), main));
@@ -1481,7 +1486,9 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         memset(&a, 0, sizeof(a));
         a.W = sd.W;
         a.G = sd.G;
-        a.ngroups = sd.ngroups;
+        const uint32_t ug = unit_groups(sd);
+        a.ngroups = sd.ngroups / ug;
+        a.gpu = ug;
         a.m = R.m;
         a.e = R.e;
         a.npre = sd.npre;
@@ -1489,30 +1496,24 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         a.pbf16 = uint32_t(dctx.pred_bf16);
         uint32_t nph = 0;
         const uint32_t gframes = sd.G * uint32_t(R.nframes);
-        const uint32_t fpi = persistent_frames_per_item(um_any);
-        auto add = [&](uint32_t type, uint32_t count, uint32_t arg) {
+        // frames per item of the frame-parallel phases: a team of threads each
+        const uint32_t C = (1u << frame_log_for(int(R.m))) / 32u;
+        const uint32_t fpi = persistent_threads(um_any) / (C < 32u ? 32u : C);
+        auto add = [&](uint32_t type, uint32_t per, uint32_t arg) {
             if (nph < uint32_t(kMaxPhases)) {
                 a.ph[nph].type = type;
-                a.ph[nph].count = count;
+                a.ph[nph].per = per;
+                a.ph[nph].count = per * ug;
                 a.ph[nph].arg = arg;
             }
             ++nph;
         };
-        add(PH_DECODE, (gframes + fpi - 1) / fpi, 0);
+        const uint32_t fitems = (gframes + fpi - 1) / fpi;
+        add(PH_DECODE, fitems, 0);
         if (R.predict) add(PH_PREDICT, 1, 0);
         for (uint32_t pi = 0; pi < sd.npasses; ++pi) add(PH_PASS, 1u << sd.passes_host[pi].nout, pi);
-        if (R.rel) {
-            // relative-bound codec: in-place encoder (exact slots, or predicted slots kept when they fit), copy
-            add(PH_ENCODE_IP, (gframes + fpi - 1) / fpi, 0);
-            add(PH_COPY, (gframes + fpi - 1) / fpi, 0);
-        } else if (R.predict) {
-            add(PH_ENCODE, (gframes + fpi - 1) / fpi, 0);
-            add(PH_FIX, 1, 0);
-            add(PH_REENCODE, (gframes + fpi - 1) / fpi, 0);
-        } else {
-            add(PH_SIZE_W, (gframes + fpi - 1) / fpi, 0);
-            add(PH_ENCODE_W, (gframes + fpi - 1) / fpi, 0);
-        }
+        add(PH_ENCODE, fitems, 0);
+        if (R.nframes > 1) add(PH_COPY, fitems, 0);
         // the last phase index is the group's finished flag
         if (nph > uint32_t(kMaxPhases) - 1)
             return set_error(QSIM_E_UNSUPPORTED, "stage has too many passes for the persistent kernel");
@@ -1523,7 +1524,7 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
             acc_items += a.ph[t].count;
         }
         a.per_group = acc_items;
-        seg_items[k] = uint64_t(sd.ngroups) * acc_items;
+        seg_items[k] = uint64_t(a.ngroups) * acc_items;
         a.passes = R.pd->passes.p + sd.pass_begin;
         a.ops = R.pd->ops.p;
         a.mats = R.pd->mats.p;
@@ -1536,12 +1537,10 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         a.acc = R.accs.p + si;
         a.dev = R.arena_dev(out_par);
         a.host = R.arena_host(out_par);
-        a.data_start = qsz_data_start(int(R.m));
         a.worst = R.worst;
         PBlockBufs &b = *bb[order[k].c];
         a.tgt = b.tgt.p;
         a.res = b.res.p;
-        a.sizes = b.sizes.p;
         a.hist = R.predict ? b.hist.p : nullptr;
         a.pparams = R.predict ? dctx.pred_params : nullptr;
         a.sf = stage_features(R.p, si, R.e);
@@ -1553,7 +1552,7 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         a.fin_flag = fin.p + 2 * k + 1;
         a.reset_bumps = R.bumps.p + 2 * in_par;  // the next stage writes where this one read
         seg_group_off[k] = group_off;
-        group_off += sd.ngroups;
+        group_off += a.ngroups;
     }
     // queue positions: one launch for everything, or one launch per segment
     {
@@ -1569,18 +1568,16 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         }
     }
     CUDA_TRY(cudaMemcpyAsync(dsegs.p, segs.data(), nseg * sizeof(PSeg), cudaMemcpyHostToDevice, main));
-    const size_t smem = persistent_smem_bytes(max_pass_bytes);
+    const size_t smem = persistent_smem_bytes(max_pass_bytes, um_any);
     if ((rc = prepare_stage_persistent(prec, smem, rel, um_any))) return set_error(rc, "persistent kernel set-up failed");
 
     PLaunch L{};
     L.wv = wv.p;
-    L.wrec = wrec.p;
+    L.side = side.p;
+    L.side_bytes = side_bytes;
     L.flen = flen.p;
     L.foff = foff.p;
-    L.im = im.p;
-    L.fwords = fwords.p;
-    L.fmixed = fmixed.p;
-    L.lb = lb.p;
+    L.fhead = fhead.p;
     L.part = part.p;
     L.ctr = ctr.p;
     L.status = status;
@@ -2035,7 +2032,7 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     std::vector<RunCtx *> rp(count);
     int rc;
     uint64_t sum_need = 0;
-    std::map<uint32_t, uint64_t> w_groups;  // working-vector sizes of the batch and their group counts
+    std::map<uint64_t, uint64_t> w_groups;  // unit sizes (amplitudes) of the batch and their unit counts
     for (size_t c = 0; c < count; ++c) {
         const qsim_plan *p = plans[c];
         if (!p) return set_error(QSIM_E_INVALID, "batch entry %zu is null", c);
@@ -2050,7 +2047,10 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
         rs[c].reset(new RunCtx());
         rp[c] = rs[c].get();
         if ((rc = prepare_run(*rs[c], p, dctx))) return rc;
-        for (const StageDev &sd : rs[c]->pd->stages) w_groups[sd.W] += sd.ngroups;
+        for (const StageDev &sd : rs[c]->pd->stages) {
+            const uint64_t ug = unit_groups(sd);
+            w_groups[ug << sd.W] += sd.ngroups / ug;
+        }
         sum_need += rs[c]->need_per_parity;
     }
     const uint64_t slot_budget = 1ull << 27;  // working-vector slots of the launch: about 1 GiB
@@ -2060,10 +2060,9 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     // working-vector slot rings (one per size) with their frame scratch
     uint64_t ring_amps = 0;
     for (const auto &kv : w_groups)
-        ring_amps += std::min<uint64_t>(kv.second, std::max<uint64_t>(2, slot_budget >> kv.first)) << kv.first;
-    const bool rel = plans[0]->cfg.codec == QSIM_CODEC_QSZR;
-    // 8 B per amplitude and a quarter for the frame scratch; the relative codec adds its 4 B imaginary words
-    const uint64_t work_bytes = ring_amps * (rel ? 14 : 10);
+        ring_amps += std::min<uint64_t>(kv.second, std::max<uint64_t>(2, slot_budget / kv.first)) * kv.first;
+    // 8 B per amplitude and a quarter for the frame scratch
+    const uint64_t work_bytes = ring_amps * 10;
     const double dev_budget = free_b > work_bytes ? 0.85 * double(free_b - work_bytes) : 0.0;
     const double host_budget = 0.3 * double(host_phys_bytes());
     // each circuit's share of both levels follows its worst-case need

@@ -38,24 +38,6 @@ __device__ __forceinline__ float mlp_forward_one(const float *w, const float *x)
     return y;
 }
 
-// the 41 inputs of block j of a batch: its SV group's code-width histogram (each 32-value chunk of the decoded
-// input counts 32 in the bin of its width; G blocks of 2^(m+1) values each, hist read through L2), the largest
-// populated bin / 32 and the stage features
-__device__ __forceinline__ void mlp_features(const uint32_t *hist, uint32_t j, uint32_t G, int m,
-                                             const StageFeatures &sf, float *x) {
-    const float inv = 1.0f / (float(G) * float(2ull << m));
-    const uint64_t g0 = uint64_t(j / G) * G;
-    int maxb = 0;
-    for (int b = 0; b < 32; ++b) {
-        uint32_t c = 0;
-        for (uint32_t jj = 0; jj < G; ++jj) c += __ldcg(hist + (g0 + jj) * 32 + b);
-        x[b] = float(c) * inv;
-        if (c) maxb = b;
-    }
-    x[32] = float(maxb) / 32.f;
-    for (int t = 0; t < 8; ++t) x[33 + t] = sf.v[t];
-}
-
 void launch_mlp_forward(const float *params, const float *x, uint32_t batch, float *y, int bf16, cudaStream_t s);
 // features from the decoder's histogram (+ stage features) -> predicted log2 bytes; feat_out (nullable) receives
 // rows of kMlpIn features followed by one target slot

@@ -5,9 +5,13 @@
 // every CTA repeatedly takes the next work item from a global queue, whose
 // order is, group after group, the group's phases
 //     decode frames -> [predict + reserve] -> gate-pass tiles (pass by pass)
-//     -> [sizing frames] -> encode frames -> [exact re-reserve -> re-encode]
+//     -> encode frames -> [copy frames to their slots]
 // and waits (bounded spin) until the group's previous phase is complete
-// before running its item. Groups are independent (Sec. 4.1), so different
+// before running its item. A "group" of the queue is a unit of one or more SV
+// groups of the stage (together about 2^22 amplitudes): items are handed out in
+// queue order, so the phases of a small SV group would follow one another at
+// the latency of a phase each, while a unit's phases are long enough to fill
+// the GPU. Groups are independent (Sec. 4.1), so different
 // CTAs work on different phases of different groups at the same time, and a
 // group's work item only waits on items that come earlier in the queue, which
 // were taken by CTAs that are already running: the schedule cannot deadlock
@@ -21,8 +25,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "codec.cuh"
 #include "codec_dev.cuh"
+#include "codec_team.cuh"
 #include "device_common.cuh"
 #include "gates.cuh"
 #include "gates_dev.cuh"
@@ -36,9 +43,8 @@ namespace {
 using cdev::FrameGeom;
 using cdev::geom;
 
-// threads per CTA: one warp per frame of a frame-parallel item
 template <bool UM>
-constexpr int kPT = 32 * int(persistent_frames_per_item(UM));
+constexpr int kPT = int(persistent_threads(UM));
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
     uint32_t v;
@@ -55,7 +61,7 @@ __device__ __forceinline__ EncTarget load_target(const EncTarget *t) {
     return r;
 }
 
-// REL: the relative-bound codec (QSZR) in the decode phase and the in-place exact phases. UM: the plan's dense ops
+// REL: the relative-bound codec (QSZR). UM: the plan's dense ops
 // of width 3 to 5 (TF32 or split BF16) and 6 (TF32) run on tcgen05 (TMEM accumulator and MMA mbarrier held by each
 // CTA for the launch).
 template <int PREC, bool REL, bool UM>
@@ -63,17 +69,16 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     constexpr int PT = kPT<UM>;
     extern __shared__ float4 dsm[];
     __shared__ gdev::PassSmem PS;
-    __shared__ uint32_t s_wb[PT / 32][64];
     __shared__ OpDev s_pre[kMaxPreOps];
     __shared__ uint2 s_pre_ab[kMaxPreOps];
     __shared__ __align__(16) PSeg S;
-    __shared__ uint32_t s_hist[PT / 32][32];
-    __shared__ uint32_t s_item, s_epoch, s_seg, s_next;
+    __shared__ cdev::TeamSmem s_team[PT / 32];
+    __shared__ float s_pred[4 * kMlpHidden];  // predictor: features, hidden layers
+    __shared__ uint32_t s_item, s_seg, s_next;
     __shared__ uint32_t s_pcache[2];  // key (segment x 256 + pass) of the pass staged in dsm; its B resident
     __shared__ int s_flag, s_abort;
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
-        s_epoch = ld_relaxed_u32(L.ctr + 2) & cdev::kEpochMask;
         s_seg = ~0u;
         s_pcache[0] = ~0u;
         s_pcache[1] = 0;
@@ -204,26 +209,32 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         const uint32_t i = r - S.ph_start[p];
         const uint32_t type = S.ph[p].type;
         const bool abort_item = s_abort != 0;
-        float2 *wv = L.wv + L.g_wv[q];
-        float2 *part = L.part + L.g_frame[q];
-        const uint32_t *ids = S.ids + uint64_t(grp) * S.G;
-        const uint64_t gb = S.gbase[grp];
-        const uint64_t bbase = uint64_t(grp) * S.G;  // per-group block arrays
-        const uint32_t sf0 = L.g_frame[q];  // the slot's first frame in wrec / flen / foff / part / lb
-        bool by_arrival = type == PH_ENCODE || type == PH_REENCODE || type == PH_SIZE_W ||
-                          type == PH_ENCODE_W || type == PH_ENCODE_IP || type == PH_COPY;
+        // the item's SV group in the unit and its place among the group's items of this phase
+        const uint32_t gi = i / S.ph[p].per, ii = i % S.ph[p].per;
+        const uint64_t sg = uint64_t(grp) * S.gpu + gi;  // SV group of the stage
+        float2 *wv = L.wv + L.g_wv[q] + (uint64_t(gi) << S.W);
+        const uint32_t *ids = S.ids + sg * S.G;
+        const uint64_t gb = S.gbase[sg];
+        const uint64_t bbase = sg * S.G;  // per-group block arrays
+        const uint32_t sf0 = L.g_frame[q] + gi * gframes;  // the group's first frame in the frame records
+        const bool by_arrival = type == PH_ENCODE || type == PH_COPY;
+        // frame-parallel items: a team per frame, each with its own tile in dsm
+        const uint32_t tn = cdev::team_threads(g.C), team = uint32_t(tid) / tn;
+        const cdev::Team tm{uint32_t(tid) % tn, tn, 1u + team};
+        uint8_t *tile = reinterpret_cast<uint8_t *>(dsm) + team * cdev::team_tile_bytes(g.C);
+        const uint32_t fi = ii * (PT / tn) + team;
+        const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
+        const uint64_t a0 = (uint64_t(jj) << S.m) + uint64_t(f) * g.F;
+        if (type != PH_PASS && tid == 0) s_pcache[0] = ~0u;  // dsm is overwritten: no pass stays staged
         if (abort_item) {
             // skip the work, keep the counts
         } else if (type == PH_DECODE) {
-            const uint32_t fi = i * (PT / 32) + warp;
             if (fi < gframes) {
-                const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
                 const BlockSlot sl = S.tab_in[ids[jj]];
-                cdev::decode_frame_warp<kMaxPreOps, false, REL>(sl.ptr, sl.bytes, g, int(S.m), f,
-                                                    wv + (uint64_t(jj) << S.m) + uint64_t(f) * g.F,
-                                                    S.hist ? S.hist + (bbase + jj) * 32 : nullptr, s_hist[warp],
-                                                    L.status, s_pre, s_pre_ab, S.npre, S.mats,
-                                                    uint64_t(jj) << S.m, gb);
+                cdev::decode_frame_team<kMaxPreOps, REL>(tm, s_team[team], tile, sl.ptr, sl.bytes, g, int(S.m), f,
+                                                         wv + a0, S.hist ? S.hist + (bbase + jj) * 32 : nullptr,
+                                                         L.status, s_pre, s_pre_ab, S.npre, S.mats,
+                                                         uint64_t(jj) << S.m, gb);
             }
         } else if (type == PH_PASS) {
             if constexpr (UM) {
@@ -231,114 +242,94 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
                 // group and phase, in this item or an earlier one of this CTA) before the CTA barrier above, so the
                 // memory model orders them after the previous phase's writes; L1 starts empty at the launch
                 mma_ok &= gdev::pass_tile<PT, 5, PREC, false, true>(wv, S.passes[S.ph[p].arg], S.blob, S.mats, S.bfr,
-                                                                   i, gb, PS, reinterpret_cast<float2 *>(dsm),
+                                                                   ii, gb, PS, reinterpret_cast<float2 *>(dsm),
                                                                    L.status, &mphase, s_pcache,
                                                                    s_seg * 256u + S.ph[p].arg);
             } else {
-                gdev::pass_tile<PT, 5, PREC, false>(wv, S.passes[S.ph[p].arg], S.blob, S.mats, S.bfr, i, gb, PS,
+                gdev::pass_tile<PT, 5, PREC, false>(wv, S.passes[S.ph[p].arg], S.blob, S.mats, S.bfr, ii, gb, PS,
                                                    reinterpret_cast<float2 *>(dsm), L.status, nullptr, s_pcache,
                                                    s_seg * 256u + S.ph[p].arg);
             }
-        } else if (REL && type == PH_ENCODE_IP) {
-            if constexpr (REL) {
-                const uint32_t fi = i * (PT / 32) + warp;
-                if (fi < gframes) {
-                    const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
-                    const uint64_t a0 = (uint64_t(jj) << S.m) + uint64_t(f) * g.F;
-                    uint32_t words, mixed;
-                    const uint32_t len = cdev::encode_frame_warp_ip<true, true>(
-                        wv + a0, L.im + L.g_wv[q] + a0, g, S.e, L.wrec + uint64_t(sf0 + fi) * kQszrSideBytes, words,
-                        mixed, part + fi, L.status);
-                    if ((tid & 31) == 0) {
-                        L.flen[sf0 + fi] = len;
-                        L.fwords[sf0 + fi] = words;
-                        L.fmixed[sf0 + fi] = mixed;
+        } else if (type == PH_ENCODE) {
+            if (fi < gframes) {
+                cdev::load_rows_team(tm, tile, wv + a0, g.C);
+                const cdev::EncFrame r = cdev::encode_frame_team<REL>(tm, s_team[team], tile, g, S.e, L.status);
+                if (g.nframes == 1) {
+                    // a block of one frame: straight to its slot
+                    if (tm.t == 0) {
+                        const uint32_t total = uint32_t(g.data_start) + r.len;
+                        const EncTarget t = cdev::reserve_block(total, S.pparams != nullptr, &S.tgt[bbase + jj], S.dev,
+                                                                S.host, S.acc, L.status);
+                        EncResult out{};
+                        out.err_sq = r.err_sq;
+                        out.norm_sq = r.norm_sq;
+                        s_team[team].bc = reinterpret_cast<uint64_t>(
+                            cdev::finish_single_frame(total, t, out, S.tab_out + ids[jj], S.acc));
+                        S.res[bbase + jj] = out;
+                        atomicAdd(&S.acc->err_sq, out.err_sq);
+                        atomicAdd(&S.acc->norm_sq, out.norm_sq);
+                    }
+                    tm.sync();
+                    cdev::store_single_frame<REL>(tm, tile, g, int(S.m), S.e, r.len,
+                                                  reinterpret_cast<uint8_t *>(s_team[team].bc));
+                } else {
+                    cdev::stage_frame(tm, tile, r, wv + a0, L.side + uint64_t(sf0 + fi) * L.side_bytes);
+                    if (tm.t == 0) {
+                        L.flen[sf0 + fi] = r.len;
+                        if (REL) L.fhead[sf0 + fi] = r.head;
+                        L.part[sf0 + fi] = make_float2(r.err_sq, r.norm_sq);
                         __threadfence();  // read by the phase's last item and the copy phase on other CTAs
                     }
                 }
             }
-        } else if (REL && type == PH_COPY) {
-            if constexpr (REL) {
-                const uint32_t fi = i * (PT / 32) + warp;
-                if (fi < gframes) {
-                    const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
-                    const uint64_t a0 = (uint64_t(jj) << S.m) + uint64_t(f) * g.F;
-                    cdev::copy_frame_warp<true>(reinterpret_cast<const uint32_t *>(wv + a0), L.im + L.g_wv[q] + a0,
-                                                L.wrec + uint64_t(sf0 + fi) * kQszrSideBytes,
-                                                __ldcg(L.fwords + sf0 + fi), __ldcg(L.fmixed + sf0 + fi),
-                                                __ldcg(L.flen + sf0 + fi), __ldcg(L.foff + sf0 + fi), g, int(S.m),
-                                                S.e, f, load_target(&S.tgt[bbase + jj]), &S.res[bbase + jj],
-                                                S.tab_out + ids[jj], S.acc);
-                }
-            }
-        } else if (type == PH_SIZE_W) {
-            const uint32_t fi = i * (PT / 32) + warp;
-            if (fi < gframes) {
-                const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
-                const uint32_t len = cdev::size_frame_warp<true>(wv + (uint64_t(jj) << S.m) + uint64_t(f) * g.F, g,
-                                                                 S.e, L.wrec + uint64_t(sf0 + fi) * 256, L.status);
-                if ((tid & 31) == 0) {
-                    L.flen[sf0 + fi] = len;
-                    __threadfence();  // read by the phase's last item on another CTA
-                }
-            }
-        } else if (type == PH_ENCODE_W) {
-            const uint32_t fi = i * (PT / 32) + warp;
-            if (fi < gframes) {
-                const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
-                cdev::encode_frame_warp_known<true>(wv + (uint64_t(jj) << S.m) + uint64_t(f) * g.F, g, int(S.m), S.e,
-                                                    f, L.wrec + uint64_t(sf0 + fi) * 256, __ldcg(L.foff + sf0 + fi),
-                                                    __ldcg(L.flen + sf0 + fi), load_target(&S.tgt[bbase + jj]),
-                                                    &S.res[bbase + jj], S.tab_out + ids[jj], S.acc, part + fi,
-                                                    L.status);
-            }
+        } else if (type == PH_COPY) {
+            if (fi < gframes)  // frames of 4096 amplitudes: teams of 128
+                cdev::copy_frame_team<REL>(tm, wv + a0, L.side + uint64_t(sf0 + fi) * L.side_bytes,
+                                           __ldcg(L.flen + sf0 + fi), REL ? __ldcg(L.fhead + sf0 + fi) : 256u,
+                                           __ldcg(L.foff + sf0 + fi), g, int(S.m), S.e, f,
+                                           load_target(&S.tgt[bbase + jj]), &S.res[bbase + jj], S.tab_out + ids[jj],
+                                           S.acc);
         } else if (type == PH_PREDICT) {
-            float *w = reinterpret_cast<float *>(dsm);
-            if (tid == 0) s_pcache[0] = ~0u;  // dsm is overwritten: no pass stays staged
+            // one SV group: its blocks share every input of the predictor, so one forward pass sizes them all. Weights in
+            // dsm, W2's rows padded to 65 words (lanes walk rows)
+            constexpr int IN = kMlpIn, HID = kMlpHidden, OB1 = HID * IN, OW2 = OB1 + HID, OB2 = OW2 + HID * (HID + 1),
+                          OW3 = OB2 + HID, OB3 = OW3 + HID, FW2 = HID * IN + HID;
+            float *w = reinterpret_cast<float *>(dsm), *x = s_pred, *h1 = s_pred + HID, *h2 = s_pred + 2 * HID;
             for (int t = tid; t < kMlpParams; t += PT) {
                 const float v = S.pparams[t];
-                w[t] = S.pbf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
+                const int o = t < FW2 ? t : t < FW2 + HID * HID ? t + (t - FW2) / HID : t + HID;
+                w[o] = S.pbf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
+            }
+            if (tid < 32) {
+                uint32_t c = 0;
+                for (uint32_t k = 0; k < S.G; ++k) c += __ldcg(S.hist + (bbase + k) * 32 + tid);
+                x[tid] = float(c) * (1.0f / (float(S.G) * float(2ull << S.m)));
+                const uint32_t nz = __ballot_sync(kFull, c != 0);
+                if (tid == 0) x[32] = float(nz ? 31 - __clz(nz) : 0) / 32.f;
+                if (tid < 8) x[33 + tid] = S.sf.v[tid];
             }
             __syncthreads();
-            for (uint32_t jj = tid; jj < S.G; jj += PT) {
-                float x[kMlpIn];
-                mlp_features(S.hist + bbase * 32, jj, S.G, int(S.m), S.sf, x);
-                double pr = double(mlp_forward_one(w, x)) + double(S.m + 3);
-                pr = pr < 0 ? 0 : (pr > 40 ? 40 : pr);
-                const double want_b = exp2(pr) * (1.0 + S.margin);
-                EncResult &rs = S.res[bbase + jj];
-                rs.total = 0;
-                rs.overflow = 0;
-                rs.err_sq = 0;
-                rs.norm_sq = 0;
-                cdev::reserve_slot(want_b >= double(S.worst) ? S.worst : uint64_t(want_b), S.dev, S.host,
-                                   &S.tgt[bbase + jj], L.status);
+            if (tid < HID) {
+                float a = w[OB1 + tid];
+                for (int j = 0; j < IN; ++j) a = fmaf(w[tid * IN + j], x[j], a);
+                h1[tid] = fmaxf(a, 0.f);
             }
             __syncthreads();
+            if (tid < HID) {
+                float a = w[OB2 + tid];
+                for (int j = 0; j < HID; ++j) a = fmaf(w[OW2 + tid * (HID + 1) + j], h1[j], a);
+                h2[tid] = fmaxf(a, 0.f) * w[OW3 + tid];
+            }
+            __syncthreads();
+            float y = w[OB3];
+            for (int j = 0; j < HID; ++j) y += h2[j];
+            double pr = double(y) + double(S.m + 3);
+            pr = pr < 0 ? 0 : (pr > 40 ? 40 : pr);
+            const double want_b = exp2(pr) * (1.0 + S.margin);
+            const uint64_t want = want_b >= double(S.worst) ? S.worst : uint64_t(want_b);
+            for (uint32_t k = tid; k < S.G; k += PT) cdev::reserve_slot(want, S.dev, S.host, &S.tgt[bbase + k], L.status);
             // the group's histograms are consumed: leave them zero for the next stage
             for (uint32_t t = tid; t < S.G * 32; t += PT) S.hist[bbase * 32 + t] = 0;
-        } else if (type == PH_ENCODE || type == PH_REENCODE) {
-            // learned sizing: one frame per warp, offsets by warp look-back
-            const uint32_t fi = i * (PT / 32) + warp;
-            const bool retry = type == PH_REENCODE;
-            if (fi < gframes) {
-                const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
-                if (!retry || __ldcg(&S.res[bbase + jj].overflow) != 0) {
-                    const uint32_t epoch = (s_epoch + 2 * q + (retry ? 1 : 0)) & cdev::kEpochMask;
-                    cdev::encode_frame_warp_lb<true>(wv + (uint64_t(jj) << S.m) + uint64_t(f) * g.F, g, int(S.m), S.e,
-                                                     f, L.lb + L.g_frame[q] + uint64_t(jj) * g.nframes, epoch,
-                                                     load_target(&S.tgt[bbase + jj]), &S.res[bbase + jj],
-                                                     S.tab_out + ids[jj], S.acc, retry ? nullptr : part + fi,
-                                                     s_wb[warp], L.status);
-                }
-            }
-        } else if (type == PH_FIX) {
-            for (uint32_t jj = tid; jj < S.G; jj += PT) {
-                EncResult &rs = S.res[bbase + jj];
-                if (__ldcg(&rs.overflow))
-                    cdev::reserve_slot(__ldcg(reinterpret_cast<const unsigned long long *>(&rs.total)), S.dev, S.host,
-                                       &S.tgt[bbase + jj], L.status);
-            }
         }
         // ---- completion ----
         __syncthreads();
@@ -360,60 +351,26 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         __syncthreads();
         if (!s_flag) continue;
         __threadfence();
-        if (abort_item) {
-            // no reservation or statistics after an error
-        } else if (type == PH_SIZE_W || type == PH_ENCODE_IP) {
-            // the group's frame lengths are complete: frame offsets (warp per block) and the group's slots (the
-            // in-place phase with learned sizing keeps every predicted slot its block fits)
-            const int lane = tid & 31;
-            for (uint32_t jj = warp; jj < S.G; jj += PT / 32) {
-                uint32_t run = uint32_t(S.data_start);
-                for (uint32_t f0 = 0; f0 < g.nframes; f0 += 32) {
-                    const uint32_t fi = sf0 + jj * g.nframes + f0 + lane;
-                    const uint32_t v = f0 + lane < g.nframes ? __ldcg(L.flen + fi) : 0u;
-                    uint32_t incl = v;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t t = __shfl_up_sync(kFull, incl, o);
-                        if (lane >= o) incl += t;
-                    }
-                    if (f0 + lane < g.nframes) L.foff[fi] = run + incl - v;
-                    run += __shfl_sync(kFull, incl, 31);
+        if (!abort_item && type == PH_ENCODE && g.nframes > 1) {
+            // the unit's frame lengths are complete: frame offsets, the blocks' slots (with learned sizing every
+            // predicted slot its block fits is kept) and the stage's error sums, a team of 128 per block
+            const uint32_t f0 = L.g_frame[q];
+            const uint64_t b0 = uint64_t(grp) * S.gpu * S.G;
+            for (uint32_t k = team; k < S.gpu * S.G; k += PT / 128) {
+                double a, b;
+                const uint32_t fk = f0 + k * g.nframes;
+                const uint32_t total = cdev::block_offsets_team(tm, s_team[team], L.flen + fk, L.part + fk, L.foff + fk,
+                                                                g.nframes, uint32_t(g.data_start), a, b);
+                if (tm.t == 0) {
+                    cdev::reserve_block(total, S.pparams != nullptr, &S.tgt[b0 + k], S.dev, S.host, S.acc, L.status);
+                    EncResult out{};
+                    out.err_sq = a;
+                    out.norm_sq = b;
+                    S.res[b0 + k] = out;
+                    atomicAdd(&S.acc->err_sq, a);
+                    atomicAdd(&S.acc->norm_sq, b);
                 }
-                if (lane == 0) {
-                    EncResult &rs = S.res[bbase + jj];
-                    rs.total = 0;
-                    rs.overflow = 0;
-                    rs.err_sq = 0;
-                    rs.norm_sq = 0;
-                    EncTarget &t = S.tgt[bbase + jj];
-                    if (type == PH_ENCODE_IP && S.pparams) {
-                        if (t.ptr == nullptr || run > t.cap) {
-                            atomicAdd(reinterpret_cast<unsigned long long *>(&S.acc->overflow_blocks), 1ull);
-                            cdev::reserve_slot(run, S.dev, S.host, &t, L.status);
-                        }
-                    } else {
-                        cdev::reserve_slot(run, S.dev, S.host, &t, L.status);
-                    }
-                }
-            }
-        }
-        if (!abort_item && (type == PH_ENCODE || type == PH_ENCODE_W || type == PH_ENCODE_IP)) {
-            // the group's frames are encoded: fold their error partials into the stage totals
-            double a = 0, b = 0;
-            for (uint32_t t = tid; t < gframes; t += PT) {
-                const float2 v = __ldcg(part + t);
-                a += double(v.x);
-                b += double(v.y);
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                a += __shfl_xor_sync(kFull, a, o);
-                b += __shfl_xor_sync(kFull, b, o);
-            }
-            if ((tid & 31) == 0) {
-                atomicAdd(&S.acc->err_sq, a);
-                atomicAdd(&S.acc->norm_sq, b);
+                tm.sync();
             }
         }
         __syncthreads();
@@ -446,14 +403,12 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
             umma::tmem_dealloc(PS.tmem, gdev::umma_pass_tmem_cols(0));
         }
     }
-    // the last CTA out resets the queue and advances the look-back epoch
+    // the last CTA out resets the queue
     if (tid == 0) {
         __threadfence();
         if (atomicAdd(L.ctr + 1, 1u) == gridDim.x - 1) {
             L.ctr[0] = 0;
             L.ctr[1] = 0;
-            __threadfence();
-            atomicExch(L.ctr + 2, (s_epoch + 2 * L.total_groups) & cdev::kEpochMask);
         }
     }
 }
@@ -535,9 +490,11 @@ int launch_codec(const PLaunch &a, int prec, size_t smem, cudaStream_t s, int *g
 
 }  // namespace
 
-size_t persistent_smem_bytes(size_t pass_bytes) {
-    const size_t mlp = size_t(kMlpParams) * sizeof(float);
-    return pass_bytes > mlp ? pass_bytes : mlp;
+size_t persistent_smem_bytes(size_t pass_bytes, bool um) {
+    const size_t mlp = size_t(kMlpParams + kMlpHidden) * sizeof(float);
+    // a tile per team: threads / max(32, C) of them, most in all at C = 32
+    const size_t tiles = size_t(persistent_threads(um) / 32) * cdev::team_tile_bytes(32);
+    return std::max(std::max(pass_bytes, mlp), tiles);
 }
 
 int prepare_stage_persistent(int prec, size_t smem, bool rel, bool um) {
