@@ -1346,6 +1346,54 @@ static uint32_t unit_groups(const StageDev &sd) {
     return uint32_t(std::min<uint64_t>(sd.ngroups, sd.W < 22 ? 1ull << (22 - sd.W) : 1ull));
 }
 
+// Circuits (indices into rs) that share the working-vector slots of one launch, with the slots' size and number.
+struct PLane {
+    std::vector<uint32_t> circuits;
+    uint64_t amps = 0, frames = 0, units = 0;  // largest unit, largest unit's frames, most units of a stage
+    uint32_t slots = 1;
+};
+
+// The lanes of a launch over stages [s0, s1) of every circuit: a lane of its own for each of the smallest circuits while
+// their slots together stay within budget amplitudes, and one lane for the others. A stage of several units gets two
+// slots, up to four while they stay within the budget.
+static std::vector<PLane> plan_lanes(const std::vector<RunCtx *> &rs, size_t s0, size_t s1, uint64_t budget) {
+    std::vector<PLane> lanes;
+    for (uint32_t c = 0; c < rs.size(); ++c) {
+        PLane l;
+        l.circuits.push_back(c);
+        for (size_t si = s0; si < std::min(s1, rs[c]->nst); ++si) {
+            const StageDev &sd = rs[c]->pd->stages[si];
+            const uint64_t ug = unit_groups(sd);
+            l.amps = std::max(l.amps, ug << sd.W);
+            l.frames = std::max<uint64_t>(l.frames, ug * sd.G * rs[c]->nframes);
+            l.units = std::max<uint64_t>(l.units, sd.ngroups / ug);
+        }
+        if (l.units) lanes.push_back(std::move(l));
+    }
+    std::stable_sort(lanes.begin(), lanes.end(), [](const PLane &x, const PLane &y) { return x.amps < y.amps; });
+    std::vector<PLane> out;
+    PLane rest;
+    uint64_t used = 0;
+    for (PLane &l : lanes) {
+        l.slots = uint32_t(std::min<uint64_t>(l.units, std::max<uint64_t>(2, std::min<uint64_t>(4, budget / 4 / l.amps))));
+        if (used + l.slots * l.amps <= budget) {
+            used += l.slots * l.amps;
+            out.push_back(std::move(l));
+            continue;
+        }
+        rest.circuits.push_back(l.circuits[0]);
+        rest.amps = std::max(rest.amps, l.amps);
+        rest.frames = std::max(rest.frames, l.frames);
+        rest.units = std::max(rest.units, l.units);
+        rest.slots = uint32_t(std::min<uint64_t>(rest.units, 2));
+    }
+    if (rest.units) {
+        std::sort(rest.circuits.begin(), rest.circuits.end());
+        out.push_back(std::move(rest));
+    }
+    return out;
+}
+
 static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cudaStream_t main, int *status,
                           Profiler &prof, const DeviceCtx &dctx, uint64_t slot_budget_amps) {
     const qsim_config &cfg0 = rs[0]->p->cfg;
@@ -1395,57 +1443,46 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
             return rc;
         if (R.predict) CUDA_TRY(cudaMemsetAsync(b.hist.p, 0, R.nblocks * 32 * sizeof(uint32_t), main));
     }
-    // Working-vector slots, planned per launch: one ring of slots per unit size (amplitudes), each ring about
-    // slot_budget_amps large (at least 2 slots, at most the launch's units of that size); a unit takes the next slot
-    // of its ring and waits for the slot's previous unit.
+    // Working-vector slots, planned per launch: every lane's slots side by side; unit u of a stage takes the lane's slot
+    // u mod slots and waits for the slot's previous unit.
     std::vector<uint64_t> g_wv(total_groups);
     std::vector<uint32_t> g_frame(total_groups), g_prev(total_groups, kNoGroup);
+    std::vector<std::vector<PLane>> lanes;  // per launch
     uint64_t wv_total = 0, frames_total = 0;
     {
-        const size_t nlaunch_plan = one_launch ? 1 : nseg;
-        uint64_t q_global = 0;
-        for (size_t l = 0; l < nlaunch_plan; ++l) {
-            const size_t k0 = one_launch ? 0 : l, k1 = one_launch ? nseg : l + 1;
-            struct Ring {
-                uint64_t amps = 0, frames = 0, groups = 0, slots = 0, used = 0, wv_base = 0, fr_base = 0;
-                std::vector<uint32_t> last;  // per slot: launch group that used it last
-            };
-            std::map<uint64_t, Ring> rings;  // by amplitudes of a unit
-            for (size_t k = k0; k < k1; ++k) {
-                const RunCtx &R = *rs[order[k].c];
-                const StageDev &sd = R.pd->stages[order[k].si];
-                const uint64_t ug = unit_groups(sd);
-                Ring &rg = rings[ug << sd.W];
-                rg.amps = ug << sd.W;
-                rg.frames = std::max<uint64_t>(rg.frames, ug * sd.G * R.nframes);
-                rg.groups += sd.ngroups / ug;
-            }
+        std::vector<uint64_t> first(nseg);  // number of a segment's first unit, over all launches
+        uint64_t n_units = 0;
+        for (size_t k = 0; k < nseg; ++k) {
+            const StageDev &sd = rs[order[k].c]->pd->stages[order[k].si];
+            first[k] = n_units;
+            n_units += sd.ngroups / unit_groups(sd);
+        }
+        for (size_t l = 0; l < (one_launch ? 1 : nseg); ++l) {
+            const size_t s0 = one_launch ? 0 : l, s1 = one_launch ? max_nst : l + 1;
+            lanes.push_back(plan_lanes(rs, s0, s1, slot_budget_amps));
+            const uint64_t q0 = one_launch ? 0 : first[l];  // unit numbers are per launch
             uint64_t wv_l = 0, fr_l = 0;
-            for (auto &kv : rings) {
-                Ring &rg = kv.second;
-                rg.slots = std::max<uint64_t>(2, std::min<uint64_t>(rg.groups, slot_budget_amps / rg.amps));
-                rg.slots = std::min<uint64_t>(rg.slots, rg.groups);
-                rg.last.assign(rg.slots, kNoGroup);
-                rg.wv_base = wv_l;
-                rg.fr_base = fr_l;
-                wv_l += rg.slots * rg.amps;
-                fr_l += rg.slots * rg.frames;
+            for (const PLane &ln : lanes.back()) {
+                std::vector<uint32_t> last(ln.slots, kNoGroup);
+                for (size_t r = s0; r < s1; ++r)
+                    for (uint32_t c : ln.circuits) {
+                        if (r >= rs[c]->nst) continue;
+                        const size_t k = seg_of[c][r];
+                        const StageDev &sd = rs[c]->pd->stages[r];
+                        for (uint32_t u = 0; u < sd.ngroups / unit_groups(sd); ++u) {
+                            const uint64_t q = first[k] + u;
+                            const uint32_t slot = u % ln.slots;
+                            g_wv[q] = wv_l + slot * ln.amps;
+                            g_frame[q] = uint32_t(fr_l + slot * ln.frames);
+                            g_prev[q] = last[slot];
+                            last[slot] = uint32_t(q - q0);
+                        }
+                    }
+                wv_l += ln.slots * ln.amps;
+                fr_l += ln.slots * ln.frames;
             }
             wv_total = std::max(wv_total, wv_l);
             frames_total = std::max(frames_total, fr_l);
-            uint32_t q_local = 0;
-            for (size_t k = k0; k < k1; ++k) {
-                const StageDev &sd = rs[order[k].c]->pd->stages[order[k].si];
-                const uint32_t ug = unit_groups(sd);
-                Ring &rg = rings[uint64_t(ug) << sd.W];
-                for (uint32_t gi = 0; gi < sd.ngroups / ug; ++gi, ++q_local, ++q_global) {
-                    const uint64_t slot = rg.used++ % rg.slots;
-                    g_wv[q_global] = rg.wv_base + slot * rg.amps;
-                    g_frame[q_global] = uint32_t(rg.fr_base + slot * rg.frames);
-                    g_prev[q_global] = rg.last[slot];
-                    rg.last[slot] = q_local;
-                }
-            }
         }
         if (frames_total >= (1ull << 32)) return set_error(QSIM_E_UNSUPPORTED, "working-vector slot plan too large");
     }
@@ -1473,7 +1510,8 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
 
     // ---- segment descriptors ----
     std::vector<PSeg> segs(nseg);
-    std::vector<uint64_t> seg_items(nseg), seg_group_off(nseg);  // group offset into the done/arrive arrays
+    std::vector<std::vector<PStep>> phases(nseg);  // of one unit (begin, seg and grp to be set)
+    std::vector<uint64_t> seg_group_off(nseg);     // group offset into the done/arrive arrays
     uint64_t group_off = 0;
     bool stall = false;
     for (size_t k = 0; k < nseg; ++k) {
@@ -1500,13 +1538,14 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         const uint32_t C = (1u << frame_log_for(int(R.m))) / 32u;
         const uint32_t fpi = persistent_threads(um_any) / (C < 32u ? 32u : C);
         auto add = [&](uint32_t type, uint32_t per, uint32_t arg) {
-            if (nph < uint32_t(kMaxPhases)) {
-                a.ph[nph].type = type;
-                a.ph[nph].per = per;
-                a.ph[nph].count = per * ug;
-                a.ph[nph].arg = arg;
-            }
-            ++nph;
+            PStep s{};
+            s.phase = nph++;
+            s.type = type;
+            s.arg = arg;
+            s.per = per;
+            s.need = phases[k].empty() ? 0u : phases[k].back().count;
+            s.count = per * ug;
+            phases[k].push_back(s);
         };
         const uint32_t fitems = (gframes + fpi - 1) / fpi;
         add(PH_DECODE, fitems, 0);
@@ -1518,13 +1557,6 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         if (nph > uint32_t(kMaxPhases) - 1)
             return set_error(QSIM_E_UNSUPPORTED, "stage has too many passes for the persistent kernel");
         a.nphases = nph;
-        uint32_t acc_items = 0;
-        for (uint32_t t = 0; t < nph; ++t) {
-            a.ph_start[t] = acc_items;
-            acc_items += a.ph[t].count;
-        }
-        a.per_group = acc_items;
-        seg_items[k] = uint64_t(a.ngroups) * acc_items;
         a.passes = R.pd->passes.p + sd.pass_begin;
         a.ops = R.pd->ops.p;
         a.mats = R.pd->mats.p;
@@ -1554,19 +1586,53 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
         seg_group_off[k] = group_off;
         group_off += a.ngroups;
     }
-    // queue positions: one launch for everything, or one launch per segment
-    {
+    // ---- the queue: every lane's steps in dependency order, the lanes merged by the fraction of their steps ----
+    std::vector<PStep> steps;
+    std::vector<size_t> step_off{0};  // per launch
+    std::vector<uint64_t> launch_items;
+    for (size_t l = 0; l < lanes.size(); ++l) {
+        const size_t s0 = one_launch ? 0 : l, s1 = one_launch ? max_nst : l + 1;
+        std::vector<std::pair<double, PStep>> all;
+        for (const PLane &ln : lanes[l]) {
+            const size_t a0 = all.size();
+            for (size_t r = s0; r < s1; ++r)
+                for (uint32_t c : ln.circuits) {
+                    if (r >= rs[c]->nst) continue;
+                    const size_t k = seg_of[c][r];
+                    for (uint32_t u0 = 0; u0 < segs[k].ngroups; u0 += ln.slots)
+                        for (PStep s : phases[k])
+                            for (uint32_t u = u0; u < std::min(segs[k].ngroups, u0 + ln.slots); ++u) {
+                                s.seg = uint32_t(one_launch ? k : 0);
+                                s.grp = u;
+                                all.emplace_back(0.0, s);
+                            }
+                }
+            for (size_t i = a0; i < all.size(); ++i)
+                all[i].first = (double(i - a0) + 0.5) / double(all.size() - a0);
+        }
+        std::stable_sort(all.begin(), all.end(),
+                         [](const std::pair<double, PStep> &x, const std::pair<double, PStep> &y) { return x.first < y.first; });
         uint64_t item = 0;
-        uint32_t group = 0;
-        for (size_t k = 0; k < nseg; ++k) {
-            if (!one_launch) item = 0, group = 0;
-            segs[k].item_begin = item;
-            segs[k].group_begin = group;
-            item += seg_items[k];
-            group += segs[k].ngroups;
+        for (auto &x : all) {
+            x.second.begin = uint32_t(item);
+            item += x.second.count;
+            steps.push_back(x.second);
             if (item >= (1ull << 32)) return set_error(QSIM_E_UNSUPPORTED, "work queue longer than 2^32 items");
         }
+        launch_items.push_back(item);
+        step_off.push_back(steps.size());
     }
+    {
+        uint32_t group = 0;
+        for (size_t k = 0; k < nseg; ++k) {
+            if (!one_launch) group = 0;
+            segs[k].group_begin = group;
+            group += segs[k].ngroups;
+        }
+    }
+    DevBuf<PStep> dsteps;
+    if ((rc = dsteps.alloc(steps.size()))) return rc;
+    CUDA_TRY(cudaMemcpyAsync(dsteps.p, steps.data(), steps.size() * sizeof(PStep), cudaMemcpyHostToDevice, main));
     CUDA_TRY(cudaMemcpyAsync(dsegs.p, segs.data(), nseg * sizeof(PSeg), cudaMemcpyHostToDevice, main));
     const size_t smem = persistent_smem_bytes(max_pass_bytes, um_any);
     if ((rc = prepare_stage_persistent(prec, smem, rel, um_any))) return set_error(rc, "persistent kernel set-up failed");
@@ -1610,8 +1676,9 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
                                one_launch ? nseg : l);
         const size_t k0 = one_launch ? 0 : l, k1 = one_launch ? nseg : l + 1;
         L.segs = dsegs.p + k0;
-        L.nseg = uint32_t(k1 - k0);
-        L.total_items = segs[k1 - 1].item_begin + seg_items[k1 - 1];
+        L.steps = dsteps.p + step_off[l];
+        L.nsteps = uint32_t(step_off[l + 1] - step_off[l]);
+        L.total_items = launch_items[l];
         L.total_groups = segs[k1 - 1].group_begin + segs[k1 - 1].ngroups;
         L.g_wv = dg_wv.p + seg_group_off[k0];
         L.g_frame = dg_frame.p + seg_group_off[k0];
@@ -2032,7 +2099,6 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     std::vector<RunCtx *> rp(count);
     int rc;
     uint64_t sum_need = 0;
-    std::map<uint64_t, uint64_t> w_groups;  // unit sizes (amplitudes) of the batch and their unit counts
     for (size_t c = 0; c < count; ++c) {
         const qsim_plan *p = plans[c];
         if (!p) return set_error(QSIM_E_INVALID, "batch entry %zu is null", c);
@@ -2047,22 +2113,19 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
         rs[c].reset(new RunCtx());
         rp[c] = rs[c].get();
         if ((rc = prepare_run(*rs[c], p, dctx))) return rc;
-        for (const StageDev &sd : rs[c]->pd->stages) {
-            const uint64_t ug = unit_groups(sd);
-            w_groups[ug << sd.W] += sd.ngroups / ug;
-        }
         sum_need += rs[c]->need_per_parity;
     }
     const uint64_t slot_budget = 1ull << 27;  // working-vector slots of the launch: about 1 GiB
     size_t free_b = 0, total_b = 0;
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     free_b += cached_dev_bytes();
-    // working-vector slot rings (one per size) with their frame scratch
-    uint64_t ring_amps = 0;
-    for (const auto &kv : w_groups)
-        ring_amps += std::min<uint64_t>(kv.second, std::max<uint64_t>(2, slot_budget / kv.first)) * kv.first;
+    // working-vector slots with their frame scratch
+    size_t max_nst = 0;
+    for (const RunCtx *R : rp) max_nst = std::max(max_nst, R->nst);
+    uint64_t slot_amps = 0;
+    for (const PLane &ln : plan_lanes(rp, 0, max_nst, slot_budget)) slot_amps += ln.slots * ln.amps;
     // 8 B per amplitude and a quarter for the frame scratch
-    const uint64_t work_bytes = ring_amps * 10;
+    const uint64_t work_bytes = slot_amps * 10;
     const double dev_budget = free_b > work_bytes ? 0.85 * double(free_b - work_bytes) : 0.0;
     const double host_budget = 0.3 * double(host_phys_bytes());
     // each circuit's share of both levels follows its worst-case need

@@ -2,23 +2,22 @@
 //
 // The paper overlaps the SV groups of a stage by dealing them round-robin to
 // CUDA streams (Sec. 4.2). Here the same overlap happens inside one launch:
-// every CTA repeatedly takes the next work item from a global queue, whose
-// order is, group after group, the group's phases
-//     decode frames -> [predict + reserve] -> gate-pass tiles (pass by pass)
-//     -> encode frames -> [copy frames to their slots]
-// and waits (bounded spin) until the group's previous phase is complete
-// before running its item. A "group" of the queue is a unit of one or more SV
-// groups of the stage (together about 2^22 amplitudes): items are handed out in
-// queue order, so the phases of a small SV group would follow one another at
-// the latency of a phase each, while a unit's phases are long enough to fill
-// the GPU. Groups are independent (Sec. 4.1), so different
-// CTAs work on different phases of different groups at the same time, and a
-// group's work item only waits on items that come earlier in the queue, which
-// were taken by CTAs that are already running: the schedule cannot deadlock
-// even when not every CTA is resident. Working vectors live in slots planned
-// on the host: one ring of slots per working-vector size, so that many small
-// groups can be in flight next to a few large ones; the first item of a group
-// also waits for the slot's previous group (earlier in the queue) to finish.
+// every CTA repeatedly takes the next work item from a global queue of steps. A
+// step is one phase of one unit: decode frames, [predict + reserve], a gate pass's
+// tiles (pass by pass), encode frames, [copy frames to their slots]. A unit is one
+// or more SV groups of the stage, together about 2^22 amplitudes, so that its
+// phases are long enough to fill the GPU. A CTA waits (bounded spin) until the
+// unit's previous phase is complete before running its item.
+//
+// Items are handed out in queue order, so the order decides what overlaps. Units
+// that share working-vector slots form a lane, whose steps are in dependency order
+// (stage after stage; within a stage as many units side by side as the lane has
+// slots, phase by phase); a batch's small circuits have a lane each, and the lanes
+// are merged by the fraction of their steps, so that while one circuit's phase
+// drains the CTAs work on the others'. (With every circuit's stage in the queue as a
+// whole, the time of a batch was the sum of its circuits' alone.) Every dependency
+// points to an earlier item of the same lane, which was taken by a CTA that is
+// already running: the schedule cannot deadlock even when not every CTA is resident.
 //
 // Data produced by other CTAs of the same launch is read through L2 (ld.cg),
 // since the per-SM L1 caches are not coherent within a launch.
@@ -74,7 +73,8 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     __shared__ __align__(16) PSeg S;
     __shared__ cdev::TeamSmem s_team[PT / 32];
     __shared__ float s_pred[4 * kMlpHidden];  // predictor: features, hidden layers
-    __shared__ uint32_t s_item, s_seg, s_next;
+    __shared__ uint32_t s_item, s_seg;
+    __shared__ PStep s_step;
     __shared__ uint32_t s_pcache[2];  // key (segment x 256 + pass) of the pass staged in dsm; its B resident
     __shared__ int s_flag, s_abort;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -116,29 +116,25 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     // thread 0: wait for the item's dependencies (the group's previous phase; for its first phase the slot's
     // previous group and the circuit's previous stage); returns 1 when the item must skip its work (a device
     // error, or a wait that ran out)
-    auto deps = [&](uint32_t it) -> int {
-        const uint32_t rel = uint32_t(it - S.item_begin);
-        const uint32_t grp = rel / S.per_group, r = rel % S.per_group;
-        const uint32_t q = S.group_begin + grp;
-        uint32_t p = 0;
-        while (p + 1 < S.nphases && r >= S.ph_start[p + 1]) ++p;
-        const uint64_t key = uint64_t(q) * kMaxPhases + p;
+    auto deps = [&]() -> int {
+        const uint32_t q = S.group_begin + s_step.grp;
+        const uint64_t key = uint64_t(q) * kMaxPhases + s_step.phase;
         if (key == dep_key) return ld_relaxed_u32(reinterpret_cast<const uint32_t *>(L.status)) != 0;
         flush();
         const uint32_t *flag = nullptr, *flag2 = nullptr;
         uint32_t need = 0;
-        if (p > 0) {
-            flag = L.done + uint64_t(q) * kMaxPhases + p - 1;
-            need = S.ph[p - 1].count;
+        if (s_step.phase > 0) {
+            flag = L.done + uint64_t(q) * kMaxPhases + s_step.phase - 1;
+            need = s_step.need;
         } else {
             const uint32_t prev = L.g_prev[q];
-            if (prev != kNoGroup) {  // the slot's previous group must have finished
+            if (prev != kNoGroup) {  // the slot's previous unit must have finished
                 flag = L.done + uint64_t(prev) * kMaxPhases + kMaxPhases - 1;
                 need = 1;
             }
             flag2 = S.prev_flag;
         }
-        if (S.stall_test && grp == 0 && p == 1) ++need;  // never reached: exercises the time limit
+        if (S.stall_test && s_step.grp == 0 && s_step.phase == 1) ++need;  // never reached: exercises the time limit
         bool met = true;
         if (flag || flag2) {
             const uint64_t t0 = global_ns();
@@ -156,33 +152,35 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         return (!met || ld_relaxed_u32(reinterpret_cast<const uint32_t *>(L.status)) != 0) ? 1 : 0;
     };
 
+    uint32_t cur = 0;  // warp 0: the step of the CTA's last item (items of a CTA only move forward)
     while (true) {
-        if (tid == 0) {
-            const uint32_t it = nx_item;
-            s_item = it;
-            // the segment holding the item: last one with item_begin <= item
-            uint32_t lo = 0;
+        if (warp == 0) {
+            const uint32_t it = __shfl_sync(kFull, nx_item, 0);
             if (it < L.total_items) {
-                nx_item = atomicAdd(L.ctr, 1u);
-                uint32_t hi = L.nseg - 1;
-                if (s_seg != ~0u && it >= S.item_begin && it - S.item_begin < uint64_t(S.ngroups) * S.per_group)
-                    lo = hi = s_seg;  // still in the segment whose descriptor is staged
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (__ldg(reinterpret_cast<const unsigned long long *>(&L.segs[mid].item_begin)) <= it)
-                        lo = mid;
-                    else
-                        hi = mid - 1;
+                for (;;) {  // the last step that begins at or before the item, 32 steps at a look
+                    const uint32_t k = cur + uint32_t(tid);
+                    const uint32_t begin = k < L.nsteps ? __ldg(&L.steps[k].begin) : 0xffffffffu;
+                    const uint32_t ahead = __popc(__ballot_sync(kFull, begin <= it)) - 1;
+                    cur += ahead;
+                    if (ahead < 31) break;
+                }
+                if (tid < int(sizeof(PStep) / 4))
+                    reinterpret_cast<uint32_t *>(&s_step)[tid] = __ldg(reinterpret_cast<const uint32_t *>(L.steps + cur) + tid);
+            }
+            __syncwarp();
+            if (tid == 0) {
+                s_item = it;
+                if (it < L.total_items) {
+                    nx_item = atomicAdd(L.ctr, 1u);
+                    // the current segment's descriptor is in S: check the dependencies before the barrier
+                    if (s_step.seg == s_seg) s_abort = deps();
                 }
             }
-            s_next = lo;
-            // the current segment's descriptor is in S: check the dependencies before the barrier
-            if (it < L.total_items && lo == s_seg) s_abort = deps(it);
         }
         __syncthreads();
         const uint32_t item = s_item;
         if (item >= L.total_items) break;
-        const uint32_t want = s_next;
+        const uint32_t want = s_step.seg;
         if (want != s_seg) {  // uniform: a new segment, load its descriptor and leading phase ops
             const unsigned long long *src = reinterpret_cast<const unsigned long long *>(L.segs + want);
             unsigned long long *dst = reinterpret_cast<unsigned long long *>(&S);
@@ -194,23 +192,17 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
             }
             if (tid == 0) {
                 s_seg = want;
-                s_abort = deps(item);
+                s_abort = deps();
             }
             __syncthreads();
         }
         const FrameGeom g = geom(int(S.m));
-        const uint32_t nph = S.nphases;
         const uint32_t gframes = S.G * g.nframes;
-        const uint32_t rel = uint32_t(item - S.item_begin);
-        const uint32_t grp = rel / S.per_group, r = rel % S.per_group;
-        const uint32_t q = S.group_begin + grp;  // the group's number in this launch
-        uint32_t p = 0;
-        while (p + 1 < nph && r >= S.ph_start[p + 1]) ++p;
-        const uint32_t i = r - S.ph_start[p];
-        const uint32_t type = S.ph[p].type;
+        const uint32_t grp = s_step.grp, q = S.group_begin + grp;  // the unit's number in the stage and the launch
+        const uint32_t p = s_step.phase, type = s_step.type, count = s_step.count, i = item - s_step.begin;
         const bool abort_item = s_abort != 0;
         // the item's SV group in the unit and its place among the group's items of this phase
-        const uint32_t gi = i / S.ph[p].per, ii = i % S.ph[p].per;
+        const uint32_t gi = i / s_step.per, ii = i % s_step.per;
         const uint64_t sg = uint64_t(grp) * S.gpu + gi;  // SV group of the stage
         float2 *wv = L.wv + L.g_wv[q] + (uint64_t(gi) << S.W);
         const uint32_t *ids = S.ids + sg * S.G;
@@ -241,14 +233,14 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
                 // tile loads by cp.async (L1-cached): the item's dependencies were acquired by thread 0 (for this
                 // group and phase, in this item or an earlier one of this CTA) before the CTA barrier above, so the
                 // memory model orders them after the previous phase's writes; L1 starts empty at the launch
-                mma_ok &= gdev::pass_tile<PT, 5, PREC, false, true>(wv, S.passes[S.ph[p].arg], S.blob, S.mats, S.bfr,
+                mma_ok &= gdev::pass_tile<PT, 5, PREC, false, true>(wv, S.passes[s_step.arg], S.blob, S.mats, S.bfr,
                                                                    ii, gb, PS, reinterpret_cast<float2 *>(dsm),
                                                                    L.status, &mphase, s_pcache,
-                                                                   s_seg * 256u + S.ph[p].arg);
+                                                                   s_seg * 256u + s_step.arg);
             } else {
-                gdev::pass_tile<PT, 5, PREC, false>(wv, S.passes[S.ph[p].arg], S.blob, S.mats, S.bfr, ii, gb, PS,
+                gdev::pass_tile<PT, 5, PREC, false>(wv, S.passes[s_step.arg], S.blob, S.mats, S.bfr, ii, gb, PS,
                                                    reinterpret_cast<float2 *>(dsm), L.status, nullptr, s_pcache,
-                                                   s_seg * 256u + S.ph[p].arg);
+                                                   s_seg * 256u + s_step.arg);
             }
         } else if (type == PH_ENCODE) {
             if (fi < gframes) {
@@ -346,7 +338,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         }
         if (tid == 0) {
             __threadfence();
-            s_flag = atomicAdd(L.arrive + uint64_t(q) * kMaxPhases + p, 1u) == S.ph[p].count - 1;
+            s_flag = atomicAdd(L.arrive + uint64_t(q) * kMaxPhases + p, 1u) == count - 1;
         }
         __syncthreads();
         if (!s_flag) continue;
@@ -376,8 +368,8 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         __syncthreads();
         if (tid == 0) {
             __threadfence();
-            atomicExch(done, S.ph[p].count);
-            if (p == nph - 1) {
+            atomicExch(done, count);
+            if (p == S.nphases - 1) {
                 // the group is finished: its slot may be reused; the stage may be complete
                 atomicExch(L.done + uint64_t(q) * kMaxPhases + kMaxPhases - 1, 1u);
                 if (atomicAdd(S.fin_count, 1u) == S.ngroups - 1) {

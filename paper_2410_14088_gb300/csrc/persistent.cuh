@@ -21,10 +21,16 @@ enum PhaseType : uint32_t {
     PH_COPY = 4      // frames_per_item staged frames copied into their slots (blocks of more than one frame)
 };
 
-struct PPhase {
-    uint32_t type, count, arg;
-    uint32_t per;  // items per SV group of the unit
+// One step of the work queue: phase `phase` of a unit, `count` items from item `begin` on.
+struct PStep {
+    uint32_t begin, seg, grp;  // first item; segment (stage of a circuit); unit of the segment
+    uint32_t phase, type, arg;
+    uint32_t per;    // items per SV group of the unit
+    uint32_t need;   // items of the unit's previous phase
+    uint32_t count;
+    uint32_t pad[3];
 };
+static_assert(sizeof(PStep) % 16 == 0, "steps are read as words");
 
 constexpr int kMaxPhases = 128;
 // threads per CTA: 128 in launches whose dense ops run on tcgen05 (one thread per index group of a width-5 op, four CTAs
@@ -32,19 +38,14 @@ constexpr int kMaxPhases = 128;
 __host__ __device__ constexpr uint32_t persistent_threads(bool um) { return um ? 128u : 256u; }
 constexpr uint32_t kNoGroup = 0xffffffffu;
 
-// One segment of the work queue: one stage of one circuit, its SV groups taken gpu at a time as units, which the queue
-// and its counters call groups. The queue holds ngroups (units) x per_group items starting at item_begin; its units take
-// the launch's numbers group_begin .. group_begin + ngroups - 1 (working-vector slot and the done/arrive counters
-// follow that number).
+// One stage of one circuit, its SV groups taken gpu at a time as units. Its units take the launch's numbers group_begin
+// and on (working-vector slot and the done/arrive counters follow that number).
 struct PSeg {
-    uint64_t item_begin;
     uint32_t group_begin;
-    uint32_t W, G, ngroups, m, nphases, per_group, npre, pre_begin, pbf16;
+    uint32_t W, G, ngroups, m, nphases, npre, pre_begin, pbf16;  // ngroups: units
     uint32_t gpu;  // SV groups per unit
     int e;
     uint32_t stall_test;  // 1: group 0's second phase waits for a count never reached (bounded-wait test)
-    PPhase ph[kMaxPhases];
-    uint32_t ph_start[kMaxPhases];
     const PassDev *passes;
     const OpDev *ops;
     const float2 *mats;
@@ -73,8 +74,9 @@ struct PSeg {
 };
 
 struct PLaunch {
-    const PSeg *segs;        // device array, ordered by item_begin
-    uint32_t nseg;
+    const PSeg *segs;
+    const PStep *steps;      // in queue order
+    uint32_t nsteps;
     uint64_t total_items;    // below 2^32
     uint32_t total_groups;
     // per unit of the launch (host-planned working-vector slots): amplitude offset of its slot in wv, frame offset of its
