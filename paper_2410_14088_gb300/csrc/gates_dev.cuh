@@ -98,6 +98,33 @@ __device__ __forceinline__ void apply_dense_k1(float2 *tile, const float2 *U, co
     }
 }
 
+// apply_dense with the width (up to 5) at run time and its inputs in local memory: a tcgen05 kernel's passes of tiles
+// below 4096 amplitudes (a plan's stages of small working vectors in a launch whose other passes run on tcgen05), which
+// are rare and small; not inlined, so that the kernel's registers are not sized for it. The same products in the same
+// order as apply_dense.
+template <int NT>
+__device__ __noinline__ void apply_dense_small(uint32_t k, float2 *tile, const float2 *U, const uint32_t *cb,
+                                               const uint32_t *osw, uint32_t T) {
+    const uint32_t D = 1u << k, ngroups = 1u << (T - k);
+    for (uint32_t g = threadIdx.x; g < ngroups; g += NT) {
+        const uint32_t sb = cb[g & 63u] ^ cb[64u + (g >> 6)];
+        float2 x[32];
+#pragma unroll 1
+        for (uint32_t c = 0; c < D; ++c) x[c] = tile[sb ^ osw[c]];
+#pragma unroll 1
+        for (uint32_t r = 0; r < D; ++r) {
+            float ar = 0.f, ai = 0.f;
+#pragma unroll 1
+            for (uint32_t c = 0; c < D; ++c) {
+                const float2 u = U[r * D + c];
+                ar = fmaf(u.x, x[c].x, ar); ar = fmaf(-u.y, x[c].y, ar);
+                ai = fmaf(u.x, x[c].y, ai); ai = fmaf(u.y, x[c].x, ai);
+            }
+            tile[sb ^ osw[r]] = make_float2(ar, ai);
+        }
+    }
+}
+
 __device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
     const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
@@ -793,9 +820,10 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
             }
             if constexpr (UM) {
                 // a tcgen05 pass (T = 12) runs every dense op of width 3 to 5 above (widths 3 and 4 come widened
-                // to 5), and width 6 in TF32; what is left here is width 1 or 2, or 6 in split BF16, on CUDA cores,
-                // so no other dense form is compiled in
+                // to 5), and width 6 in TF32; what is left here is width 1 or 2, 6 in split BF16, and the passes of
+                // smaller tiles in a launch of the persistent kernel, on CUDA cores
                 if (k <= 2) apply_dense_dispatch<NT, 2, PREC>(k, tile, M, bfr + op.bfrag, cb, osw, T);
+                else if (k <= 5) apply_dense_small<NT>(k, tile, M, cb, osw, T);
                 else if constexpr (KMAX >= 6) apply_dense<NT, 6>(tile, M, cb, osw, T);
             } else if constexpr (KMAX >= 1) {
                 apply_dense_dispatch<NT, KMAX, PREC>(k, tile, M, bfr + op.bfrag, cb, osw, T);

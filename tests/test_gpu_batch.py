@@ -102,3 +102,17 @@ def test_batch_rejects_malformed():
     with pytest.raises(qsim.QsimError) as ei:
         qsim.run_batch([raw])
     assert ei.value.code == qsim.E_INVALID
+
+
+@pytest.mark.parametrize("prec", [qsim.PREC_TF32, qsim.PREC_BF16X3], ids=["tf32", "bf16x3"])
+def test_batch_on_tcgen05_with_small_working_vectors(prec):
+    """Working vectors below 4096 amplitudes (their tiles are too) beside larger ones whose dense ops run on tcgen05:
+    every dense op of the small passes is applied, in the products' order of the stream engine."""
+    plans = [(c, qsim.plan_stages(c, m=m, inner=2, k=5, eps=1e-3, prec=prec, tcgen05=1, reorder=2, diag_exempt=1))
+             for c, m in ((inputs.random_brick(13, 6, 2), 9), (inputs.random_brick(16, 6, 3), 12),
+                          (inputs.qft_rz_cx(11, 2, 4), 7), (inputs.grover(12, 3, 77), 8))]
+    states, _ = qsim.run_batch([p for _, p in plans])
+    for (c, p), st in zip(plans, states):
+        ref = qsim.run(p)
+        assert streams_of(ref, 1 << (c.n - p.cfg.m)) == streams_of(st, 1 << (c.n - p.cfg.m)), c.family
+        assert st.fidelity(oracle.simulate(c)) >= 0.99
