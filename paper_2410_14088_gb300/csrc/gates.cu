@@ -32,6 +32,7 @@ namespace {
 
 using namespace gdev;
 constexpr int NT = 128;
+constexpr int kPassSmemMost = 220 * 1024;  // dynamic shared memory of a pass, 6 KB of PassSmem beside it
 
 // One wave of resident CTAs, each looping over tiles of all the launch's groups
 // (one tile buffer per CTA; several resident CTAs per SM keep loads, ops and
@@ -42,24 +43,30 @@ constexpr int NT = 128;
 // on load/store-only passes.)
 // UM: the pass's k = 5 dense ops run on tcgen05 (a separate instantiation, so that the warp-MMA kernels
 // keep their own register allocation)
+// Teams of 128 threads per CTA, a tile each, at most. Without tcgen05 four share one pass blob: a blob of many ops (56 KB
+// in the 28-op passes of a random circuit) beside every 32 KB tile left two tiles, 8 warps, per SM; four tiles beside one
+// blob are the 16 warps that 128 registers a thread allow. The split-BF16 warp MMAs take 168 registers (three teams),
+// width 6 takes 255, and the tcgen05 forms size TMEM and B by the tile.
 template <int KMAX, int PREC, bool UM>
-__host__ __device__ constexpr int pass_threads() {
-    return NT;
+__host__ __device__ constexpr int pass_teams() {
+    return UM || KMAX >= 6 ? 1 : PREC == QSIM_PREC_BF16X3 && KMAX >= 4 ? 3 : 4;
 }
+// CTAs of one team that fit an SM by registers
 template <int KMAX, int PREC, bool UM>
 __host__ __device__ constexpr int pass_min_blocks() {
-    return KMAX >= 6 ? 2 : (PREC == QSIM_PREC_BF16X3 && KMAX >= 4) ? 3 : 4;
+    return pass_teams<KMAX, PREC, UM>() > 1 ? 1 : KMAX >= 6 ? 2 : (PREC == QSIM_PREC_BF16X3 && KMAX >= 4) ? 3 : 4;
 }
 
 template <int KMAX, int PREC, bool UM>
-__global__ void __launch_bounds__(pass_threads<KMAX, PREC, UM>(), pass_min_blocks<KMAX, PREC, UM>())
+__global__ void __launch_bounds__(NT * pass_teams<KMAX, PREC, UM>(), pass_min_blocks<KMAX, PREC, UM>())
     k_pass(float2 *__restrict__ wv, uint32_t W, uint64_t ntiles, const __grid_constant__ PassDev P,
            const uint4 *__restrict__ blob, const float2 *__restrict__ mats, const uint32_t *__restrict__ bfr,
            const uint64_t *__restrict__ gbase, uint32_t *ctr, int *status) {
     extern __shared__ float4 dyn_smem[];
-    __shared__ PassSmem S;
-    pass_tiles<pass_threads<KMAX, PREC, UM>(), KMAX, PREC, UM>(wv, W, ntiles, P, blob, mats, bfr, gbase, S,
-                                                                reinterpret_cast<float2 *>(dyn_smem), ctr, status);
+    constexpr int TEAMS = pass_teams<KMAX, PREC, UM>();
+    __shared__ PassSmem S[TEAMS];
+    pass_tiles<NT, KMAX, PREC, UM, TEAMS>(wv, W, ntiles, P, blob, mats, bfr, gbase, S[threadIdx.x / NT],
+                                          reinterpret_cast<float2 *>(dyn_smem), ctr, status);
 }
 
 // Resident CTAs per SM of one k_pass instantiation at a given dynamic shared memory size (cached), from the
@@ -67,22 +74,22 @@ __global__ void __launch_bounds__(pass_threads<KMAX, PREC, UM>(), pass_min_block
 // 228 KB of shared memory with 1 KB reserved per CTA). (The runtime's occupancy query answered 1 here where
 // 4 CTAs per SM were resident.)
 template <int KMAX, int PREC, bool UM>
-int pass_blocks_per_sm(size_t smem) {
+int pass_blocks_per_sm(size_t smem, int nt) {
     static std::mutex mu;
-    static std::map<size_t, int> cache;
+    static std::map<std::pair<size_t, int>, int> cache;
     std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(smem);
+    const std::pair<size_t, int> key(smem, nt);
+    auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     cudaFuncAttributes fa{};
     int nb = 1;
-    constexpr int nt = pass_threads<KMAX, PREC, UM>();
     if (cudaFuncGetAttributes(&fa, k_pass<KMAX, PREC, UM>) == cudaSuccess) {
         const int regs = ((fa.numRegs > 0 ? fa.numRegs : 255) + 7) & ~7;
         const int by_regs = 65536 / (regs * nt);
         const int by_smem = int((228u * 1024u) / (smem + fa.sharedSizeBytes + 1024u));
         nb = std::max(1, std::min(std::min(by_regs, by_smem), std::min(2048 / nt, 32)));
     }
-    cache[smem] = nb;
+    cache[key] = nb;
     return nb;
 }
 
@@ -98,39 +105,40 @@ int num_sms() {
 }
 
 template <int KMAX, int PREC, bool UM>
-void launch_pass_ku(dim3 grid, size_t smem, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P,
-                    const uint4 *blob, const float2 *mats, const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr,
-                    int *status) {
+void launch_pass_ku(dim3 grid, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
+                    const float2 *mats, const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {
     static bool attr_set = false;
     if (!attr_set) {
-        cudaFuncSetAttribute(k_pass<KMAX, PREC, UM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_pass<KMAX, PREC, UM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmemMost);
         // the whole unified L1/shared array as shared memory: the resident CTAs are limited by their tiles
         cudaFuncSetAttribute(k_pass<KMAX, PREC, UM>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              int(cudaSharedmemCarveoutMaxShared));
         attr_set = true;
     }
+    int teams = pass_teams<KMAX, PREC, UM>();
+    while (teams > 1 && pass_smem_bytes(P, teams) > size_t(kPassSmemMost)) --teams;  // tiles of 2^13 amplitudes
+    const size_t smem = pass_smem_bytes(P, teams);
     // grid.x tiles per group, grid.y groups: the resident CTAs loop over all of them. The grid is twice the
     // resident count so that an underestimate of it cannot leave SMs short of CTAs (measured on the 32-qubit
     // QAOA passes: one CTA per SM 0.85 ms, one resident wave 0.41 ms, two 0.41 ms, one tile per CTA 0.46 ms);
-    // CTAs that start after the tiles have run out leave at once.
+    // CTAs that start after the tiles have run out leave at once. CTAs of several teams: one wave.
     const uint64_t ntiles = uint64_t(grid.x) * grid.y;
-    const uint64_t resident = 2ull * uint64_t(pass_blocks_per_sm<KMAX, PREC, UM>(smem)) * num_sms();
+    const uint64_t resident = (teams > 1 ? 1ull : 2ull) * uint64_t(pass_blocks_per_sm<KMAX, PREC, UM>(smem, NT * teams)) * num_sms();
     const uint32_t nctas = uint32_t(ntiles < resident ? ntiles : resident);
-    k_pass<KMAX, PREC, UM><<<nctas, pass_threads<KMAX, PREC, UM>(), smem, s>>>(wv, W, ntiles, P, blob, mats, bfr,
-                                                                              gbase, ctr, status);
+    k_pass<KMAX, PREC, UM><<<nctas, NT * teams, smem, s>>>(wv, W, ntiles, P, blob, mats, bfr, gbase, ctr, status);
 }
 
 template <int KMAX, int PREC>
-void launch_pass_k(dim3 grid, size_t smem, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P,
+void launch_pass_k(dim3 grid, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P,
                    const uint4 *blob, const float2 *mats, const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr,
                    int *status) {
     if constexpr ((PREC == QSIM_PREC_TF32 || PREC == QSIM_PREC_BF16X3) && KMAX >= 5) {
         if (P.umma) {
-            launch_pass_ku<KMAX, PREC, true>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status);
+            launch_pass_ku<KMAX, PREC, true>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status);
             return;
         }
     }
-    launch_pass_ku<KMAX, PREC, false>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status);
+    launch_pass_ku<KMAX, PREC, false>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status);
 }
 
 template <int PREC, int H>
@@ -181,17 +189,17 @@ void launch_reg_prec(uint64_t ntiles, cudaStream_t s, float2 *wv, uint32_t W, co
 }
 
 template <int PREC>
-void launch_pass_prec(uint32_t kmax, dim3 grid, size_t smem, cudaStream_t s, float2 *wv, uint32_t W,
+void launch_pass_prec(uint32_t kmax, dim3 grid, cudaStream_t s, float2 *wv, uint32_t W,
                       const PassDev &P, const uint4 *blob, const float2 *mats, const uint32_t *bfr,
                       const uint64_t *gbase, uint32_t *ctr, int *status) {
     switch (kmax) {
-        case 0: launch_pass_k<0, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        case 1: launch_pass_k<1, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        case 2: launch_pass_k<2, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        case 3: launch_pass_k<3, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        case 4: launch_pass_k<4, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        case 5: launch_pass_k<5, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
-        default: launch_pass_k<6, PREC>(grid, smem, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 0: launch_pass_k<0, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 1: launch_pass_k<1, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 2: launch_pass_k<2, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 3: launch_pass_k<3, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 4: launch_pass_k<4, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        case 5: launch_pass_k<5, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
+        default: launch_pass_k<6, PREC>(grid, s, wv, W, P, blob, mats, bfr, gbase, ctr, status); break;
     }
 }
 
@@ -272,10 +280,10 @@ size_t umma_pass_smem(uint32_t umma_bits) {
     return (umma_bits & 1u) ? size_t(umma_pass_b_bytes(umma_bits)) + 1024 : 0;
 }
 
-size_t pass_smem_bytes(const PassDev &P) {
+size_t pass_smem_bytes(const PassDev &P, int teams) {
     const size_t um = umma_pass_smem(P.umma);
-    return (size_t(1) << P.T) * sizeof(float2) + um + size_t(P.blob_words) * 16 +
-           size_t(P.mat_elems) * sizeof(float2);
+    return (size_t(teams) << P.T) * sizeof(float2) + um + size_t(P.blob_words) * 16 +
+           size_t(teams) * P.mat_elems * sizeof(float2);
 }
 
 // (the reload form keeps three CTAs per SM up to 75 KB each)
@@ -348,15 +356,14 @@ void launch_pass(float2 *wv, uint32_t W, uint32_t ngroups, const PassDev *pass_h
         count_launch();
         return;
     }
-    const size_t smem = pass_smem_bytes(P);
     dim3 grid(1u << P.nout, ngroups);
     const uint32_t kmax = P.kmax;
     if (prec == QSIM_PREC_TF32 && kmax >= 3)
-        launch_pass_prec<QSIM_PREC_TF32>(kmax, grid, smem, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
+        launch_pass_prec<QSIM_PREC_TF32>(kmax, grid, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
     else if (prec == QSIM_PREC_BF16X3 && kmax >= 3)
-        launch_pass_prec<QSIM_PREC_BF16X3>(kmax, grid, smem, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
+        launch_pass_prec<QSIM_PREC_BF16X3>(kmax, grid, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
     else
-        launch_pass_prec<QSIM_PREC_FP32>(kmax, grid, smem, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
+        launch_pass_prec<QSIM_PREC_FP32>(kmax, grid, s, wv, W, P, blob_dev, mats_dev, bfr_dev, gbase_dev, ctr, status);
     count_launch();
 }
 

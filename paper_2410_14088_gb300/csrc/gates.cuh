@@ -126,6 +126,6 @@ void launch_pass(float2 *wv, uint32_t W, uint32_t ngroups, const PassDev *pass_h
 bool reg_pass_fits(const PassDev &P, int prec);
 
 // dynamic shared memory of one tile pass (tile, B operand and alignment when on tcgen05, blob, matrices)
-size_t pass_smem_bytes(const PassDev &P);
+size_t pass_smem_bytes(const PassDev &P, int teams = 1);
 
 }  // namespace qsim

@@ -20,13 +20,29 @@ __device__ __forceinline__ uint32_t swz(uint32_t i) {
     return i ^ (((i >> 4) ^ (i >> 8) ^ (i >> 12)) & 15u);
 }
 
-// CTA-cooperative copy of a descriptor (4-byte words; src may be kernel-parameter or global memory)
+// A tile belongs to a team of NT threads, NT to the power of two: the whole CTA, or one of several in a pass kernel whose
+// teams share the pass blob. team_tid numbers its threads and team_sync is its barrier (ids as constants: an id in a
+// register would reserve all sixteen barriers; 0 stays the CTA's).
+template <int NT>
+__device__ __forceinline__ uint32_t team_tid() {
+    return threadIdx.x & uint32_t(NT - 1);
+}
+template <int NT>
+__device__ __forceinline__ void team_sync() {
+    const uint32_t team = threadIdx.x / uint32_t(NT);
+    if (team == 0) asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    else if (team == 1) asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
+    else if (team == 2) asm volatile("bar.sync 3, %0;" ::"n"(NT) : "memory");
+    else asm volatile("bar.sync 4, %0;" ::"n"(NT) : "memory");
+}
+
+// Team-cooperative copy of a descriptor (4-byte words; src may be kernel-parameter or global memory)
 template <int NT, class T>
 __device__ __forceinline__ void coop_copy(T &dst, const T &src) {
     static_assert(sizeof(T) % 4 == 0, "descriptor size");
     const uint32_t *s = reinterpret_cast<const uint32_t *>(&src);
     uint32_t *d = reinterpret_cast<uint32_t *>(&dst);
-    for (int t = threadIdx.x; t < int(sizeof(T) / 4); t += NT) d[t] = s[t];
+    for (int t = team_tid<NT>(); t < int(sizeof(T) / 4); t += NT) d[t] = s[t];
 }
 
 struct PassSmem {
@@ -48,39 +64,71 @@ struct PassSmem {
 };
 static_assert(sizeof(OpDev) % 16 == 0, "op descriptors are copied as 16-byte words");
 
-template <int NT, int K>
-__device__ __forceinline__ void apply_dense(float2 *tile, const float2 *U, const uint32_t *cb, const uint32_t *osw,
-                                            uint32_t T) {
+// Dense op of width K on CUDA cores, GP index groups per thread at a time and two matrix rows. The matrix comes from
+// shared memory, every lane the same element, and a 16-byte load of it takes as long to reach the registers (512 bytes
+// a warp at 128 a cycle) as four FMAs per lane take to issue: with one group per thread the loads of U bound the op
+// (width 4 on 2^26 amplitudes: 284 us against 107 us of FMAs). GP groups share each load; width 4 holds two groups'
+// 32 inputs in 64 registers, width 5 has room for one. Two rows double the independent FMA chains, which is what a
+// launch of few tiles waits for.
+template <int NT, int K, int GP>
+__device__ __forceinline__ void apply_dense_groups(float2 *tile, const float2 *U, const uint32_t *cb,
+                                                   const uint32_t *osw, uint32_t T) {
     constexpr int D = 1 << K;
     const uint32_t ngroups = 1u << (T - K);
-    for (uint32_t g = threadIdx.x; g < ngroups; g += NT) {
-        const uint32_t sb = cb[g & 63u] ^ cb[64u + (g >> 6)];
-        float2 x[D];
+    for (uint32_t g = team_tid<NT>(); g < ngroups; g += NT * GP) {
+        uint32_t sb[GP];
+        float2 x[GP][D];
 #pragma unroll
-        for (int c = 0; c < D; ++c) x[c] = tile[sb ^ osw[c]];
+        for (int p = 0; p < GP; ++p) {
+            const uint32_t gp = g + NT * p;
+            sb[p] = cb[gp & 63u] ^ cb[64u + (gp >> 6)];
+#pragma unroll
+            for (int c = 0; c < D; ++c) x[p][c] = tile[sb[p] ^ osw[c]];
+        }
 #pragma unroll 1
-        for (int r = 0; r < D; ++r) {
+        for (int r = 0; r < D; r += 2) {
             const float4 *row = reinterpret_cast<const float4 *>(U + r * D);
-            float ar = 0.f, ai = 0.f;
-            if constexpr (D == 2) {
-                float4 u = row[0];
-                ar = fmaf(u.x, x[0].x, ar); ar = fmaf(-u.y, x[0].y, ar);
-                ai = fmaf(u.x, x[0].y, ai); ai = fmaf(u.y, x[0].x, ai);
-                ar = fmaf(u.z, x[1].x, ar); ar = fmaf(-u.w, x[1].y, ar);
-                ai = fmaf(u.z, x[1].y, ai); ai = fmaf(u.w, x[1].x, ai);
-            } else {
+            float ar[2][GP] = {}, ai[2][GP] = {};
 #pragma unroll
-                for (int c = 0; c < D; c += 2) {
-                    float4 u = row[c / 2];
-                    ar = fmaf(u.x, x[c].x, ar); ar = fmaf(-u.y, x[c].y, ar);
-                    ai = fmaf(u.x, x[c].y, ai); ai = fmaf(u.y, x[c].x, ai);
-                    ar = fmaf(u.z, x[c + 1].x, ar); ar = fmaf(-u.w, x[c + 1].y, ar);
-                    ai = fmaf(u.z, x[c + 1].y, ai); ai = fmaf(u.w, x[c + 1].x, ai);
+            for (int c = 0; c < D; c += 2) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float4 u = row[q * (D / 2) + c / 2];
+#pragma unroll
+                    for (int p = 0; p < GP; ++p) {
+                        ar[q][p] = fmaf(u.x, x[p][c].x, ar[q][p]);
+                        ar[q][p] = fmaf(-u.y, x[p][c].y, ar[q][p]);
+                        ai[q][p] = fmaf(u.x, x[p][c].y, ai[q][p]);
+                        ai[q][p] = fmaf(u.y, x[p][c].x, ai[q][p]);
+                        ar[q][p] = fmaf(u.z, x[p][c + 1].x, ar[q][p]);
+                        ar[q][p] = fmaf(-u.w, x[p][c + 1].y, ar[q][p]);
+                        ai[q][p] = fmaf(u.z, x[p][c + 1].y, ai[q][p]);
+                        ai[q][p] = fmaf(u.w, x[p][c + 1].x, ai[q][p]);
+                    }
                 }
             }
-            tile[sb ^ osw[r]] = make_float2(ar, ai);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int p = 0; p < GP; ++p) tile[sb[p] ^ osw[r + q]] = make_float2(ar[q][p], ai[q][p]);
         }
     }
+}
+
+// The groups of a 4096-amplitude tile divide evenly over the threads at every width up to 5; smaller tiles may leave
+// threads without one.
+template <int NT, int K, int MOST = 4>
+__device__ __forceinline__ void apply_dense(float2 *tile, const float2 *U, const uint32_t *cb, const uint32_t *osw,
+                                            uint32_t T) {
+    constexpr int per_thread = (4096 >> K) / NT, most = MOST == 1 ? 1 : K <= 3 ? 4 : K == 4 ? 2 : 1;
+    constexpr int GP = per_thread < 1 ? 1 : per_thread < most ? per_thread : most;
+    if constexpr (GP > 1) {
+        if (T == 12) {
+            apply_dense_groups<NT, K, GP>(tile, U, cb, osw, T);
+            return;
+        }
+    }
+    apply_dense_groups<NT, K, 1>(tile, U, cb, osw, T);
 }
 
 template <int NT>
@@ -88,7 +136,7 @@ __device__ __forceinline__ void apply_dense_k1(float2 *tile, const float2 *U, co
                                                uint32_t T) {
     const uint32_t ngroups = 1u << (T - 1);
     const float2 u00 = U[0], u01 = U[1], u10 = U[2], u11 = U[3];
-    for (uint32_t g = threadIdx.x; g < ngroups; g += NT) {
+    for (uint32_t g = team_tid<NT>(); g < ngroups; g += NT) {
         const uint32_t i0 = cb[g & 63u] ^ cb[64u + (g >> 6)], i1 = i0 ^ osw[1];
         const float2 x0 = tile[i0], x1 = tile[i1];
         tile[i0] = make_float2(u00.x * x0.x - u00.y * x0.y + u01.x * x1.x - u01.y * x1.y,
@@ -106,7 +154,7 @@ template <int NT>
 __device__ __noinline__ void apply_dense_small(uint32_t k, float2 *tile, const float2 *U, const uint32_t *cb,
                                                const uint32_t *osw, uint32_t T) {
     const uint32_t D = 1u << k, ngroups = 1u << (T - k);
-    for (uint32_t g = threadIdx.x; g < ngroups; g += NT) {
+    for (uint32_t g = team_tid<NT>(); g < ngroups; g += NT) {
         const uint32_t sb = cb[g & 63u] ^ cb[64u + (g >> 6)];
         float2 x[32];
 #pragma unroll 1
@@ -199,7 +247,7 @@ __device__ __forceinline__ void apply_dense_mma(float2 *tile, const uint32_t *__
     constexpr uint32_t ROWS = (1u << (12 - K)) / (NT / 32);    // index groups per warp
     constexpr uint32_t MT = ROWS / 16;                         // m16 tiles per warp
     static_assert(MT >= 1, "tensor-core tile needs 16 rows per warp");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = team_tid<NT>() >> 5;
     const uint32_t gq = lane >> 2, tq = lane & 3;
     const uint32_t row0 = warp * ROWS;
     uint32_t base[MT][2];  // swizzled bases of the lane's index groups
@@ -610,20 +658,20 @@ __device__ __forceinline__ void apply_dense_dispatch(uint32_t k, float2 *tile, c
 template <int NT>
 __device__ __forceinline__ void pass_setup(const PassDev &pd, PassSmem &S) {
     coop_copy<NT>(S.p, pd);
-    __syncthreads();
+    team_sync<NT>();
     const uint32_t T = S.p.T;
     constexpr uint32_t A = NT == 256 ? 8 : 7;
     if (T == 12) {
         // element i = tid + NT u: tile bits 0..A-1 from tid (thread_tile_offset), A..11 from u (disjoint working
         // bits)
-        const uint32_t x = threadIdx.x;
+        const uint32_t x = team_tid<NT>();
         if (x < (4096u / NT)) {
             uint32_t h = 0;
             for (uint32_t t = A; t < 12; ++t) h |= ((x >> (t - A)) & 1u) << S.p.tile_pos[t];
             S.off12[x] = h;
         }
     }
-    __syncthreads();
+    team_sync<NT>();
 }
 
 constexpr uint32_t kCgBatch = 16;
@@ -636,7 +684,7 @@ __device__ __forceinline__ uint32_t thread_tile_offset(const PassSmem &S) {
     constexpr uint32_t A = NT == 256 ? 8 : 7;
     uint32_t o = 0;
 #pragma unroll
-    for (uint32_t t = 0; t < A; ++t) o |= ((uint32_t(threadIdx.x) >> t) & 1u) << S.p.tile_pos[t];
+    for (uint32_t t = 0; t < A; ++t) o |= ((team_tid<NT>() >> t) & 1u) << S.p.tile_pos[t];
     return o;
 }
 
@@ -677,7 +725,7 @@ template <int NT, bool CG>
 __device__ __forceinline__ void tile_load(const float2 *__restrict__ g, uint64_t base, const PassSmem &S,
                                           float2 *tile) {
     const uint32_t T = S.p.T, L = S.p.L, lmask = (1u << L) - 1;
-    const int tid = threadIdx.x;
+    const int tid = team_tid<NT>();
     if (fast12<NT>(S)) {
         const float2 *gt = g + (base | uint64_t(thread_tile_offset<NT>(S)));
         const uint32_t tq = swz_thread<NT>(tid);
@@ -721,39 +769,43 @@ __device__ __forceinline__ void tile_store(float2 *__restrict__ g, uint64_t base
                                            const float2 *tile) {
     const uint32_t T = S.p.T, L = S.p.L, lmask = (1u << L) - 1;
     if (fast12<NT>(S)) {
-        const uint32_t tid = threadIdx.x, tq = swz_thread<NT>(tid);
+        const uint32_t tid = team_tid<NT>(), tq = swz_thread<NT>(tid);
         float2 *gt = g + (base | uint64_t(thread_tile_offset<NT>(S)));
 #pragma unroll
         for (uint32_t u = 0; u < 4096u / NT; ++u) gt[S.off12[u]] = tile[(tq ^ swz_u<NT>(u)) + NT * u];
         return;
     }
-    for (uint32_t i = threadIdx.x; i < (1u << T); i += NT) g[base | (i & lmask) | hi_off(S, i >> L)] = tile[swz(i)];
+    for (uint32_t i = team_tid<NT>(); i < (1u << T); i += NT) g[base | (i & lmask) | hi_off(S, i >> L)] = tile[swz(i)];
 }
 
 // The pass blob (op descriptors, diagonal ops' index tables and phases, small
 // dense matrices) staged in shared memory with 16-byte cp.async.
-template <int NT>
 __device__ __forceinline__ void blob_load(const uint4 *__restrict__ gblob, uint32_t words, uint4 *sblob) {
-    for (uint32_t t = threadIdx.x; t < words; t += NT) cp_async16(sblob + t, gblob + t);
+    for (uint32_t t = threadIdx.x; t < words; t += blockDim.x) cp_async16(sblob + t, gblob + t);
 }
 
 // The pass's ops on a staged tile; blob: the staged pass blob; mat: the matrix
-// area for dense ops whose matrix is not in the blob. Starts with a CTA
+// area for dense ops whose matrix is not in the blob. Starts with a team
 // barrier, so the tile's and blob's loads need only have completed per thread.
-template <int NT, int KMAX, int PREC, bool UM = false>
+// SMALL: a tcgen05 launch (UM) that may hold passes of smaller tiles too.
+template <int NT, int KMAX, int PREC, bool UM = false, bool SMALL = false>
 __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2 *mat,
                                          const float2 *__restrict__ mats, const uint32_t *__restrict__ bfr,
                                          uint64_t base, uint64_t gb, PassSmem &S, uint4 *bbuf, int *status,
                                          uint32_t &phase, bool b_resident = false) {
     // b_resident: the pass's only tcgen05 op has its B operand in bbuf already (staged once per CTA)
     // phase: parity of the next MMA-completion phase (tcgen05 dense ops); false after a wait ran out
-    const int tid = threadIdx.x;
+    const int tid = team_tid<NT>();
+    auto sync = [&]() {
+        if constexpr (UM) __syncthreads();  // one team per CTA
+        else team_sync<NT>();
+    };
     const uint32_t T = S.p.T;
     const OpDev *bops = reinterpret_cast<const OpDev *>(blob);
     const float2 *bf2 = reinterpret_cast<const float2 *>(blob);
     const uint8_t *bb = reinterpret_cast<const uint8_t *>(blob);
     for (uint32_t oi = 0; oi < S.p.op_count;) {
-        __syncthreads();
+        sync();
         const OpDev &op = bops[oi];
         const uint32_t type = op.type, k = op.k;
         uint32_t adv = 1;
@@ -803,7 +855,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                     S.cb[half][v] = swz(b);
                 }
             }
-            if (op.dlut == kNoTab || !tc) __syncthreads();  // tables built above, or the matrix area filled
+            if (op.dlut == kNoTab || !tc) sync();  // tables built above, or the matrix area filled
             if constexpr (UM) {
                 if (um) {
                     bool done;
@@ -822,9 +874,15 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                 // a tcgen05 pass (T = 12) runs every dense op of width 3 to 5 above (widths 3 and 4 come widened
                 // to 5), and width 6 in TF32; what is left here is width 1 or 2, 6 in split BF16, and the passes of
                 // smaller tiles in a launch of the persistent kernel, on CUDA cores
-                if (k <= 2) apply_dense_dispatch<NT, 2, PREC>(k, tile, M, bfr + op.bfrag, cb, osw, T);
-                else if (k <= 5) apply_dense_small<NT>(k, tile, M, cb, osw, T);
-                else if constexpr (KMAX >= 6) apply_dense<NT, 6>(tile, M, cb, osw, T);
+                if (k == 1) {
+                    apply_dense_k1<NT>(tile, M, cb, osw, T);
+                } else if (k == 2) {
+                    apply_dense<NT, 2, 1>(tile, M, cb, osw, T);
+                } else if (k <= 5) {
+                    if constexpr (SMALL) apply_dense_small<NT>(k, tile, M, cb, osw, T);
+                } else if constexpr (KMAX >= 6) {
+                    apply_dense<NT, 6>(tile, M, cb, osw, T);
+                }
             } else if constexpr (KMAX >= 1) {
                 apply_dense_dispatch<NT, KMAX, PREC>(k, tile, M, bfr + op.bfrag, cb, osw, T);
             }
@@ -844,7 +902,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                 }
                 S.dconst[tid] = idx;
             }
-            __syncthreads();
+            sync();
             uint32_t dc[kDiagRun], tb[kDiagRun], lb[kDiagRun];
 #pragma unroll
             for (uint32_t d = 0; d < kDiagRun; ++d) {
@@ -898,7 +956,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
             // this tile's A_t and C: the pass constants, then every term whose constant bits are 1 over this tile,
             // the records shared out over the CTA (shared atomic adds, exact modulo 2^32)
             if (tid < 13) S.pA[tid] = pw[tid < 12 ? 192 + tid : 204];
-            __syncthreads();
+            sync();
             {
                 const uint32_t *tr = pw + kPolyHeadWords;
                 for (uint32_t i = tid; i < op.ncst; i += NT) {
@@ -908,7 +966,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                     if (b1 & b2) atomicAdd(&S.pA[t == kPolyConst ? 12u : t], tr[4 * i + 3]);
                 }
             }
-            __syncthreads();
+            sync();
             if (T == 12) {
                 // element i = tid + NT u: tile bits 0..LB-1 from tid, LB..11 from u
                 constexpr uint32_t LB = NT == 256 ? 8 : 7, HB = 12 - LB;
@@ -961,7 +1019,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                                     : 0u;
                 }
             }
-            __syncthreads();
+            sync();
             // branches that are the identity (bit b of idm) leave their amplitudes as they are
             const uint32_t idm = ((op.cctl & kCtlId0) ? 1u : 0u) | ((op.cctl & kCtlId1) ? 2u : 0u);
             const bool ctile = !(op.cctl & kCtlConst);
@@ -978,7 +1036,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
                 const float2 h = phi[x], kb = S.ck[b];
                 csq[x] = make_float2(h.x * kb.x - h.y * kb.y, h.x * kb.y + h.y * kb.x);
             }
-            __syncthreads();
+            sync();
             if (T == 12) {
                 const uint32_t tq = swz_thread<NT>(tid), lo = uint32_t(tid) & 127u, hib = uint32_t(tid) >> 7;
                 const float2 pl0 = plo[lo], pl1 = plo[128 + lo];
@@ -1064,7 +1122,7 @@ __device__ __forceinline__ bool pass_tile(float2 *__restrict__ g, const PassDev 
     if (hit) {
         b_res = cache[1] != 0;
     } else {
-        blob_load<NT>(gblob + S.p.blob_off, S.p.blob_words, blob);
+        blob_load(gblob + S.p.blob_off, S.p.blob_words, blob);
         if (cache) {
             // a pass with a single tcgen05 op keeps that op's B operand staged for the calls that hit the cache
             if constexpr (UM) {
@@ -1097,7 +1155,7 @@ __device__ __forceinline__ bool pass_tile(float2 *__restrict__ g, const PassDev 
     cp_async_wait_all();
     uint32_t phase = phase_io ? *phase_io : 0u;
     const bool ok =
-        tile_ops<NT, KMAX, PREC, UM>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
+        tile_ops<NT, KMAX, PREC, UM, UM>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
     __syncthreads();
     tile_store<NT>(g, base, S, tile);
     if (phase_io) {
@@ -1117,41 +1175,46 @@ __device__ __forceinline__ bool pass_tile(float2 *__restrict__ g, const PassDev 
     return ok;
 }
 
-// One pass over many tiles (streams mode): CTA c takes tiles c, c + gridDim.x, ... of the launch's groups
-// (tile t: group t >> nout, tile index t & (2^nout - 1)). The pass descriptor, the pass blob, the TMEM
-// accumulator and the MMA mbarrier are set up once per CTA instead of once per tile, and when the pass has a
-// single tcgen05 op its B operand is staged once too; each tile is then loaded, updated and stored as in
-// pass_tile, with several CTAs per SM keeping loads, ops and stores of different tiles in flight.
+// One pass over many tiles (streams mode), blockDim.x / NT (at most TEAMS) teams of NT threads per CTA, each with a tile of
+// its own; the pass blob
+// (shared by the teams), the descriptor, the TMEM accumulator and the MMA mbarrier are set up once per CTA instead of
+// once per tile, and when the pass has a single tcgen05 op its B operand is staged once too; each tile is then loaded,
+// updated and stored as in pass_tile, with several teams per SM keeping loads, ops and stores of different tiles in
+// flight. Tile t is tile index t & (2^nout - 1) of group t >> nout.
 // Tiles are handed out in launch order from a counter (ctr[0]; ctr[1] counts the CTAs that finished, and the last
 // one zeroes both for the next launch on the stream), so the tiles in flight stay a narrow window of the working
 // vector: its 64-byte rows that share DRAM pages are read and written close together in time.
-template <int NT, int KMAX, int PREC, bool UM = false>
+// S: a team's; dyn: the teams' tiles, B operand, blob, then the teams' matrix areas.
+template <int NT, int KMAX, int PREC, bool UM, int TEAMS>
 __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, uint64_t ntiles, const PassDev &pd,
                                            const uint4 *__restrict__ gblob, const float2 *__restrict__ mats,
                                            const uint32_t *__restrict__ bfr, const uint64_t *__restrict__ gbase,
                                            PassSmem &S, float2 *dyn, uint32_t *ctr, int *status) {
-    // the CTA's next tile, in a slot by iteration parity: thread 0 writes slot (it + 1) & 1 while a slower warp may
+    // a team's next tile, in a slot by iteration parity: its thread 0 writes slot (it + 1) & 1 while a slower warp may
     // still be reading slot it & 1 after the end-of-iteration barrier; that slot is next written two barriers later
-    __shared__ uint32_t s_next[2];
+    __shared__ uint32_t s_next[TEAMS][2];
+    const uint32_t team = threadIdx.x / uint32_t(NT), tid = team_tid<NT>();
+    const uint32_t teams = TEAMS > 1 ? blockDim.x / uint32_t(NT) : 1u;
     pass_setup<NT>(pd, S);
     const uint32_t T = S.p.T;
-    static_assert(!UM || ((PREC == QSIM_PREC_TF32 || PREC == QSIM_PREC_BF16X3) && NT == 128 && KMAX >= 5),
+    static_assert(!UM || ((PREC == QSIM_PREC_TF32 || PREC == QSIM_PREC_BF16X3) && NT == 128 && KMAX >= 5 && TEAMS == 1),
                   "tcgen05 passes: TF32 or split BF16, k = 5");
     bool um = false;
     if constexpr (UM) um = S.p.umma != 0;
-    float2 *tile = dyn;
+    float2 *tiles = dyn;
     uint4 *bbuf = nullptr;
     if (um) {
         const uint32_t pad = (1024u - (umma::smem_addr(dyn) & 1023u)) & 1023u;
-        tile = reinterpret_cast<float2 *>(reinterpret_cast<uint8_t *>(dyn) + pad);
-        bbuf = reinterpret_cast<uint4 *>(tile + 4096);
+        tiles = reinterpret_cast<float2 *>(reinterpret_cast<uint8_t *>(dyn) + pad);
+        bbuf = reinterpret_cast<uint4 *>(tiles + 4096);
         if (threadIdx.x < 32) umma::tmem_alloc(umma::smem_addr(&S.tmem), umma_pass_tmem_cols(S.p.umma));
         if (threadIdx.x == 0) umma::mbar_init(umma::smem_addr(&S.mbar), 1);
         umma::fence_before_sync();
     }
-    uint4 *blob = reinterpret_cast<uint4 *>(tile + (1u << T)) + (um ? umma_pass_b_bytes(S.p.umma) / 16 : 0u);
-    float2 *mat = reinterpret_cast<float2 *>(blob + S.p.blob_words);
-    blob_load<NT>(gblob + S.p.blob_off, S.p.blob_words, blob);
+    float2 *tile = tiles + (size_t(team) << T);
+    uint4 *blob = reinterpret_cast<uint4 *>(tiles + (size_t(teams) << T)) + (um ? umma_pass_b_bytes(S.p.umma) / 16 : 0u);
+    float2 *mat = reinterpret_cast<float2 *>(blob + S.p.blob_words) + team * S.p.mat_elems;
+    blob_load(gblob + S.p.blob_off, S.p.blob_words, blob);
     cp_async_wait_all();
     __syncthreads();
     // a single tcgen05 op: its B operand stays in bbuf for every tile of this CTA
@@ -1177,8 +1240,9 @@ __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, 
     bool ok = true;
     const uint64_t tmask = (1ull << S.p.nout) - 1;
     uint32_t it = 0;
-    for (uint64_t t = blockIdx.x; t < ntiles; ++it) {
-        if (threadIdx.x == 0) s_next[it & 1u] = gridDim.x + atomicAdd(ctr, 1u);  // read after the barrier below
+    // the first tiles go to the CTAs' first teams: a launch of few tiles spreads over the SMs
+    for (uint64_t t = uint64_t(team) * gridDim.x + blockIdx.x; t < ntiles; ++it) {
+        if (tid == 0) s_next[team][it & 1u] = gridDim.x * teams + atomicAdd(ctr, 1u);  // read after the barrier below
         const uint64_t grp = t >> S.p.nout, cta = t & tmask;
         float2 *g = wv + (grp << W);
         const uint64_t gb = gbase ? gbase[grp] : 0ull;
@@ -1186,12 +1250,13 @@ __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, 
         tile_load<NT, false>(g, base, S, tile);
         cp_async_wait_all();
         ok = tile_ops<NT, KMAX, PREC, UM>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
-        __syncthreads();
+        team_sync<NT>();
         tile_store<NT>(g, base, S, tile);
-        __syncthreads();  // the next tile's loads overwrite the tile; s_next[it & 1] is visible
+        team_sync<NT>();  // the next tile's loads overwrite the tile; s_next[team][it & 1] is visible
         if (!ok) break;   // uniform: the MMA wait ran out (status set)
-        t = s_next[it & 1u];
+        t = s_next[team][it & 1u];
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
         // every tile counter increment of this CTA precedes its arrival; the last CTA to arrive resets both
         __threadfence();
