@@ -44,18 +44,33 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_decode(const BlockSlot *__restr
     __shared__ uint2 s_pre_ab[NP > 0 ? NP : 1];
     __shared__ TeamSmem S;
     const Team tm{threadIdx.x, blockDim.x, 1};
-    if (NP > 0 && threadIdx.x < pre.count) {
-        s_pre[threadIdx.x] = pre.ops[threadIdx.x];
-        s_pre_ab[threadIdx.x] = pre_setup(pre.ops[threadIdx.x]);
+    // the leading ops' descriptors and tables, staged once per CTA beside its tile
+    uint8_t *tabs = tile + team_tile_bytes(g.C);
+    if (NP > 0) {
+        constexpr uint32_t W = sizeof(OpDev) / 4;
+        for (uint32_t i = threadIdx.x; i < pre.count * W; i += blockDim.x)
+            reinterpret_cast<uint32_t *>(s_pre)[i] = __ldg(reinterpret_cast<const uint32_t *>(pre.ops) + i);
+        __syncthreads();
+        for (uint32_t o = 0; o < pre.count; ++o) {
+            const bool diag = s_pre[o].type == OP_DIAG;
+            if (threadIdx.x == 0)
+                s_pre_ab[o] = make_uint2(o * kPreTabBytes, diag ? o * kPreTabBytes + 160u : kPreFlip);
+            if (!diag) continue;
+            uint64_t *d = reinterpret_cast<uint64_t *>(tabs + o * kPreTabBytes);
+            const uint64_t *lut = reinterpret_cast<const uint64_t *>(pre.mats + s_pre[o].dlut);
+            const uint64_t *ph = reinterpret_cast<const uint64_t *>(pre.mats + s_pre[o].mat);
+            for (uint32_t i = threadIdx.x; i < 20u + (1u << s_pre[o].k); i += blockDim.x)
+                d[i] = __ldg(i < 20u ? lut + i : ph + (i - 20u));
+        }
+        __syncthreads();
     }
-    if (NP > 0) __syncthreads();
     const uint64_t items = uint64_t(nblocks) * g.nframes;
     for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t j = uint32_t(item / g.nframes), f = uint32_t(item % g.nframes);
         const BlockSlot sl = table[ids ? ids[j] : b0 + j];
         decode_frame_team<NP, REL>(tm, S, tile, sl.ptr, sl.bytes, g, m, f, wv + (uint64_t(j) << m) + uint64_t(f) * g.F,
                                    hist ? hist + uint64_t(j) * 32 : nullptr, status, s_pre, s_pre_ab, pre.count,
-                                   pre.mats, pre.count ? (uint64_t(j % pre.G) << m) : 0,
+                                   tabs, pre.count ? (uint64_t(j % pre.G) << m) : 0,
                                    pre.count ? pre.gbase[j / pre.G] : 0);
         tm.sync();
     }
@@ -214,20 +229,28 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_encode_block(const float2 *__re
     const FrameGeom g = geom(m);
     __shared__ TeamSmem S;
     const Team tm{threadIdx.x, blockDim.x, 1};
-    if (tm.t == 0) {
-        S.bc = atomicAdd(scr.ticket, 1u);
-        S.bc2 = ld_relaxed_u32(scr.epoch) & kEpochMask;
+    uint32_t f = 0, epoch = 0;
+    if (g.nframes > 1) {
+        if (tm.t == 0) {
+            S.bc = atomicAdd(scr.ticket, 1u);
+            S.bc2 = ld_relaxed_u32(scr.epoch) & kEpochMask;
+        }
+        tm.sync();
+        f = uint32_t(S.bc);
+        epoch = uint32_t(S.bc2);
     }
-    tm.sync();
-    const uint32_t f = uint32_t(S.bc), epoch = uint32_t(S.bc2);
     load_rows_team(tm, tile, amps + uint64_t(f) * g.F, g.C);
     const EncFrame r = encode_frame_team<REL>(tm, S, tile, g, e, res.status);
-    if (tm.t < 32) {
-        const uint32_t excl = lookback_warp(scr.state, f, epoch, r.len, res.status);
-        if (tm.t == 0) S.flag = excl;
+    uint32_t excl = 0;
+    if (g.nframes > 1) {
+        if (tm.t < 32) {
+            const uint32_t x = lookback_warp(scr.state, f, epoch, r.len, res.status);
+            if (tm.t == 0) S.flag = x;
+        }
+        tm.sync();
+        excl = S.flag;
     }
-    tm.sync();
-    const uint64_t off = g.data_start + S.flag, total = off + r.len;
+    const uint64_t off = g.data_start + excl, total = off + r.len;
     if (total <= cap) {
         uint4 *d = reinterpret_cast<uint4 *>(out + off);
         for (uint32_t i = tm.t; i < r.len / 16u; i += tm.n) d[i] = reinterpret_cast<const uint4 *>(tile)[i];
@@ -242,7 +265,7 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_encode_block(const float2 *__re
         }
         if (tm.t == 0) res.record->bytes = total;
     }
-    if (call_done(res, tm, gridDim.x)) {
+    if (call_done(res, tm, gridDim.x) && g.nframes > 1) {
         *scr.ticket = 0;
         atomicExch(scr.epoch, (epoch + 1) & kEpochMask);
     }
@@ -403,12 +426,19 @@ static void decode_table(const BlockSlot *table, const uint32_t *ids, uint64_t b
     const TeamShape ts = team_shape(m);
     // with leading phase ops each CTA copies their descriptors once and takes several frames
     const unsigned grid = grid_for(items, pre.count ? 152 * 5 * 3 : kMaxGrid);
+    const size_t smem = ts.smem + pre.count * cdev::kPreTabBytes;
+    static bool attr_set = false;  // kMaxPreOps tables beside the largest tile: 52.5 KB
+    if (pre.count > 2 && !attr_set) {
+        cudaFuncSetAttribute(k_decode<kMaxPreOps, REL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(cdev::team_tile_bytes(128) + kMaxPreOps * cdev::kPreTabBytes));
+        attr_set = true;
+    }
     if (pre.count == 0)
-        k_decode<0, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
+        k_decode<0, REL><<<grid, ts.threads, smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
     else if (pre.count <= 2)
-        k_decode<2, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
+        k_decode<2, REL><<<grid, ts.threads, smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
     else
-        k_decode<kMaxPreOps, REL><<<grid, ts.threads, ts.smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
+        k_decode<kMaxPreOps, REL><<<grid, ts.threads, smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
 }
 
 void launch_decode(const BlockSlot *table, uint64_t b0, uint32_t nblocks, int m, float2 *wv, int *status,

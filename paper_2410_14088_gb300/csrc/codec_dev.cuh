@@ -87,23 +87,23 @@ __device__ __forceinline__ int32_t unzigzag(uint32_t z) {
 }
 
 // ---------------------------------------------------------------------------
-// Decode: one CTA per frame (grid-stride over all frames of all blocks).
-// ---------------------------------------------------------------------------
 // Leading phase ops of a stage, applied by the decoder. The phase index of a
 // diagonal op splits into bits fixed for the frame (working bits >= the frame
 // log, and outer qubits from the group), the lane's bits 0..4 and the chunk's
 // bits 5.. ; the host builds the lane and chunk parts as byte tables (32 + 128
 // bytes at float2 offset op.dlut of the phase area). pre_setup gives each op
-// its launch-wide table offsets (shared memory), pre_frame its per-lane
-// register for the frame, and pre_chunk applies the ops to one chunk's
-// amplitude.
+// its tables' place (in the phase area, or staged in shared memory), pre_frame
+// its per-lane register for the frame, and pre_chunk applies the ops to one
+// chunk's amplitude.
+// ---------------------------------------------------------------------------
 constexpr uint32_t kPreFlip = 0xFFFFFFFFu;  // pre_ab[o].y of a phase flip
 constexpr uint32_t kPreNone = 0xFFFFFFFFu;  // register of a flip whose amplitude is not in this lane
+constexpr uint32_t kPreTabBytes = 160u + 8u * 256u;  // an op's staged tables: index bytes, phases
 
-// ab.x: byte offset of a diagonal op's chunk table in the phase area; ab.y: float2 offset of its phase
-// table, or kPreFlip for a phase flip.
+// ab.x: byte offset of a diagonal op's lane and chunk tables from the tables' base; ab.y: of its phases, or kPreFlip for
+// a phase flip.
 __device__ __forceinline__ uint2 pre_setup(const OpDev &op) {
-    return op.type == OP_DIAG ? make_uint2(uint32_t(op.dlut) * 8u + 32u, uint32_t(op.mat)) : make_uint2(0u, kPreFlip);
+    return op.type == OP_DIAG ? make_uint2(uint32_t(op.dlut) * 8u, uint32_t(op.mat) * 8u) : make_uint2(0u, kPreFlip);
 }
 
 // Per-lane register of each op for the frame whose first working index is w0f: a diagonal op's frame
@@ -111,8 +111,8 @@ __device__ __forceinline__ uint2 pre_setup(const OpDev &op) {
 // holds it (kPreNone elsewhere).
 template <int NP>
 __device__ __forceinline__ void pre_frame(uint32_t (&cl)[NP > 0 ? NP : 1], const OpDev *ops, uint32_t nops,
-                                          uint64_t w0f, uint32_t fl, uint32_t lane, uint64_t gb,
-                                          const float2 *__restrict__ mats) {
+                                          const uint2 *pre_ab, const uint8_t *tabs, uint64_t w0f, uint32_t fl,
+                                          uint32_t lane, uint64_t gb) {
 #pragma unroll
     for (int o = 0; o < NP; ++o) {
         cl[o] = kPreNone;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void pre_frame(uint32_t (&cl)[NP > 0 ? NP : 1], const
                 const uint64_t bit = src < 64 ? (w0f >> src) & 1ull : (gb >> (src - 64)) & 1ull;
                 idx |= uint32_t(bit) << j;
             }
-            cl[o] = idx | __ldg(reinterpret_cast<const uint8_t *>(mats + op.dlut) + lane);
+            cl[o] = idx | tabs[pre_ab[o].x + lane];
         } else if (op.basis_in_stage && gb == op.basis_outer && op.basis_w >= w0f &&
                    op.basis_w - w0f < (uint64_t(1) << fl)) {
             const uint32_t off = uint32_t(op.basis_w - w0f);
@@ -137,14 +137,14 @@ __device__ __forceinline__ void pre_frame(uint32_t (&cl)[NP > 0 ? NP : 1], const
 
 template <int NP>
 __device__ __forceinline__ float2 pre_chunk(float2 v, const uint32_t (&cl)[NP > 0 ? NP : 1], const uint2 *pre_ab,
-                                            uint32_t nops, uint32_t c, const float2 *__restrict__ mats) {
+                                            uint32_t nops, uint32_t c, const uint8_t *tabs) {
 #pragma unroll
     for (int o = 0; o < NP; ++o) {
         if (uint32_t(o) >= nops) break;
         const uint2 ab = pre_ab[o];
         if (ab.y != kPreFlip) {
-            const uint32_t idx = cl[o] | __ldg(reinterpret_cast<const uint8_t *>(mats) + ab.x + c);
-            const float2 ph = __ldg(mats + ab.y + idx);
+            const uint32_t idx = cl[o] | tabs[ab.x + 32u + c];
+            const float2 ph = reinterpret_cast<const float2 *>(tabs + ab.y)[idx];
             v = make_float2(ph.x * v.x - ph.y * v.y, ph.x * v.y + ph.y * v.x);
         } else if (c == cl[o]) {
             v = make_float2(-v.x, -v.y);

@@ -106,10 +106,12 @@ constexpr int32_t kRoundBits = 0x4B400000;
 __device__ __forceinline__ bool call_done(const CallResult &res, const Team &tm, uint32_t nctas) {
     tm.sync();  // every thread's raise_status came before
     if (tm.t != 0) return false;
-    __threadfence();
-    if (atomicAdd(res.done, 1u) != nctas - 1) return false;
-    __threadfence();
-    *res.done = 0;
+    if (nctas > 1) {  // a call of one frame has nobody to wait for
+        __threadfence();
+        if (atomicAdd(res.done, 1u) != nctas - 1) return false;
+        __threadfence();
+        *res.done = 0;
+    }
     res.record->status = atomicExch(res.status, 0);
     __threadfence_system();
     return true;
@@ -242,14 +244,15 @@ __device__ __forceinline__ float2 amplitude_warp(const uint8_t *sp, uint64_t byt
 }
 
 // Frame f of one block (stream sp, `bytes` long) into dst (F amplitudes). tile: team_tile_bytes(C), 16-byte aligned.
-// hist_j (nullable): the block's code-width histogram. pre_*: leading phase ops, as decode of a stage. The team may
+// hist_j (nullable): the block's code-width histogram. pre_*: leading phase ops, their tables at byte offsets pre_ab of
+// tabs. The team may
 // reuse tile and S after its next sync().
 template <int NP, bool REL>
 __device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, uint8_t *tile, const uint8_t *sp,
                                                   uint64_t bytes, const FrameGeom &g, int m, uint32_t f,
                                                   float2 *__restrict__ dst, uint32_t *hist_j, int *status,
                                                   const OpDev *pre_ops, const uint2 *pre_ab, uint32_t npre,
-                                                  const float2 *__restrict__ mats, uint64_t wbase, uint64_t gb) {
+                                                  const uint8_t *tabs, uint64_t wbase, uint64_t gb) {
     const uint32_t t = tm.t, lane = t & 31u, warp = t >> 5, nw = tm.n >> 5, C = g.C;
     const uint32_t padw = (2u * C + 15u) & ~15u;
     const uint32_t tbp = REL ? ((((2u * C + 3u) / 4u) + 15u) & ~15u) : 0u;  // sign chunk types, padded
@@ -420,8 +423,8 @@ __device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, u
     uint32_t p0[NP > 0 ? NP : 1], p1[NP > 0 ? NP : 1];
     if (NP > 0 && npre) {
         const uint64_t w0f = wbase | (uint64_t(f) * g.F);
-        pre_frame<NP>(p0, pre_ops, npre, w0f, g.fl, 2u * (t & 15u), gb, mats);
-        pre_frame<NP>(p1, pre_ops, npre, w0f, g.fl, 2u * (t & 15u) + 1u, gb, mats);
+        pre_frame<NP>(p0, pre_ops, npre, pre_ab, tabs, w0f, g.fl, 2u * (t & 15u), gb);
+        pre_frame<NP>(p1, pre_ops, npre, pre_ab, tabs, w0f, g.fl, 2u * (t & 15u) + 1u, gb);
     }
     tm.sync();
     const uint8_t *col = tile + 16u * (t & 15u);
@@ -429,8 +432,8 @@ __device__ __forceinline__ void decode_frame_team(const Team &tm, TeamSmem &S, u
     for (uint32_t i = t; i < 16u * C; i += tm.n) {
         float4 v = *reinterpret_cast<const float4 *>(col + kRowBytes * (i >> 4));
         if (NP > 0 && npre) {
-            const float2 a = pre_chunk<NP>(make_float2(v.x, v.y), p0, pre_ab, npre, i >> 4, mats);
-            const float2 b = pre_chunk<NP>(make_float2(v.z, v.w), p1, pre_ab, npre, i >> 4, mats);
+            const float2 a = pre_chunk<NP>(make_float2(v.x, v.y), p0, pre_ab, npre, i >> 4, tabs);
+            const float2 b = pre_chunk<NP>(make_float2(v.z, v.w), p1, pre_ab, npre, i >> 4, tabs);
             v = make_float4(a.x, a.y, b.x, b.y);
         }
         if (wide_dst) {

@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
                 const BlockSlot sl = S.tab_in[ids[jj]];
                 cdev::decode_frame_team<kMaxPreOps, REL>(tm, s_team[team], tile, sl.ptr, sl.bytes, g, int(S.m), f,
                                                          wv + a0, S.hist ? S.hist + (bbase + jj) * 32 : nullptr,
-                                                         L.status, s_pre, s_pre_ab, S.npre, S.mats,
+                                                         L.status, s_pre, s_pre_ab, S.npre,
+                                                         reinterpret_cast<const uint8_t *>(S.mats),
                                                          uint64_t(jj) << S.m, gb);
             }
         } else if (type == PH_PASS) {
