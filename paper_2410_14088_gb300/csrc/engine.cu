@@ -247,7 +247,21 @@ struct DevBuf {
         p = nullptr;
         n = 0;
     }
+    T *take() {  // the caller owns it (dev_free)
+        T *r = p;
+        p = nullptr;
+        n = 0;
+        return r;
+    }
     ~DevBuf() { release(); }
+};
+
+// pinned host buffer from the library's cache
+template <class T>
+struct HostBuf {
+    T *p = nullptr;
+    int alloc(size_t count) { return host_alloc(reinterpret_cast<void **>(&p), count * sizeof(T)); }
+    ~HostBuf() { host_free(p); }
 };
 
 // ---------------------------------------------------------------------------
@@ -1017,7 +1031,8 @@ struct qsim_state {
     int e = 0;
     uint8_t *dev_arena = nullptr;
     uint8_t *host_arena = nullptr;
-    qsim::BlockSlot *table = nullptr;  // device, 2^(n-m) entries
+    qsim::BlockSlot *table = nullptr;  // device, 2^(n-m) entries, in table_mem
+    qsim::BlockSlot *table_mem = nullptr;
     std::vector<qsim::StageAccum> stage_acc;
     std::vector<qsim_kernel_stat> kstats;
     std::vector<float> train_rows;  // collect mode: rows of 41 features + target
@@ -1711,22 +1726,45 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
     return QSIM_OK;
 }
 
+// Wait for the runs' end on `main`, their stage totals and the status word read back in the same wait: pinned copies, one
+// synchronisation. accs[c] points into `host`.
+static int collect_run(const std::vector<RunCtx *> &rs, int *status, cudaStream_t main, HostBuf<StageAccum> &host,
+                       std::vector<const StageAccum *> &accs, const char *what) {
+    size_t n = 1;  // the status word
+    for (const RunCtx *R : rs) n += R->nst + 1;
+    int rc = host.alloc(n);
+    if (rc) return rc;
+    size_t at = 1;
+    for (const RunCtx *R : rs) {
+        accs.push_back(host.p + at);
+        CUDA_TRY(cudaMemcpyAsync(host.p + at, R->accs.p, (R->nst + 1) * sizeof(StageAccum), cudaMemcpyDeviceToHost, main));
+        at += R->nst + 1;
+    }
+    CUDA_TRY(cudaMemcpyAsync(host.p, status, sizeof(int), cudaMemcpyDeviceToHost, main));
+    CUDA_TRY(cudaStreamSynchronize(main));
+    int code;
+    memcpy(&code, host.p, sizeof(int));
+    if (!code) return QSIM_OK;
+    CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), main));
+    CUDA_TRY(cudaStreamSynchronize(main));
+    return set_error(code, "%s: %s", what, status_text(code));
+}
+
 // The run's state handle and statistics (after the stream has been synchronised).
-static int finish_run(RunCtx &R, int dev, double ms, Profiler *prof, qsim_stats *stats, qsim_state **out) {
+static int finish_run(RunCtx &R, int dev, double ms, const StageAccum *accs, Profiler *prof, qsim_stats *stats,
+                      qsim_state **out) {
     const qsim_plan *p = R.p;
     PlanDev *pd = R.pd;
     const size_t nst = R.nst;
     const bool raw = R.raw, predict = R.predict;
     const uint64_t nblocks = R.nblocks;
-    int rc;
     qsim_state *S = new qsim_state();
     S->device = dev;
     S->n = R.n;
     S->m = R.m;
     S->codec = p->cfg.codec;
     S->e = R.e;
-    S->stage_acc.resize(nst + 1);
-    CUDA_TRY(cudaMemcpy(S->stage_acc.data(), R.accs.p, (nst + 1) * sizeof(StageAccum), cudaMemcpyDeviceToHost));
+    S->stage_acc.assign(accs, accs + nst + 1);
     if (R.collect && R.log_next) {
         S->train_rows.resize(R.log_next * (kMlpIn + 1));
         CUDA_TRY(cudaMemcpy(S->train_rows.data(), R.log_rows.p, S->train_rows.size() * sizeof(float),
@@ -1738,11 +1776,8 @@ static int finish_run(RunCtx &R, int dev, double ms, Profiler *prof, qsim_stats 
     R.dev_arena[fin] = nullptr;
     R.host_arena[fin] = nullptr;
     R.free_arenas();
-    if ((rc = dev_alloc(reinterpret_cast<void **>(&S->table), nblocks * sizeof(BlockSlot)))) {
-        qsim_state_free(S);
-        return rc;
-    }
-    CUDA_TRY(cudaMemcpy(S->table, R.tables.p + fin * nblocks, nblocks * sizeof(BlockSlot), cudaMemcpyDeviceToDevice));
+    S->table_mem = R.tables.take();
+    S->table = S->table_mem + fin * nblocks;
 
     if (prof && prof->on) {
         double secs[P_NCAT];
@@ -1845,8 +1880,21 @@ struct StreamsRun {
     }
 };
 
-// Validation, the compressed store's tiers, the per-stream buffers and the initial store (Sec. 4.2); the start
-// event is recorded on `main` before the initial store.
+// The run's work is ordered on its first stream, sw[0].s: it starts after what `main` holds (streams_fork), and main
+// waits for it (streams_join) where the caller takes over. A stage whose groups make one batch needs no event at all.
+static int streams_fork(StreamsRun &S) {
+    CUDA_TRY(cudaEventRecord(S.ev_fork, S.main));
+    CUDA_TRY(cudaStreamWaitEvent(S.sw[0].s, S.ev_fork, 0));
+    return QSIM_OK;
+}
+static int streams_join(StreamsRun &S) {
+    CUDA_TRY(cudaEventRecord(S.sw[0].done, S.sw[0].s));
+    CUDA_TRY(cudaStreamWaitEvent(S.main, S.sw[0].done, 0));
+    return QSIM_OK;
+}
+
+// Validation, the compressed store's tiers, the per-stream buffers and the initial store (Sec. 4.2), which is left on
+// sw[0].s; the start event is recorded on `main` before it.
 static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
     const qsim_config &cfg = p->cfg;
     CUDA_TRY(cudaGetDevice(&S.dev));
@@ -1882,16 +1930,16 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
 
     // ---- per-stream work buffers ----
     std::vector<StreamWork> &sw = S.sw;
-    sw.resize(nstreams);
-    uint64_t max_batch_blocks = 0;
+    uint64_t max_batch_blocks = 0, most_batches = 1;
     for (const StageDev &sd : pd->stages) {
         uint64_t gpb = std::min<uint64_t>(std::max<uint64_t>(1, batch_amps >> sd.W), 32768);
         gpb = std::min<uint64_t>(gpb, sd.ngroups);
         max_batch_blocks = std::max<uint64_t>(max_batch_blocks, gpb * sd.G);
+        most_batches = std::max<uint64_t>(most_batches, (sd.ngroups + gpb - 1) / gpb);
     }
+    sw.resize(std::min<uint64_t>(nstreams, most_batches));  // no more streams than a stage has batches for
     max_batch_blocks = std::max<uint64_t>(max_batch_blocks, 2);
-    for (uint32_t i = 0; i < nstreams; ++i) {
-        StreamWork &w = sw[i];
+    for (StreamWork &w : sw) {
         CUDA_TRY(cudaStreamCreateWithFlags(&w.s, cudaStreamNonBlocking));
         CUDA_TRY(cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming));
         if (!persistent && (rc = w.alloc_codec(max_batch_blocks, m, nframes, RC.rel, main))) return rc;
@@ -1904,19 +1952,12 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
     CUDA_TRY(cudaEventRecord(S.ev_start, main));
 
     // ---- initial store ----
-    {
-        StreamWork &w = sw[0];
-        CUDA_TRY(cudaEventRecord(S.ev_fork, main));
-        CUDA_TRY(cudaStreamWaitEvent(w.s, S.ev_fork, 0));
-        if ((rc = init_store(RC, &w, S.status, w.s))) return rc;
-        CUDA_TRY(cudaEventRecord(w.done, w.s));
-        CUDA_TRY(cudaStreamWaitEvent(main, w.done, 0));
-    }
-    return QSIM_OK;
+    if ((rc = streams_fork(S))) return rc;
+    return init_store(RC, &sw[0], S.status, sw[0].s);
 }
 
 // Stage si over `ngroups` SV groups: ids_stage holds their block ids (group-major, G per group), gb_stage their
-// outer bits (device arrays). Work runs on the run's streams, joined back to S.main.
+// outer bits (device arrays). Work runs on the run's streams, joined back to sw[0].s.
 static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, const uint64_t *gb_stage,
                          uint64_t ngroups) {
     RunCtx &RC = S.RC;
@@ -1946,12 +1987,13 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
         const int in_par = si & 1, out_par = (si + 1) & 1;
         BlockSlot *tab_in = tables_p + in_par * nblocks;
         BlockSlot *tab_out = tables_p + out_par * nblocks;
-        CUDA_TRY(cudaMemsetAsync(bumps_p + 2 * out_par, 0, 2 * sizeof(uint64_t), main));
-        CUDA_TRY(cudaEventRecord(ev_fork, main));
-        for (auto &w : sw) CUDA_TRY(cudaStreamWaitEvent(w.s, ev_fork, 0));
+        CUDA_TRY(cudaMemsetAsync(bumps_p + 2 * out_par, 0, 2 * sizeof(uint64_t), sw[0].s));
         const uint64_t gpb = std::min<uint64_t>(std::min<uint64_t>(std::max<uint64_t>(1, batch_amps >> sd.W), 32768),
                                                 std::max<uint64_t>(1, ngroups));
         const uint64_t nbatches = (ngroups + gpb - 1) / gpb;
+        const uint32_t used = uint32_t(std::min<uint64_t>(nbatches, sw.size()));  // streams of this stage
+        if (used > 1) CUDA_TRY(cudaEventRecord(ev_fork, sw[0].s));
+        for (uint32_t i = 1; i < used; ++i) CUDA_TRY(cudaStreamWaitEvent(sw[i].s, ev_fork, 0));
         S.groups_run += ngroups;
         StageAccum *acc = accs_p + si;
         StageFeatures sf{};
@@ -2044,23 +2086,24 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
                 }
             }
         }
-        for (auto &w : sw) {
-            CUDA_TRY(cudaEventRecord(w.done, w.s));
-            CUDA_TRY(cudaStreamWaitEvent(main, w.done, 0));
+        for (uint32_t i = 1; i < used; ++i) {
+            CUDA_TRY(cudaEventRecord(sw[i].done, sw[i].s));
+            CUDA_TRY(cudaStreamWaitEvent(sw[0].s, sw[i].done, 0));
         }
-        }
+    }
     return QSIM_OK;
 }
 
-// The run's end: stop event, status, and the state handle with the statistics.
+// The run's end (its work joined to main): stop event, status, and the state handle with the statistics.
 static int streams_finish(StreamsRun &S, qsim_state **out, qsim_stats *stats) {
     CUDA_TRY(cudaEventRecord(S.ev_stop, S.main));
-    CUDA_TRY(cudaEventSynchronize(S.ev_stop));
+    HostBuf<StageAccum> host;
+    std::vector<const StageAccum *> accs;
+    int rc = collect_run({&S.RC}, S.status, S.main, host, accs, "qsim_run");
+    if (rc) return rc;
     float ms = 0;
     CUDA_TRY(cudaEventElapsedTime(&ms, S.ev_start, S.ev_stop));
-    int st_code = read_status(S.status, S.main);
-    if (st_code) return set_error(st_code, "qsim_run: %s", status_text(st_code));
-    return finish_run(S.RC, S.dev, ms, &S.prof, stats, out);
+    return finish_run(S.RC, S.dev, ms, accs[0], &S.prof, stats, out);
 }
 
 static int run_plan(const qsim_plan *p, cudaStream_t main, qsim_state **out, qsim_stats *stats) {
@@ -2071,13 +2114,14 @@ static int run_plan(const qsim_plan *p, cudaStream_t main, qsim_state **out, qsi
     PlanDev *pd = S.RC.pd;
     if (S.RC.persistent) {
         std::vector<RunCtx *> one{&S.RC};
-        if ((rc = run_persistent(one, false, main, S.status, S.prof, *S.dctx, 1ull << 25))) return rc;
+        if ((rc = streams_join(S)) || (rc = run_persistent(one, false, main, S.status, S.prof, *S.dctx, 1ull << 25))) return rc;
     } else {
         for (size_t si = 0; si < S.RC.nst; ++si) {
             const StageDev &sd = pd->stages[si];
             if ((rc = streams_stage(S, si, pd->ids.p + pd->ids_off[si], pd->gbase.p + pd->gbase_off[si], sd.ngroups)))
                 return rc;
         }
+        if ((rc = streams_join(S))) return rc;
     }
     return streams_finish(S, out, stats);
 }
@@ -2144,16 +2188,17 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     if (rc) return rc;
     if ((rc = run_persistent(rp, true, main, status, prof, dctx, slot_budget))) return rc;
     CUDA_TRY(cudaEventRecord(ev_stop, main));
-    CUDA_TRY(cudaEventSynchronize(ev_stop));
+    HostBuf<StageAccum> host;
+    std::vector<const StageAccum *> accs;
+    rc = collect_run(rp, status, main, host, accs, "qsim_run_batch");
     float ms = 0;
-    CUDA_TRY(cudaEventElapsedTime(&ms, ev_start, ev_stop));
+    if (!rc) CUDA_TRY(cudaEventElapsedTime(&ms, ev_start, ev_stop));
     cudaEventDestroy(ev_start);
     cudaEventDestroy(ev_stop);
-    int st_code = read_status(status, main);
-    if (st_code) return set_error(st_code, "qsim_run_batch: %s", status_text(st_code));
+    if (rc) return rc;
     double alg_bytes = 0, alg_flops = 0;
     for (size_t c = 0; c < count; ++c) {
-        if ((rc = finish_run(*rs[c], dev, ms, nullptr, stats ? stats + c : nullptr, out + c))) {
+        if ((rc = finish_run(*rs[c], dev, ms, accs[c], nullptr, stats ? stats + c : nullptr, out + c))) {
             for (size_t d = 0; d < c; ++d) {
                 qsim_state_free(out[d]);
                 out[d] = nullptr;
@@ -2464,7 +2509,7 @@ int qsim_shard_begin(const qsim_plan *plan, const uint32_t *rank_qubits, uint32_
         R->rank = rank;
         R->rq.assign(rank_qubits, rank_qubits + nst * log2_ranks);
         int rc = streams_begin(R->S, plan, static_cast<cudaStream_t>(cuda_stream));
-        if (rc) return rc;
+        if (rc || (rc = streams_join(R->S))) return rc;
         const uint64_t nblocks = R->S.RC.nblocks;
         R->held.assign(nblocks, 0);
         if (nst)
@@ -2514,7 +2559,9 @@ int qsim_shard_stage(qsim_shard_run *R, size_t stage) {
         if (bool(R->held[b]) != (shard_owner(R, stage, b) == R->rank))
             return set_error(QSIM_E_INVALID, "stage %zu: block %llu is %s this rank, the rank qubits say otherwise",
                              stage, (unsigned long long)b, R->held[b] ? "on" : "not on");
-    int rc = streams_stage(R->S, stage, R->ids.p + R->ids_off[stage], R->gb.p + R->gb_off[stage], R->ngroups[stage]);
+    int rc = streams_fork(R->S);
+    if (!rc) rc = streams_stage(R->S, stage, R->ids.p + R->ids_off[stage], R->gb.p + R->gb_off[stage], R->ngroups[stage]);
+    if (!rc) rc = streams_join(R->S);
     if (rc) {
         R->failed = true;
         return rc;
@@ -2810,7 +2857,7 @@ void qsim_state_free(qsim_state *st) {
     if (!st) return;
     dev_free(st->dev_arena);
     host_free(st->host_arena);
-    dev_free(st->table);
+    dev_free(st->table_mem);
     delete st;
 }
 
