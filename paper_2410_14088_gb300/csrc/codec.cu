@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_decode(const BlockSlot *__restr
     __shared__ uint2 s_pre_ab[NP > 0 ? NP : 1];
     __shared__ TeamSmem S;
     const Team tm{threadIdx.x, blockDim.x, 1};
+    if (pre.reset && blockIdx.x == 0 && threadIdx.x < 2) pre.reset[threadIdx.x] = 0;
     // the leading ops' descriptors and tables, staged once per CTA beside its tile
     uint8_t *tabs = tile + team_tile_bytes(g.C);
     if (NP > 0) {

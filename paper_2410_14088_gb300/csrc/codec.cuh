@@ -116,6 +116,7 @@ struct PreOps {
     uint32_t G = 1;                   // blocks per group
     const float2 *mats = nullptr;
     const uint64_t *gbase = nullptr;  // per group of the batch
+    uint64_t *reset = nullptr;        // two words set to zero by the launch (null: none)
 };
 // decode with the block references read from table[ids[j]]
 void launch_decode_table(const BlockSlot *table, const uint32_t *ids, uint32_t nblocks, int m, float2 *wv,

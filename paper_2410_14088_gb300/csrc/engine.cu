@@ -1972,7 +1972,6 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
     const uint32_t nstreams = uint32_t(S.sw.size());
     std::vector<StreamWork> &sw = S.sw;
     const uint64_t batch_amps = S.batch_amps;
-    cudaStream_t main = S.main;
     cudaEvent_t ev_fork = S.ev_fork;
     Profiler &prof = S.prof;
     int *status = S.status;
@@ -1987,11 +1986,13 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
         const int in_par = si & 1, out_par = (si + 1) & 1;
         BlockSlot *tab_in = tables_p + in_par * nblocks;
         BlockSlot *tab_out = tables_p + out_par * nblocks;
-        CUDA_TRY(cudaMemsetAsync(bumps_p + 2 * out_par, 0, 2 * sizeof(uint64_t), sw[0].s));
         const uint64_t gpb = std::min<uint64_t>(std::min<uint64_t>(std::max<uint64_t>(1, batch_amps >> sd.W), 32768),
                                                 std::max<uint64_t>(1, ngroups));
         const uint64_t nbatches = (ngroups + gpb - 1) / gpb;
         const uint32_t used = uint32_t(std::min<uint64_t>(nbatches, sw.size()));  // streams of this stage
+        // the output arena starts empty: reset by the decoder of a stage's only batch, else ahead of all of them
+        const bool reset_in_decode = nbatches == 1 && !raw;
+        if (!reset_in_decode) CUDA_TRY(cudaMemsetAsync(bumps_p + 2 * out_par, 0, 2 * sizeof(uint64_t), sw[0].s));
         if (used > 1) CUDA_TRY(cudaEventRecord(ev_fork, sw[0].s));
         for (uint32_t i = 1; i < used; ++i) CUDA_TRY(cudaStreamWaitEvent(sw[i].s, ev_fork, 0));
         S.groups_run += ngroups;
@@ -2035,6 +2036,7 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
                 pre.G = sd.G;
                 pre.mats = pd->mats.p;
                 pre.gbase = gb_stage + g0;
+                pre.reset = reset_in_decode ? bumps_p + 2 * out_par : nullptr;
                 uint32_t *hist = (predict || collect) ? w.hist.p : nullptr;
                 if (hist) CUDA_TRY(cudaMemsetAsync(hist, 0, size_t(nb) * 32 * sizeof(uint32_t), w.s));
                 launch_decode_table(tab_in, ids, nb, m, w.wv.p, hist, status, pre, w.s, RC.rel);
