@@ -4,8 +4,8 @@
 // The paper handles the unpredictable size of compressed blocks with a second
 // memory level (Sec. 4.4). Here the size of each block's next stream is
 // predicted from cheap statistics so that a slot can be reserved before the
-// block is encoded, without a sizing pass; an under-estimate falls back to an
-// exact re-encode.
+// block is encoded; a block whose size was under-estimated gets a slot of its
+// exact size.
 //
 // Inputs (x, 41 floats): the 32-bin histogram of code bit lengths
 // (bit length of |q|, as fractions of the 2^(m+1) values of each block of the
@@ -117,32 +117,47 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
 // through distributed shared memory (each CTA sums an eighth of the parameters over the eight partials, in rank
 // order, so the result is deterministic), and the same CTA applies Adam to that eighth, whose moments it keeps in
 // registers, and writes the new weights into all eight copies. Two cluster barriers per step, no launch and no global
-// round trip. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases: latency bounds it, so the split is
-// the smallest that leaves every phase two outputs per thread (8 samples x 64 units on 256 threads). W2's rows are
-// padded to 65 words: both directions through it read conflict-free.
+// round trip. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases: latency and shared-memory reads
+// bound it, so the split is the smallest that leaves every phase two outputs per thread (8 samples x 64 units on 256
+// threads) and every product is tiled in registers over 128-bit reads.
 // ---------------------------------------------------------------------------
 constexpr int CR = 8;                            // CTAs of the cluster
 constexpr int SB = 8;                            // samples a CTA takes at a time (one warp each in the output layer)
 constexpr int TT = 256;                          // threads
 constexpr int SHARD = 868;                       // parameters per CTA (8 x 868 >= NP), four per thread at most
-constexpr int W2S = HID + 1;
+constexpr int XS = (IN + 15) / 16 * 16;          // words of an input row and of a row of W1, zeros past IN
+constexpr int W2S = HID + 16;                    // words of a row of W2
+static_assert(XS % 32 == 16 && W2S % 32 == 16, "two rows read together must fall on different halves of the banks");
 
-struct __align__(16) TrainSmem {
-    float w1[HID * IN], b1[HID], w2[HID * W2S], b2[HID], w3[HID], b3[4];
-    float g[CR * SHARD];                         // partial gradient, flat parameter order
+struct __align__(16) TrainParams {
+    float w1[HID * XS], b1[HID], w2[HID * W2S], b2[HID], w3[HID], b3[4];
+};
+struct __align__(16) TrainSmem : TrainParams {
+    TrainParams g;                               // partial gradient
+    float x[SB][XS];
     float h1[SB][HID], h2[SB][HID], d1[SB][HID], d2[SB][HID];
-    float x[SB * IN], t[SB], dy[SB], sq[SB];
+    float t[SB], dy[SB], sq[SB];
     float loss;
 };
 
-// parameter i's place in the weights' shared copy
-__device__ __forceinline__ float *train_weight(TrainSmem &S, int i) {
-    if (i < OB1) return S.w1 + i;
-    if (i < OW2) return S.b1 + (i - OB1);
-    if (i < OB2) return S.w2 + ((i - OW2) / HID) * W2S + (i - OW2) % HID;
-    if (i < OW3) return S.b2 + (i - OB2);
-    if (i < OB3) return S.w3 + (i - OW3);
-    return S.b3;
+// parameter i's place in a TrainParams, in floats
+__device__ __forceinline__ int train_place(int i) {
+    constexpr int P1 = HID * XS, P2 = P1 + HID, P3 = P2 + HID * W2S;
+    if (i < OB1) return i / IN * XS + i % IN;
+    if (i < OW2) return P1 + (i - OB1);
+    if (i < OB2) return P2 + (i - OW2) / HID * W2S + (i - OW2) % HID;
+    return P3 + (i - OB2);  // b2, W3 and b3 follow one another
+}
+
+__device__ __forceinline__ float *train_flat(TrainParams &p) { return reinterpret_cast<float *>(&p); }
+
+// The weights into S, zeros into the rows' ends.
+__device__ __forceinline__ void train_load(TrainSmem &S, const float *params) {
+    float *w = train_flat(S);
+    for (int i = threadIdx.x; i < HID * XS; i += TT) w[i] = 0.f;
+    for (int i = threadIdx.x; i < SB * XS; i += TT) S.x[0][i] = 0.f;
+    __syncthreads();
+    for (int i = threadIdx.x; i < NP; i += TT) w[train_place(i)] = params[i];
 }
 
 // The rows of the samples a CTA takes at once, two values per thread (IN features and the target per sample), held in
@@ -168,34 +183,121 @@ __device__ __forceinline__ void train_put(TrainSmem &S, const TrainRows &r) {
     for (int k = 0; k < 2; ++k) {
         const uint32_t i = threadIdx.x + TT * k, b = i / (IN + 1), j = i % (IN + 1);
         if (b >= uint32_t(SB)) continue;
-        if (j < uint32_t(IN)) S.x[b * IN + j] = r.v[k];
+        if (j < uint32_t(IN)) S.x[b][j] = r.v[k];
         else S.t[b] = r.v[k];
+    }
+}
+
+// The sums over K terms of v[b][k] * w[u * S + k] for the 8 samples and 64 units, put(b, u, sum) for each. The phase is
+// bound by shared-memory reads: a thread takes two units of four samples over a quarter of the terms in 128-bit reads,
+// K / 16 * 6 of them for 2 K products (one unit of two samples at a time took 3 K reads for the same 2 K). The
+// quarters are neighbouring lanes, whose reads of two rows of w fill the 32 banks (S = 16 mod 32).
+template <int K, int S, class F>
+__device__ __forceinline__ void train_rows(const float *w, const float *v, int vs, F put) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3;
+    const int u0 = (lane >> 2) + 8 * (warp & 3), b0 = 4 * (warp >> 2);
+    float acc[2][4] = {};
+#pragma unroll
+    for (int t = 0; t < K / 16; ++t) {
+        const int k = 16 * t + 4 * q;
+        const float4 wa = *reinterpret_cast<const float4 *>(w + u0 * S + k);
+        const float4 wb = *reinterpret_cast<const float4 *>(w + (u0 + HID / 2) * S + k);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const float4 x = *reinterpret_cast<const float4 *>(v + (b0 + b) * vs + k);
+            acc[0][b] = fmaf(wa.w, x.w, fmaf(wa.z, x.z, fmaf(wa.y, x.y, fmaf(wa.x, x.x, acc[0][b]))));
+            acc[1][b] = fmaf(wb.w, x.w, fmaf(wb.z, x.z, fmaf(wb.y, x.y, fmaf(wb.x, x.x, acc[1][b]))));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {  // lane q of the four ends with sample b0 + q
+        float r[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float keep = q & 2 ? acc[i][2 + j] : acc[i][j], give = q & 2 ? acc[i][j] : acc[i][2 + j];
+            r[j] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+        }
+        const float keep = q & 1 ? r[1] : r[0], give = q & 1 ? r[0] : r[1];
+        put(b0 + q, u0 + HID / 2 * i, keep + __shfl_xor_sync(0xffffffffu, give, 1));
+    }
+}
+
+// The sums over i of d2[b][i] * W2[i][j], put(b, j, sums of j and j + 1). As above with the threads along W2's rows: four
+// units of two samples over a quarter of the terms.
+template <class F>
+__device__ __forceinline__ void train_cols(const TrainSmem &S, F put) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 3;
+    const int j0 = 4 * ((lane & 7) + 8 * (warp & 1)), b0 = 2 * (warp >> 1);
+    float acc[2][4] = {};
+#pragma unroll
+    for (int t = 0; t < HID / 16; ++t) {
+        const int k = HID / 4 * q + 4 * t;
+        float x[2][4];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const float4 d = *reinterpret_cast<const float4 *>(&S.d2[b0 + b][k]);
+            x[b][0] = d.x;
+            x[b][1] = d.y;
+            x[b][2] = d.z;
+            x[b][3] = d.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 w = *reinterpret_cast<const float4 *>(S.w2 + (k + i) * W2S + j0);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                acc[b][0] = fmaf(w.x, x[b][i], acc[b][0]);
+                acc[b][1] = fmaf(w.y, x[b][i], acc[b][1]);
+                acc[b][2] = fmaf(w.z, x[b][i], acc[b][2]);
+                acc[b][3] = fmaf(w.w, x[b][i], acc[b][3]);
+            }
+        }
+    }
+    float r[4], s[2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {  // quarters 2 and 3 end with sample b0 + 1
+        const float keep = q & 2 ? acc[1][j] : acc[0][j], give = q & 2 ? acc[0][j] : acc[1][j];
+        r[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {  // odd quarters with units j0 + 2 and j0 + 3
+        const float keep = q & 1 ? r[2 + j] : r[j], give = q & 1 ? r[j] : r[2 + j];
+        s[j] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+    put(b0 + (q >> 1), j0 + 2 * (q & 1), s[0], s[1]);
+}
+
+// What a thread writes of the partial gradient: four neighbours, first ? v : what is there + v.
+__device__ __forceinline__ void train_put4(float *at, bool first, const float *v) {
+    float4 o = make_float4(v[0], v[1], v[2], v[3]);
+    if (!first) {
+        const float4 w = *reinterpret_cast<float4 *>(at);
+        o = make_float4(o.x + w.x, o.y + w.y, o.z + w.z, o.w + w.w);
+    }
+    *reinterpret_cast<float4 *>(at) = o;
+}
+
+// The outer products of a and x, four by four (rows r0 .., columns c0 ..), summed over the samples.
+__device__ __forceinline__ void train_outer(const float *a, const float *x, int xs, int r0, int c0, float (&acc)[4][4]) {
+#pragma unroll
+    for (int b = 0; b < SB; ++b) {
+        const float4 d = *reinterpret_cast<const float4 *>(a + b * HID + r0);
+        const float4 e = *reinterpret_cast<const float4 *>(x + b * xs + c0);
+        const float dd[4] = {d.x, d.y, d.z, d.w}, xx[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], xx[j], acc[i][j]);
     }
 }
 
 // Forward pass of the n (<= SB) samples in S.x; each sample's residual y - t to S.dy (0 past n). Ends unsynchronised:
 // warp b wrote sample b's.
 __device__ __forceinline__ void train_forward(TrainSmem &S, uint32_t n) {
-    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID, lane = tid & 31, warp = tid >> 5;
-    float a0 = S.b1[h], a1 = a0;
-#pragma unroll
-    for (int j = 0; j < IN; ++j) {
-        const float w = S.w1[h * IN + j];
-        a0 = fmaf(w, S.x[q * IN + j], a0);
-        a1 = fmaf(w, S.x[(q + 4) * IN + j], a1);
-    }
-    S.h1[q][h] = fmaxf(a0, 0.f);
-    S.h1[q + 4][h] = fmaxf(a1, 0.f);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    train_rows<XS, XS>(S.w1, S.x[0], XS, [&](int b, int u, float v) { S.h1[b][u] = fmaxf(v + S.b1[u], 0.f); });
     __syncthreads();
-    a0 = a1 = S.b2[h];
-#pragma unroll 16
-    for (int j = 0; j < HID; ++j) {
-        const float w = S.w2[h * W2S + j];
-        a0 = fmaf(w, S.h1[q][j], a0);
-        a1 = fmaf(w, S.h1[q + 4][j], a1);
-    }
-    S.h2[q][h] = fmaxf(a0, 0.f);
-    S.h2[q + 4][h] = fmaxf(a1, 0.f);
+    train_rows<HID, W2S>(S.w2, S.h1[0], HID, [&](int b, int u, float v) { S.h2[b][u] = fmaxf(v + S.b2[u], 0.f); });
     __syncthreads();
     float y = S.w3[lane] * S.h2[warp][lane] + S.w3[lane + 32] * S.h2[warp][lane + 32];
 #pragma unroll
@@ -219,34 +321,17 @@ __device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_
         S.d2[warp][lane + 32] = S.h2[warp][lane + 32] > 0.f ? dy * S.w3[lane + 32] : 0.f;
     }
     __syncthreads();
-    // back through W2
-    float a0 = 0.f, a1 = 0.f;
-#pragma unroll 16
-    for (int i = 0; i < HID; ++i) {
-        const float w = S.w2[i * W2S + h];
-        a0 = fmaf(S.d2[q][i], w, a0);
-        a1 = fmaf(S.d2[q + 4][i], w, a1);
-    }
-    S.d1[q][h] = S.h1[q][h] > 0.f ? a0 : 0.f;
-    S.d1[q + 4][h] = S.h1[q + 4][h] > 0.f ? a1 : 0.f;
-    auto put = [&](int i, float v) { S.g[i] = first ? v : S.g[i] + v; };
+    train_cols(S, [&](int b, int j, float v0, float v1) {  // back through W2
+        const float2 a = *reinterpret_cast<const float2 *>(&S.h1[b][j]);
+        *reinterpret_cast<float2 *>(&S.d1[b][j]) = make_float2(a.x > 0.f ? v0 : 0.f, a.y > 0.f ? v1 : 0.f);
+    });
+    auto put = [&](float *at, float v) { *at = first ? v : *at + v; };
     {  // W2: a 4 x 4 tile per thread
         const int r0 = (tid >> 4) * 4, c0 = (tid & 15) * 4;
         float acc[4][4] = {};
+        train_outer(S.d2[0], S.h1[0], HID, r0, c0, acc);
 #pragma unroll
-        for (int b = 0; b < SB; ++b) {
-            const float4 d = *reinterpret_cast<const float4 *>(&S.d2[b][r0]);
-            const float4 x = *reinterpret_cast<const float4 *>(&S.h1[b][c0]);
-            const float dd[4] = {d.x, d.y, d.z, d.w}, xx[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], xx[j], acc[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) put(OW2 + (r0 + i) * HID + c0 + j, acc[i][j]);
+        for (int i = 0; i < 4; ++i) train_put4(S.g.w2 + (r0 + i) * W2S + c0, first, acc[i]);
     }
     if (q == 0) {  // W3, b2 and b3
         float gw = 0.f, gb = 0.f;
@@ -255,8 +340,8 @@ __device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_
             gw = fmaf(S.dy[b], S.h2[b][h], gw);
             gb += S.d2[b][h];
         }
-        put(OW3 + h, gw);
-        put(OB2 + h, gb);
+        put(S.g.w3 + h, gw);
+        put(S.g.b2 + h, gb);
         if (h == 0) {
             float g3 = 0.f, ls = 0.f;
 #pragma unroll
@@ -264,30 +349,27 @@ __device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_
                 g3 += S.dy[b];
                 ls += S.sq[b];
             }
-            put(OB3, g3);
+            put(S.g.b3, g3);
             S.loss = first ? ls : S.loss + ls;
         }
     }
     __syncthreads();
-    {  // W1 and b1: four threads per unit
-        const int u = tid >> 2, j0 = tid & 3;
-        float d[SB];
+    constexpr int T1 = XS / 4;  // tiles along a row of W1
+    if (tid < 16 * T1) {        // W1
+        const int r0 = tid / T1 * 4, c0 = tid % T1 * 4;
+        float acc[4][4] = {};
+        train_outer(S.d1[0], S.x[0], XS, r0, c0, acc);
 #pragma unroll
-        for (int b = 0; b < SB; ++b) d[b] = S.d1[b][u];
-        for (int j = j0; j < IN; j += 4) {
-            float v = 0.f;
+        for (int i = 0; i < 4; ++i) train_put4(S.g.w1 + (r0 + i) * XS + c0, first, acc[i]);
+    } else if (tid - 16 * T1 < HID) {  // b1
+        const int u = tid - 16 * T1;
+        float v = 0.f;
 #pragma unroll
-            for (int b = 0; b < SB; ++b) v = fmaf(d[b], S.x[b * IN + j], v);
-            put(OW1 + u * IN + j, v);
-        }
-        if (j0 == 0) {
-            float v = 0.f;
-#pragma unroll
-            for (int b = 0; b < SB; ++b) v += d[b];
-            put(OB1 + u, v);
-        }
+        for (int b = 0; b < SB; ++b) v += S.d1[b][u];
+        put(S.g.b1 + u, v);
     }
 }
+static_assert(16 * (XS / 4) + HID <= TT, "W1's tiles and b1 share the threads");
 
 // Samples [r0, r0 + per) of a batch of nb belong to rank r.
 __device__ __forceinline__ void train_share(uint32_t nb, uint32_t rank, uint32_t &r0, uint32_t &per) {
@@ -310,14 +392,15 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
     cg::cluster_group cl = cg::this_cluster();
     const uint32_t rank = cl.block_rank();
     const int tid = threadIdx.x;
-    for (int i = tid; i < NP; i += TT) *train_weight(S, i) = params[i];
+    train_load(S, params);
     // the thread's parameters: SHARD * rank + tid + 256 k
     float p[4] = {}, ma[4] = {}, mb[4] = {};
-    int own[4];
+    int own[4], place[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int o = tid + TT * k, i = SHARD * int(rank) + o;
         own[k] = o < SHARD && i < NP ? i : -1;
+        place[k] = train_place(max(own[k], 0));
         if (own[k] >= 0) {
             p[k] = params[own[k]];
             if (TRAIN) {
@@ -355,24 +438,28 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
             train_chunk(S, n, inv_b, c == 0);
             __syncthreads();
         }
-        cl.sync();  // every rank's partial gradient is complete
         ++step;
         const float c1 = TRAIN ? 1.f - powf(beta1, float(step)) : 1.f, c2 = TRAIN ? 1.f - powf(beta2, float(step)) : 1.f;
+        cl.sync();  // every rank's partial gradient is complete
+        float part[4][CR];  // every remote read in flight before the first sum
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int r = 0; r < CR; ++r) part[k][r] = cl.map_shared_rank(train_flat(S.g), r)[place[k]];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             if (own[k] < 0) continue;
             float g = 0.f;
 #pragma unroll
-            for (int r = 0; r < CR; ++r) g += cl.map_shared_rank(S.g, r)[own[k]];
+            for (int r = 0; r < CR; ++r) g += part[k][r];
             if (TRAIN) {
                 const float a = beta1 * ma[k] + (1.f - beta1) * g;
                 const float b = beta2 * mb[k] + (1.f - beta2) * g * g;
                 ma[k] = a;
                 mb[k] = b;
                 p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
-                float *w = train_weight(S, own[k]);
 #pragma unroll
-                for (int r = 0; r < CR; ++r) *cl.map_shared_rank(w, r) = p[k];
+                for (int r = 0; r < CR; ++r) cl.map_shared_rank(train_flat(S), r)[place[k]] = p[k];
             } else {
                 grad[own[k]] = g;
             }
@@ -403,7 +490,7 @@ __global__ void __launch_bounds__(TT) k_mlp_loss(const float *__restrict__ param
                                                  uint64_t count, double *loss) {
     extern __shared__ __align__(16) uint8_t train_smem[];
     TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
-    for (int i = threadIdx.x; i < NP; i += TT) *train_weight(S, i) = params[i];
+    train_load(S, params);
     double sum = 0;
     for (uint64_t c = uint64_t(blockIdx.x) * SB; c < count; c += uint64_t(gridDim.x) * SB) {
         const uint32_t n = uint32_t(min(count - c, uint64_t(SB)));
