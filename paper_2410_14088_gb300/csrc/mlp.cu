@@ -124,7 +124,10 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
 constexpr int CR = 8;                            // CTAs of the cluster
 constexpr int SB = 8;                            // samples a CTA takes at a time (one warp each in the output layer)
 constexpr int TT = 256;                          // threads
-constexpr int SHARD = 868;                       // parameters per CTA (8 x 868 >= NP), four per thread at most
+constexpr int IN4 = (IN + 3) / 4;                // float4s of a row of W1
+constexpr int NV = HID * IN4 + HID / 4 + HID * HID / 4 + (2 * HID + 4) / 4;  // float4s of the parameters in shared memory
+constexpr int SHARD = (NV + CR - 1) / CR;        // of them a CTA's, one per thread
+static_assert(SHARD <= TT, "a thread owns at most one");
 constexpr int XS = (IN + 15) / 16 * 16;          // words of an input row and of a row of W1, zeros past IN
 constexpr int W2S = HID + 16;                    // words of a row of W2
 static_assert(XS % 32 == 16 && W2S % 32 == 16, "two rows read together must fall on different halves of the banks");
@@ -149,6 +152,23 @@ __device__ __forceinline__ int train_place(int i) {
     return P3 + (i - OB2);  // b2, W3 and b3 follow one another
 }
 
+// the place of the v-th float4 of the parameters (rows' ends past IN / 4 and HID / 4 left out)
+__device__ __forceinline__ int train_vec(int v) {
+    constexpr int P1 = HID * XS, P2 = P1 + HID, P3 = P2 + HID * W2S;
+    constexpr int V1 = HID * IN4, V2 = V1 + HID / 4, V3 = V2 + HID * HID / 4;
+    if (v < V1) return v / IN4 * XS + v % IN4 * 4;
+    if (v < V2) return P1 + (v - V1) * 4;
+    if (v < V3) return P2 + (v - V2) / (HID / 4) * W2S + (v - V2) % (HID / 4) * 4;
+    return P3 + (v - V3) * 4;
+}
+// the parameter at a place train_vec names or the three after it; -1: none (a row's end)
+__device__ __forceinline__ int train_param(int at) {
+    constexpr int P1 = HID * XS, P2 = P1 + HID, P3 = P2 + HID * W2S;
+    if (at < P1) return at % XS < IN ? at / XS * IN + at % XS : -1;
+    if (at < P2) return OB1 + (at - P1);
+    if (at < P3) return OW2 + (at - P2) / W2S * HID + (at - P2) % W2S;
+    return OB2 + (at - P3) < NP ? OB2 + (at - P3) : -1;
+}
 __device__ __forceinline__ float *train_flat(TrainParams &p) { return reinterpret_cast<float *>(&p); }
 
 // The weights into S, zeros into the rows' ends.
@@ -156,25 +176,38 @@ __device__ __forceinline__ void train_load(TrainSmem &S, const float *params) {
     float *w = train_flat(S);
     for (int i = threadIdx.x; i < HID * XS; i += TT) w[i] = 0.f;
     for (int i = threadIdx.x; i < SB * XS; i += TT) S.x[0][i] = 0.f;
+    if (threadIdx.x < 4) S.b3[threadIdx.x] = S.g.b3[threadIdx.x] = 0.f;
     __syncthreads();
     for (int i = threadIdx.x; i < NP; i += TT) w[train_place(i)] = params[i];
 }
 
 // The rows of the samples a CTA takes at once, two values per thread (IN features and the target per sample), held in
-// registers so that a step's rows are on their way while the step before it is computed.
+// registers so that a step's rows are on their way while the step before it is computed: first where they are (the
+// sample order is a load of its own), half a step later the rows.
 struct TrainRows {
     float v[2];
 };
+struct TrainAt {
+    uint64_t s[2];
+    uint32_t n;
+};
+__device__ __forceinline__ TrainAt train_at(const uint32_t *perm, uint64_t first, uint32_t n) {
+    TrainAt a{{0, 0}, n};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t b = (threadIdx.x + TT * k) / (IN + 1);
+        if (b < n && b < uint32_t(SB)) a.s[k] = perm ? __ldg(perm + first + b) : first + b;
+    }
+    return a;
+}
 __device__ __forceinline__ TrainRows train_fetch(const float *x, uint32_t xstride, const float *t, uint32_t tstride,
-                                                 const uint32_t *perm, uint64_t first, uint32_t n) {
+                                                 const TrainAt &a) {
     TrainRows r{{0.f, 0.f}};
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const uint32_t i = threadIdx.x + TT * k, b = i / (IN + 1), j = i % (IN + 1);
-        if (b < n && b < uint32_t(SB)) {
-            const uint64_t s = perm ? __ldg(perm + first + b) : first + b;
-            r.v[k] = j < uint32_t(IN) ? __ldg(x + s * xstride + j) : __ldg(t + s * tstride);
-        }
+        if (b < a.n && b < uint32_t(SB))
+            r.v[k] = j < uint32_t(IN) ? __ldg(x + a.s[k] * xstride + j) : __ldg(t + a.s[k] * tstride);
     }
     return r;
 }
@@ -306,10 +339,13 @@ __device__ __forceinline__ void train_forward(TrainSmem &S, uint32_t n) {
     __syncwarp();
 }
 
-// Gradient of the chunk in S.x (n samples), written to S.g (first) or added; the loss terms go to S.loss.
-__device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_b, bool first) {
+// Gradient of the chunk in S.x (n samples), written to S.g (first) or added; the loss terms go to S.loss. `half` is
+// called between the forward and the backward pass.
+template <class F>
+__device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_b, bool first, F half) {
     const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID, lane = tid & 31, warp = tid >> 5;
     train_forward(S, n);
+    half();
     {
         const float r = S.dy[warp], dy = r * inv_b;
         __syncwarp();
@@ -381,7 +417,7 @@ __device__ __forceinline__ void train_share(uint32_t nb, uint32_t rank, uint32_t
 // `total` samples in the order of perm (null: as they are), `batch` per step; TRAIN: Adam's step number t0 + 1 and on,
 // params, m1 and m2 updated at the end. Else one batch of all samples: gradient and loss.
 template <bool TRAIN>
-__global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
+__global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT, 1)
     k_mlp_train(float *__restrict__ params, const float *__restrict__ x, uint32_t xstride, const float *__restrict__ t,
                 uint32_t tstride, const uint32_t *__restrict__ perm, uint64_t total, uint32_t epoch, uint32_t batch,
                 float *__restrict__ m1, float *__restrict__ m2, int t0, float lr, float beta1, float beta2, float eps,
@@ -393,20 +429,19 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
     const uint32_t rank = cl.block_rank();
     const int tid = threadIdx.x;
     train_load(S, params);
-    // the thread's parameters: SHARD * rank + tid + 256 k
+    // the thread's parameters: float4 SHARD * rank + tid of them
+    const int vec = SHARD * int(rank) + tid;
+    const bool owner = tid < SHARD && vec < NV;
+    const int place = owner ? train_vec(vec) : 0;
     float p[4] = {}, ma[4] = {}, mb[4] = {};
-    int own[4], place[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int o = tid + TT * k, i = SHARD * int(rank) + o;
-        own[k] = o < SHARD && i < NP ? i : -1;
-        place[k] = train_place(max(own[k], 0));
-        if (own[k] >= 0) {
-            p[k] = params[own[k]];
-            if (TRAIN) {
-                ma[k] = m1[own[k]];
-                mb[k] = m2[own[k]];
-            }
+        const int i = train_param(place + k);
+        if (!owner || i < 0) continue;
+        p[k] = params[i];
+        if (TRAIN) {
+            ma[k] = m1[i];
+            mb[k] = m2[i];
         }
     }
     // batches do not cross epochs: the last one of an epoch may be smaller
@@ -416,7 +451,7 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
     auto batch_at = [&](uint32_t e) { return min(batch, epoch - e); };
     uint32_t r0, per;
     train_share(batch_at(0), rank, r0, per);
-    TrainRows next = train_fetch(x, xstride, t, tstride, perm, r0, min(per, uint32_t(SB)));
+    TrainRows next = train_fetch(x, xstride, t, tstride, train_at(perm, r0, min(per, uint32_t(SB))));
     cl.sync();
     while (pos < total) {
         const uint32_t nb = batch_at(in_epoch);
@@ -431,38 +466,38 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
             const uint32_t n = per > c ? min(per - c, uint32_t(SB)) : 0u;
             train_put(S, next);
             __syncthreads();
-            if (c + SB < per)
-                next = train_fetch(x, xstride, t, tstride, perm, pos + r0 + c + SB, min(per - c - SB, uint32_t(SB)));
-            else if (npos < total)
-                next = train_fetch(x, xstride, t, tstride, perm, npos + nr0, min(nper, uint32_t(SB)));
-            train_chunk(S, n, inv_b, c == 0);
+            TrainAt at{{0, 0}, 0};
+            if (c + SB < per) at = train_at(perm, pos + r0 + c + SB, min(per - c - SB, uint32_t(SB)));
+            else if (npos < total) at = train_at(perm, npos + nr0, min(nper, uint32_t(SB)));
+            train_chunk(S, n, inv_b, c == 0, [&] { next = train_fetch(x, xstride, t, tstride, at); });
             __syncthreads();
         }
         ++step;
         const float c1 = TRAIN ? 1.f - powf(beta1, float(step)) : 1.f, c2 = TRAIN ? 1.f - powf(beta2, float(step)) : 1.f;
         cl.sync();  // every rank's partial gradient is complete
-        float part[4][CR];  // every remote read in flight before the first sum
+        float4 part[CR];  // every remote read in flight before the first sum
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int r = 0; r < CR; ++r) part[k][r] = cl.map_shared_rank(train_flat(S.g), r)[place[k]];
+        for (int r = 0; r < CR; ++r) part[r] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(train_flat(S.g), r) + place);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (own[k] < 0) continue;
             float g = 0.f;
 #pragma unroll
-            for (int r = 0; r < CR; ++r) g += part[k][r];
+            for (int r = 0; r < CR; ++r) g += k == 0 ? part[r].x : k == 1 ? part[r].y : k == 2 ? part[r].z : part[r].w;
+            const int i = train_param(place + k);
             if (TRAIN) {
                 const float a = beta1 * ma[k] + (1.f - beta1) * g;
                 const float b = beta2 * mb[k] + (1.f - beta2) * g * g;
                 ma[k] = a;
                 mb[k] = b;
-                p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
-#pragma unroll
-                for (int r = 0; r < CR; ++r) cl.map_shared_rank(train_flat(S), r)[place[k]] = p[k];
-            } else {
-                grad[own[k]] = g;
+                if (i >= 0) p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+            } else if (owner && i >= 0) {
+                grad[i] = g;
             }
+        }
+        if (TRAIN && owner) {
+            const float4 w = make_float4(p[0], p[1], p[2], p[3]);
+#pragma unroll
+            for (int r = 0; r < CR; ++r) *reinterpret_cast<float4 *>(cl.map_shared_rank(train_flat(S), r) + place) = w;
         }
         if (!TRAIN && rank == 0 && tid == 0 && loss_out) {
             float ls = 0.f;
@@ -476,10 +511,10 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT)
     if (TRAIN) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (own[k] >= 0) {
-                params[own[k]] = p[k];
-                m1[own[k]] = ma[k];
-                m2[own[k]] = mb[k];
+            if (const int i = train_param(place + k); owner && i >= 0) {
+                params[i] = p[k];
+                m1[i] = ma[k];
+                m2[i] = mb[k];
             }
     }
 }
@@ -494,7 +529,7 @@ __global__ void __launch_bounds__(TT) k_mlp_loss(const float *__restrict__ param
     double sum = 0;
     for (uint64_t c = uint64_t(blockIdx.x) * SB; c < count; c += uint64_t(gridDim.x) * SB) {
         const uint32_t n = uint32_t(min(count - c, uint64_t(SB)));
-        train_put(S, train_fetch(x, xstride, t, tstride, nullptr, c, n));
+        train_put(S, train_fetch(x, xstride, t, tstride, train_at(nullptr, c, n)));
         __syncthreads();
         train_forward(S, n);
         __syncthreads();
