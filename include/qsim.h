@@ -74,11 +74,12 @@ typedef struct qsim_gate {
 #define QSIM_CODEC_QSZR 2u /* compressed blocks under a point-wise relative bound eps (Sec. 4.3,
                               Eq. 1-2, Algorithm 2); both modes, exact or learned sizing */
 
-#define QSIM_SIZING_EXACT 0u   /* every block gets a slot of its exact size: in streams mode the encoder
-                                  codes the frames in place in one read of the working vector and then
-                                  reserves the exact slots; the persistent kernel sizes the frames in
-                                  one read and encodes at the known offsets in a second */
-#define QSIM_SIZING_PREDICT 1u /* learned size predictor reserves space; overflow re-encodes */
+#define QSIM_SIZING_EXACT 0u   /* every block gets a slot of its exact size: the encoder codes the frames
+                                  in one read of the working vector, the slot is reserved when the
+                                  block's last frame is coded and the frames are moved there (blocks
+                                  of one frame are written to their slot at once) */
+#define QSIM_SIZING_PREDICT 1u /* learned size predictor reserves space; a block that does not fit
+                                  gets a slot of its exact size */
 
 #define QSIM_REORDER_NONE 0u   /* Algorithm 1 over the gates in circuit order */
 #define QSIM_REORDER_STAGES 1u /* commutation-aware stage partition */
@@ -299,9 +300,9 @@ void qsim_shard_free(qsim_shard_run *run);
 /* Read the final state (Sec. 4.2's loop leaves it compressed, block by
  * block): gather `count` amplitudes, indices idx (host, each < 2^n), into
  * out_interleaved (HOST, 2*count floats, re then im per amplitude). Only the
- * blocks holding them are decompressed, into library scratch on the state's
- * device. Errors: INVALID (null pointer, index out of range), NOMEM, CUDA,
- * CORRUPT. */
+ * 32-value chunks holding them are decoded; the indices and the amplitudes
+ * pass through library scratch on the state's device. Errors: INVALID (null
+ * pointer, index out of range), NOMEM, CUDA, CORRUPT. */
 int qsim_amplitudes(const qsim_state *st, const uint64_t *idx, size_t count, float *out_interleaved);
 
 /* Fidelity |<ref|sim>| / (||ref|| ||sim||) (Sec. 5.3 definition, normalised),
@@ -383,9 +384,8 @@ int qsim_compress_block_noalloc(const float *d_amps, uint32_t m, double eb, void
  * input x satisfies |x' - x| <= rel |x| with the sign of x kept; zeros stay
  * zero; subnormal inputs get an absolute error below 2^(k-150) (k the code
  * shift, the largest integer with 2^(k-24) <= rel / (1 + rel)).
- * d_amps is not modified (the block is copied to library scratch, grown by
- * cudaMalloc when a larger m is first used). Synchronises cuda_stream and
- * writes the stream size to *out_bytes (host).
+ * d_amps is not modified. Synchronises cuda_stream and writes the stream size
+ * to *out_bytes (host).
  * Errors: INVALID (m outside 5..26, rel outside (2^-23, 1), NaN/Inf input),
  * RANGE (|x| >= 2^64), CAPACITY (*out_bytes = the size needed), NOMEM, CUDA.
  */

@@ -1048,7 +1048,7 @@ __global__ void k_init_blocks(float2 *wv, int m, uint64_t local_index) {
         wv[i] = make_float2(i == local_index ? 1.f : 0.f, 0.f);
 }
 
-// every block except b0 gets its own copy of the zero stream (Sec. 4.2)
+// uncompressed store: every block except b0 gets its own copy of the zero block (Sec. 4.2)
 __global__ void k_replicate_zero(BlockSlot *table, uint32_t nblocks, uint32_t b0, const BlockSlot *zero_slot,
                                  ArenaDev dev, ArenaDev host, int *status) {
     __shared__ uint8_t *dst;
@@ -1344,11 +1344,11 @@ static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
     return QSIM_OK;
 }
 
-// Mode B: the persistent stage kernel over a queue of segments (one stage of
-// one circuit each). One circuit: one launch per stage (optionally the stage
+// Mode B: the persistent stage kernel over a queue of steps; a segment is one
+// stage of one circuit. One circuit: one launch per stage (optionally the stage
 // loop captured in one CUDA graph). Several circuits: one launch for all of
-// them, stages dealt round-robin over the circuits so that one circuit's stage
-// boundary overlaps the other circuits' work.
+// them, the circuits' steps merged so that one circuit's stage boundary overlaps
+// the other circuits' work.
 struct PBlockBufs {
     DevBuf<EncTarget> tgt;
     DevBuf<EncResult> res;
@@ -1756,7 +1756,7 @@ static int finish_run(RunCtx &R, int dev, double ms, const StageAccum *accs, Pro
     const qsim_plan *p = R.p;
     PlanDev *pd = R.pd;
     const size_t nst = R.nst;
-    const bool raw = R.raw, predict = R.predict;
+    const bool raw = R.raw;
     const uint64_t nblocks = R.nblocks;
     qsim_state *S = new qsim_state();
     S->device = dev;
@@ -1791,7 +1791,7 @@ static int finish_run(RunCtx &R, int dev, double ms, const StageAccum *accs, Pro
             const StageDev &sd = pd->stages[i];
             bytes[raw ? P_COPY_IN : P_DECODE] += in_store + 8 * amps;
             bytes[P_PASS] += 16 * amps * sd.npasses;
-            bytes[P_STAGE] += in_store + out_store + 8 * amps * (2 + (predict ? 0 : 1)) + 16 * amps * sd.npasses;
+            bytes[P_STAGE] += in_store + 16 * amps + 3 * out_store + 16 * amps * sd.npasses;
             for (const Op &op : p->stages[i].ops) {
                 const double fl = (op.type == OP_DENSE ? 8.0 * double(1u << op.k)
                                    : op.type == OP_DIAG ? 6.0 : op.type == OP_CSEP ? 12.0 : 0.0) * amps;

@@ -46,7 +46,7 @@ bool qsz_step_exponent(double eb, int *e);
 constexpr uint32_t kQszrMagic = 0x525A5351u;  // "QSZR"
 constexpr int kQszrKMin = 1;
 constexpr int kQszrKMax = 22;
-constexpr uint32_t kQszrSideBytes = 2048;  // per-frame side record of the in-place encoder
+constexpr uint32_t kQszrSideBytes = 2048;  // per-frame side record of the QSZR encoder
 inline uint64_t qszr_worst_case(int m) {
     uint64_t F = uint64_t(1) << frame_log_for(m), C = F / 32;
     return qsz_data_start(m) + qsz_nframes(m) * (pad16(2 * C) + pad16((2 * C + 3) / 4) + pad16(8 * C) + 8 * F);
