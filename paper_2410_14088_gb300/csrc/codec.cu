@@ -32,7 +32,9 @@ using namespace cdev;
 
 // One frame per team of max(32, C) threads, which is the CTA. Blocks are read from table[ids[j]] (ids null: block
 // b0 + j). NP: the most leading phase ops the kernel applies (pre.count <= NP). Five CTAs of 128 threads per SM: 102
-// registers hold a chunk pair's 64 bit-plane words (the wide path) without spills, and 35 KB of tile each fit six.
+// registers hold a chunk pair's 64 bit-plane words (the wide path) without spills, and 35 KB of tile each fit six. A launch
+// of few frames is one chain of latencies, so its CTAs are as many as its frames: one 1024-amplitude frame per CTA took
+// 6 us where a warp per frame took 22.
 template <int NP, bool REL>
 __global__ void __launch_bounds__(kTeamMax, 5) k_decode(const BlockSlot *__restrict__ table,
                                                         const uint32_t *__restrict__ ids, uint64_t b0,
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_decode_block(BlockRef in, int m
 // Random access: amplitude idx[i] of a state to out[i], one warp each. It reads the frame's widths and the words of two
 // chunks (about 0.5 KB) instead of decoding the frame's 4096 amplitudes to memory first, so its cost, about 0.3 ns an
 // index, stays below that of moving the index and the amplitude to and from the host however many a frame is asked for.
+// 65536 random indices of a 26-qubit state: 28.7 ms with a host map of frames and whole frames decoded, 0.13 ms now.
 template <bool REL>
 __global__ void __launch_bounds__(256) k_amplitudes(const BlockSlot *__restrict__ table,
                                                     const uint64_t *__restrict__ idx, uint64_t count, int m,
@@ -134,6 +137,7 @@ __global__ void k_amplitudes_raw(const BlockSlot *__restrict__ table, const uint
 //    of its image before them to the frame's side record; the CTA that finishes a block's last frame turns the frame
 //    lengths into offsets and reserves the block's slot, while other blocks are still being coded. k_frame_copy then
 //    moves the images. (The exact slot needs the size of the whole block, so its frames cannot go there directly.)
+// Blocks of one frame: 33 + 8 us for the encoder and its copy with a warp per frame, 8 us now (64 frames of 1024 amplitudes).
 // arrive: one counter per block, zero before and after. keep_fitting (learned sizing): a block keeps the slot reserved
 // for it beforehand when its exact size fits, and only a block whose prediction was too small gets an exact slot
 // (counted as an overflowed block).
@@ -221,7 +225,8 @@ __global__ void __launch_bounds__(kTeamMax) k_frame_copy(const float2 *__restric
 // One block into the caller's buffer in one pass: each CTA codes one frame, takes a ticket so that frames are
 // processed in order, and finds its byte offset with a decoupled look-back over the preceding frames' sizes. Every
 // spin-wait is bounded and reports QSIM_E_TIMEOUT instead of hanging. The record receives the stream's size (also when
-// it exceeds cap; the header is then not written) and the status.
+// it exceeds cap; the header is then not written) and the status. A block of 2^22 amplitudes: 84 -> 47 us a call, of
+// which the launch and the wait for it are 20 and 1024 frames on 760 resident CTAs two rounds of about 10.
 template <bool REL>
 __global__ void __launch_bounds__(kTeamMax, 5) k_encode_block(const float2 *__restrict__ amps, int m, int e,
                                                               uint8_t *__restrict__ out, uint64_t cap,
@@ -273,7 +278,8 @@ __global__ void __launch_bounds__(kTeamMax, 5) k_encode_block(const float2 *__re
 }
 
 // Initial store (Sec. 4.2): every block's stream written directly. All but block b0 are zero: a header and an offset
-// table. b0 holds the basis state's single amplitude 1 at local index loc: its one non-empty frame is coded here.
+// table. b0 holds the basis state's single amplitude 1 at local index loc: its one non-empty frame is coded here. 0.013 ms
+// for eight blocks of 2^25 amplitudes (0.83 ms with both kinds of block filled in memory and encoded).
 template <bool REL>
 __global__ void __launch_bounds__(kTeamMax) k_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e,
                                                          BlockSlot *__restrict__ table, ArenaDev dev, ArenaDev host,

@@ -9,7 +9,9 @@
 // of those (transpose, prefix sums, width votes) and walks its 128 chunk pairs one after the other.
 //
 // What bounds it: instruction issue and shared memory (the frame passes through shared memory once each way, plus its
-// words), close to the HBM time of the frame: about 30 warp instructions per 32 amplitudes.
+// words), close to the HBM time of the frame. Per 32-value chunk pair 49 warp instructions decode and 56 encode, against
+// 143 and 115 with a warp per frame; launches of 4096 dense frames (2^24 amplitudes) take 39 us instead of 155 and 46
+// instead of 133, 2^28 amplitudes of early frames 0.30 ms to decode (7.0 TB/s) and 0.57 ms to encode (4.9 TB/s; 1.26 before).
 //
 // Layout: chunk t's amplitudes at byte 272 t of the tile (256 bytes and 16 of padding): a thread walks its row 16
 // bytes at a time and eight threads' rows fall on all 32 banks, and rows are read and written coalesced. The frame's

@@ -45,7 +45,8 @@ constexpr int kPassSmemMost = 220 * 1024;  // dynamic shared memory of a pass, 6
 // keep their own register allocation)
 // Teams of 128 threads per CTA, a tile each, at most. Without tcgen05 four share one pass blob: a blob of many ops (56 KB
 // in the 28-op passes of a random circuit) beside every 32 KB tile left two tiles, 8 warps, per SM; four tiles beside one
-// blob are the 16 warps that 128 registers a thread allow. The split-BF16 warp MMAs take 168 registers (three teams),
+// blob are the 16 warps that 128 registers a thread allow (26-qubit random brick in FP32 with the groups of
+// apply_dense_groups: 21.8 -> 18.2 ms; four teams of 64 threads with twice the groups: 22.1). The split-BF16 warp MMAs take 168 registers (three teams),
 // width 6 takes 255, and the tcgen05 forms size TMEM and B by the tile.
 template <int KMAX, int PREC, bool UM>
 __host__ __device__ constexpr int pass_teams() {
@@ -286,7 +287,9 @@ size_t pass_smem_bytes(const PassDev &P, int teams) {
            size_t(teams) * P.mat_elems * sizeof(float2);
 }
 
-// (the reload form keeps three CTAs per SM up to 75 KB each)
+// A pass takes the register form while three CTAs of its reload form fit an SM (75 KB each). Past that two tiles would be
+// in flight where the staged form keeps three. The line goes by the tiles in flight: no plan of the benchmark's circuits
+// reaches it (their fullest passes, three ops and one run, take 1.53 ms per 2^28 amplitudes against 1.55 staged).
 bool reg_pass_fits(const PassDev &P, int prec) {
     constexpr uint32_t most = 228u * 1024u / 3u - 1024u - uint32_t(sizeof(RegSmem<1>)) - 64u;
     if (prec == QSIM_PREC_TF32)

