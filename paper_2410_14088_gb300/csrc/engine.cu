@@ -1150,6 +1150,7 @@ struct StreamWork {
     DevBuf<uint32_t> ctr;    // gate-pass tile counter (two words, left zero)
     DevBuf<float2> part;
     DevBuf<uint32_t> hist;   // per block: 32-bin histogram of code bit lengths (decoder)
+    DevBuf<float> pred;      // per block: predicted log2 stream bytes
     DevBuf<uint8_t> side;               // per frame: its image before the bit-plane words
     DevBuf<uint32_t> flen, foff, fhead;  // per frame: stream bytes, offset, bytes in `side`
     FrameRecords records(bool rel) const {
@@ -1161,7 +1162,7 @@ struct StreamWork {
         const uint64_t nf = nframes > 1 ? blocks * nframes : 0;  // one-frame blocks keep no frame records
         if ((rc = wv.alloc(blocks << m)) || (rc = refs.alloc(blocks)) || (rc = tgt.alloc(blocks)) ||
             (rc = res.alloc(blocks)) || (rc = sizes.alloc(blocks)) || (rc = hist.alloc(blocks * 32)) ||
-            (rc = part.alloc(nf)) || (rc = side.alloc(nf * (rel ? kQszrSideBytes : 256))) ||
+            (rc = pred.alloc(blocks)) || (rc = part.alloc(nf)) || (rc = side.alloc(nf * (rel ? kQszrSideBytes : 256))) ||
             (rc = flen.alloc(nf)) || (rc = foff.alloc(nf)) || (rel && (rc = fhead.alloc(nf))) || (rc = ctr.alloc(2)))
             return rc;
         CUDA_TRY(cudaMemsetAsync(ctr.p, 0, 2 * sizeof(uint32_t), st));
@@ -1329,7 +1330,8 @@ static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
     static const uint32_t h_ids[2] = {0, 1};
     CUDA_TRY(cudaMemcpyAsync(R.init_ids.p, h_ids, sizeof(h_ids), cudaMemcpyHostToDevice, s));
     // tmpl[0] is the basis block, tmpl[1] the zero template
-    launch_reserve(2, R.worst, R.arena_dev(0), R.arena_host(0), w->tgt.p, w->res.p, status, s);
+    launch_reserve(2, nullptr, R.worst, nullptr, 0, R.worst, R.arena_dev(0), R.arena_host(0), w->tgt.p, w->res.p, 0,
+                   status, s);
     launch_copy_out(w->wv.p, 2, m, w->tgt.p, R.init_ids.p, R.tmpl.p, nullptr, status, s);
     k_copy_slot<<<1, 1, 0, s>>>(tab0 + b0, R.tmpl.p + 0);
     count_launch();
@@ -2044,14 +2046,8 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
             float *log_ptr = collect ? RC.log_rows.p + RC.log_next * (kMlpIn + 1) : nullptr;
             if (predict || collect) {
                 prof.begin(P_PREDICT, w.s);
-                // learned sizing: 2^pred (1 + margin) bytes per block ahead of the encoder, which keeps every slot its
-                // block fits and reserves exact slots for under-estimated blocks. Reserved by the predictor's launch: a
-                // kernel of its own waited for the other stream's resident pass CTAs (0.8 ms a group on the 32-qubit
-                // QAOA)
-                const PredictSlots slots{cfg.predictor_margin, worst, arena_dev(out_par), arena_host(out_par),
-                                         w.tgt.p, w.res.p, status};
                 launch_predict_sizes(w.hist.p, nb, sd.G, m, sf, predict ? dctx.pred_params : nullptr,
-                                     dctx.pred_bf16, slots, log_ptr, w.s);
+                                     dctx.pred_bf16, w.pred.p, log_ptr, w.s);
                 prof.end(w.s);
             }
             for (uint32_t pi = 0; pi < sd.npasses; ++pi) {
@@ -2062,12 +2058,21 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
             }
             if (raw) {
                 prof.begin(P_RESERVE, w.s);
-                launch_reserve(nb, worst, arena_dev(out_par), arena_host(out_par), w.tgt.p, w.res.p, status, w.s);
+                launch_reserve(nb, nullptr, worst, nullptr, 0, worst, arena_dev(out_par), arena_host(out_par),
+                               w.tgt.p, w.res.p, 0, status, w.s);
                 prof.end(w.s);
                 prof.begin(P_COPY_OUT, w.s);
                 launch_copy_out(w.wv.p, nb, m, w.tgt.p, ids, tab_out, acc, status, w.s);
                 prof.end(w.s);
             } else {
+                if (predict) {
+                    // learned sizing: 2^pred (1 + margin) bytes per block ahead of the encoder, which keeps every
+                    // slot its block fits and reserves exact slots for under-estimated blocks
+                    prof.begin(P_RESERVE, w.s);
+                    launch_reserve(nb, nullptr, 0, w.pred.p, cfg.predictor_margin, worst, arena_dev(out_par),
+                                   arena_host(out_par), w.tgt.p, w.res.p, 0, status, w.s);
+                    prof.end(w.s);
+                }
                 const FrameRecords fr = w.records(RC.rel);
                 prof.begin(P_ENCODE, w.s);
                 launch_encode(w.wv.p, nb, int(m), e, arena_dev(out_par), arena_host(out_par), w.tgt.p, w.res.p, ids,

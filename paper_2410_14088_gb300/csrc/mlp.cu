@@ -22,7 +22,6 @@
 #include <atomic>
 
 #include "codec.cuh"
-#include "codec_dev.cuh"
 #include "device_common.cuh"
 #include "mlp.cuh"
 
@@ -61,7 +60,7 @@ __global__ void k_mlp_forward(const float *__restrict__ params, const float *__r
 __global__ void __launch_bounds__(128) k_predict_sizes(const uint32_t *__restrict__ hist, uint32_t nblocks,
                                                        uint32_t G, int m, StageFeatures sf,
                                                        const float *__restrict__ params, int bf16,
-                                                       PredictSlots slots, float *__restrict__ feat_out) {
+                                                       float *__restrict__ pred, float *__restrict__ feat_out) {
     __shared__ float w[NP];
     __shared__ float xs[4][IN + 1];
     __shared__ float hs[4][HID];
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(128) k_predict_sizes(const uint32_t *__restric
         __syncwarp();
         if (feat_out)
             for (int t = lane; t < IN; t += 32) feat_out[uint64_t(j) * (IN + 1) + t] = xs[wi][t];
-        if (params) {
+        if (params && pred) {
             float a0 = w[OB1 + lane], a1 = w[OB1 + lane + 32];
             for (int t = 0; t < IN; ++t) {
                 const float x = xs[wi][t];
@@ -100,14 +99,7 @@ __global__ void __launch_bounds__(128) k_predict_sizes(const uint32_t *__restric
             float y = w[OW3 + lane] * fmaxf(b0, 0.f) + w[OW3 + lane + 32] * fmaxf(b1, 0.f);
 #pragma unroll
             for (int o = 16; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-            if (lane == 0) {
-                double p = double(y + w[OB3] + float(m + 3));
-                p = p < 0 ? 0 : (p > 40 ? 40 : p);
-                const double b = exp2(p) * (1.0 + slots.margin);
-                slots.res[j] = EncResult{};
-                cdev::reserve_slot(b >= double(slots.worst) ? slots.worst : uint64_t(b), slots.dev, slots.host,
-                                   slots.tgt + j, slots.status);
-            }
+            if (lane == 0) pred[j] = y + w[OB3] + float(m + 3);
         }
         __syncwarp();
     }
@@ -572,9 +564,9 @@ void launch_mlp_forward(const float *params, const float *x, uint32_t batch, flo
 }
 
 void launch_predict_sizes(const uint32_t *hist, uint32_t nblocks, uint32_t G, int m, const StageFeatures &sf,
-                          const float *params, int bf16, const PredictSlots &slots, float *feat_out, cudaStream_t s) {
+                          const float *params, int bf16, float *pred, float *feat_out, cudaStream_t s) {
     const unsigned grid = (nblocks + 3) / 4;
-    k_predict_sizes<<<grid ? grid : 1, 128, 0, s>>>(hist, nblocks, G, m, sf, params, bf16, slots, feat_out);
+    k_predict_sizes<<<grid ? grid : 1, 128, 0, s>>>(hist, nblocks, G, m, sf, params, bf16, pred, feat_out);
     count_launch();
 }
 

@@ -39,19 +39,10 @@ __device__ __forceinline__ float mlp_forward_one(const float *w, const float *x)
 }
 
 void launch_mlp_forward(const float *params, const float *x, uint32_t batch, float *y, int bf16, cudaStream_t s);
-// features from the decoder's histogram (+ stage features) -> predicted log2 bytes -> a slot of 2^pred (1 + margin)
-// bytes (at most worst) for each block (params null: no prediction, no slot); feat_out (nullable) receives rows of
-// kMlpIn features followed by one target slot
-struct PredictSlots {
-    double margin;
-    uint64_t worst;
-    ArenaDev dev, host;
-    EncTarget *tgt;
-    EncResult *res;  // cleared
-    int *status;
-};
+// features from the decoder's histogram (+ stage features) -> predicted log2 bytes; feat_out (nullable) receives
+// rows of kMlpIn features followed by one target slot
 void launch_predict_sizes(const uint32_t *hist, uint32_t nblocks, uint32_t G, int m, const StageFeatures &sf,
-                          const float *params, int bf16, const PredictSlots &slots, float *feat_out, cudaStream_t s);
+                          const float *params, int bf16, float *pred, float *feat_out, cudaStream_t s);
 void launch_log_targets(const EncResult *res, uint32_t nblocks, int m, float *rows, cudaStream_t s);
 int launch_mlp_loss_grad(const float *params, const float *x, uint32_t xstride, const float *t, uint32_t tstride,
                          uint32_t count, float *grad, float *loss, cudaStream_t s);
