@@ -325,33 +325,25 @@ __global__ void __launch_bounds__(kTeamMax) k_init_store(uint64_t nblocks, uint6
 
 // ---------------------------------------------------------------------------
 // Slot reservation from the two-tier pool: device arena first, then the
-// pinned host arena. need[j] bytes (plus the fixed header/offsets part when
-// add_data_start is set); the slot is padded to 256 bytes.
+// pinned host arena. 2^pred_log2[j] (1 + margin) bytes, at most `worst`, or
+// `worst` without predictions; the slot is padded to 256 bytes.
 // ---------------------------------------------------------------------------
-__global__ void k_reserve(uint32_t nblocks, const uint64_t *__restrict__ need, uint64_t add_const,
-                          const float *__restrict__ pred_log2, double margin, uint64_t worst,
+__global__ void k_reserve(uint32_t nblocks, const float *__restrict__ pred_log2, double margin, uint64_t worst,
                           ArenaDev dev, ArenaDev host, EncTarget *__restrict__ tgt, EncResult *__restrict__ res,
-                          int retry_overflowed, int *status) {
+                          int *status) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= nblocks) return;
-    uint64_t want;
-    if (retry_overflowed) {
-        if (res[j].overflow == 0) return;
-        want = res[j].total;
-    } else if (pred_log2) {
+    uint64_t want = worst;
+    if (pred_log2) {
         double p = double(pred_log2[j]);
         p = p < 0 ? 0 : (p > 40 ? 40 : p);
         double b = exp2(p) * (1.0 + margin);
         want = b >= double(worst) ? worst : uint64_t(b);
-    } else {
-        want = (need ? need[j] : 0) + add_const;
     }
-    if (!retry_overflowed) {
-        res[j].total = 0;
-        res[j].overflow = 0;
-        res[j].err_sq = 0;
-        res[j].norm_sq = 0;
-    }
+    res[j].total = 0;
+    res[j].overflow = 0;
+    res[j].err_sq = 0;
+    res[j].norm_sq = 0;
     reserve_slot(want, dev, host, &tgt[j], status);
 }
 
@@ -533,11 +525,9 @@ void launch_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e
     count_launch();
 }
 
-void launch_reserve(uint32_t nblocks, const uint64_t *need, uint64_t add_const, const float *pred_log2,
-                    double margin, uint64_t worst, const ArenaDev &dev, const ArenaDev &host, EncTarget *tgt,
-                    EncResult *res, int retry_overflowed, int *status, cudaStream_t s) {
-    k_reserve<<<(nblocks + 127) / 128, 128, 0, s>>>(nblocks, need, add_const, pred_log2, margin, worst, dev, host,
-                                                    tgt, res, retry_overflowed, status);
+void launch_reserve(uint32_t nblocks, const float *pred_log2, double margin, uint64_t worst, const ArenaDev &dev,
+                    const ArenaDev &host, EncTarget *tgt, EncResult *res, int *status, cudaStream_t s) {
+    k_reserve<<<(nblocks + 127) / 128, 128, 0, s>>>(nblocks, pred_log2, margin, worst, dev, host, tgt, res, status);
     count_launch();
 }
 

@@ -1330,8 +1330,7 @@ static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
     static const uint32_t h_ids[2] = {0, 1};
     CUDA_TRY(cudaMemcpyAsync(R.init_ids.p, h_ids, sizeof(h_ids), cudaMemcpyHostToDevice, s));
     // tmpl[0] is the basis block, tmpl[1] the zero template
-    launch_reserve(2, nullptr, R.worst, nullptr, 0, R.worst, R.arena_dev(0), R.arena_host(0), w->tgt.p, w->res.p, 0,
-                   status, s);
+    launch_reserve(2, nullptr, 0, R.worst, R.arena_dev(0), R.arena_host(0), w->tgt.p, w->res.p, status, s);
     launch_copy_out(w->wv.p, 2, m, w->tgt.p, R.init_ids.p, R.tmpl.p, nullptr, status, s);
     k_copy_slot<<<1, 1, 0, s>>>(tab0 + b0, R.tmpl.p + 0);
     count_launch();
@@ -2058,8 +2057,8 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
             }
             if (raw) {
                 prof.begin(P_RESERVE, w.s);
-                launch_reserve(nb, nullptr, worst, nullptr, 0, worst, arena_dev(out_par), arena_host(out_par),
-                               w.tgt.p, w.res.p, 0, status, w.s);
+                launch_reserve(nb, nullptr, 0, worst, arena_dev(out_par), arena_host(out_par), w.tgt.p, w.res.p,
+                               status, w.s);
                 prof.end(w.s);
                 prof.begin(P_COPY_OUT, w.s);
                 launch_copy_out(w.wv.p, nb, m, w.tgt.p, ids, tab_out, acc, status, w.s);
@@ -2069,8 +2068,8 @@ static int streams_stage(StreamsRun &S, size_t si, const uint32_t *ids_stage, co
                     // learned sizing: 2^pred (1 + margin) bytes per block ahead of the encoder, which keeps every
                     // slot its block fits and reserves exact slots for under-estimated blocks
                     prof.begin(P_RESERVE, w.s);
-                    launch_reserve(nb, nullptr, 0, w.pred.p, cfg.predictor_margin, worst, arena_dev(out_par),
-                                   arena_host(out_par), w.tgt.p, w.res.p, 0, status, w.s);
+                    launch_reserve(nb, w.pred.p, cfg.predictor_margin, worst, arena_dev(out_par),
+                                   arena_host(out_par), w.tgt.p, w.res.p, status, w.s);
                     prof.end(w.s);
                 }
                 const FrameRecords fr = w.records(RC.rel);
