@@ -426,12 +426,8 @@ static void decode_table(const BlockSlot *table, const uint32_t *ids, uint64_t b
     // with leading phase ops each CTA copies their descriptors once and takes several frames
     const unsigned grid = grid_for(items, pre.count ? 152 * 5 * 3 : kMaxGrid);
     const size_t smem = ts.smem + pre.count * cdev::kPreTabBytes;
-    static bool attr_set = false;  // kMaxPreOps tables beside the largest tile: 52.5 KB
-    if (pre.count > 2 && !attr_set) {
-        cudaFuncSetAttribute(k_decode<kMaxPreOps, REL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(cdev::team_tile_bytes(128) + kMaxPreOps * cdev::kPreTabBytes));
-        attr_set = true;
-    }
+    if (pre.count > 2)  // kMaxPreOps tables beside the largest tile: 52.5 KB
+        allow_smem<k_decode<kMaxPreOps, REL>>(int(cdev::team_tile_bytes(128) + kMaxPreOps * cdev::kPreTabBytes));
     if (pre.count == 0)
         k_decode<0, REL><<<grid, ts.threads, smem, s>>>(table, ids, b0, nblocks, m, wv, hist, status, pre);
     else if (pre.count <= 2)

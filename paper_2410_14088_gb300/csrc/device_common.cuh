@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace qsim {
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -64,6 +66,22 @@ __device__ __forceinline__ uint32_t warp_bit_transpose(uint32_t x, int lane) {
         x = (x & keep) | (got & ~keep);
     }
     return x;
+}
+
+// Host: lets a kernel take `bytes` of dynamic shared memory, with `most` out of the largest carveout of the unified array.
+// The setting is the device's, so it is made once per kernel and device. False when the runtime refuses it.
+template <auto *kernel>
+bool allow_smem(int bytes, bool most = false) {
+    static std::atomic<uint64_t> done{0};  // a bit per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load() & bit) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    if (most)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
+    done.fetch_or(bit);
+    return true;
 }
 
 }  // namespace qsim

@@ -108,14 +108,7 @@ int num_sms() {
 template <int KMAX, int PREC, bool UM>
 void launch_pass_ku(dim3 grid, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
                     const float2 *mats, const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_pass<KMAX, PREC, UM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmemMost);
-        // the whole unified L1/shared array as shared memory: the resident CTAs are limited by their tiles
-        cudaFuncSetAttribute(k_pass<KMAX, PREC, UM>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             int(cudaSharedmemCarveoutMaxShared));
-        attr_set = true;
-    }
+    allow_smem<k_pass<KMAX, PREC, UM>>(kPassSmemMost, true);  // the resident CTAs are limited by their tiles
     int teams = pass_teams<KMAX, PREC, UM>();
     while (teams > 1 && pass_smem_bytes(P, teams) > size_t(kPassSmemMost)) --teams;  // tiles of 2^13 amplitudes
     const size_t smem = pass_smem_bytes(P, teams);
@@ -166,13 +159,7 @@ bool reg_two(const PassDev &P) {
 template <int PREC, int H>
 void launch_reg(uint64_t ntiles, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
                 const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_pass_reg<PREC, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_pass_reg<PREC, H>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             int(cudaSharedmemCarveoutMaxShared));
-        attr_set = true;
-    }
+    allow_smem<k_pass_reg<PREC, H>>(200 * 1024, true);
     const uint32_t smem = reg_shape<PREC, H>(P.reg_dense, P.reg_poly, P.reg_flags, P.reg_words).bytes;
     const uint64_t by_smem = (228u * 1024u) / (smem + sizeof(RegSmem<H>) + 1024u);
     const uint64_t per_sm = std::max<uint64_t>(1, std::min<uint64_t>(by_smem, 4 / H));

@@ -19,8 +19,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "codec.cuh"
 #include "device_common.cuh"
 #include "mlp.cuh"
@@ -575,23 +573,9 @@ void launch_log_targets(const EncResult *res, uint32_t nblocks, int m, float *ro
     count_launch();
 }
 
-// dynamic shared memory of a training kernel, allowed once per kernel and device
-template <auto *kernel>
-static int train_smem_ok() {
-    static std::atomic<uint64_t> done{0};  // per kernel: a bit per device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return QSIM_E_CUDA;
-    if (done.load() >> (dev & 63) & 1) return QSIM_OK;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(TrainSmem))) != cudaSuccess)
-        return QSIM_E_CUDA;
-    done.fetch_or(1ull << (dev & 63));
-    return QSIM_OK;
-}
-
 int launch_mlp_loss_grad(const float *params, const float *x, uint32_t xstride, const float *t, uint32_t tstride,
                          uint32_t count, float *grad, float *loss, cudaStream_t s) {
-    int rc = train_smem_ok<k_mlp_train<false>>();
-    if (rc) return rc;
+    if (!allow_smem<k_mlp_train<false>>(int(sizeof(TrainSmem)))) return QSIM_E_CUDA;
     k_mlp_train<false><<<CR, TT, sizeof(TrainSmem), s>>>(const_cast<float *>(params), x, xstride, t, tstride, nullptr,
                                                          count, count, count, nullptr, nullptr, 0, 0.f, 0.f, 0.f, 0.f,
                                                          grad, loss);
@@ -602,8 +586,7 @@ int launch_mlp_loss_grad(const float *params, const float *x, uint32_t xstride, 
 int launch_mlp_train(float *params, const float *rows, uint32_t stride, const uint32_t *perm, uint64_t total,
                      uint32_t epoch, uint32_t batch, float *m1, float *m2, int t0, float lr, float beta1, float beta2,
                      float eps, cudaStream_t s) {
-    int rc = train_smem_ok<k_mlp_train<true>>();
-    if (rc) return rc;
+    if (!allow_smem<k_mlp_train<true>>(int(sizeof(TrainSmem)))) return QSIM_E_CUDA;
     k_mlp_train<true><<<CR, TT, sizeof(TrainSmem), s>>>(params, rows, stride, rows + IN, stride, perm, total, epoch,
                                                         batch, m1, m2, t0, lr, beta1, beta2, eps, nullptr, nullptr);
     count_launch();
@@ -612,8 +595,7 @@ int launch_mlp_train(float *params, const float *rows, uint32_t stride, const ui
 
 int launch_mlp_loss(const float *params, const float *rows, uint32_t stride, uint64_t count, double *loss,
                     cudaStream_t s) {
-    int rc = train_smem_ok<k_mlp_loss>();
-    if (rc) return rc;
+    if (!allow_smem<k_mlp_loss>(int(sizeof(TrainSmem)))) return QSIM_E_CUDA;
     const uint64_t chunks = (count + SB - 1) / SB;
     k_mlp_loss<<<unsigned(chunks < 304 ? chunks : 304), TT, sizeof(TrainSmem), s>>>(params, rows, stride, rows + IN,
                                                                                    stride, count, loss);

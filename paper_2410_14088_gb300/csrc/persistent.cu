@@ -409,25 +409,29 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
 }
 
 template <int PREC, bool REL, bool UM>
-struct LaunchShape {
-    static int grid;
-    static size_t attr_smem;
+struct LaunchShape {  // of a device
+    int grid = 0;
+    size_t attr_smem = 0;
+    static LaunchShape &current() {
+        static LaunchShape shapes[64];
+        int dev = 0;
+        cudaGetDevice(&dev);
+        return shapes[dev & 63];
+    }
 };
-template <int PREC, bool REL, bool UM> int LaunchShape<PREC, REL, UM>::grid = 0;
-template <int PREC, bool REL, bool UM> size_t LaunchShape<PREC, REL, UM>::attr_smem = 0;
 
 // kernel attributes and the grid (one wave of resident CTAs); done outside any stream capture
 template <int PREC, bool REL, bool UM>
 int prepare_prec(size_t smem) {
-    using Shape = LaunchShape<PREC, REL, UM>;
-    if (Shape::attr_smem < smem) {
+    LaunchShape<PREC, REL, UM> &shape = LaunchShape<PREC, REL, UM>::current();
+    if (shape.attr_smem < smem) {
         if (cudaFuncSetAttribute(k_stage_persistent<PREC, REL, UM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(smem)) != cudaSuccess)
             return QSIM_E_CUDA;
-        Shape::attr_smem = smem;
-        Shape::grid = 0;
+        shape.attr_smem = smem;
+        shape.grid = 0;
     }
-    if (!Shape::grid) {
+    if (!shape.grid) {
         // resident CTAs per SM from the kernel's registers and shared memory and the SM's limits (65536 registers,
         // 2048 threads, 228 KB of shared memory with 1 KB reserved per CTA); the runtime's occupancy query was
         // seen to answer 1 where more CTAs were resident
@@ -446,16 +450,16 @@ int prepare_prec(size_t smem) {
             if (UM && per_sm > int(512u / gdev::umma_pass_tmem_cols(0))) per_sm = int(512u / gdev::umma_pass_tmem_cols(0));
             if (per_sm < 1) per_sm = 1;
         }
-        Shape::grid = (sms > 0 ? sms : 1) * per_sm;
+        shape.grid = (sms > 0 ? sms : 1) * per_sm;
     }
     return QSIM_OK;
 }
 
 template <int PREC, bool REL, bool UM>
 int launch_stage_prec(const PLaunch &a, size_t smem, cudaStream_t s, int *grid_out) {
-    using Shape = LaunchShape<PREC, REL, UM>;
-    if (Shape::attr_smem < smem || !Shape::grid) return QSIM_E_INVALID;
-    const int grid = Shape::grid;
+    const LaunchShape<PREC, REL, UM> &shape = LaunchShape<PREC, REL, UM>::current();
+    if (shape.attr_smem < smem || !shape.grid) return QSIM_E_INVALID;
+    const int grid = shape.grid;
     k_stage_persistent<PREC, REL, UM><<<grid, kPT<UM>, smem, s>>>(a);
     if (grid_out) *grid_out = grid;
     count_launch();
