@@ -110,35 +110,33 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
 }
 
 // ---------------------------------------------------------------------------
-// Training. One cluster of eight CTAs runs a whole sequence of steps: each CTA takes an eighth of a batch's samples
-// through the forward and backward pass with its own copy of the weights in shared memory, the gradient is reduced
-// through distributed shared memory (each CTA sums an eighth of the parameters over the eight partials, in rank
-// order, so the result is deterministic), and the same CTA applies Adam to that eighth, whose moments it keeps in
-// registers, and writes the new weights into all eight copies. Two cluster barriers per step, no launch and no global
-// round trip. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases: latency and shared-memory reads
-// bound it, so the split is the smallest that leaves every phase two outputs per thread (8 samples x 64 units on 256
-// threads) and every product is tiled in registers over 128-bit reads. 800 steps of 64 samples: 72 ms with two launches
-// and one CTA per step, 5.9 ms of kernel now (8.1 ms the call).
+// Training. One cluster of eight CTAs runs a whole sequence of steps. A batch is taken in chunks of 64 samples: each CTA
+// takes eight of them through the forward and backward pass with its own copy of the weights in shared memory, then every
+// CTA collects what its eighth of the weight rows needs of all 64 through distributed shared memory, sums the gradient
+// of those rows over the samples, applies Adam to them, whose moments it keeps in registers, and writes the new weights
+// into all eight copies. Two cluster barriers per chunk, no launch and no global round trip. Every sum runs in the order
+// of a loop over its terms (inputs, units or samples): a training run amplifies the rounding of its first steps, so a sum
+// split over threads or CTAs ends in other weights. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases:
+// latency and shared-memory reads bound it. 800 steps of 64 samples: 72 ms with two launches and one CTA per step,
+// 8.3 ms now (the call).
 // ---------------------------------------------------------------------------
 constexpr int CR = 8;                            // CTAs of the cluster
-constexpr int SB = 8;                            // samples a CTA takes at a time (one warp each in the output layer)
+constexpr int SB = 8;                            // samples a CTA takes at a time
+constexpr int CH = CR * SB;                      // of a chunk
 constexpr int TT = 256;                          // threads
-constexpr int IN4 = (IN + 3) / 4;                // float4s of a row of W1
-constexpr int NV = HID * IN4 + HID / 4 + HID * HID / 4 + (2 * HID + 4) / 4;  // float4s of the parameters in shared memory
-constexpr int SHARD = (NV + CR - 1) / CR;        // of them a CTA's, one per thread
-static_assert(SHARD <= TT, "a thread owns at most one");
-constexpr int XS = (IN + 15) / 16 * 16;          // words of an input row and of a row of W1, zeros past IN
-constexpr int W2S = HID + 16;                    // words of a row of W2
-static_assert(XS % 32 == 16 && W2S % 32 == 16, "two rows read together must fall on different halves of the banks");
+constexpr int RW = HID / CR;                     // weight rows a CTA owns, one per warp
+constexpr int XS = 44, W2S = HID + 4, H2S = HID + 4;  // words of a row: eight rows' 16-byte reads fall on all banks
+static_assert(XS >= IN && RW == TT / 32 && IN > 32 && IN <= 32 + 9, "a warp's lanes cover a row of W1 in two rounds");
 
 struct __align__(16) TrainParams {
     float w1[HID * XS], b1[HID], w2[HID * W2S], b2[HID], w3[HID], b3[4];
 };
 struct __align__(16) TrainSmem : TrainParams {
-    TrainParams g;                               // partial gradient
-    float x[SB][XS];
-    float h1[SB][HID], h2[SB][HID], d1[SB][HID], d2[SB][HID];
-    float t[SB], dy[SB], sq[SB];
+    // this CTA's samples
+    float x[SB][XS], h1[SB][HID], h2[SB][H2S], d1[SB][HID], d2[SB][HID], dy[SB], t[SB], sq[SB];
+    // the chunk's, where it is about this CTA's weight rows by row
+    float ax[CH][XS], ah1[CH][HID], at1[RW][CH], at2[RW][CH], ah2[RW][CH], ady[CH];
+    float one[4];
     float loss;
 };
 
@@ -150,34 +148,14 @@ __device__ __forceinline__ int train_place(int i) {
     if (i < OB2) return P2 + (i - OW2) / HID * W2S + (i - OW2) % HID;
     return P3 + (i - OB2);  // b2, W3 and b3 follow one another
 }
-
-// the place of the v-th float4 of the parameters (rows' ends past IN / 4 and HID / 4 left out)
-__device__ __forceinline__ int train_vec(int v) {
-    constexpr int P1 = HID * XS, P2 = P1 + HID, P3 = P2 + HID * W2S;
-    constexpr int V1 = HID * IN4, V2 = V1 + HID / 4, V3 = V2 + HID * HID / 4;
-    if (v < V1) return v / IN4 * XS + v % IN4 * 4;
-    if (v < V2) return P1 + (v - V1) * 4;
-    if (v < V3) return P2 + (v - V2) / (HID / 4) * W2S + (v - V2) % (HID / 4) * 4;
-    return P3 + (v - V3) * 4;
-}
-// the parameter at a place train_vec names or the three after it; -1: none (a row's end)
-__device__ __forceinline__ int train_param(int at) {
-    constexpr int P1 = HID * XS, P2 = P1 + HID, P3 = P2 + HID * W2S;
-    if (at < P1) return at % XS < IN ? at / XS * IN + at % XS : -1;
-    if (at < P2) return OB1 + (at - P1);
-    if (at < P3) return OW2 + (at - P2) / W2S * HID + (at - P2) % W2S;
-    return OB2 + (at - P3) < NP ? OB2 + (at - P3) : -1;
-}
 __device__ __forceinline__ float *train_flat(TrainParams &p) { return reinterpret_cast<float *>(&p); }
 
-// The weights into S, zeros into the rows' ends.
 __device__ __forceinline__ void train_load(TrainSmem &S, const float *params) {
+    for (int i = threadIdx.x; i < SB * XS; i += TT) S.x[0][i] = 0.f;  // the rows' ends too
+    if (threadIdx.x == 0) S.one[0] = 1.f, S.loss = 0.f;
     float *w = train_flat(S);
-    for (int i = threadIdx.x; i < HID * XS; i += TT) w[i] = 0.f;
-    for (int i = threadIdx.x; i < SB * XS; i += TT) S.x[0][i] = 0.f;
-    if (threadIdx.x < 4) S.b3[threadIdx.x] = S.g.b3[threadIdx.x] = 0.f;
-    __syncthreads();
     for (int i = threadIdx.x; i < NP; i += TT) w[train_place(i)] = params[i];
+    __syncthreads();
 }
 
 // The rows of the samples a CTA takes at once, two values per thread (IN features and the target per sample), held in
@@ -220,197 +198,75 @@ __device__ __forceinline__ void train_put(TrainSmem &S, const TrainRows &r) {
     }
 }
 
-// The sums over K terms of v[b][k] * w[u * S + k] for the 8 samples and 64 units, put(b, u, sum) for each. The phase is
-// bound by shared-memory reads: a thread takes two units of four samples over a quarter of the terms in 128-bit reads,
-// K / 16 * 6 of them for 2 K products (one unit of two samples at a time took 3 K reads for the same 2 K). The
-// quarters are neighbouring lanes, whose reads of two rows of w fill the 32 banks (S = 16 mod 32).
-template <int K, int S, class F>
-__device__ __forceinline__ void train_rows(const float *w, const float *v, int vs, F put) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3;
-    const int u0 = (lane >> 2) + 8 * (warp & 3), b0 = 4 * (warp >> 2);
-    float acc[2][4] = {};
-#pragma unroll
-    for (int t = 0; t < K / 16; ++t) {
-        const int k = 16 * t + 4 * q;
-        const float4 wa = *reinterpret_cast<const float4 *>(w + u0 * S + k);
-        const float4 wb = *reinterpret_cast<const float4 *>(w + (u0 + HID / 2) * S + k);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const float4 x = *reinterpret_cast<const float4 *>(v + (b0 + b) * vs + k);
-            acc[0][b] = fmaf(wa.w, x.w, fmaf(wa.z, x.z, fmaf(wa.y, x.y, fmaf(wa.x, x.x, acc[0][b]))));
-            acc[1][b] = fmaf(wb.w, x.w, fmaf(wb.z, x.z, fmaf(wb.y, x.y, fmaf(wb.x, x.x, acc[1][b]))));
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {  // lane q of the four ends with sample b0 + q
-        float r[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float keep = q & 2 ? acc[i][2 + j] : acc[i][j], give = q & 2 ? acc[i][j] : acc[i][2 + j];
-            r[j] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
-        }
-        const float keep = q & 1 ? r[1] : r[0], give = q & 1 ? r[0] : r[1];
-        put(b0 + q, u0 + HID / 2 * i, keep + __shfl_xor_sync(0xffffffffu, give, 1));
-    }
+__device__ __forceinline__ float train_fma4(const float4 &a, const float4 &b, float c) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
 }
 
-// The sums over i of d2[b][i] * W2[i][j], put(b, j, sums of j and j + 1). As above with the threads along W2's rows: four
-// units of two samples over a quarter of the terms.
-template <class F>
-__device__ __forceinline__ void train_cols(const TrainSmem &S, F put) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 3;
-    const int j0 = 4 * ((lane & 7) + 8 * (warp & 1)), b0 = 2 * (warp >> 1);
-    float acc[2][4] = {};
-#pragma unroll
-    for (int t = 0; t < HID / 16; ++t) {
-        const int k = HID / 4 * q + 4 * t;
-        float x[2][4];
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const float4 d = *reinterpret_cast<const float4 *>(&S.d2[b0 + b][k]);
-            x[b][0] = d.x;
-            x[b][1] = d.y;
-            x[b][2] = d.z;
-            x[b][3] = d.w;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 w = *reinterpret_cast<const float4 *>(S.w2 + (k + i) * W2S + j0);
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                acc[b][0] = fmaf(w.x, x[b][i], acc[b][0]);
-                acc[b][1] = fmaf(w.y, x[b][i], acc[b][1]);
-                acc[b][2] = fmaf(w.z, x[b][i], acc[b][2]);
-                acc[b][3] = fmaf(w.w, x[b][i], acc[b][3]);
-            }
-        }
-    }
-    float r[4], s[2];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {  // quarters 2 and 3 end with sample b0 + 1
-        const float keep = q & 2 ? acc[1][j] : acc[0][j], give = q & 2 ? acc[0][j] : acc[1][j];
-        r[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {  // odd quarters with units j0 + 2 and j0 + 3
-        const float keep = q & 1 ? r[2 + j] : r[j], give = q & 1 ? r[j] : r[2 + j];
-        s[j] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-    }
-    put(b0 + (q >> 1), j0 + 2 * (q & 1), s[0], s[1]);
-}
-
-// What a thread writes of the partial gradient: four neighbours, first ? v : what is there + v.
-__device__ __forceinline__ void train_put4(float *at, bool first, const float *v) {
-    float4 o = make_float4(v[0], v[1], v[2], v[3]);
-    if (!first) {
-        const float4 w = *reinterpret_cast<float4 *>(at);
-        o = make_float4(o.x + w.x, o.y + w.y, o.z + w.z, o.w + w.w);
-    }
-    *reinterpret_cast<float4 *>(at) = o;
-}
-
-// The outer products of a and x, four by four (rows r0 .., columns c0 ..), summed over the samples.
-__device__ __forceinline__ void train_outer(const float *a, const float *x, int xs, int r0, int c0, float (&acc)[4][4]) {
-#pragma unroll
-    for (int b = 0; b < SB; ++b) {
-        const float4 d = *reinterpret_cast<const float4 *>(a + b * HID + r0);
-        const float4 e = *reinterpret_cast<const float4 *>(x + b * xs + c0);
-        const float dd[4] = {d.x, d.y, d.z, d.w}, xx[4] = {e.x, e.y, e.z, e.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], xx[j], acc[i][j]);
-    }
-}
-
-// Forward pass of the n (<= SB) samples in S.x; each sample's residual y - t to S.dy (0 past n). Ends unsynchronised:
-// warp b wrote sample b's.
+// Forward pass of the n (<= SB) samples in S.x; each sample's residual y - t to S.dy (0 past n). A thread takes one unit
+// of two samples. Ends unsynchronised: thread b wrote sample b's.
 __device__ __forceinline__ void train_forward(TrainSmem &S, uint32_t n) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    train_rows<XS, XS>(S.w1, S.x[0], XS, [&](int b, int u, float v) { S.h1[b][u] = fmaxf(v + S.b1[u], 0.f); });
-    __syncthreads();
-    train_rows<HID, W2S>(S.w2, S.h1[0], HID, [&](int b, int u, float v) { S.h2[b][u] = fmaxf(v + S.b2[u], 0.f); });
-    __syncthreads();
-    float y = S.w3[lane] * S.h2[warp][lane] + S.w3[lane + 32] * S.h2[warp][lane + 32];
+    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID;
+    float a0 = S.b1[h], a1 = a0;
+    const float *w = S.w1 + h * XS;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-    if (lane == 0) S.dy[warp] = uint32_t(warp) < n ? y + S.b3[0] - S.t[warp] : 0.f;
-    __syncwarp();
+    for (int j = 0; j < IN / 4 * 4; j += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(w + j);
+        a0 = train_fma4(v, *reinterpret_cast<const float4 *>(&S.x[q][j]), a0);
+        a1 = train_fma4(v, *reinterpret_cast<const float4 *>(&S.x[q + 4][j]), a1);
+    }
+#pragma unroll
+    for (int j = IN / 4 * 4; j < IN; ++j) {
+        a0 = fmaf(w[j], S.x[q][j], a0);
+        a1 = fmaf(w[j], S.x[q + 4][j], a1);
+    }
+    S.h1[q][h] = fmaxf(a0, 0.f);
+    S.h1[q + 4][h] = fmaxf(a1, 0.f);
+    __syncthreads();
+    a0 = a1 = S.b2[h];
+    w = S.w2 + h * W2S;
+#pragma unroll
+    for (int j = 0; j < HID; j += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(w + j);
+        a0 = train_fma4(v, *reinterpret_cast<const float4 *>(&S.h1[q][j]), a0);
+        a1 = train_fma4(v, *reinterpret_cast<const float4 *>(&S.h1[q + 4][j]), a1);
+    }
+    S.h2[q][h] = fmaxf(a0, 0.f);
+    S.h2[q + 4][h] = fmaxf(a1, 0.f);
+    __syncthreads();
+    if (tid < SB) {
+        float y = S.b3[0];
+#pragma unroll
+        for (int j = 0; j < HID; j += 4)
+            y = train_fma4(*reinterpret_cast<const float4 *>(S.w3 + j), *reinterpret_cast<const float4 *>(&S.h2[tid][j]), y);
+        S.dy[tid] = uint32_t(tid) < n ? y - S.t[tid] : 0.f;
+    }
 }
 
-// Gradient of the chunk in S.x (n samples), written to S.g (first) or added; the loss terms go to S.loss. `half` is
-// called between the forward and the backward pass.
+// Forward and backward pass of the n samples in S.x (inv_b: 1 / the batch's samples); `half` is called in between.
 template <class F>
-__device__ __forceinline__ void train_chunk(TrainSmem &S, uint32_t n, float inv_b, bool first, F half) {
-    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID, lane = tid & 31, warp = tid >> 5;
+__device__ __forceinline__ void train_samples(TrainSmem &S, uint32_t n, float inv_b, F half) {
+    const int tid = threadIdx.x, h = tid & (HID - 1), q = tid / HID;
     train_forward(S, n);
+    if (tid < SB) {
+        const float r = S.dy[tid];
+        S.dy[tid] = r * inv_b;
+        S.sq[tid] = 0.5f * r * r * inv_b;
+    }
     half();
-    {
-        const float r = S.dy[warp], dy = r * inv_b;
-        __syncwarp();
-        if (lane == 0) {
-            S.dy[warp] = dy;
-            S.sq[warp] = 0.5f * r * dy;
-        }
-        S.d2[warp][lane] = S.h2[warp][lane] > 0.f ? dy * S.w3[lane] : 0.f;
-        S.d2[warp][lane + 32] = S.h2[warp][lane + 32] > 0.f ? dy * S.w3[lane + 32] : 0.f;
-    }
     __syncthreads();
-    train_cols(S, [&](int b, int j, float v0, float v1) {  // back through W2
-        const float2 a = *reinterpret_cast<const float2 *>(&S.h1[b][j]);
-        *reinterpret_cast<float2 *>(&S.d1[b][j]) = make_float2(a.x > 0.f ? v0 : 0.f, a.y > 0.f ? v1 : 0.f);
-    });
-    auto put = [&](float *at, float v) { *at = first ? v : *at + v; };
-    {  // W2: a 4 x 4 tile per thread
-        const int r0 = (tid >> 4) * 4, c0 = (tid & 15) * 4;
-        float acc[4][4] = {};
-        train_outer(S.d2[0], S.h1[0], HID, r0, c0, acc);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) train_put4(S.g.w2 + (r0 + i) * W2S + c0, first, acc[i]);
-    }
-    if (q == 0) {  // W3, b2 and b3
-        float gw = 0.f, gb = 0.f;
-#pragma unroll
-        for (int b = 0; b < SB; ++b) {
-            gw = fmaf(S.dy[b], S.h2[b][h], gw);
-            gb += S.d2[b][h];
-        }
-        put(S.g.w3 + h, gw);
-        put(S.g.b2 + h, gb);
-        if (h == 0) {
-            float g3 = 0.f, ls = 0.f;
-#pragma unroll
-            for (int b = 0; b < SB; ++b) {
-                g3 += S.dy[b];
-                ls += S.sq[b];
-            }
-            put(S.g.b3, g3);
-            S.loss = first ? ls : S.loss + ls;
-        }
-    }
+    for (int b = q; b < SB; b += 4) S.d2[b][h] = S.h2[b][h] > 0.f ? S.dy[b] * S.w3[h] : 0.f;
     __syncthreads();
-    constexpr int T1 = XS / 4;  // tiles along a row of W1
-    if (tid < 16 * T1) {        // W1
-        const int r0 = tid / T1 * 4, c0 = tid % T1 * 4;
-        float acc[4][4] = {};
-        train_outer(S.d1[0], S.x[0], XS, r0, c0, acc);
+    float a0 = 0.f, a1 = 0.f;  // back through W2
 #pragma unroll
-        for (int i = 0; i < 4; ++i) train_put4(S.g.w1 + (r0 + i) * XS + c0, first, acc[i]);
-    } else if (tid - 16 * T1 < HID) {  // b1
-        const int u = tid - 16 * T1;
-        float v = 0.f;
-#pragma unroll
-        for (int b = 0; b < SB; ++b) v += S.d1[b][u];
-        put(S.g.b1 + u, v);
+    for (int i = 0; i < HID; i += 4) {
+        const float4 w = make_float4(S.w2[i * W2S + h], S.w2[(i + 1) * W2S + h], S.w2[(i + 2) * W2S + h],
+                                     S.w2[(i + 3) * W2S + h]);
+        a0 = train_fma4(*reinterpret_cast<const float4 *>(&S.d2[q][i]), w, a0);
+        a1 = train_fma4(*reinterpret_cast<const float4 *>(&S.d2[q + 4][i]), w, a1);
     }
-}
-static_assert(16 * (XS / 4) + HID <= TT, "W1's tiles and b1 share the threads");
-
-// Samples [r0, r0 + per) of a batch of nb belong to rank r.
-__device__ __forceinline__ void train_share(uint32_t nb, uint32_t rank, uint32_t &r0, uint32_t &per) {
-    const uint32_t each = (nb + CR - 1) / CR;
-    r0 = min(each * rank, nb);
-    per = min(each, nb - r0);
+    S.d1[q][h] = S.h1[q][h] > 0.f ? a0 : 0.f;
+    S.d1[q + 4][h] = S.h1[q + 4][h] > 0.f ? a1 : 0.f;
 }
 
 // `total` samples in the order of perm (null: as they are), `batch` per step; TRAIN: Adam's step number t0 + 1 and on,
@@ -426,21 +282,30 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT, 1)
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const uint32_t rank = cl.block_rank();
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, row = tid >> 5, lane = tid & 31, unit = RW * int(rank) + row;
     train_load(S, params);
-    // the thread's parameters: float4 SHARD * rank + tid of them
-    const int vec = SHARD * int(rank) + tid;
-    const bool owner = tid < SHARD && vec < NV;
-    const int place = owner ? train_vec(vec) : 0;
-    float p[4] = {}, ma[4] = {}, mb[4] = {};
+    // the thread's parameters, of weight rows `unit`: two neighbours of W2, one of W1, and one of the row's end of W1, of
+    // b2, b1, W3 or b3
+    int own[4] = {OW2 + unit * HID + 2 * lane, OW2 + unit * HID + 2 * lane + 1, OW1 + unit * IN + lane, -1};
+    if (lane < IN - 32) own[3] = OW1 + unit * IN + 32 + lane;
+    else if (lane == 9) own[3] = OB2 + unit;
+    else if (lane == 10) own[3] = OB1 + unit;
+    else if (lane == 11) own[3] = OW3 + unit;
+    else if (lane == 12 && unit == 0) own[3] = OB3;
+    // the last one's factors by sample
+    const float *pf = lane == 9 ? S.at2[row] : lane == 11 || lane == 12 ? S.ady : S.at1[row];
+    const float *qf = lane < IN - 32 ? &S.ax[0][32 + lane] : lane == 11 ? S.ah2[row] : S.one;
+    const int qs = lane < IN - 32 ? XS : lane == 11 ? 1 : 0;
+    int place[4];
+    float p[4] = {}, ma[4] = {}, mb[4] = {}, g[4] = {};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int i = train_param(place + k);
-        if (!owner || i < 0) continue;
-        p[k] = params[i];
+        place[k] = train_place(max(own[k], 0));
+        if (own[k] < 0) continue;
+        p[k] = params[own[k]];
         if (TRAIN) {
-            ma[k] = m1[i];
-            mb[k] = m2[i];
+            ma[k] = m1[own[k]];
+            mb[k] = m2[own[k]];
         }
     }
     // batches do not cross epochs: the last one of an epoch may be smaller
@@ -448,72 +313,113 @@ __global__ void __cluster_dims__(CR, 1, 1) __launch_bounds__(TT, 1)
     uint32_t in_epoch = 0;
     int step = t0;
     auto batch_at = [&](uint32_t e) { return min(batch, epoch - e); };
-    uint32_t r0, per;
-    train_share(batch_at(0), rank, r0, per);
-    TrainRows next = train_fetch(x, xstride, t, tstride, train_at(perm, r0, min(per, uint32_t(SB))));
+    // this CTA's samples of the chunk that starts `left` samples before its batch's end
+    auto share = [&](uint32_t left) { return left > SB * rank ? min(left - SB * rank, uint32_t(SB)) : 0u; };
+    TrainRows next = train_fetch(x, xstride, t, tstride, train_at(perm, SB * rank, share(batch_at(0))));
     cl.sync();
     while (pos < total) {
         const uint32_t nb = batch_at(in_epoch);
-        train_share(nb, rank, r0, per);
         const float inv_b = 1.0f / float(nb);
         const uint64_t npos = pos + nb;
         const uint32_t nin = in_epoch + nb == epoch ? 0u : in_epoch + nb;
-        uint32_t nr0 = 0, nper = 0;
-        if (npos < total) train_share(batch_at(nin), rank, nr0, nper);
-        // at least one chunk: a rank without samples contributes zeros
-        for (uint32_t c = 0; c == 0 || c < per; c += SB) {
-            const uint32_t n = per > c ? min(per - c, uint32_t(SB)) : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) g[k] = 0.f;
+        for (uint32_t c = 0; c < nb; c += CH) {
+            if (c) cl.sync();  // every CTA has collected the chunk before
             train_put(S, next);
             __syncthreads();
             TrainAt at{{0, 0}, 0};
-            if (c + SB < per) at = train_at(perm, pos + r0 + c + SB, min(per - c - SB, uint32_t(SB)));
-            else if (npos < total) at = train_at(perm, npos + nr0, min(nper, uint32_t(SB)));
-            train_chunk(S, n, inv_b, c == 0, [&] { next = train_fetch(x, xstride, t, tstride, at); });
+            if (c + CH < nb) at = train_at(perm, pos + c + CH + SB * rank, share(nb - c - CH));
+            else if (npos < total) at = train_at(perm, npos + SB * rank, share(batch_at(nin)));
+            train_samples(S, share(nb - c), inv_b, [&] { next = train_fetch(x, xstride, t, tstride, at); });
+            cl.sync();  // every CTA's samples are done
+            {           // collect: sample b of the chunk is sample b % SB of CTA b / SB
+                float4 vh[CH * HID / 4 / TT], vx[3], vd[3];
+#pragma unroll
+                for (int k = 0; k < CH * HID / 4 / TT; ++k) {
+                    const int i = tid + TT * k, b = i / (HID / 4);
+                    vh[k] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(&S.h1[b % SB][i % (HID / 4) * 4], b / SB));
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int i = tid + TT * k, b = i / (XS / 4);
+                    if (b < CH)
+                        vx[k] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(&S.x[b % SB][i % (XS / 4) * 4], b / SB));
+                }
+                const int b = (tid / 2) & (CH - 1), o = RW * int(rank) + 4 * (tid & 1);  // threads 0 .. 127
+                float yv = 0.f;
+                if (tid < 2 * CH) {
+                    vd[0] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(&S.d1[b % SB][o], b / SB));
+                    vd[1] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(&S.d2[b % SB][o], b / SB));
+                    vd[2] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(&S.h2[b % SB][o], b / SB));
+                    yv = *cl.map_shared_rank(&S.dy[b % SB], b / SB);
+                }
+#pragma unroll
+                for (int k = 0; k < CH * HID / 4 / TT; ++k)
+                    reinterpret_cast<float4 *>(S.ah1[0])[tid + TT * k] = vh[k];
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if ((tid + TT * k) / (XS / 4) < CH) reinterpret_cast<float4 *>(S.ax[0])[tid + TT * k] = vx[k];
+                if (tid < 2 * CH) {
+                    const int r = 4 * (tid & 1);
+                    S.at1[r][b] = vd[0].x, S.at1[r + 1][b] = vd[0].y, S.at1[r + 2][b] = vd[0].z, S.at1[r + 3][b] = vd[0].w;
+                    S.at2[r][b] = vd[1].x, S.at2[r + 1][b] = vd[1].y, S.at2[r + 2][b] = vd[1].z, S.at2[r + 3][b] = vd[1].w;
+                    S.ah2[r][b] = vd[2].x, S.ah2[r + 1][b] = vd[2].y, S.ah2[r + 2][b] = vd[2].z, S.ah2[r + 3][b] = vd[2].w;
+                    if (!(tid & 1)) S.ady[b] = yv;
+                }
+            }
+            if (!TRAIN && tid == 0)
+                for (int b = 0; b < SB; ++b) S.loss += S.sq[b];
             __syncthreads();
+            float a[4] = {};  // samples past the batch's end have zero derivatives
+            const int cn = int(min(nb - c, uint32_t(CH)));
+#pragma unroll 4
+            for (int b = 0; b < cn; ++b) {
+                const float2 hv = *reinterpret_cast<const float2 *>(&S.ah1[b][2 * lane]);
+                const float e2 = S.at2[row][b];
+                a[0] = fmaf(e2, hv.x, a[0]);
+                a[1] = fmaf(e2, hv.y, a[1]);
+                a[2] = fmaf(S.at1[row][b], S.ax[b][lane], a[2]);
+                a[3] = fmaf(pf[b], qf[b * qs], a[3]);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k] += a[k];
         }
         ++step;
         const float c1 = TRAIN ? 1.f - powf(beta1, float(step)) : 1.f, c2 = TRAIN ? 1.f - powf(beta2, float(step)) : 1.f;
-        cl.sync();  // every rank's partial gradient is complete
-        float4 part[CR];  // every remote read in flight before the first sum
-#pragma unroll
-        for (int r = 0; r < CR; ++r) part[r] = *reinterpret_cast<const float4 *>(cl.map_shared_rank(train_flat(S.g), r) + place);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            float g = 0.f;
-#pragma unroll
-            for (int r = 0; r < CR; ++r) g += k == 0 ? part[r].x : k == 1 ? part[r].y : k == 2 ? part[r].z : part[r].w;
-            const int i = train_param(place + k);
+            if (own[k] < 0) continue;
             if (TRAIN) {
-                const float a = beta1 * ma[k] + (1.f - beta1) * g;
-                const float b = beta2 * mb[k] + (1.f - beta2) * g * g;
+                const float gi = g[k];
+                const float a = beta1 * ma[k] + (1.f - beta1) * gi;
+                const float b = beta2 * mb[k] + (1.f - beta2) * gi * gi;
                 ma[k] = a;
                 mb[k] = b;
-                if (i >= 0) p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
-            } else if (owner && i >= 0) {
-                grad[i] = g;
+                p[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+#pragma unroll
+                for (int r = 0; r < CR; ++r) cl.map_shared_rank(train_flat(S), r)[place[k]] = p[k];
+            } else {
+                grad[own[k]] = g[k];
             }
         }
-        if (TRAIN && owner) {
-            const float4 w = make_float4(p[0], p[1], p[2], p[3]);
-#pragma unroll
-            for (int r = 0; r < CR; ++r) *reinterpret_cast<float4 *>(cl.map_shared_rank(train_flat(S), r) + place) = w;
-        }
+        cl.sync();  // the new weights are in every copy, the chunk has been collected
         if (!TRAIN && rank == 0 && tid == 0 && loss_out) {
             float ls = 0.f;
             for (int r = 0; r < CR; ++r) ls += *cl.map_shared_rank(&S.loss, r);
             *loss_out = ls;
         }
-        cl.sync();  // the new weights are in every copy, the partials have been read
         pos = npos;
         in_epoch = nin;
     }
+    if (!TRAIN) cl.sync();  // no CTA leaves while its loss may be read
     if (TRAIN) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (const int i = train_param(place + k); owner && i >= 0) {
-                params[i] = p[k];
-                m1[i] = ma[k];
-                m2[i] = mb[k];
+            if (own[k] >= 0) {
+                params[own[k]] = p[k];
+                m1[own[k]] = ma[k];
+                m2[own[k]] = mb[k];
             }
     }
 }
