@@ -501,22 +501,24 @@ int qsim_state_kernel_stats(const qsim_state *st, qsim_kernel_stat *out, size_t 
 /* ---- a batch of independent circuits ----------------------------------------
  * Runs `count` planned circuits together: their initial stores, then ONE launch
  * of the persistent stage kernel whose work queue holds every stage of every
- * circuit. Stages are dealt round-robin over the circuits (stage 0 of each,
- * then stage 1 of each, ...); a circuit's stage waits on the device for all
+ * circuit (two launches when plans with tcgen05 set and plans whose
+ * tensor-core ops run without it are mixed). The circuits' steps are merged by
+ * how far each circuit is; a circuit's stage waits on the device for all
  * groups of its previous stage (a bounded wait, QSIM_E_TIMEOUT), so one
  * circuit's stage boundary overlaps the other circuits' work. The paper runs
  * one circuit at a time; this extends its group pipeline (Sec. 4.2) to many
  * independent state vectors, each with its own block size, fused width and
  * error bound.
- *   plans   host array of `count` plans. Each must use codec QSZ1, k <= 5 and
- *           no row collection; all must use the same precision. Their mode and
+ *   plans   host array of `count` plans. Each must use a compressed codec (the
+ *           same one), k <= 5 (6 in TF32 with tcgen05) and no row collection;
+ *           all must use the same precision. Their mode and
  *           streams fields are ignored; sizing is exact or predict per plan
  *           (predict needs trained weights); the first plan's `graph` flag
  *           decides whether the launch is captured in a CUDA graph.
  *   states  out: host array of `count` handles, each freed by qsim_state_free.
  *   stats   nullable: `count` entries; `seconds` is the whole batch's time.
- *   launch  nullable: event time, algorithmic bytes and flops of the batch's
- *           persistent launch.
+ *   launch  nullable: number, event time, algorithmic bytes and flops of the
+ *           batch's persistent launches.
  * Memory: each circuit gets a share of the device and pinned-host levels in
  * proportion to its worst-case store size.
  * Errors: INVALID (empty batch, mixed precision, a plan the persistent kernel

@@ -1409,10 +1409,9 @@ static std::vector<PLane> plan_lanes(const std::vector<RunCtx *> &rs, size_t s0,
     return out;
 }
 
-static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cudaStream_t main, int *status,
+static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, bool graph, cudaStream_t main, int *status,
                           Profiler &prof, const DeviceCtx &dctx, uint64_t slot_budget_amps) {
-    const qsim_config &cfg0 = rs[0]->p->cfg;
-    const int prec = int(cfg0.prec);
+    const int prec = int(rs[0]->p->cfg.prec);
     // ---- segments in queue order ----
     struct SegRef {
         uint32_t c, si;
@@ -1664,7 +1663,6 @@ static int run_persistent(const std::vector<RunCtx *> &rs, bool one_launch, cuda
     L.status = status;
     L.wait_ns = stall ? 200000000ull : 2000000000ull;  // 0.2 s in the bounded-wait test, else 2 s
 
-    const bool graph = cfg0.graph != 0;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
     // the caller's stream may be the legacy default stream, which cannot be captured: capture on our own
@@ -2116,7 +2114,7 @@ static int run_plan(const qsim_plan *p, cudaStream_t main, qsim_state **out, qsi
     PlanDev *pd = S.RC.pd;
     if (S.RC.persistent) {
         std::vector<RunCtx *> one{&S.RC};
-        if ((rc = streams_join(S)) || (rc = run_persistent(one, false, main, S.status, S.prof, *S.dctx, 1ull << 25))) return rc;
+        if ((rc = streams_join(S)) || (rc = run_persistent(one, false, p->cfg.graph != 0, main, S.status, S.prof, *S.dctx, 1ull << 25))) return rc;
     } else {
         for (size_t si = 0; si < S.RC.nst; ++si) {
             const StageDev &sd = pd->stages[si];
@@ -2128,8 +2126,27 @@ static int run_plan(const qsim_plan *p, cudaStream_t main, qsim_state **out, qsi
     return streams_finish(S, out, stats);
 }
 
-// A batch of circuits: initial stores, then one persistent launch over every
-// stage of every circuit.
+// The launches of a batch, each over every stage of its circuits. A launch with a pass on tcgen05 runs the kernel that
+// holds those products and no warp-level MMAs; the circuits that need the latter (tensor-core ops in passes planned
+// without tcgen05) then get a launch of their own. Every other batch is one launch.
+static std::vector<std::vector<RunCtx *>> batch_launches(const std::vector<RunCtx *> &rp) {
+    bool tcgen05 = false;
+    std::vector<RunCtx *> warp, others;
+    for (RunCtx *R : rp) {
+        bool w = false;
+        const uint32_t min_k = R->p->cfg.prec == QSIM_PREC_TF32 ? 3u : 4u;
+        for (const StageDev &sd : R->pd->stages)
+            for (const PassDev &ps : sd.passes_host) {
+                tcgen05 |= (ps.umma & 1u) != 0;
+                w |= R->p->cfg.prec != QSIM_PREC_FP32 && ps.T == 12 && !(ps.umma & 1u) && ps.kmax >= min_k;
+            }
+        (w ? warp : others).push_back(R);
+    }
+    if (!tcgen05 || warp.empty()) return {rp};
+    return {others, warp};
+}
+
+// A batch of circuits: initial stores, then the persistent launches (one, or the two of batch_launches).
 static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t main, qsim_state **out,
                      qsim_stats *stats, qsim_kernel_stat *launch_stat) {
     NvtxRange batch_range("qsim_run_batch %zu circuits", count);
@@ -2168,8 +2185,10 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     // working-vector slots with their frame scratch
     size_t max_nst = 0;
     for (const RunCtx *R : rp) max_nst = std::max(max_nst, R->nst);
-    uint64_t slot_amps = 0;
-    for (const PLane &ln : plan_lanes(rp, 0, max_nst, slot_budget)) slot_amps += ln.slots * ln.amps;
+    const std::vector<std::vector<RunCtx *>> launch_sets = batch_launches(rp);
+    uint64_t slot_amps = 0;  // of all launches: the cache keeps the first one's buffers
+    for (const std::vector<RunCtx *> &set : launch_sets)
+        for (const PLane &ln : plan_lanes(set, 0, max_nst, slot_budget)) slot_amps += ln.slots * ln.amps;
     // 8 B per amplitude and a quarter for the frame scratch
     const uint64_t work_bytes = slot_amps * 10;
     const double dev_budget = free_b > work_bytes ? 0.85 * double(free_b - work_bytes) : 0.0;
@@ -2188,7 +2207,8 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     CUDA_TRY(cudaEventRecord(ev_start, main));
     for (size_t c = 0; c < count && !rc; ++c) rc = init_store(*rs[c], nullptr, status, main);
     if (rc) return rc;
-    if ((rc = run_persistent(rp, true, main, status, prof, dctx, slot_budget))) return rc;
+    for (const std::vector<RunCtx *> &set : launch_sets)
+        if ((rc = run_persistent(set, true, plans[0]->cfg.graph != 0, main, status, prof, dctx, slot_budget))) return rc;
     CUDA_TRY(cudaEventRecord(ev_stop, main));
     HostBuf<StageAccum> host;
     std::vector<const StageAccum *> accs;

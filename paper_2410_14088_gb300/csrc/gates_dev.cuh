@@ -873,7 +873,8 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
             if constexpr (UM) {
                 // a tcgen05 pass (T = 12) runs every dense op of width 3 to 5 above (widths 3 and 4 come widened
                 // to 5), and width 6 in TF32; what is left here is width 1 or 2, 6 in split BF16, and the passes of
-                // smaller tiles in a launch of the persistent kernel, on CUDA cores
+                // smaller tiles in a launch of the persistent kernel, on CUDA cores. (A wider op of a 4096-amplitude pass
+                // planned without tcgen05 has no matrix staged; such passes are not in a tcgen05 launch.)
                 if (k == 1) {
                     apply_dense_k1<NT>(tile, M, cb, osw, T);
                 } else if (k == 2) {

@@ -418,8 +418,8 @@ def run(plan: Plan, stream=None) -> State:
 
 
 def run_batch(plans, stream=None):
-    """Run several plans in one persistent launch (qsim_run_batch). Returns
-    (states, launch) where launch is the persistent launch's kernel statistic."""
+    """Run several plans in one persistent launch, or two (qsim_run_batch). Returns
+    (states, launch) where launch is the persistent launches' kernel statistic."""
     n = len(plans)
     handles = (_VP * n)(*[p.handle for p in plans])
     outs = (_VP * n)()
