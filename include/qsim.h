@@ -301,7 +301,8 @@ void qsim_shard_free(qsim_shard_run *run);
  * block): gather `count` amplitudes, indices idx (host, each < 2^n), into
  * out_interleaved (HOST, 2*count floats, re then im per amplitude). Only the
  * 32-value chunks holding them are decoded; the indices and the amplitudes
- * pass through library scratch on the state's device. Errors: INVALID (null
+ * pass through library scratch on the state's device. out_interleaved is
+ * written as a whole or, on an error, not at all. Errors: INVALID (null
  * pointer, index out of range), NOMEM, CUDA, CORRUPT. */
 int qsim_amplitudes(const qsim_state *st, const uint64_t *idx, size_t count, float *out_interleaved);
 

@@ -2909,21 +2909,23 @@ int qsim_amplitudes(const qsim_state *st, const uint64_t *idx, size_t count, flo
     uint64_t any = 0;
     for (size_t i = 0; i < count; ++i) any |= idx[i];
     if (any >> st->n) return set_error(QSIM_E_INVALID, "amplitude index out of range");
-    // at most 2^24 indices at a time (256 MB of scratch)
+    // at most 2^24 indices at a time (128 MB of scratch); the caller's buffer is written once every status is good
     const size_t chunk = std::min<size_t>(count, size_t(1) << 24);
     DevBuf<uint64_t> d_idx;
     DevBuf<float2> d_out;
     int rc;
-    if ((rc = d_idx.alloc(chunk)) || (rc = d_out.alloc(chunk))) return rc;
+    if ((rc = d_idx.alloc(chunk)) || (rc = d_out.alloc(count))) return rc;
     cudaStream_t s = nullptr;
     CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     int *status = device_ctx(st->device).status;
     for (size_t i = 0; i < count; i += chunk) {
         const size_t cnt = std::min(chunk, count - i);
         CUDA_TRY(cudaMemcpyAsync(d_idx.p, idx + i, cnt * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-        launch_amplitudes(st->table, d_idx.p, cnt, int(st->m), d_out.p, status, s, st->codec);
-        if ((rc = read_status(status, s))) break;  // out is written only where the status is good
-        CUDA_TRY(cudaMemcpyAsync(out + 2 * i, d_out.p, cnt * sizeof(float2), cudaMemcpyDeviceToHost, s));
+        launch_amplitudes(st->table, d_idx.p, cnt, int(st->m), d_out.p + i, status, s, st->codec);
+    }
+    rc = read_status(status, s);
+    if (!rc) {
+        CUDA_TRY(cudaMemcpyAsync(out, d_out.p, count * sizeof(float2), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
     }
     cudaStreamDestroy(s);
