@@ -2889,13 +2889,15 @@ int qsim_state_decompress(const qsim_state *st, float *d_out, void *cuda_stream)
     const uint64_t nblocks = 1ull << (st->n - st->m);
     DevBuf<BlockRef> refs;
     int rc;
-    if (st->codec == QSIM_CODEC_NONE && (rc = refs.alloc(nblocks))) return rc;
+    // launches of at most 2^28 blocks (32-bit block and grid counts); an uncompressed state's go through a list of 2^16
+    // block references (1 MB), which the stream's order lets every launch use again
+    const bool raw = st->codec == QSIM_CODEC_NONE;
+    const uint64_t most = raw ? 1ull << 16 : 1ull << 28;
+    if (raw && (rc = refs.alloc(std::min(nblocks, most)))) return rc;
     int *status = device_ctx(st->device).status;
-    // launches of at most 2^28 blocks (32-bit block and grid counts)
     for (uint64_t b = 0, cnt; b < nblocks; b += cnt) {
-        cnt = std::min<uint64_t>(nblocks - b, 1ull << 28);
-        rc = decode_state_blocks(st, b, uint32_t(cnt), reinterpret_cast<float2 *>(d_out) + (b << st->m), refs.p + b,
-                                 status, s);
+        cnt = std::min<uint64_t>(nblocks - b, most);
+        rc = decode_state_blocks(st, b, uint32_t(cnt), reinterpret_cast<float2 *>(d_out) + (b << st->m), refs.p, status, s);
         if (rc) return rc;
     }
     int code = read_status(status, s);

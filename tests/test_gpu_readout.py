@@ -36,3 +36,18 @@ def test_amplitudes_written_whole_or_not_at_all(codec):
         assert call() == qsim.OK
         want = st.amplitudes(idx[-2:])
         assert (out.view(np.complex64)[:-1] == want[0]).all() and out.view(np.complex64)[-1] == want[1]
+
+
+def test_decompressing_an_uncompressed_state_takes_little_scratch():
+    c = inputs.random_brick(24, 1, 3)
+    st = qsim.run(qsim.plan_stages(c, m=5, inner=2, k=2, codec=qsim.CODEC_NONE))  # 2^19 blocks
+    small = qsim.run(qsim.plan_stages(inputs.random_brick(10, 1, 3), m=5, inner=2, k=2, codec=qsim.CODEC_NONE))
+    small.decompress()  # the kernels are loaded
+    out = torch.empty(1 << 24, dtype=torch.complex64, device="cuda")
+    torch.cuda.synchronize()
+    qsim.release_cached_memory()
+    free, _ = torch.cuda.mem_get_info()
+    st.decompress(out=out)
+    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20  # 2^16 references of 16 bytes, in the driver's units of 2 MB
+    idx = np.array([0, 31, 32, (1 << 21) - 1, 1 << 21, (1 << 24) - 1], dtype=np.uint64)  # across the lists' ends
+    np.testing.assert_array_equal(out.cpu().numpy()[idx.astype(np.int64)], st.amplitudes(idx))
