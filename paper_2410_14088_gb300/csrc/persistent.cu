@@ -313,11 +313,11 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
             if (tid < HID) {
                 float a = w[OB2 + tid];
                 for (int j = 0; j < HID; ++j) a = fmaf(w[OW2 + tid * (HID + 1) + j], h1[j], a);
-                h2[tid] = fmaxf(a, 0.f) * w[OW3 + tid];
+                h2[tid] = fmaxf(a, 0.f);
             }
             __syncthreads();
             float y = w[OB3];
-            for (int j = 0; j < HID; ++j) y += h2[j];
+            for (int j = 0; j < HID; ++j) y = fmaf(w[OW3 + j], h2[j], y);  // as mlp_forward_one
             double pr = double(y) + double(S.m + 3);
             pr = pr < 0 ? 0 : (pr > 40 ? 40 : pr);
             const double want_b = exp2(pr) * (1.0 + S.margin);
