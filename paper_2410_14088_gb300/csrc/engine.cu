@@ -1364,7 +1364,8 @@ static uint32_t unit_groups(const StageDev &sd) {
 // Circuits (indices into rs) that share the working-vector slots of one launch, with the slots' size and number.
 struct PLane {
     std::vector<uint32_t> circuits;
-    uint64_t amps = 0, frames = 0, units = 0;  // largest unit, largest unit's frames, most units of a stage
+    // largest unit, its frame records at most (blocks of one frame keep none), most units of a stage
+    uint64_t amps = 0, frames = 0, units = 0;
     uint32_t slots = 1;
 };
 
@@ -1380,7 +1381,7 @@ static std::vector<PLane> plan_lanes(const std::vector<RunCtx *> &rs, size_t s0,
             const StageDev &sd = rs[c]->pd->stages[si];
             const uint64_t ug = unit_groups(sd);
             l.amps = std::max(l.amps, ug << sd.W);
-            l.frames = std::max<uint64_t>(l.frames, ug * sd.G * rs[c]->nframes);
+            if (rs[c]->nframes > 1) l.frames = std::max<uint64_t>(l.frames, ug * sd.G * rs[c]->nframes);
             l.units = std::max<uint64_t>(l.units, sd.ngroups / ug);
         }
         if (l.units) lanes.push_back(std::move(l));
