@@ -424,7 +424,7 @@ static void decode_table(const BlockSlot *table, const uint32_t *ids, uint64_t b
     const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
     const TeamShape ts = team_shape(m);
     // with leading phase ops each CTA copies their descriptors once and takes several frames
-    const unsigned grid = grid_for(items, pre.count ? 152 * 5 * 3 : kMaxGrid);
+    const unsigned grid = grid_for(items, pre.count ? num_sms() * 5 * 3 : kMaxGrid);
     const size_t smem = ts.smem + pre.count * cdev::kPreTabBytes;
     if (pre.count > 2)  // kMaxPreOps tables beside the largest tile: 52.5 KB
         allow_smem<k_decode<kMaxPreOps, REL>>(int(cdev::team_tile_bytes(128) + kMaxPreOps * cdev::kPreTabBytes));
@@ -454,11 +454,11 @@ void launch_decode_block(const BlockRef &in, int m, float2 *out, const CallResul
 void launch_amplitudes(const BlockSlot *table, const uint64_t *idx, uint64_t count, int m, float2 *out, int *status,
                        cudaStream_t s, uint32_t codec) {
     if (codec == QSIM_CODEC_NONE)
-        k_amplitudes_raw<<<grid_for((count + 255) / 256, 152 * 16), 256, 0, s>>>(table, idx, count, m, out, status);
+        k_amplitudes_raw<<<grid_for((count + 255) / 256, num_sms() * 16), 256, 0, s>>>(table, idx, count, m, out, status);
     else if (codec == QSIM_CODEC_QSZR)
-        k_amplitudes<true><<<grid_for((count + 7) / 8, 152 * 64), 256, 0, s>>>(table, idx, count, m, out, status);
+        k_amplitudes<true><<<grid_for((count + 7) / 8, num_sms() * 64), 256, 0, s>>>(table, idx, count, m, out, status);
     else
-        k_amplitudes<false><<<grid_for((count + 7) / 8, 152 * 64), 256, 0, s>>>(table, idx, count, m, out, status);
+        k_amplitudes<false><<<grid_for((count + 7) / 8, num_sms() * 64), 256, 0, s>>>(table, idx, count, m, out, status);
     count_launch();
 }
 
@@ -513,7 +513,7 @@ void launch_init_store(uint64_t nblocks, uint64_t b0, uint64_t loc, int m, int e
                        const ArenaDev &dev, const ArenaDev &host, StageAccum *acc, int *status, cudaStream_t s,
                        bool rel) {
     const TeamShape ts = team_shape(m);
-    const unsigned grid = grid_for(nblocks, 152 * 8);
+    const unsigned grid = grid_for(nblocks, num_sms() * 8);
     if (rel)
         k_init_store<true><<<grid, ts.threads, ts.smem, s>>>(nblocks, b0, loc, m, e, table, dev, host, acc, status);
     else
@@ -530,14 +530,14 @@ void launch_reserve(uint32_t nblocks, const float *pred_log2, double margin, uin
 void launch_copy_out(const float2 *wv, uint32_t nblocks, int m, const EncTarget *tgt, const uint32_t *ids,
                      BlockSlot *table, StageAccum *acc, int *status, cudaStream_t s) {
     const uint64_t items = (uint64_t(nblocks) << m) / 2;
-    k_copy_blocks_out<<<grid_for((items + 255) / 256, 152 * 16), 256, 0, s>>>(wv, nblocks, m, tgt, ids, table, acc,
+    k_copy_blocks_out<<<grid_for((items + 255) / 256, num_sms() * 16), 256, 0, s>>>(wv, nblocks, m, tgt, ids, table, acc,
                                                                             status);
     count_launch();
 }
 
 void launch_copy_in(const BlockRef *in, uint32_t nblocks, int m, float2 *wv, int *status, cudaStream_t s) {
     const uint64_t items = (uint64_t(nblocks) << m) / 2;
-    k_copy_blocks_in<<<grid_for((items + 255) / 256, 152 * 16), 256, 0, s>>>(in, nblocks, m, wv, status);
+    k_copy_blocks_in<<<grid_for((items + 255) / 256, num_sms() * 16), 256, 0, s>>>(in, nblocks, m, wv, status);
     count_launch();
 }
 

@@ -84,4 +84,17 @@ bool allow_smem(int bytes, bool most = false) {
     return true;
 }
 
+// Host: SMs of the current device (asked once per device; callers on several threads store the same value).
+inline int num_sms() {
+    static std::atomic<int> sms[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    std::atomic<int> &n = sms[dev & 63];
+    int v = n.load();
+    if (v) return v;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
+    n.store(v);
+    return v;
+}
+
 }  // namespace qsim

@@ -1335,7 +1335,7 @@ static int init_store(RunCtx &R, StreamWork *w, int *status, cudaStream_t s) {
     k_copy_slot<<<1, 1, 0, s>>>(tab0 + b0, R.tmpl.p + 0);
     count_launch();
     // the zero template slot stays allocated in arena 0 until stage 0 has read its copies
-    k_replicate_zero<<<unsigned(std::min<uint64_t>(R.nblocks, 152 * 8)), 128, 0, s>>>(
+    k_replicate_zero<<<unsigned(std::min<uint64_t>(R.nblocks, num_sms() * 8)), 128, 0, s>>>(
         tab0, uint32_t(R.nblocks), uint32_t(b0), R.tmpl.p + 1, R.arena_dev(0), R.arena_host(0), status);
     count_launch();
     k_sum_table<<<64, 256, 0, s>>>(tab0, R.nblocks, R.accs.p + R.nst);
@@ -2626,7 +2626,7 @@ int qsim_shard_export(qsim_shard_run *R, const uint64_t *blocks, size_t count, v
     cudaStream_t s = R->S.main;
     CUDA_TRY(cudaMemcpyAsync(R->xbuf.p, lists.data(), 2 * count * 8, cudaMemcpyHostToDevice, s));
     BlockSlot *cur = R->S.RC.tables.p + (R->next & 1) * R->S.RC.nblocks;
-    k_export_streams<<<unsigned(std::min<size_t>(count, 152 * 8)), 256, 0, s>>>(cur, R->xbuf.p, R->xbuf.p + count,
+    k_export_streams<<<unsigned(std::min<size_t>(count, num_sms() * 8)), 256, 0, s>>>(cur, R->xbuf.p, R->xbuf.p + count,
                                                                                uint32_t(count), static_cast<uint8_t *>(d_packed));
     count_launch();
     CUDA_TRY(cudaStreamSynchronize(s));
@@ -2657,7 +2657,7 @@ int qsim_shard_import(qsim_shard_run *R, const uint64_t *blocks, const uint64_t 
     CUDA_TRY(cudaMemcpyAsync(R->xbuf.p, lists.data(), 3 * count * 8, cudaMemcpyHostToDevice, s));
     const int par = int(R->next & 1);
     BlockSlot *cur = R->S.RC.tables.p + par * nblocks;
-    k_import_streams<<<unsigned(std::min<size_t>(count, 152 * 8)), 256, 0, s>>>(
+    k_import_streams<<<unsigned(std::min<size_t>(count, num_sms() * 8)), 256, 0, s>>>(
         cur, R->xbuf.p, R->xbuf.p + count, R->xbuf.p + 2 * count, uint32_t(count),
         static_cast<const uint8_t *>(d_packed), R->S.RC.arena_dev(par), R->S.RC.arena_host(par), R->S.status);
     count_launch();
@@ -2974,7 +2974,7 @@ static int reduce_state(const qsim_state *st, const double *ref, double acc_out[
                 r = rbuf.p;
             }
         }
-        k_reduce_fid<<<unsigned(std::min<uint64_t>(152 * 4, (amps + 255) / 256)), 256, 0, s>>>(r, blocks.p, amps, acc.p);
+        k_reduce_fid<<<unsigned(std::min<uint64_t>(num_sms() * 4, (amps + 255) / 256)), 256, 0, s>>>(r, blocks.p, amps, acc.p);
         count_launch();
     }
     CUDA_TRY(cudaMemcpyAsync(acc_out, acc.p, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));

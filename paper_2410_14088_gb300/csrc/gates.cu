@@ -94,17 +94,6 @@ int pass_blocks_per_sm(size_t smem, int nt) {
     return nb;
 }
 
-int num_sms() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0, v = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        n = v > 0 ? v : 1;
-    }
-    return n;
-}
-
 template <int KMAX, int PREC, bool UM>
 void launch_pass_ku(dim3 grid, cudaStream_t s, float2 *wv, uint32_t W, const PassDev &P, const uint4 *blob,
                     const float2 *mats, const uint32_t *bfr, const uint64_t *gbase, uint32_t *ctr, int *status) {

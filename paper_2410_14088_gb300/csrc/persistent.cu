@@ -27,6 +27,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "codec.cuh"
 #include "codec_dev.cuh"
@@ -409,7 +410,8 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
 }
 
 template <int PREC, bool REL, bool UM>
-struct LaunchShape {  // of a device
+struct LaunchShape {  // of a device; mu guards the two values (runs on several threads)
+    std::mutex mu;
     int grid = 0;
     size_t attr_smem = 0;
     static LaunchShape &current() {
@@ -424,6 +426,7 @@ struct LaunchShape {  // of a device
 template <int PREC, bool REL, bool UM>
 int prepare_prec(size_t smem) {
     LaunchShape<PREC, REL, UM> &shape = LaunchShape<PREC, REL, UM>::current();
+    std::lock_guard<std::mutex> lk(shape.mu);
     if (shape.attr_smem < smem) {
         if (cudaFuncSetAttribute(k_stage_persistent<PREC, REL, UM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(smem)) != cudaSuccess)
@@ -435,9 +438,7 @@ int prepare_prec(size_t smem) {
         // resident CTAs per SM from the kernel's registers and shared memory and the SM's limits (65536 registers,
         // 2048 threads, 228 KB of shared memory with 1 KB reserved per CTA); the runtime's occupancy query was
         // seen to answer 1 where more CTAs were resident
-        int dev = 0, sms = 0, per_sm = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int per_sm = 1;
         cudaFuncAttributes fa{};
         if (cudaFuncGetAttributes(&fa, k_stage_persistent<PREC, REL, UM>) == cudaSuccess) {
             const int regs = ((fa.numRegs > 0 ? fa.numRegs : 255) + 7) & ~7;
@@ -450,16 +451,20 @@ int prepare_prec(size_t smem) {
             if (UM && per_sm > int(512u / gdev::umma_pass_tmem_cols(0))) per_sm = int(512u / gdev::umma_pass_tmem_cols(0));
             if (per_sm < 1) per_sm = 1;
         }
-        shape.grid = (sms > 0 ? sms : 1) * per_sm;
+        shape.grid = num_sms() * per_sm;
     }
     return QSIM_OK;
 }
 
 template <int PREC, bool REL, bool UM>
 int launch_stage_prec(const PLaunch &a, size_t smem, cudaStream_t s, int *grid_out) {
-    const LaunchShape<PREC, REL, UM> &shape = LaunchShape<PREC, REL, UM>::current();
-    if (shape.attr_smem < smem || !shape.grid) return QSIM_E_INVALID;
-    const int grid = shape.grid;
+    LaunchShape<PREC, REL, UM> &shape = LaunchShape<PREC, REL, UM>::current();
+    int grid;
+    {
+        std::lock_guard<std::mutex> lk(shape.mu);
+        if (shape.attr_smem < smem || !shape.grid) return QSIM_E_INVALID;
+        grid = shape.grid;
+    }
     k_stage_persistent<PREC, REL, UM><<<grid, kPT<UM>, smem, s>>>(a);
     if (grid_out) *grid_out = grid;
     count_launch();
