@@ -43,14 +43,17 @@ constexpr int kPassSmemMost = 220 * 1024;  // dynamic shared memory of a pass, 6
 // on load/store-only passes.)
 // UM: the pass's k = 5 dense ops run on tcgen05 (a separate instantiation, so that the warp-MMA kernels
 // keep their own register allocation)
-// Teams of 128 threads per CTA, a tile each, at most. Without tcgen05 four share one pass blob: a blob of many ops (56 KB
+// Teams of 128 threads per CTA, a tile each, at most. On CUDA cores four share one pass blob: a blob of many ops (56 KB
 // in the 28-op passes of a random circuit) beside every 32 KB tile left two tiles, 8 warps, per SM; four tiles beside one
 // blob are the 16 warps that 128 registers a thread allow (26-qubit random brick in FP32 with the groups of
-// apply_dense_groups: 21.8 -> 18.2 ms; four teams of 64 threads with twice the groups: 22.1). The split-BF16 warp MMAs take 168 registers (three teams),
-// width 6 takes 255, and the tcgen05 forms size TMEM and B by the tile.
+// apply_dense_groups: 21.8 -> 18.2 ms; four teams of 64 threads with twice the groups: 22.1). One team per CTA elsewhere:
+// width 6 takes 255 registers, the tcgen05 forms size TMEM and B by the tile, and the warp-level MMAs hold their matrix
+// in registers, where a team's own tile, barrier and counters cost spills (whole runs of 26 qubits, several teams and
+// one: random brick in TF32 at width 5 13.2 and 11.75 ms, at width 3 16.8 and 15.6, in split BF16 at width 5 21.7 and
+// 19.3, at width 4 19.6 and 17.5; QFT in split BF16 21.4 and 18.8).
 template <int KMAX, int PREC, bool UM>
 __host__ __device__ constexpr int pass_teams() {
-    return UM || KMAX >= 6 ? 1 : PREC == QSIM_PREC_BF16X3 && KMAX >= 4 ? 3 : 4;
+    return UM || KMAX >= 6 || PREC != QSIM_PREC_FP32 ? 1 : 4;
 }
 // CTAs of one team that fit an SM by registers
 template <int KMAX, int PREC, bool UM>

@@ -116,7 +116,7 @@ __device__ __forceinline__ void apply_dense_groups(float2 *tile, const float2 *U
 }
 
 // The groups of a 4096-amplitude tile divide evenly over the threads at every width up to 5; smaller tiles may leave
-// threads without one.
+// threads without one. MOST = 1: one group at a time, in kernels whose registers are needed elsewhere (the MMA forms).
 template <int NT, int K, int MOST = 4>
 __device__ __forceinline__ void apply_dense(float2 *tile, const float2 *U, const uint32_t *cb, const uint32_t *osw,
                                             uint32_t T) {
@@ -626,25 +626,25 @@ __device__ __forceinline__ void apply_dense_dispatch(uint32_t k, float2 *tile, c
     const bool tc_ok = TC && k >= min_k && k <= 5 && T == 12;  // 16+ index groups per warp for NT <= 256
     switch (k) {
         case 1: apply_dense_k1<NT>(tile, mat, cb, osw, T); break;
-        case 2: if constexpr (KMAX >= 2) apply_dense<NT, 2>(tile, mat, cb, osw, T); break;
+        case 2: if constexpr (KMAX >= 2) apply_dense<NT, 2, TC ? 1 : 4>(tile, mat, cb, osw, T); break;
         case 3:
             if constexpr (KMAX >= 3) {
                 if constexpr (PREC == QSIM_PREC_TF32) {
                     if (tc_ok) { apply_dense_mma<NT, 3, PREC>(tile, bfr, cb, osw, T); break; }
                 }
-                apply_dense<NT, 3>(tile, mat, cb, osw, T);
+                apply_dense<NT, 3, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
         case 4:
             if constexpr (KMAX >= 4) {
                 if (tc_ok) apply_dense_mma<NT, 4, PREC>(tile, bfr, cb, osw, T);
-                else apply_dense<NT, 4>(tile, mat, cb, osw, T);
+                else apply_dense<NT, 4, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
         case 5:
             if constexpr (KMAX >= 5) {
                 if (tc_ok) apply_dense_mma<NT, 5, PREC>(tile, bfr, cb, osw, T);
-                else apply_dense<NT, 5>(tile, mat, cb, osw, T);
+                else apply_dense<NT, 5, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
         default:
@@ -787,8 +787,9 @@ __device__ __forceinline__ void blob_load(const uint4 *__restrict__ gblob, uint3
 // The pass's ops on a staged tile; blob: the staged pass blob; mat: the matrix
 // area for dense ops whose matrix is not in the blob. Starts with a team
 // barrier, so the tile's and blob's loads need only have completed per thread.
-// SMALL: a tcgen05 launch (UM) that may hold passes of smaller tiles too.
-template <int NT, int KMAX, int PREC, bool UM = false, bool SMALL = false>
+// SMALL: a tcgen05 launch (UM) that may hold passes of smaller tiles too. ONE: the CTA has one team, whose barrier is
+// the CTA's.
+template <int NT, int KMAX, int PREC, bool UM = false, bool SMALL = false, bool ONE = UM>
 __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2 *mat,
                                          const float2 *__restrict__ mats, const uint32_t *__restrict__ bfr,
                                          uint64_t base, uint64_t gb, PassSmem &S, uint4 *bbuf, int *status,
@@ -797,7 +798,7 @@ __device__ __forceinline__ bool tile_ops(float2 *tile, const uint4 *blob, float2
     // phase: parity of the next MMA-completion phase (tcgen05 dense ops); false after a wait ran out
     const int tid = team_tid<NT>();
     auto sync = [&]() {
-        if constexpr (UM) __syncthreads();  // one team per CTA
+        if constexpr (ONE) __syncthreads();
         else team_sync<NT>();
     };
     const uint32_t T = S.p.T;
@@ -1203,7 +1204,11 @@ __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, 
     // a team's next tile, in a slot by iteration parity: its thread 0 writes slot (it + 1) & 1 while a slower warp may
     // still be reading slot it & 1 after the end-of-iteration barrier; that slot is next written two barriers later
     __shared__ uint32_t s_next[TEAMS][2];
-    const uint32_t team = threadIdx.x / uint32_t(NT), tid = team_tid<NT>();
+    const uint32_t team = TEAMS > 1 ? threadIdx.x / uint32_t(NT) : 0u, tid = team_tid<NT>();
+    auto sync = [&]() {
+        if constexpr (TEAMS > 1) team_sync<NT>();
+        else __syncthreads();
+    };
     const uint32_t teams = TEAMS > 1 ? blockDim.x / uint32_t(NT) : 1u;
     pass_setup<NT>(pd, S);
     const uint32_t T = S.p.T;
@@ -1226,14 +1231,18 @@ __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, 
     float2 *mat = reinterpret_cast<float2 *>(blob + S.p.blob_words) + team * S.p.mat_elems;
     // Every tile has a team of its own in the first round: no counter is needed. A launch of 16 tiles is one chain of
     // latencies, which loses the atomics, the fence and one load's wait by this and the next comment's overlap (with the
-    // arena reset folded into the decoder, 48 stages of a 16-qubit run 1.405 -> 1.312 ms).
-    const bool single = ntiles <= uint64_t(gridDim.x) * teams;
+    // arena reset folded into the decoder, 48 stages of a 16-qubit run 1.405 -> 1.312 ms). The warp-level MMA forms do
+    // without both, for their registers: the second copy of the load and the flag are live across the MMAs (26-qubit
+    // random brick at width 5, with and without: 12.45 and 11.75 ms in TF32, 20.3 and 19.3 in split BF16; a 16-qubit
+    // run takes 1.32 ms either way).
+    constexpr bool AHEAD = PREC == QSIM_PREC_FP32 || UM;
+    const bool single = AHEAD && ntiles <= uint64_t(gridDim.x) * teams;
     blob_load(gblob + S.p.blob_off, S.p.blob_words, blob);
     const uint64_t tmask = (1ull << S.p.nout) - 1;
     // the first tiles go to the CTAs' first teams: a launch of few tiles spreads over the SMs. The first one's loads
     // travel with the blob's
     uint64_t t = uint64_t(team) * gridDim.x + blockIdx.x;
-    if (t < ntiles) tile_load<NT, false>(wv + ((t >> S.p.nout) << W), tile_base(S, t & tmask), S, tile);
+    if (AHEAD && t < ntiles) tile_load<NT, false>(wv + ((t >> S.p.nout) << W), tile_base(S, t & tmask), S, tile);
     cp_async_wait_all();
     __syncthreads();
     // a single tcgen05 op: its B operand stays in bbuf for every tile of this CTA
@@ -1264,13 +1273,14 @@ __device__ __forceinline__ void pass_tiles(float2 *__restrict__ wv, uint32_t W, 
         float2 *g = wv + (grp << W);
         const uint64_t gb = gbase ? gbase[grp] : 0ull;
         const uint64_t base = tile_base(S, cta);
-        if (it) tile_load<NT, false>(g, base, S, tile);
+        if (!AHEAD || it) tile_load<NT, false>(g, base, S, tile);
         cp_async_wait_all();
-        ok = tile_ops<NT, KMAX, PREC, UM>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
-        team_sync<NT>();
+        ok = tile_ops<NT, KMAX, PREC, UM, false, TEAMS == 1>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase,
+                                                             b_res);
+        sync();
         tile_store<NT>(g, base, S, tile);
         if (single) break;
-        team_sync<NT>();  // the next tile's loads overwrite the tile; s_next[team][it & 1] is visible
+        sync();  // the next tile's loads overwrite the tile; s_next[team][it & 1] is visible
         if (!ok) break;   // uniform: the MMA wait ran out (status set)
         t = s_next[team][it & 1u];
     }
