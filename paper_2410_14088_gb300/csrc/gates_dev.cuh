@@ -616,6 +616,22 @@ __device__ __forceinline__ bool apply_dense_umma3(float2 *tile, uint32_t bsm, co
     return true;
 }
 
+// apply_dense_mma as a called function where it is a kernel's largest part by registers: split BF16 in the persistent
+// kernel (256 threads of 128 registers). Called, it spills nothing; inlined among that kernel's other phases its loops do
+// (26-qubit random brick at width 5: 23.0 ms inlined, 22.6 called). TF32, which needs fewer, is faster inlined (16.1
+// and 19.8 ms), and so is the stream engine's kernel, which holds nothing else.
+template <int NT, int K, int PREC>
+__device__ __noinline__ void apply_dense_mma_call(float2 *tile, const uint32_t *bfr, const uint32_t *cb, const uint32_t *osw,
+                                                  uint32_t T) {
+    apply_dense_mma<NT, K, PREC>(tile, bfr, cb, osw, T);
+}
+template <int NT, int K, int PREC>
+__device__ __forceinline__ void apply_dense_mma_any(float2 *tile, const uint32_t *bfr, const uint32_t *cb, const uint32_t *osw,
+                                                    uint32_t T) {
+    if constexpr (PREC == QSIM_PREC_BF16X3 && NT == 256) apply_dense_mma_call<NT, K, PREC>(tile, bfr, cb, osw, T);
+    else apply_dense_mma<NT, K, PREC>(tile, bfr, cb, osw, T);
+}
+
 // Dense op of width k (<= KMAX) on the shared-memory tile; the tensor-core
 // form needs 4096-amplitude tiles and at least 16 index groups per warp.
 template <int NT, int KMAX, int PREC>
@@ -630,20 +646,20 @@ __device__ __forceinline__ void apply_dense_dispatch(uint32_t k, float2 *tile, c
         case 3:
             if constexpr (KMAX >= 3) {
                 if constexpr (PREC == QSIM_PREC_TF32) {
-                    if (tc_ok) { apply_dense_mma<NT, 3, PREC>(tile, bfr, cb, osw, T); break; }
+                    if (tc_ok) { apply_dense_mma_any<NT, 3, PREC>(tile, bfr, cb, osw, T); break; }
                 }
                 apply_dense<NT, 3, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
         case 4:
             if constexpr (KMAX >= 4) {
-                if (tc_ok) apply_dense_mma<NT, 4, PREC>(tile, bfr, cb, osw, T);
+                if (tc_ok) apply_dense_mma_any<NT, 4, PREC>(tile, bfr, cb, osw, T);
                 else apply_dense<NT, 4, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
         case 5:
             if constexpr (KMAX >= 5) {
-                if (tc_ok) apply_dense_mma<NT, 5, PREC>(tile, bfr, cb, osw, T);
+                if (tc_ok) apply_dense_mma_any<NT, 5, PREC>(tile, bfr, cb, osw, T);
                 else apply_dense<NT, 5, TC ? 1 : 4>(tile, mat, cb, osw, T);
             }
             break;
@@ -1166,7 +1182,7 @@ __device__ __forceinline__ bool pass_tile(float2 *__restrict__ g, const PassDev 
     cp_async_wait_all();
     uint32_t phase = phase_io ? *phase_io : 0u;
     const bool ok =
-        tile_ops<NT, KMAX, PREC, UM, UM>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
+        tile_ops<NT, KMAX, PREC, UM, UM, true>(tile, blob, mat, mats, bfr, base, gb, S, bbuf, status, phase, b_res);
     __syncthreads();
     tile_store<NT>(g, base, S, tile);
     if (phase_io) {

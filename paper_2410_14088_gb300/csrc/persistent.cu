@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
         s_seg = ~0u;
+        s_step.begin = s_step.count = 0;
         s_pcache[0] = ~0u;
         s_pcache[1] = 0;
     }
@@ -96,24 +97,30 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     __syncthreads();
     if constexpr (UM) umma::fence_after_sync();
 
-    // thread 0: the next item, claimed one item ahead so that the claim's latency hides under the current item
-    // (every dependency points to an earlier item, and the grid is one wave of resident CTAs, so the smallest
-    // unfinished item is always some CTA's current item and the queue keeps moving)
-    uint32_t nx_item = 0;
-    // thread 0: the (launch group, phase) whose dependencies this CTA last saw met; later items of the same
-    // phase of the same group skip the wait (the counters only grow within a launch)
-    uint64_t dep_key = ~0ull;
-    if (tid == 0) nx_item = atomicAdd(L.ctr, 1u);
-    // thread 0: a done counter of a per-item phase whose increments this CTA holds back, and their number; they are
-    // added (after a fence) when the CTA completes an item of another phase, before it waits on any dependency and
-    // when it leaves, so a CTA that waits never holds counts another CTA waits for
-    uint32_t *pend_done = nullptr;
-    uint32_t pend_cnt = 0;
+    // Thread 0's words (cur: warp 0's), in shared memory: the passes are short of registers, and what is held through
+    // an item in each thread's is spilled inside their loops.
+    struct Own {
+        // the (launch group, phase) whose dependencies this CTA last saw met; later items of the same phase of the
+        // same group skip the wait (the counters only grow within a launch)
+        uint64_t dep_key;
+        // a done counter of a per-item phase whose increments this CTA holds back, and their number; they are added
+        // (after a fence) when the CTA completes an item of another phase, before it waits on any dependency and when
+        // it leaves, so a CTA that waits never holds counts another CTA waits for
+        uint32_t *pend_done;
+        uint32_t pend_cnt;
+        // the next item, claimed one item ahead so that the claim's latency hides under the current item (every
+        // dependency points to an earlier item, and the grid is one wave of resident CTAs, so the smallest unfinished
+        // item is always some CTA's current item and the queue keeps moving)
+        uint32_t nx_item;
+        uint32_t cur;  // the step in s_step
+    };
+    __shared__ Own own;
+    if (tid == 0) own = Own{~0ull, nullptr, 0u, atomicAdd(L.ctr, 1u), 0u};
     auto flush = [&]() {
-        if (pend_cnt) {
+        if (own.pend_cnt) {
             __threadfence();
-            atomicAdd(pend_done, pend_cnt);
-            pend_cnt = 0;
+            atomicAdd(own.pend_done, own.pend_cnt);
+            own.pend_cnt = 0;
         }
     };
     // thread 0: wait for the item's dependencies (the group's previous phase; for its first phase the slot's
@@ -122,7 +129,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
     auto deps = [&]() -> int {
         const uint32_t q = S.group_begin + s_step.grp;
         const uint64_t key = uint64_t(q) * kMaxPhases + s_step.phase;
-        if (key == dep_key) return ld_relaxed_u32(reinterpret_cast<const uint32_t *>(L.status)) != 0;
+        if (key == own.dep_key) return ld_relaxed_u32(reinterpret_cast<const uint32_t *>(L.status)) != 0;
         flush();
         const uint32_t *flag = nullptr, *flag2 = nullptr;
         uint32_t need = 0;
@@ -150,16 +157,18 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
                 __nanosleep(256);
             }
         }
-        if (met) dep_key = key;
+        if (met) own.dep_key = key;
         // after any device error the remaining items only keep the schedule going
         return (!met || ld_relaxed_u32(reinterpret_cast<const uint32_t *>(L.status)) != 0) ? 1 : 0;
     };
 
-    uint32_t cur = 0;  // warp 0: the step of the CTA's last item (items of a CTA only move forward)
     while (true) {
         if (warp == 0) {
-            const uint32_t it = __shfl_sync(kFull, nx_item, 0);
-            if (it < L.total_items) {
+            __syncwarp();  // thread 0 has written own and read s_step
+            const uint32_t it = own.nx_item;
+            // a CTA's items only move forward, mostly within one step: then s_step holds it
+            if (it < L.total_items && it - s_step.begin >= s_step.count) {
+                uint32_t cur = own.cur;
                 for (;;) {  // the last step that begins at or before the item, 32 steps at a look
                     const uint32_t k = cur + uint32_t(tid);
                     const uint32_t begin = k < L.nsteps ? __ldg(&L.steps[k].begin) : 0xffffffffu;
@@ -167,6 +176,8 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
                     cur += ahead;
                     if (ahead < 31) break;
                 }
+                __syncwarp();
+                if (tid == 0) own.cur = cur;
                 if (tid < int(sizeof(PStep) / 4))
                     reinterpret_cast<uint32_t *>(&s_step)[tid] = __ldg(reinterpret_cast<const uint32_t *>(L.steps + cur) + tid);
             }
@@ -174,7 +185,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
             if (tid == 0) {
                 s_item = it;
                 if (it < L.total_items) {
-                    nx_item = atomicAdd(L.ctr, 1u);
+                    own.nx_item = atomicAdd(L.ctr, 1u);
                     // the current segment's descriptor is in S: check the dependencies before the barrier
                     if (s_step.seg == s_seg) s_abort = deps();
                 }
@@ -202,10 +213,13 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         const FrameGeom g = geom(int(S.m));
         const uint32_t gframes = S.G * g.nframes;
         const uint32_t grp = s_step.grp, q = S.group_begin + grp;  // the unit's number in the stage and the launch
-        const uint32_t p = s_step.phase, type = s_step.type, count = s_step.count, i = item - s_step.begin;
+        const uint32_t type = s_step.type, i = item - s_step.begin;
         const bool abort_item = s_abort != 0;
-        // the item's SV group in the unit and its place among the group's items of this phase
-        const uint32_t gi = i / s_step.per, ii = i % s_step.per;
+        // the item's SV group in the unit and its place among the group's items of this phase. Every divisor here is a
+        // power of two: shifts, except in the tcgen05 forms, where they cost registers (26-qubit random brick in one
+        // group: 26.1 -> 25.5 ms in FP32, 16.7 -> 16.3 in TF32 warp MMAs; tcgen05 1 to 2 % slower with them)
+        const uint32_t gi = UM ? i / s_step.per : S.gpu == 1u ? 0u : i / s_step.per;
+        const uint32_t ii = UM ? i % s_step.per : i - gi * s_step.per;
         const uint64_t sg = uint64_t(grp) * S.gpu + gi;  // SV group of the stage
         float2 *wv = L.wv + L.g_wv[q] + (uint64_t(gi) << S.W);
         const uint32_t *ids = S.ids + sg * S.G;
@@ -214,11 +228,13 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         const uint32_t sf0 = L.g_frame[q] + gi * gframes;  // the group's first frame in the frame records
         const bool by_arrival = type == PH_ENCODE || type == PH_COPY;
         // frame-parallel items: a team per frame, each with its own tile in dsm
-        const uint32_t tn = cdev::team_threads(g.C), team = uint32_t(tid) / tn;
-        const cdev::Team tm{uint32_t(tid) % tn, tn, 1u + team};
+        const uint32_t tl = 31u - uint32_t(__clz(cdev::team_threads(g.C)));
+        const uint32_t tn = UM ? cdev::team_threads(g.C) : 1u << tl, team = UM ? uint32_t(tid) / tn : uint32_t(tid) >> tl;
+        const cdev::Team tm{UM ? uint32_t(tid) % tn : uint32_t(tid) & (tn - 1u), tn, 1u + team};
         uint8_t *tile = reinterpret_cast<uint8_t *>(dsm) + team * cdev::team_tile_bytes(g.C);
-        const uint32_t fi = ii * (PT / tn) + team;
-        const uint32_t jj = fi / g.nframes, f = fi % g.nframes;
+        const uint32_t fi = ii * (UM ? PT / tn : PT >> tl) + team;
+        const uint32_t jj = UM ? fi / g.nframes : fi >> (S.m - uint32_t(g.fl));
+        const uint32_t f = UM ? fi % g.nframes : fi & (g.nframes - 1u);
         const uint64_t a0 = (uint64_t(jj) << S.m) + uint64_t(f) * g.F;
         if (type != PH_PASS && tid == 0) s_pcache[0] = ~0u;  // dsm is overwritten: no pass stays staged
         if (abort_item) {
@@ -329,20 +345,24 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         }
         // ---- completion ----
         __syncthreads();
-        uint32_t *done = L.done + uint64_t(q) * kMaxPhases + p;
+        // The step's numbers are read from s_step again. Warp 0 overwrites it at the loop's top: after thread 0's reads
+        // here, and after one more barrier where every thread reads.
         if (!by_arrival) {
             if (tid == 0) {
-                if (done != pend_done) {
+                uint32_t *done = L.done + uint64_t(S.group_begin + s_step.grp) * kMaxPhases + s_step.phase;
+                if (done != own.pend_done) {
                     flush();
-                    pend_done = done;
+                    own.pend_done = done;
                 }
-                ++pend_cnt;
+                ++own.pend_cnt;
             }
             continue;
         }
+        const uint32_t p = s_step.phase, count = s_step.count, dq = S.group_begin + s_step.grp;
+        uint32_t *done = L.done + uint64_t(dq) * kMaxPhases + p;
         if (tid == 0) {
             __threadfence();
-            s_flag = atomicAdd(L.arrive + uint64_t(q) * kMaxPhases + p, 1u) == count - 1;
+            s_flag = atomicAdd(L.arrive + uint64_t(dq) * kMaxPhases + p, 1u) == count - 1;
         }
         __syncthreads();
         if (!s_flag) continue;
@@ -350,7 +370,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
         if (!abort_item && type == PH_ENCODE && g.nframes > 1) {
             // the unit's frame lengths are complete: frame offsets, the blocks' slots (with learned sizing every
             // predicted slot its block fits is kept) and the stage's error sums, a team of 128 per block
-            const uint32_t f0 = L.g_frame[q];
+            const uint32_t f0 = L.g_frame[dq];
             const uint64_t b0 = uint64_t(grp) * S.gpu * S.G;
             for (uint32_t k = team; k < S.gpu * S.G; k += PT / 128) {
                 double a, b;
@@ -375,7 +395,7 @@ __global__ void __launch_bounds__(kPT<UM>, 512 / kPT<UM>) k_stage_persistent(PLa
             atomicExch(done, count);
             if (p == S.nphases - 1) {
                 // the group is finished: its slot may be reused; the stage may be complete
-                atomicExch(L.done + uint64_t(q) * kMaxPhases + kMaxPhases - 1, 1u);
+                atomicExch(L.done + uint64_t(dq) * kMaxPhases + kMaxPhases - 1, 1u);
                 if (atomicAdd(S.fin_count, 1u) == S.ngroups - 1) {
                     if (S.reset_bumps) {
                         // every group of the stage has read its input arena: the next stage writes there
