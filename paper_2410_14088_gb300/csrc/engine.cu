@@ -1868,8 +1868,12 @@ struct StreamsRun {
     int *status = nullptr;
     uint64_t batch_amps = 0;
     uint64_t groups_run = 0;  // SV groups processed (all stages)
+    bool drained = true;      // nothing of the run is in flight
     ~StreamsRun() {
+        // a run that is left early: its buffers go back to the cache below, for runs on any stream
+        if (!drained) cudaStreamSynchronize(main);
         for (auto &x : sw) {
+            if (x.s && !drained) cudaStreamSynchronize(x.s);
             if (x.s) cudaStreamDestroy(x.s);
             if (x.done) cudaEventDestroy(x.done);
         }
@@ -1925,6 +1929,7 @@ static int streams_begin(StreamsRun &S, const qsim_plan *p, cudaStream_t main) {
     const uint64_t work_bytes = nstreams * batch_amps * 8 * 2;
     const uint64_t dev_budget = free_b > work_bytes ? uint64_t(0.85 * double(free_b - work_bytes)) : 0;
     // the pinned-host level holds at most 30 % of the host's memory per stage parity
+    S.drained = false;
     if ((rc = alloc_run(RC, dev_budget, uint64_t(0.3 * double(host_phys_bytes())), main))) return rc;
 
     // ---- per-stream work buffers ----
@@ -2102,6 +2107,7 @@ static int streams_finish(StreamsRun &S, qsim_state **out, qsim_stats *stats) {
     std::vector<const StageAccum *> accs;
     int rc = collect_run({&S.RC}, S.status, S.main, host, accs, "qsim_run");
     if (rc) return rc;
+    S.drained = true;
     float ms = 0;
     CUDA_TRY(cudaEventElapsedTime(&ms, S.ev_start, S.ev_stop));
     return finish_run(S.RC, S.dev, ms, accs[0], &S.prof, stats, out);
@@ -2207,9 +2213,14 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
     prof.on = (g_profile.load() != 0 || launch_stat) && !plans[0]->cfg.graph;
     CUDA_TRY(cudaEventRecord(ev_start, main));
     for (size_t c = 0; c < count && !rc; ++c) rc = init_store(*rs[c], nullptr, status, main);
-    if (rc) return rc;
-    for (const std::vector<RunCtx *> &set : launch_sets)
-        if ((rc = run_persistent(set, true, plans[0]->cfg.graph != 0, main, status, prof, dctx, slot_budget))) return rc;
+    for (size_t k = 0; k < launch_sets.size() && !rc; ++k)
+        rc = run_persistent(launch_sets[k], true, plans[0]->cfg.graph != 0, main, status, prof, dctx, slot_budget);
+    if (rc) {  // the circuits' arenas go back to the cache, for runs on any stream
+        cudaStreamSynchronize(main);
+        cudaEventDestroy(ev_start);
+        cudaEventDestroy(ev_stop);
+        return rc;
+    }
     CUDA_TRY(cudaEventRecord(ev_stop, main));
     HostBuf<StageAccum> host;
     std::vector<const StageAccum *> accs;

@@ -32,3 +32,19 @@ def test_batch_of_both_tensor_core_forms(prec, graph):
     assert graph or launch["launches"] == 1
     for p, st in zip([plans[1], plans[4], plans[5], plans[6]], states):
         assert streams_of(st) == streams_of(qsim.run(p))
+
+
+def test_run_after_a_refused_batch():
+    """A batch is refused after its initial stores are launched; what it allocated may be another run's the moment the
+    call returns, on whichever stream: the stores are waited for first."""
+    torch = pytest.importorskip("torch")
+    c = inputs.random_brick(20, 2, 9)
+    kw = dict(m=6, inner=2, k=2, eps=1e-3)
+    plan, other = qsim.plan_stages(c, **kw), torch.cuda.Stream()
+    wide = qsim.plan_stages(inputs.random_brick(20, 2, 1), m=6, inner=2, k=6, eps=1e-3)
+    want = qsim.run(plan).decompress()
+    for _ in range(5):
+        with pytest.raises(qsim.QsimError) as ei:
+            qsim.run_batch([plan, plan, wide])
+        assert ei.value.code == qsim.E_INVALID
+        assert torch.equal(qsim.run(plan, stream=other).decompress(), want)
