@@ -1749,6 +1749,14 @@ static int collect_run(const std::vector<RunCtx *> &rs, int *status, cudaStream_
     return set_error(code, "%s: %s", what, status_text(code));
 }
 
+// Bytes that stage i of a finished run moves in the persistent kernel: its input streams and the decoded amplitudes, the
+// passes, the amplitudes read by the encoder, and the output streams (staged and copied where a block has several frames).
+static double stage_bytes(const RunCtx &R, const qsim_state *S, size_t i) {
+    const double in_store = double(i == 0 ? S->stage_acc[R.nst].store_bytes : S->stage_acc[i - 1].store_bytes);
+    return in_store + std::ldexp(16.0, int(R.n)) * (1 + R.pd->stages[i].npasses) +
+           double(S->stage_acc[i].store_bytes) * (R.nframes > 1 ? 3 : 1);
+}
+
 // The run's state handle and statistics (after the stream has been synchronised).
 static int finish_run(RunCtx &R, int dev, double ms, const StageAccum *accs, Profiler *prof, qsim_stats *stats,
                       qsim_state **out) {
@@ -1790,7 +1798,7 @@ static int finish_run(RunCtx &R, int dev, double ms, const StageAccum *accs, Pro
             const StageDev &sd = pd->stages[i];
             bytes[raw ? P_COPY_IN : P_DECODE] += in_store + 8 * amps;
             bytes[P_PASS] += 16 * amps * sd.npasses;
-            bytes[P_STAGE] += in_store + 16 * amps + 3 * out_store + 16 * amps * sd.npasses;
+            bytes[P_STAGE] += stage_bytes(R, S, i);
             for (const Op &op : p->stages[i].ops) {
                 const double fl = (op.type == OP_DENSE ? 8.0 * double(1u << op.k)
                                    : op.type == OP_DIAG ? 6.0 : op.type == OP_CSEP ? 12.0 : 0.0) * amps;
@@ -2243,10 +2251,7 @@ static int run_batch(const qsim_plan *const *plans, size_t count, cudaStream_t m
         const qsim_state *S = out[c];
         const double amps = std::ldexp(1.0, int(R.n));
         for (size_t i = 0; i < R.nst; ++i) {
-            const double in_store = double(i == 0 ? S->stage_acc[R.nst].store_bytes : S->stage_acc[i - 1].store_bytes);
-            const double out_store = double(S->stage_acc[i].store_bytes);
-            alg_bytes += in_store + out_store + 8 * amps * (2 + (R.predict ? 0 : 1)) +
-                         16 * amps * R.pd->stages[i].npasses;
+            alg_bytes += stage_bytes(R, S, i);
             for (const Op &op : R.p->stages[i].ops)
                 alg_flops += (op.type == OP_DENSE ? 8.0 * double(1u << op.k)
                               : op.type == OP_DIAG ? 6.0 : op.type == OP_CSEP ? 12.0 : 0.0) * amps;

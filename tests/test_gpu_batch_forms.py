@@ -48,3 +48,16 @@ def test_run_after_a_refused_batch():
             qsim.run_batch([plan, plan, wide])
         assert ei.value.code == qsim.E_INVALID
         assert torch.equal(qsim.run(plan, stream=other).decompress(), want)
+
+
+def test_batch_bytes_are_its_circuits():
+    plans = [qsim.plan_stages(c, m=m, inner=2, k=4, eps=1e-3, mode=qsim.MODE_PERSISTENT)
+             for c, m in ((inputs.random_brick(15, 4, 1), 13), (inputs.qft_rz_cx(12, 1, 2), 9))]
+    _, launch = qsim.run_batch(plans)
+    qsim.profile_enable(True)
+    try:
+        single = [qsim.run(p).kernel_stats()[launch["name"]] for p in plans]
+    finally:
+        qsim.profile_enable(False)
+    assert launch["alg_bytes"] == sum(s["alg_bytes"] for s in single)
+    assert launch["alg_flops"] == sum(s["alg_flops"] for s in single)
