@@ -114,9 +114,10 @@ __global__ void k_log_targets(const EncResult *__restrict__ res, uint32_t nblock
 // takes eight of them through the forward and backward pass with its own copy of the weights in shared memory, then every
 // CTA collects what its eighth of the weight rows needs of all 64 through distributed shared memory, sums the gradient
 // of those rows over the samples, applies Adam to them, whose moments it keeps in registers, and writes the new weights
-// into all eight copies. Two cluster barriers per chunk, no launch and no global round trip. Every sum runs in the order
-// of a loop over its terms (inputs, units or samples): a training run amplifies the rounding of its first steps, so a sum
-// split over threads or CTAs ends in other weights. A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases:
+// into all eight copies. Two cluster barriers per chunk, no launch and no global round trip. Every sum that the weights
+// depend on runs in the order of a loop over its terms: inputs, units, and samples within a chunk, whose sums are added
+// in the chunks' order. A training run amplifies the rounding of its first steps, so a sum split over threads or CTAs
+// ends in other weights. (The reported loss is no such sum: k_mlp_loss adds its CTAs' shares in any order, in FP64.) A step of 64 samples is 1.3 MFLOP in a chain of six dependent phases:
 // latency and shared-memory reads bound it. 800 steps of 64 samples: 72 ms with two launches and one CTA per step,
 // 8.3 ms now (the call).
 // ---------------------------------------------------------------------------
