@@ -31,8 +31,9 @@ namespace {
 using namespace cdev;
 
 // One frame per team of max(32, C) threads, which is the CTA. Blocks are read from table[ids[j]] (ids null: block
-// b0 + j). NP: the most leading phase ops the kernel applies (pre.count <= NP). Five CTAs of 128 threads per SM: 102
-// registers hold a chunk pair's 64 bit-plane words (the wide path) without spills, and 35 KB of tile each fit six. A launch
+// b0 + j). NP: the most leading phase ops the kernel applies (pre.count <= NP). Five CTAs of 128 threads per SM (35 KB of tile
+// each would fit six) leave 102 registers, of which a chunk pair's 64 bit-plane words (the wide path) and the rest take
+// 91 to 96; only the relative codec's form with more than two leading ops spills (68 bytes a thread). A launch
 // of few frames is one chain of latencies, so its CTAs are as many as its frames: one 1024-amplitude frame per CTA took
 // 6 us where a warp per frame took 22.
 template <int NP, bool REL>
@@ -423,7 +424,8 @@ static void decode_table(const BlockSlot *table, const uint32_t *ids, uint64_t b
                          uint32_t *hist, int *status, const PreOps &pre, cudaStream_t s) {
     const uint64_t items = uint64_t(nblocks) * qsz_nframes(m);
     const TeamShape ts = team_shape(m);
-    // with leading phase ops each CTA copies their descriptors once and takes several frames
+    // with leading phase ops each CTA copies their tables (up to 18 KB) once and takes several frames: three CTAs for
+    // each of the five resident ones, so that the last ones to finish are short
     const unsigned grid = grid_for(items, pre.count ? num_sms() * 5 * 3 : kMaxGrid);
     const size_t smem = ts.smem + pre.count * cdev::kPreTabBytes;
     if (pre.count > 2)  // kMaxPreOps tables beside the largest tile: 52.5 KB

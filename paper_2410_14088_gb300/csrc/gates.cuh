@@ -83,6 +83,7 @@ constexpr uint32_t kPassBlobMax = 40960;    // bytes of one pass blob (shared me
 //       word offset of its B operand in the plan's B array
 //   runs: kPolyHeadWords words as OP_POLY's, in the index bits of the dense op before it (else after it): bits 0..6 the
 //       group number's, 7..11 the matrix bits; its term records; its table T (words 205 and 206 of the head)
+// The head has room for 24 steps and four runs; a pass with more stays staged (its tables would not fit either).
 constexpr uint32_t kRegHead = 64, kRegDense = 136, kRegMaxSteps = 24, kRegMaxPoly = 4, kRegPoly = 0x10000u;
 constexpr uint32_t kRegRow = 33;  // words per row of a run's table T: rows read by one warp fall on different banks
 constexpr uint32_t kRegIn = 1u, kRegOut = 2u;
@@ -122,7 +123,8 @@ void launch_pass(float2 *wv, uint32_t W, uint32_t ngroups, const PassDev *pass_h
                  const float2 *mats_dev, const uint32_t *bfr_dev, const uint64_t *gbase_dev, int prec,
                  cudaStream_t s, uint32_t *ctr, int *status);
 
-// whether a pass with register tables (reg_words) gets at least two CTAs' worth of threads per SM in that form
+// whether a pass with register tables (reg_words) keeps enough tiles in flight per SM in that form: two CTAs of two tiles,
+// or three of one (75 KB each)
 bool reg_pass_fits(const PassDev &P, int prec);
 
 // dynamic shared memory of one tile pass (tile, B operand and alignment when on tcgen05, blob, matrices)

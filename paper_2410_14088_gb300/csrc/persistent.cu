@@ -16,7 +16,7 @@
 // are merged by the fraction of their steps, so that while one circuit's phase
 // drains the CTAs work on the others'. (With every circuit's stage in the queue as a
 // whole, the time of a batch was the sum of its circuits' alone: 16 circuits of 17 to 22
-// qubits took 14.4 ms, 6.6 ms as lanes; 48 ms with a warp per frame and a group per
+// qubits took 14.4 ms, 6.4 ms as lanes; 48 ms with a warp per frame and a group per
 // unit.) Every dependency
 // points to an earlier item of the same lane, which was taken by a CTA that is
 // already running: the schedule cannot deadlock even when not every CTA is resident.
@@ -491,7 +491,7 @@ int launch_stage_prec(const PLaunch &a, size_t smem, cudaStream_t s, int *grid_o
     return QSIM_OK;
 }
 
-// tcgen05 (um) only for TF32: the split-BF16 form keeps 128-thread CTAs, which this kernel does not have
+// um: the tcgen05 forms, TF32 and split BF16, with 128-thread CTAs; the others have 256 threads
 template <bool REL>
 int prepare_codec(int prec, size_t smem, bool um) {
     if (prec == QSIM_PREC_TF32)

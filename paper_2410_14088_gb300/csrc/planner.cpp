@@ -724,7 +724,10 @@ void layout_passes(Stage &st, uint32_t tile_bits, bool fold_leading_diag) {
 
 // Modelled time of a stage's tile passes, to choose between two layouts of the same stage (relative units:
 // one pass over 2^28 amplitudes, in ms on GB300). A pass costs its load and store plus its ops; the
-// coefficients are the k_pass times the ncu launch list gave for 28-qubit QAOA passes of every composition
+// coefficients are the times of the staged form (k_pass, one tile per CTA) that the ncu launch list gave for
+// 28-qubit QAOA passes of every composition, and were not refitted since tcgen05 passes of width-5 ops and
+// phase polynomials run in the register form (gates_reg.cuh: one op 0.75, two 0.90, two and a run 1.31) and
+// CUDA-core passes share their op data between four tiles
 // (TF32 dense ops of width 3 to 5 on tcgen05; the warp-level MMA form runs these passes at about the same rate):
 // with 4 resident CTAs per SM 0.61 per pass and 0.213 per tensor-core dense op; with 3 (a pass whose op data
 // pushes a CTA's shared memory past a quarter of the SM's) 0.72 and 0.315 (scaled by the ratio measured before
