@@ -48,6 +48,6 @@ def test_decompressing_an_uncompressed_state_takes_little_scratch():
     qsim.release_cached_memory()
     free, _ = torch.cuda.mem_get_info()
     st.decompress(out=out)
-    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20  # 2^16 references of 16 bytes, in the driver's units of 2 MB
+    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20  # 2^16 references of 16 bytes, in cudaMalloc's units of 2 MB
     idx = np.array([0, 31, 32, (1 << 21) - 1, 1 << 21, (1 << 24) - 1], dtype=np.uint64)  # across the lists' ends
     np.testing.assert_array_equal(out.cpu().numpy()[idx.astype(np.int64)], st.amplitudes(idx))
